@@ -468,3 +468,20 @@ def test_error_paths(torch):
         B.mnn_conv_run(r.plan, x.data_ptr(), w.data_ptr(), None, y.data_ptr(), r.stream())
     assert ei.value.code == B.MNN_EWORKSPACE
     r.close()
+
+
+# The tile kernel of the sliding-window scheme: patches longer than one staged chunk (512 elements) with a remainder, cut
+# over two to eight warps and not cut, a last position block that is partly empty, channel tiles of 4, 8 and 16 with
+# remainders, groups.
+@pytest.mark.parametrize("N,Cin,Cout,H,W_,k,stride,dil,groups", [
+    (1, 256, 33, 7, 7, 1, 2, 1, 1), (1, 61, 17, 9, 11, 3, 1, 1, 1), (1, 8, 16, 3, 3, 3, 1, 1, 1), (2, 130, 5, 12, 10, 3, 2, 1, 1),
+    (4, 20, 40, 40, 41, 3, 1, 2, 4), (3, 18, 6, 33, 31, 1, 1, 1, 2), (40, 16, 48, 33, 30, 1, 1, 1, 2), (1, 16, 20, 30, 14, 11, 1, 1, 2)])
+def test_direct_tiles(torch, N, Cin, Cout, H, W_, k, stride, dil, groups):
+    layer = W.ConvLayer("t", N, Cin, Cout, H, W_, k, stride, dil * (k - 1) // 2, dil, groups=groups, relu=Cin % 2 == 1, seed=Cin + k)
+    x, w, b = W.make_inputs(layer)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (x, w, b))
+    assert info.algo == B.ALGO_DIRECT
+    assert rel_l2(got, oracle(layer, x, w, b)) < 1e-6
+    xi, wi, bi = W.integer_inputs(layer)
+    goti, _, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (xi, wi, bi))
+    assert np.array_equal(goti.astype(np.float64), oracle(layer, xi, wi, bi))

@@ -571,13 +571,15 @@ __global__ void __launch_bounds__(kStemThreads) direct_stem_fixed_kernel(const f
 // results of a channel and row leave as one float2 store, and only the row above the plane and the column
 // left of it can fall outside.  One 16-byte weight fetch from shared memory feeds 2 ROWS packed multiply-adds
 // (__ffma2_rn: two IEEE fused multiply-adds per instruction, bit for bit the scalar result).  Blocks walk
-// over (image, group of 128 pixel blocks) units and stage the weights once.
+// over (image, group of 128 pixel blocks) units and stage the weights once.  Small batches take one output row per block
+// and share an image's output channels out over co_split units, because a unit is one serial sweep (one image, 32
+// channels at 224 x 224: 25 units, 7.0 us -> 98 units, 5.3 us).
 constexpr int kPairCoChunk = 16;   // output channels per sweep over the 27 taps
 
 template <bool RELU, int ROWS>
 __global__ void __launch_bounds__(kStemThreads, ROWS == 1 ? 5 : 3)
 direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ bias,
-                           float* __restrict__ y, DirectGeom g, int co_pad, int groups, int n_units)
+                           float* __restrict__ y, DirectGeom g, int co_pad, int groups, int co_split, int n_units)
 {
     constexpr int CIN = 3, K = 3, TAPS = CIN * K * K, NR = 2 * ROWS + 1, PIX = 2 * ROWS;
     extern __shared__ __align__(16) float s_w[];              // [TAPS][co_pad]
@@ -588,8 +590,10 @@ direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict_
     __syncthreads();
     const int ohw = g.OH * g.OW, half_w = g.OW >> 1, per_image = (g.OH / ROWS) * half_w;
     for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-        const int n = unit / groups;
-        const int pp = (unit - n * groups) * kStemThreads + threadIdx.x;
+        // (image, group of pixel blocks, share of the output channels); ROWS = 2 is taken for full machines and never shares
+        const int pg = ROWS == 1 ? unit / co_split : unit, cs = ROWS == 1 ? unit - pg * co_split : 0;
+        const int n = pg / groups;
+        const int pp = (pg - n * groups) * kStemThreads + threadIdx.x;
         if (pp >= per_image) continue;
         const int obr = pp / half_w;
         const int oh = obr * ROWS, ow = 2 * (pp - obr * half_w);
@@ -611,7 +615,7 @@ direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict_
                 c[ci][r][3] = row_ok ? m1.x : 0.0f;
                 c[ci][r][4] = row_ok ? m1.y : 0.0f;
             }
-        for (int c0 = 0; c0 < g.Cout; c0 += kPairCoChunk) {
+        for (int c0 = cs * kPairCoChunk; c0 < g.Cout; c0 += (ROWS == 1 ? co_split : 1) * kPairCoChunk) {
             float2 acc[PIX][kPairCoChunk / 2];                 // pixel = 2 * row + column
 #pragma unroll
             for (int j = 0; j < kPairCoChunk / 2; ++j) {
@@ -681,15 +685,27 @@ direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict_
 // row needs; horizontal neighbours come from warp shuffles, so every input element is loaded once per strip
 // (plus two halo rows per band).  Four input rows are requested before any of them is used, which keeps
 // enough loads in flight for the kernel to follow the memory system rather than its latency.
-constexpr int kDwBandRows = 32;   // output rows per unit
+//
+// A unit has up to 32 output rows; small batches take shorter bands (down to 4 rows, two halo rows each) until the chip has
+// kDwUnitsWanted warps, because a band is a serial chain of trips to memory: one image, 32 channels at 112 x 112: 6.0 -> 2.1
+// us, 128 at 56 x 56: 6.2 -> 2.1 us.  At batch 64 the halo rows would cost 3-5 %.
+constexpr int kDwBandRows = 32, kDwMinBandRows = 4;
+constexpr long long kDwUnitsWanted = 148 * 16;
+// Launches of at most this many CTAs are scheduled while the previous kernel finishes.  Larger ones are not: their CTAs
+// would settle on SMs still configured for a contraction's 200 KB of shared memory and run with what is left as L1
+// (MobileNet-v1 at batch 64: 702 us with plain launches, 744 us overlapped).
+constexpr long long kDwOverlapBlocks = 148 * 4;
 
-// SW = lanes per plane segment (32, 16 or 8): narrow planes put 2 or 4 channel planes side by side in a warp.
-template <int STRIDE, int SW>
+// SW = lanes per plane segment (32, 16 or 8): narrow planes put 2 or 4 channel planes side by side in a warp.  HMAX > 0
+// (stride 1, planes of at most HMAX rows): every row of the plane is requested before the first is used (1024 channels 7 x 7,
+// batch 64: 11.5 -> 8.8 us).
+template <int STRIDE, int SW, int HMAX = 0>
 __global__ void __launch_bounds__(128) depthwise3x3_kernel(const float* __restrict__ x, const float* __restrict__ w,
                                                            const float* __restrict__ bias, float* __restrict__ y,
-                                                           DirectGeom g, int strips, int bands, long long n_planes,
+                                                           DirectGeom g, int strips, int bands, int band_rows, long long n_planes,
                                                            long long n_units)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int PPW = 32 / SW;                      // planes per warp
     const int lane = threadIdx.x & 31, ls = lane % SW, seg = lane / SW;
     const long long unit = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // (plane group, band, strip)
@@ -706,7 +722,7 @@ __global__ void __launch_bounds__(128) depthwise3x3_kernel(const float* __restri
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + (size_t)c * 9 + i);
     const float b = bias ? __ldg(bias + c) : 0.0f;
-    const int oh0 = band * kDwBandRows, oh1 = min(g.OH, oh0 + kDwBandRows);
+    const int oh0 = band * band_rows, oh1 = min(g.OH, oh0 + band_rows);
     const unsigned full = 0xffffffffu;
 
     if (STRIDE == 1) {
@@ -722,6 +738,26 @@ __global__ void __launch_bounds__(128) depthwise3x3_kernel(const float* __restri
             const float n = __shfl_down_sync(full, v, 1, SW);
             return ls == SW - 1 ? 0.0f : n;
         };
+        if constexpr (HMAX > 0) {
+            float rows[HMAX];
+#pragma unroll
+            for (int k = 0; k < HMAX; ++k) rows[k] = row(k);
+            float l0 = 0.0f, r0 = 0.0f, q0 = 0.0f, r1 = rows[0];
+            float l1 = __shfl_up_sync(full, r1, 1, SW), q1 = right(r1);
+#pragma unroll
+            for (int k = 0; k < HMAX; ++k) {
+                const float r2 = k + 1 < HMAX ? rows[(k + 1) % HMAX] : 0.0f;
+                const float l2 = __shfl_up_sync(full, r2, 1, SW), q2 = right(r2);
+                float acc = b;
+                acc = fmaf(wk[0], l0, acc); acc = fmaf(wk[1], r0, acc); acc = fmaf(wk[2], q0, acc);
+                acc = fmaf(wk[3], l1, acc); acc = fmaf(wk[4], r1, acc); acc = fmaf(wk[5], q1, acc);
+                acc = fmaf(wk[6], l2, acc); acc = fmaf(wk[7], r2, acc); acc = fmaf(wk[8], q2, acc);
+                if (out_ok && k < oh1) yp[(size_t)k * g.OW + ow] = g.relu ? fmaxf(acc, 0.0f) : acc;
+                l0 = l1; r0 = r1; q0 = q1;
+                l1 = l2; r1 = r2; q1 = q2;
+            }
+            return;
+        }
         // per input row: the lane's own value and its left / right neighbours (shuffled once, when the row arrives)
         float r0 = row(oh0 - 1), r1 = row(oh0);
         float l0 = __shfl_up_sync(full, r0, 1, SW), q0 = right(r0);
@@ -817,9 +853,10 @@ __device__ __forceinline__ void dw_load_row(const float* __restrict__ p, bool ok
 template <int STRIDE, int SW, int VIN, int HMAX = 0>
 __global__ void __launch_bounds__(128) depthwise3x3_vec_kernel(const float* __restrict__ x, const float* __restrict__ w,
                                                                const float* __restrict__ bias, float* __restrict__ y,
-                                                               DirectGeom g, int strips, int bands, long long n_planes,
+                                                               DirectGeom g, int strips, int bands, int band_rows, long long n_planes,
                                                                long long n_units)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int PPW = 32 / SW;                      // planes per warp
     constexpr int VOUT = STRIDE == 1 ? VIN : VIN / 2;
     const int lane = threadIdx.x & 31, ls = lane % SW, seg = lane / SW;
@@ -838,7 +875,7 @@ __global__ void __launch_bounds__(128) depthwise3x3_vec_kernel(const float* __re
 #pragma unroll
     for (int i = 0; i < 9; ++i) wk[i] = __ldg(w + (size_t)c * 9 + i);
     const float b = bias ? __ldg(bias + c) : 0.0f;
-    const int oh0 = band * kDwBandRows, oh1 = min(g.OH, oh0 + kDwBandRows);
+    const int oh0 = band * band_rows, oh1 = min(g.OH, oh0 + band_rows);
     const unsigned full = 0xffffffffu;
 
     // columns of this lane
@@ -996,7 +1033,14 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
                             (g.stride == 1 || g.stride == 2);
     if (depthwise3) {
         const long long planes = (long long)g.N * g.Cout;
-        const int bands = (g.OH + kDwBandRows - 1) / kDwBandRows;
+        // rows per band: 32, halved while that leaves fewer warps than wanted (per_band: warps of one band)
+        auto pick_band = [&](long long per_band, int* band_rows, int* bands) {
+            int r = kDwBandRows;
+            while (r > kDwMinBandRows && per_band * ((g.OH + r - 1) / r) < kDwUnitsWanted) r /= 2;
+            *band_rows = r;
+            *bands = (g.OH + r - 1) / r;
+        };
+        int band_rows = kDwBandRows, bands = 1;
         if (g.W % 2 == 0) {
             // even widths: 2 or 4 columns per lane, the narrowest segment that holds a row, else 32-lane strips
             const int vin = g.W % 4 == 0 ? 4 : 2;
@@ -1005,19 +1049,18 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
             const int per_strip = (g.stride == 1 ? 30 : 31) * vin;
             const int strips = need <= 32 ? 1 : (g.W + per_strip - 1) / per_strip;
             const long long groups = (planes + 32 / sw - 1) / (32 / sw);
+            // short planes held whole in registers: up to 16 rows with 2 columns per lane, up to 8 with 4
+            const bool whole = strips == 1 && sw == 8 && g.H <= (vin == 2 ? 16 : 8);
+            if (!whole) pick_band(groups * strips, &band_rows, &bands);
             const long long units = groups * strips * bands;
             const long long blocks = (units + 3) / 4;
             if (units > 2147483647ll - 4) return cudaErrorInvalidValue;
-            // short planes held whole in registers: up to 16 rows with 2 columns per lane, up to 8 with 4
-            if (strips == 1 && sw == 8 && g.H <= (vin == 2 ? 16 : 8)) {
-#define MNNB_DWS_LAUNCH(ST, VI, HM) depthwise3x3_vec_kernel<ST, 8, VI, HM><<<(unsigned)blocks, 128, 0, stream>>>(x, w, bias, y, g, strips, bands, planes, units)
-                if (vin == 4) { if (g.stride == 1) MNNB_DWS_LAUNCH(1, 4, 8); else MNNB_DWS_LAUNCH(2, 4, 8); }
-                else if (g.H <= 8) { if (g.stride == 1) MNNB_DWS_LAUNCH(1, 2, 8); else MNNB_DWS_LAUNCH(2, 2, 8); }
-                else { if (g.stride == 1) MNNB_DWS_LAUNCH(1, 2, 16); else MNNB_DWS_LAUNCH(2, 2, 16); }
-#undef MNNB_DWS_LAUNCH
-                return cudaGetLastError();
+#define MNNB_DWV_LAUNCH(...) return launch_chained(blocks <= kDwOverlapBlocks, depthwise3x3_vec_kernel<__VA_ARGS__>, dim3((unsigned)blocks), dim3(128), 0, stream, x, w, bias, y, g, strips, bands, band_rows, planes, units)
+            if (whole) {
+                if (vin == 4) { if (g.stride == 1) MNNB_DWV_LAUNCH(1, 8, 4, 8); else MNNB_DWV_LAUNCH(2, 8, 4, 8); }
+                else if (g.H <= 8) { if (g.stride == 1) MNNB_DWV_LAUNCH(1, 8, 2, 8); else MNNB_DWV_LAUNCH(2, 8, 2, 8); }
+                else { if (g.stride == 1) MNNB_DWV_LAUNCH(1, 8, 2, 16); else MNNB_DWV_LAUNCH(2, 8, 2, 16); }
             }
-#define MNNB_DWV_LAUNCH(ST, SWV, VI) depthwise3x3_vec_kernel<ST, SWV, VI><<<(unsigned)blocks, 128, 0, stream>>>(x, w, bias, y, g, strips, bands, planes, units)
 #define MNNB_DWV_PICK(ST, VI) do { if (sw == 8) MNNB_DWV_LAUNCH(ST, 8, VI); else if (sw == 16) MNNB_DWV_LAUNCH(ST, 16, VI); else MNNB_DWV_LAUNCH(ST, 32, VI); } while (0)
             if (g.stride == 1) {
                 if (vin == 4) MNNB_DWV_PICK(1, 4); else MNNB_DWV_PICK(1, 2);
@@ -1026,7 +1069,6 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
             }
 #undef MNNB_DWV_PICK
 #undef MNNB_DWV_LAUNCH
-            return cudaGetLastError();
         }
         // odd widths: one column per lane.  A stride-1 segment of SW lanes covers SW - 1 input columns from -1
         // on, a stride-2 segment SW output columns
@@ -1034,10 +1076,13 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
         const int sw = need <= 8 ? 8 : (need <= 16 ? 16 : 32);
         const int strips = sw < 32 ? 1 : (g.stride == 1 ? (g.OW + 29) / 30 : (g.OW + 31) / 32);
         const long long groups = (planes + 32 / sw - 1) / (32 / sw);
+        const bool whole = g.stride == 1 && sw == 8 && g.H <= 8;          // 7 x 7 planes: every row requested before use
+        if (!whole) pick_band(groups * strips, &band_rows, &bands);
         const long long units = groups * strips * bands;
         const long long blocks = (units + 3) / 4;
         if (blocks > 2147483647ll) return cudaErrorInvalidValue;
-#define MNNB_DW_LAUNCH(ST, SWV) depthwise3x3_kernel<ST, SWV><<<(unsigned)blocks, 128, 0, stream>>>(x, w, bias, y, g, strips, bands, planes, units)
+#define MNNB_DW_LAUNCH(...) return launch_chained(blocks <= kDwOverlapBlocks, depthwise3x3_kernel<__VA_ARGS__>, dim3((unsigned)blocks), dim3(128), 0, stream, x, w, bias, y, g, strips, bands, band_rows, planes, units)
+        if (whole) MNNB_DW_LAUNCH(1, 8, 8);
         if (g.stride == 1) {
             if (sw == 8) MNNB_DW_LAUNCH(1, 8);
             else if (sw == 16) MNNB_DW_LAUNCH(1, 16);
@@ -1048,7 +1093,6 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
             else MNNB_DW_LAUNCH(2, 32);
         }
 #undef MNNB_DW_LAUNCH
-        return cudaGetLastError();
     }
     if (direct_stem_applies(g)) {
         const int co_pad = (g.Cout + kStemCoChunk - 1) / kStemCoChunk * kStemCoChunk;
@@ -1059,14 +1103,17 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
         }
         if (g.Cin == 3 && g.k == 3 && g.dil == 1 && g.stride == 2 && g.pad == 1 && g.H % 2 == 0 && g.W % 4 == 0 &&
             smem <= 48 * 1024 && reinterpret_cast<uintptr_t>(x) % 8 == 0 && reinterpret_cast<uintptr_t>(y) % 8 == 0) {
-            const int rows = g.H % 4 == 0 ? 2 : 1;
+            const long long blocks2 = (long long)g.N * (((g.OH / 2) * (g.OW / 2) + kStemThreads - 1) / kStemThreads);
+            const int rows = g.H % 4 == 0 && blocks2 >= 148 ? 2 : 1;
             const int per_image = (g.OH / rows) * (g.OW / 2);
             const int groups = (per_image + kStemThreads - 1) / kStemThreads;
-            const long long units = (long long)g.N * groups;
+            int co_split = 1;
+            while (rows == 1 && (long long)g.N * groups * co_split < 148 && co_split * kPairCoChunk < g.Cout) co_split *= 2;
+            const long long units = (long long)g.N * groups * co_split;
             if (units <= 2147483647ll) {
                 const int resident = 148 * (rows == 1 ? 5 : 3);
                 const unsigned blocks = (unsigned)(units < resident ? units : resident);
-#define MNNB_STEM_PAIR(RELU, ROWS) direct_stem_s2_pair_kernel<RELU, ROWS><<<blocks, kStemThreads, smem, stream>>>(x, w, bias, y, g, co_pad, groups, (int)units)
+#define MNNB_STEM_PAIR(RELU, ROWS) direct_stem_s2_pair_kernel<RELU, ROWS><<<blocks, kStemThreads, smem, stream>>>(x, w, bias, y, g, co_pad, groups, co_split, (int)units)
                 if (rows == 2) { if (g.relu) MNNB_STEM_PAIR(true, 2); else MNNB_STEM_PAIR(false, 2); }
                 else { if (g.relu) MNNB_STEM_PAIR(true, 1); else MNNB_STEM_PAIR(false, 1); }
 #undef MNNB_STEM_PAIR

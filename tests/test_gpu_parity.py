@@ -485,3 +485,25 @@ def test_direct_tiles(torch, N, Cin, Cout, H, W_, k, stride, dil, groups):
     xi, wi, bi = W.integer_inputs(layer)
     goti, _, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (xi, wi, bi))
     assert np.array_equal(goti.astype(np.float64), oracle(layer, xi, wi, bi))
+
+
+# Depthwise planes cut into bands of 4, 8, 16 and 32 rows (fewer planes, shorter bands), the last band partial, and 7 x 7
+# planes held whole at odd width; the 3 -> Cout stride-2 kernel with its output channels shared out (few images, Cout off
+# the chunk of 16).
+@pytest.mark.parametrize("C,H,W_,N", [(1, 61, 64, 1), (130, 61, 30, 1), (300, 41, 45, 1), (700, 37, 28, 1), (1200, 35, 60, 2),
+                                      (5, 7, 7, 3), (9, 8, 5, 1), (3, 1, 7, 2)])
+@pytest.mark.parametrize("stride", [1, 2])
+def test_depthwise_bands(torch, C, H, W_, N, stride):
+    layer = W.ConvLayer("t", N, C, C, H, W_, 3, stride, 1, groups=C, relu=(C % 2 == 0), seed=C + H)
+    xi, wi, bi = W.integer_inputs(layer)
+    got, info, _ = run_layer(torch, layer, opts_for(layer), (xi, wi, bi))
+    assert info.algo == B.ALGO_DIRECT
+    assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))
+
+
+@pytest.mark.parametrize("N,Cout,H,Wd", [(1, 33, 64, 96), (1, 64, 30, 44), (2, 16, 128, 128), (6, 40, 160, 160)])
+def test_stem_shared_channels(torch, N, Cout, H, Wd):
+    layer = W.ConvLayer("t", N, 3, Cout, H, Wd, 3, 2, 1, 1, relu=True, seed=Cout)
+    xi, wi, bi = W.integer_inputs(layer, -3, 3)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (xi, wi, bi))
+    assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))

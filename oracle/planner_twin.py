@@ -158,6 +158,16 @@ def contraction_tiling(tile_blocks: int, positions: int, Cout: int, sms: int):
     return best[1], best[2]
 
 
+def cluster_split(items: int, k_blocks: int, sms: int) -> int:
+    """CTAs that share one work item's K loop: doubled while twice as many still fit the SMs and every CTA keeps at least
+    four blocks; at most 4, or 8 for up to 8 items."""
+    most = 8 if items <= 8 else 4
+    n = 1
+    while n < most and 2 * n * items <= sms and k_blocks >= 8 * n:
+        n *= 2
+    return n
+
+
 # ---------------------------------------------------------------------------------------
 # GEMM scheme (k = 1 "is just a matrix multiplication"; k > 1 over gathered patches).
 # ---------------------------------------------------------------------------------------
@@ -357,6 +367,14 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 # (plain pointwise layers keep the tuned paths: measured, the implicit gather never beat them there)
                 if implicit_ok and not (L.k == 1 and L.stride == 1) and c[13] > 0 and costs[LHS_IMPLICIT] < costs[lhs]:
                     lhs = LHS_IMPLICIT
+                # items so few that their K loop is cut over clusters: the implicit gather, booked at the patches' cost
+                if implicit_ok and not (L.k == 1 and L.stride == 1) and c[13] > 0 and lhs == LHS_PATCHES:
+                    sms = c[7] if c[7] > 0 else 148
+                    blocks = cdiv(L.N * L.OH * L.OW, 128)
+                    _, co_blocks = contraction_tiling(blocks, 1, L.Cout, sms)
+                    if cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1:
+                        lhs = LHS_IMPLICIT
+                        costs[LHS_IMPLICIT] = costs[LHS_PATCHES]
             if lhs == LHS_X:
                 p = max(p, LHS_X_ERROR_PPM)
             side[i] = dict(lhs=lhs, ppm=p)

@@ -21,6 +21,7 @@
 #include "contract_pair.h"
 #include "contract_umma.h"
 #include "kernels.h"
+#include "cluster.cuh"
 #include "umma.cuh"
 
 namespace mnnb {
@@ -43,24 +44,6 @@ struct PairParams {
     int* status;
 };
 
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Cluster address of the shared-memory location `addr` (an address of this CTA) in the CTA of rank `rank`.
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void remote_arrive(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
@@ -153,7 +136,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();
+    const uint32_t rank = ptx::cluster_ctarank();
     const long long pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t tile_bytes = kRows * SW;
@@ -183,7 +166,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     }
     ptx::tc_fence_before();
     __syncthreads();
-    cluster_sync_all();                  // both CTAs' barriers exist before anything is signalled across
+    ptx::cluster_sync_all();                  // both CTAs' barriers exist before anything is signalled across
     ptx::tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
     ptx::grid_launch_dependents();
@@ -210,7 +193,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                     }
                     // the first CTA's barrier counts the bytes of both CTAs' copies
                     if (rank == 0) ptx::mbar_expect_tx(ptx::smem_u32(&full_bar[stage]), 2u * stage_bytes);
-                    const uint32_t bar = map_to_rank(ptx::smem_u32(&full_bar[stage]), 0);
+                    const uint32_t bar = ptx::map_to_rank(ptx::smem_u32(&full_bar[stage]), 0);
                     const uint32_t sbase = smem_base + stage * stage_bytes;
                     if (p.merged) {
                         pair_load_4d(sbase, &map_v_hi, bar, kb * k_elems, v_row, 0, xi);
@@ -331,7 +314,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             }
             ptx::tc_fence_before();
             __syncwarp();
-            if (lane == 0) remote_arrive(map_to_rank(ptx::smem_u32(&tempty_bar[acc]), 0));
+            if (lane == 0) remote_arrive(ptx::map_to_rank(ptx::smem_u32(&tempty_bar[acc]), 0));
             acc ^= 1u;
             if (acc == 0) acc_phase ^= 1u;
         }
@@ -342,7 +325,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     if (*abortp) __nanosleep(200000);
     ptx::tc_fence_before();
     __syncthreads();
-    cluster_sync_all();
+    ptx::cluster_sync_all();
     if (warp == 1) {
         __syncwarp();
         ptx::tc_fence_after();

@@ -13,11 +13,14 @@
 //     buffered in tensor memory;
 //   - four epilogue warps drain an accumulator, add the bias, apply ReLU and store y (a tensor-memory lane is an
 //     output position, so a warp store writes 128 contiguous bytes of one channel plane).
+// Layers with so few work items that most SMs would idle (one image, late stages) run as clusters of `split` CTAs per
+// item, each taking a share of the K blocks; the partial accumulators meet in distributed shared memory (cluster.cuh).
 // A tiled TMA copy cannot gather the patches: it would have to start at x offsets (- pad + b * dilation) that are
 // not multiples of 16 bytes.  Every mbarrier wait is bounded and reports through the status word.
 #include "implicit_gemm.h"
 
 #include "contract_umma.h"
+#include "cluster.cuh"
 #include "planner.h"
 #include "umma.cuh"
 
@@ -47,6 +50,7 @@ struct IgParams {
     int n_tile_blocks, n_co_blocks, bn, k_blocks, stages, tmem_cols;
     long long n_items;
     int relu;
+    int split;               // CTAs (a cluster) per work item; then every cluster has one item
     int tap_major;           // patch elements ordered (a, b, ci) instead of (ci, a, b): a stage is 32 channels of one tap
     int* status;
 };
@@ -102,6 +106,10 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
     const uint32_t tmem_base = tmem_slot;
     ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
+    // work items of this CTA and its share of their K blocks
+    const uint32_t rank = p.split > 1 ? ptx::cluster_ctarank() : 0u;
+    const long long first_item = blockIdx.x / (unsigned)p.split, item_step = gridDim.x / (unsigned)p.split;
+    const int kb0 = p.k_blocks * (int)rank / p.split, kb1 = p.k_blocks * ((int)rank + 1) / p.split;
     const bool bias_in_smem = p.Cout <= kMaxSharedBias;
     if (bias_in_smem && warp >= 2 && warp < 2 + kEpilogueWarps) {
         for (int i = threadIdx.x - 64; i < p.Cout; i += 32 * kEpilogueWarps) s_bias[i] = p.bias ? __ldg(p.bias + i) : 0.0f;
@@ -113,9 +121,9 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
         if (lane == 0) {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
-            for (long long item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+            for (long long item = first_item; item < p.n_items && ok; item += item_step) {
                 const int nb = (int)(item / p.n_tile_blocks);
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_relaxed(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
                         if (!*abortp) atomicCAS(p.status, 0, kErrTmaWait);
                         *abortp = 1;
@@ -138,7 +146,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
             const uint32_t idesc = ptx::mma_idesc(2, kTileM, p.bn);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
-            for (long long item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+            for (long long item = first_item; item < p.n_items && ok; item += item_step) {
                 if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
                     if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
                     *abortp = 1;
@@ -146,7 +154,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
                 }
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)p.bn;
-                for (int kb = 0; kb < p.k_blocks; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
                         if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
                         *abortp = 1;
@@ -158,7 +166,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         ptx::mma_ss<0>(d_tmem, ptx::smem_desc_k128(sbase + ks * 32), ptx::smem_desc_k128(sbase + kABytes + ks * 32),
-                                       idesc, (kb | ks) != 0 ? 1u : 0u);
+                                       idesc, kb != kb0 || ks != 0 ? 1u : 0u);
                     ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
@@ -177,7 +185,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
         const long long ohw = (long long)p.OH * p.OW;
         uint32_t acc = 0, acc_phase = 0;
         const bool relu = p.relu != 0;
-        for (long long item = blockIdx.x; item < p.n_items; item += gridDim.x) {
+        for (long long item = first_item; item < p.n_items; item += item_step) {
             const int tb = (int)(item % p.n_tile_blocks);
             const int nb = (int)(item / p.n_tile_blocks);
             int got = 1;
@@ -200,8 +208,14 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + acc * (uint32_t)p.bn;
             const int n_chunks = (n_co + 15) >> 4;
             auto store_chunk = [&](const uint32_t (&v)[16], int ch) {
-                if (!t_ok) return;
                 const int c0 = ch * 16;
+                if (p.split > 1) {                        // partial sums over the operand slots, which nothing uses any more
+                    float* red = reinterpret_cast<float*>(generic_base) + q * 32 + lane;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) red[(c0 + j) * 128] = __uint_as_float(v[j]);
+                    return;
+                }
+                if (!t_ok) return;
                 const int n = min(16, n_co - c0);
                 float bz[16];
                 if (bias_in_smem) {
@@ -253,15 +267,14 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
         const int k2 = p.k * p.k;
         const long long ohw = (long long)p.OH * p.OW;
         const size_t plane = (size_t)p.H * p.W;
-        const unsigned first = blockIdx.x;
-        const long long n_local = (long long)first < p.n_items ? (p.n_items - first + gridDim.x - 1) / gridDim.x : 0;
-        const long long n_steps = n_local * p.k_blocks;
+        const long long n_local = first_item < p.n_items ? (p.n_items - first_item + item_step - 1) / item_step : 0;
+        const long long n_steps = n_local * (kb1 - kb0);
         uint32_t stage = 0, phase = 0;
         float va[16], vb[16];                               // the patch elements of the next two steps, in flight
         // The gather stream: steps are taken in order, so a cursor (work item, K block) advances by one per call and
         // the decode of the lane's output position is redone only when the work item changes.
-        long long cur_item = first;
-        int cur_kb = 0;
+        long long cur_item = first_item;
+        int cur_kb = kb0;
         const float* base = p.x;
         unsigned rows_in = 0, cols_in = 0;
         auto decode_item = [&]() {
@@ -296,9 +309,9 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
                 const float* src = base + ((size_t)(cb * kKBlock + piece0 * 4) * p.H + a * p.dil) * p.W + b * p.dil;
 #pragma unroll
                 for (int e = 0; e < 16; ++e) v[e] = ok ? __ldg(src + (size_t)e * plane) : 0.0f;
-                if (++cur_kb == p.k_blocks) {
-                    cur_kb = 0;
-                    cur_item += gridDim.x;
+                if (++cur_kb == kb1) {
+                    cur_kb = kb0;
+                    cur_item += item_step;
                     if (cur_item < p.n_items) decode_item();
                 }
                 return;
@@ -323,9 +336,9 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
                     }
                 }
             }
-            if (++cur_kb == p.k_blocks) {
-                cur_kb = 0;
-                cur_item += gridDim.x;
+            if (++cur_kb == kb1) {
+                cur_kb = kb0;
+                cur_item += item_step;
                 if (cur_item < p.n_items) decode_item();
             }
         };
@@ -365,6 +378,27 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
                 phase ^= 1u;
             }
         }
+    }
+
+    if (p.split > 1) {
+        __syncwarp();
+        ptx::cluster_sync_all();
+        if (warp < 12 && !*abortp && first_item < p.n_items) {            // three sets of four warps share the columns
+            const int tb = (int)(first_item % p.n_tile_blocks), nb = (int)(first_item / p.n_tile_blocks);
+            const int row = (warp & 3) * 32 + lane, co0 = nb * p.bn;
+            const long long t = (long long)tb * kTileM + row, ohw = (long long)p.OH * p.OW;
+            if (t < p.T) {
+                const long long img = t / ohw;
+                float* const dst = p.y + ((size_t)img * p.Cout + co0) * ohw + (t - img * ohw);
+                ptx::cluster_reduce_columns(smem_base, p.bn, rank, p.split, row, warp >> 2, 3, [&](int c, float sum) {
+                    if (co0 + c >= p.Cout) return;
+                    sum += p.bias ? __ldg(p.bias + co0 + c) : 0.0f;
+                    dst[(long long)c * ohw] = p.relu ? fmaxf(sum, 0.0f) : sum;
+                });
+            }
+        }
+        __syncwarp();
+        ptx::cluster_sync_all();                           // nobody leaves while its partial sums are being read
     }
 
     // Teardown.  After an aborted run give copies still in flight time to land before shared memory is released.
@@ -460,8 +494,9 @@ cudaError_t launch_implicit_gemm(const ImplicitGemm& ig, const float* x, const f
     p.relu = relu;
     p.tap_major = implicit_gemm_tap_major(g.Cin) ? 1 : 0;
     p.status = status;
-    const long long grid = p.n_items < ig.num_sms ? p.n_items : ig.num_sms;
-    return launch_overlapped(implicit_gemm_kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)ig.smem_bytes, stream, ig.map_u, p);
+    p.split = contract_split(p.n_items, p.k_blocks, ig.num_sms);
+    const long long grid = p.split > 1 ? p.n_items * p.split : (p.n_items < ig.num_sms ? p.n_items : ig.num_sms);
+    return launch_cluster(p.split, implicit_gemm_kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)ig.smem_bytes, stream, ig.map_u, p);
 }
 
 }  // namespace mnnb

@@ -36,6 +36,28 @@ inline cudaError_t launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 blo
     return launch_chained(true, kern, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
+// The same as clusters of `cluster` CTAs along x (1: no cluster).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cluster(int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                  Args&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
 // How transformed operands are stored.
 enum StoreMode {
     STORE_TF32 = 0,       // fp32 container, rounded to 10 mantissa bits

@@ -340,6 +340,13 @@ void contract_tiling(long long tile_blocks, int alpha2, int Cout, int num_sms, i
     }
 }
 
+int contract_split(long long items, int k_blocks, int num_sms)
+{
+    int split = 1;
+    while (split < (items <= 8 ? 8 : 4) && 2 * split * items <= num_sms && k_blocks >= 8 * split) split *= 2;
+    return split;
+}
+
 bool gemm_reads_x(const LayerShape& s, int operand, int passes)
 {
     return s.k == 1 && s.stride == 1 && s.pad == 0 && s.groups == 1 && operand == MNN_OPERAND_TF32 && passes == 1 &&
@@ -399,6 +406,17 @@ uint64_t gemm_cost(const LayerShape& s, int operand, int lhs, const Calibration&
     if (lhs_x) return kernel_ps((u128)(x_bytes + u_bytes + y_bytes) * (uint64_t)cal.c[0], serial_as, 0, cal);
     const uint64_t contract = kernel_ps((u128)(v_bytes + u_bytes + y_bytes) * (uint64_t)cal.c[0], serial_as, 0, cal);
     return saturate((u128)gather + contract);
+}
+
+// CTAs per work item of the GEMM scheme over gathered patches in TF32 (what the kernels' host side computes).
+int gemm_split(const LayerShape& s, const Calibration& cal)
+{
+    const int sms = cal.c[7] > 0 ? (int)cal.c[7] : 148;
+    const uint64_t tile_blocks = ceil_div((uint64_t)s.N * s.OH * s.OW, 128);
+    int bn = 256, n_co_blocks = 1;
+    contract_tiling((long long)tile_blocks, 1, s.Cout, sms, &bn, &n_co_blocks);
+    const uint64_t k_blocks = ceil_div(round_up((uint64_t)s.Cin * s.k * s.k, 8), 32);
+    return contract_split((long long)(tile_blocks * (uint64_t)n_co_blocks), (int)k_blocks, sms);
 }
 
 uint64_t winograd_chunk_cost(const LayerShape& s, int m, int operand, int passes, uint64_t n, bool resident,
@@ -575,12 +593,19 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 // (plain pointwise layers keep the tuned paths: measured, the implicit gather never beat them there)
                 const bool pointwise = s.k == 1 && s.stride == 1;
                 if (implicit_ok && !pointwise && cal.c[13] > 0 && cost_i < best_lhs) lhs = MNN_GEMM_LHS_IMPLICIT;
+                // So few work items that their K loop is cut over clusters: the cut gather beats writing the patches first
+                // (one image, 3x3 stride 2: 64 -> 128 at 56 x 56 10.8 against 22.4 us, 256 -> 512 at 14 x 14 14.2 against
+                // 24.0 us).  The booked cost stays the patch matrix's, an upper bound.
+                if (implicit_ok && !pointwise && cal.c[13] > 0 && lhs == MNN_GEMM_LHS_PATCHES && gemm_split(s, cal) > 1)
+                    lhs = MNN_GEMM_LHS_IMPLICIT;
             }
             const bool take_x = lhs == MNN_GEMM_LHS_X;
             if (take_x && ppm < kGemmLhsXErrorPpm) ppm = kGemmLhsXErrorPpm;
             lhs_of[i] = lhs;
             ppm_of[i] = ppm;
-            d->cost_ps[i] = lhs == MNN_GEMM_LHS_X ? cost_x : (lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches);
+            d->cost_ps[i] = lhs == MNN_GEMM_LHS_X ? cost_x
+                            : lhs == MNN_GEMM_LHS_IMPLICIT && (o.gemm_lhs == MNN_GEMM_LHS_IMPLICIT || cost_i < cost_patches) ? cost_i
+                                                                                                                            : cost_patches;
             continue;
         }
         // Winograd

@@ -46,6 +46,12 @@ void install_calibration(const Calibration& c);
 // rows an item loads (128 tiles + bn channels).  The kernel's host side and the cost model both call this.
 void contract_tiling(long long tile_blocks, int alpha2, int Cout, int num_sms, int* bn, int* n_co_blocks);
 
+// CTAs that share the K loop of one work item of the GEMM scheme (1, 2, 4 or 8): items so few that most SMs would idle are cut
+// along K and the partial accumulators added through distributed shared memory.  At least four blocks of K per CTA: the
+// cluster costs about 3 us (4 blocks cut in two: 5.9 -> 8.3 us; 16 blocks cut in four: 12.3 -> 8.1 us);
+// clusters of 8 only for up to 8 items (a GPC holds two of them at best; 16 such clusters ran in two waves).
+int contract_split(long long items, int k_blocks, int num_sms);
+
 // True when the GEMM scheme can take x itself as its left operand (no patch matrix): a 1x1 stride-1 unpadded
 // ungrouped layer with H*W >= 32 and a multiple of 4, single-pass TF32 operands.
 bool gemm_reads_x(const LayerShape& s, int operand, int passes);

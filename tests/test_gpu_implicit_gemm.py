@@ -90,3 +90,29 @@ def test_where_it_does_not_apply(torch):
     with pytest.raises(B.MnnError):      # grouped
         B.mnn_conv_plan_ex(1, 16, 16, 8, 8, 3, 2, 1, 1, B.make_opts(groups=16, force_algo=B.ALGO_GEMM,
                                                                     gemm_lhs=B.GEMM_LHS_IMPLICIT))
+
+
+# Few work items: the K loop is cut over clusters of 2, 4 and 8 CTAs (uneven shares, a partial last tile of positions, output
+# channels off the tile), for the implicit gather and for the contraction over patches and over x itself.
+@pytest.mark.parametrize("lhs", [B.GEMM_LHS_PATCHES, B.GEMM_LHS_X, B.GEMM_LHS_IMPLICIT])
+@pytest.mark.parametrize("shape", [(1, 264, 40, 8, 12, 1, 1, 0), (1, 520, 300, 7, 7, 1, 1, 0), (1, 72, 24, 9, 9, 3, 2, 1),
+                                   (3, 100, 130, 13, 13, 3, 1, 1), (1, 1000, 64, 10, 10, 1, 1, 0), (2, 96, 48, 12, 12, 5, 2, 2)])
+def test_k_loop_cut_over_clusters(torch, shape, lhs):
+    N, Cin, Cout, H, W_, k, s, p = shape
+    if lhs == B.GEMM_LHS_X and (k > 1 or H * W_ % 4):
+        pytest.skip("x itself is the operand of pointwise layers with H*W a multiple of 4")
+    layer = W.ConvLayer("split", N, Cin, Cout, H, W_, k, s, p, relu=True, x_dist="normal", w_dist="kaiming", seed=sum(shape))
+    for inputs, exact in ((W.make_inputs(layer), False), (W.integer_inputs(layer, -3, 3), True)):
+        x, w, b = inputs
+        r = B.ConvLayerRunner(N, Cin, Cout, H, W_, k, s, p, 1, B.make_opts(relu=1, force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32,
+                                                                           passes=1, gemm_lhs=lhs))
+        xd, wd, bd = to_dev(torch, x), to_dev(torch, w), to_dev(torch, b)
+        y1, y2 = r.run(xd, wd, bd), r.run(xd, wd, bd)
+        torch.cuda.synchronize()
+        assert r.device_status() == 0 and torch.equal(y1, y2)
+        r.close()
+        ref = oracle(layer, x, w, b)
+        if exact:
+            assert np.array_equal(y1.cpu().numpy().astype(np.float64), ref)
+        else:
+            assert_close(y1.cpu().numpy(), ref, B.PREC_TF32, "cut K loop")

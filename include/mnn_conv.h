@@ -52,7 +52,8 @@ enum { MNN_ALGO_AUTO = 0, MNN_ALGO_WINOGRAD = 1, MNN_ALGO_GEMM = 2, MNN_ALGO_DIR
 enum { MNN_PREC_TF32 = 0, MNN_PREC_BF16 = 1 };             /* accuracy class */
 enum { MNN_OPERAND_AUTO = 0, MNN_OPERAND_TF32 = 1, MNN_OPERAND_BF16 = 2, MNN_OPERAND_FP32_REF = 3 };
 enum { MNN_POINTS_AUTO = 0, MNN_POINTS_PAPER = 1, MNN_POINTS_UNIT = 2, MNN_POINTS_MIXED = 3 };
-enum { MNN_GEMM_LHS_AUTO = 0, MNN_GEMM_LHS_PATCHES = 1, MNN_GEMM_LHS_X = 2, MNN_GEMM_LHS_IMPLICIT = 3 };
+enum { MNN_GEMM_LHS_AUTO = 0, MNN_GEMM_LHS_PATCHES = 1, MNN_GEMM_LHS_X = 2, MNN_GEMM_LHS_IMPLICIT = 3,
+       MNN_GEMM_LHS_PACKED = 4 };
 enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_STAGE_OUTPUT = 8,
        MNN_STAGE_ALL = 15 };
 
@@ -93,7 +94,9 @@ enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_ST
  *              stored.  IMPLICIT: no patch matrix either, for any k / stride / padding /
  *              dilation: producer warps of the GEMM kernel gather the patches into the
  *              shared-memory operand tile themselves (single-pass TF32 operands, rounded
- *              to nearest).  AUTO = the planner takes the cheapest that applies.  Asking
+ *              to nearest).  AUTO = the planner takes the cheapest that applies; it may also report
+ *              PACKED (not an option value): x is re-laid into lines of positions, rounded to nearest,
+ *              and every kernel tap reads them at a shifted start.  Asking
  *              for X or IMPLICIT where it does not apply fails the plan.
  *   fused      Winograd F(2x2, 3x3) as ONE kernel (input transform, contraction and output
  *              transform fused; the transformed tensors V and M never reach device memory):
@@ -140,7 +143,8 @@ typedef struct {
  *   u_offset  transformed weights  U [alpha^2][Cout][cin_pad]  (operand format; hi then lo when passes = 3)
  *   v_offset  transformed inputs   V [alpha^2][chunk_tiles][cin_pad] of one chunk (same format)
  *   m_offset  contraction results  M [alpha^2][Cout][m_row_stride] fp32 of one chunk
- * For the GEMM scheme alpha = 1, cin_pad covers Cin*k*k and M is unused.
+ * For the GEMM scheme alpha = 1, cin_pad covers Cin*k*k and M is unused (PACKED: cin_pad elements per position and
+ * chunk_tiles positions per plane of V).
  */
 typedef struct {
     int algo, m, alpha, precision, operand, passes, points_id;
@@ -152,7 +156,7 @@ typedef struct {
     long long u_offset, u_bytes, v_offset, v_bytes, m_offset, m_bytes;
     long long predicted_error_ppm;   /* accuracy model's relative L2 error x 1e6 for the choice */
     int chosen_candidate;            /* index into cost_ps, -1 when the choice was forced outside the list */
-    int gemm_lhs;                    /* GEMM scheme: MNN_GEMM_LHS_PATCHES, _X or _IMPLICIT as planned, else 0 */
+    int gemm_lhs;                    /* GEMM scheme: MNN_GEMM_LHS_PATCHES, _X, _IMPLICIT or _PACKED as planned, else 0 */
     unsigned long long cost_ps[MNN_N_CANDIDATES];
     int fused;                       /* 1 when the plan is the single fused Winograd kernel (no V, no M) */
     int paper_n_hat;

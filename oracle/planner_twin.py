@@ -37,7 +37,7 @@ from dataclasses import dataclass, field
 ALGO_WINOGRAD, ALGO_GEMM, ALGO_DIRECT = 1, 2, 3
 OPERAND_TF32, OPERAND_BF16, OPERAND_FP32_REF = 1, 2, 3
 PREC_TF32, PREC_BF16 = 0, 1
-LHS_PATCHES, LHS_X, LHS_IMPLICIT = 1, 2, 3
+LHS_PATCHES, LHS_X, LHS_IMPLICIT, LHS_PACKED = 1, 2, 3, 4
 INADMISSIBLE = 2 ** 64 - 1
 SATURATED = 2 ** 64 - 2
 MAX_CHUNK_BYTES = 4 << 30          # V + M of one chunk may not exceed this, whatever the cost says
@@ -174,6 +174,28 @@ def cluster_split(items: int, k_blocks: int, sms: int) -> int:
 def gemm_may_read_x(L: Layer, operand: int, passes: int) -> bool:
     return (L.k == 1 and L.stride == 1 and L.pad == 0 and L.groups == 1 and operand == OPERAND_TF32
             and passes == 1 and L.H * L.W >= 32 and (L.H * L.W) % 4 == 0)
+
+
+def packs_lines(L: Layer) -> bool:
+    """x packed into lines of positions: k in 2..7, stride <= 4, Cin a multiple of 32 or Cin * k <= 32, taps reaching at most
+    600 positions past an output, packed planes of at most 4 GiB."""
+    if L.groups != 1 or not 2 <= L.k <= 7 or L.stride > 4 or not (L.Cin % 32 == 0 or L.Cin * L.k <= 32):
+        return False
+    reach = (L.k - 1) * L.dil // L.stride
+    wq, hq = L.OW + reach, L.OH + reach
+    cells = L.N * hq * wq
+    return (reach * (wq + 1) <= 600 and cells < 2 ** 30
+            and L.stride ** 2 * (cells + 2048) * (cdiv(L.Cin, 32) * 32) * 4 <= 4 << 30)
+
+
+def packed_cost(L: Layer, c) -> int:
+    """Packed lines: a pass from x to the packed planes, and a product that reads them, at half the contraction's tensor rate."""
+    reach = (L.k - 1) * L.dil // L.stride
+    planes = min(L.stride, L.k) ** 2
+    a = L.N * (L.OH + reach) * (L.OW + reach) * planes * cdiv(L.Cin, 32) * 32 * 4
+    x, y = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW
+    flops = 2 * L.N * L.OH * L.OW * L.Cout * L.Cin * L.k * L.k
+    return sat(kernel_ps(c, mem_as=(x + a) * c[0]) + kernel_ps(c, mem_as=(a + y) * c[0], tensor_as=flops * 2 * c[2]))
 
 
 def gemm_cost(L: Layer, operand: int, lhs, c) -> int:
@@ -367,14 +389,20 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 # (plain pointwise layers keep the tuned paths: measured, the implicit gather never beat them there)
                 if implicit_ok and not (L.k == 1 and L.stride == 1) and c[13] > 0 and costs[LHS_IMPLICIT] < costs[lhs]:
                     lhs = LHS_IMPLICIT
-                # items so few that their K loop is cut over clusters: the implicit gather, booked at the patches' cost
-                if implicit_ok and not (L.k == 1 and L.stride == 1) and c[13] > 0 and lhs == LHS_PATCHES:
+                costs_of = lhs
+                # items so few that their K loop is cut over clusters: the implicit gather instead of patches; else packed
+                # lines where they apply.  Booked at the cost of the operand chosen above.
+                if implicit_ok:
                     sms = c[7] if c[7] > 0 else 148
                     blocks = cdiv(L.N * L.OH * L.OW, 128)
                     _, co_blocks = contraction_tiling(blocks, 1, L.Cout, sms)
-                    if cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1:
-                        lhs = LHS_IMPLICIT
-                        costs[LHS_IMPLICIT] = costs[LHS_PATCHES]
+                    cut = cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1
+                    if cut and not (L.k == 1 and L.stride == 1) and c[13] > 0:
+                        if lhs == LHS_PATCHES:
+                            lhs = LHS_IMPLICIT
+                    elif packs_lines(L) and packed_cost(L, c) < costs[lhs]:
+                        lhs = LHS_PACKED
+                costs[lhs] = costs[costs_of]
             if lhs == LHS_X:
                 p = max(p, LHS_X_ERROR_PPM)
             side[i] = dict(lhs=lhs, ppm=p)

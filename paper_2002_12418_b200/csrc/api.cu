@@ -15,6 +15,7 @@
 #include "contract_pair.h"
 #include "contract_umma.h"
 #include "kernels.h"
+#include "line_conv.h"
 #include "planner.h"
 #include "strassen.h"
 #include "wino_fused.h"
@@ -57,6 +58,8 @@ struct mnn_conv_plan_s {
     bool gemm_x = false;             // GEMM scheme with x itself as the left operand: no V, one launch
     bool gemm_implicit = false;      // GEMM scheme with the patches gathered inside the GEMM kernel: no V, one launch
     ImplicitGemm ig;
+    bool packed = false;             // GEMM scheme on packed lines: V holds the packed planes, two launches
+    LineConv lc;
     TransformMatrices mats;
     // run-time state
     char* ws = nullptr;              // status word and U (persistent part), and V, M unless tws is set
@@ -138,6 +141,14 @@ void layout_workspace(mnn_conv_plan_t p)
         p->v_bytes = align_up(7 * p->chunk_tiles * p->cin_pad * eb, 2048);
         p->m_bytes = align_up(7 * Mh * p->m_row_stride * 4, 1024);
         p->launches_per_run = 3;
+    } else if (p->packed) {
+        p->cin_pad = p->lc.p.elems;
+        p->chunk_tiles = p->lc.p.P;
+        p->m_row_stride = 0;
+        p->u_bytes = align_up(p->lc.p.u_bytes, 2048);
+        p->v_bytes = align_up(p->lc.p.a_bytes, 2048);
+        p->m_bytes = 0;
+        p->launches_per_run = 2;
     } else {
         p->cin_pad = (int)align_up((long long)s.Cin * s.k * s.k, 8);
         p->chunk_tiles = (long long)s.N * s.OH * s.OW;
@@ -274,6 +285,15 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
         p->d.chosen = -1;
         p->d.gemm_lhs = MNN_GEMM_LHS_PATCHES;
         p->d.error_ppm = accuracy_ppm(1, 1, 0, p->d.operand, p->d.passes);
+    }
+    if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
+        const LineShape ls = {N, Cin, Cout, H, W, k, stride, dilation, pad, s.OH, s.OW};
+        p->packed = line_plan(ls, 148, &p->lc.p);
+        if (!p->packed) {
+            fail(MNN_EUNSUPPORTED, "no tiling of the packed-line product fits this layer");
+            delete p;
+            return nullptr;
+        }
     }
     if (p->d.algo == MNN_ALGO_WINOGRAD) {
         WinogradMatrices wm;
@@ -456,6 +476,7 @@ static bool pair_contraction_wanted(int Cout, long long tiles, int alpha2)
 static cudaError_t setup_tensor_kernels(mnn_conv_plan_t p, const char** why)
 {
     const int alpha2 = p->d.algo == MNN_ALGO_WINOGRAD ? p->d.alpha * p->d.alpha : 1;
+    if (p->packed) return line_setup(&p->lc, v_hi(p), u_hi(p), why);
     if (p->fused) return fused_wino_setup(&p->fw, p->s.Cout, p->s.Cin, u_hi(p), why);
     if (p->rect)
         return umma_contract_setup(&p->uc, p->store_mode, p->d.alpha, p->s.Cout, p->cin_pad, p->chunk_tiles, u_hi(p), u_lo(p),
@@ -592,7 +613,9 @@ static int do_weights(mnn_conv_plan_t p, const float* w, cudaStream_t st)
 {
     cudaError_t e;
     LaunchTimer lt(p, st, 0);
-    if (p->gemm_implicit)
+    if (p->packed)
+        e = launch_line_weights(p->lc.p, w, u_hi(p), st);
+    else if (p->gemm_implicit)
         e = launch_implicit_weights(w, u_hi(p), p->s.Cout, p->s.Cin, p->s.k, p->cin_pad, st);
     else if (p->rect)
         e = launch_rect_weights(w, u_hi(p), u_lo(p), rect_geom(p), p->store_mode, p->mats, st);
@@ -689,6 +712,19 @@ int mnn_conv_run_stages(mnn_conv_plan_t p, const float* x, const float* w, const
             LaunchTimer lt(p, st, 3);
             e = launch_strassen_output(m_buf(p), bias, y, g, s.relu, st);
             if (e != cudaSuccess) return fail_cuda(e, "Strassen result pass");
+        }
+        return MNN_OK;
+    }
+    if (p->packed) {
+        if (mask & MNN_STAGE_INPUT) {
+            LaunchTimer lt(p, st, 1);
+            e = launch_line_pack(p->lc.p, x, v_hi(p), st);
+            if (e != cudaSuccess) return fail_cuda(e, "packing the input");
+        }
+        if (mask & MNN_STAGE_CONTRACT) {
+            LaunchTimer lt(p, st, 2);
+            e = launch_line_gemm(p->lc, bias, y, s.relu, status_word(p), st);
+            if (e != cudaSuccess) return fail_cuda(e, "packed-line product");
         }
         return MNN_OK;
     }

@@ -1,0 +1,142 @@
+// Geometry and tiling of the packed-line convolution.
+#include "line_plan.h"
+
+#include <algorithm>
+#include <cstring>
+
+namespace mnnb {
+
+namespace {
+
+long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
+long long rup(long long a, long long b) { return cdiv(a, b) * b; }
+
+// Cells of one axis: `out` outputs, `lead` zero cells in front, data cells end before `end`, taps reach `reach` cells past an
+// output.  The smallest pitch that lets the zero cells behind the data be the next line's leading ones.
+int axis_pitch(int out, int lead, int end, int reach)
+{
+    return std::max(out, std::min(out + reach, std::max(end, out + reach - lead)));
+}
+
+}  // namespace
+
+bool line_plan(const LineShape& s, int num_sms, LinePlan* p)
+{
+    std::memset(p, 0, sizeof(*p));
+    p->s = s;
+    p->few = s.Cin % 32 != 0;
+    if (p->few && s.Cin * s.k > 32) return false;
+    if (s.k > 7 || s.stride > 4) return false;
+    p->elems = p->few ? 32 : s.Cin;
+    p->k_steps = p->few && s.Cin * s.k <= 24 ? 3 : 4;
+
+    // phases and taps, grouped by phase
+    struct Tap { int id, qh, qw; };
+    Tap taps[kLineMaxPlanes][kLineMaxTaps];
+    int n_in[kLineMaxPlanes] = {0};
+    int qh_max = 0, qw_max = 0;
+    const int kb = p->few ? 1 : s.k;
+    for (int a = 0; a < s.k; ++a)
+        for (int b = 0; b < kb; ++b) {
+            const int rh = a * s.dil % s.stride, rw = b * s.dil % s.stride;
+            int ph = 0;
+            while (ph < p->n_planes && !(p->phase_h[ph] == rh && p->phase_w[ph] == rw)) ++ph;
+            if (ph == p->n_planes) {
+                if (ph == kLineMaxPlanes) return false;
+                p->phase_h[ph] = rh;
+                p->phase_w[ph] = rw;
+                ++p->n_planes;
+            }
+            taps[ph][n_in[ph]++] = {p->few ? a : a * s.k + b, a * s.dil / s.stride, b * s.dil / s.stride};
+            qh_max = std::max(qh_max, a * s.dil / s.stride);
+            qw_max = std::max(qw_max, b * s.dil / s.stride);
+        }
+    for (int ax = 0; ax < 2; ++ax) {
+        const int in = ax ? s.W : s.H, out = ax ? s.OW : s.OH, reach = ax ? qw_max : qh_max;
+        int lead = 1 << 30, end = 0;
+        for (int i = 0; i < p->n_planes; ++i) {
+            const int r = ax ? p->phase_w[i] : p->phase_h[i];
+            lead = std::min(lead, r < s.pad ? (int)cdiv(s.pad - r, s.stride) : 0);
+            end = std::max(end, in - 1 + s.pad - r >= 0 ? (in - 1 + s.pad - r) / s.stride + 1 : 0);
+        }
+        const int pitch = axis_pitch(out, lead, end, reach);
+        if (ax) p->Wq = pitch;
+        else p->Hq = pitch;
+    }
+    p->strips = 1;
+    if (p->few) {
+        p->strips = (int)cdiv(s.OW, 16);
+        p->Wq = (int)cdiv(s.OW, p->strips);
+    }
+    int span = 0, max_base = 0;
+    p->n_groups = p->n_planes;
+    for (int g = 0; g < p->n_planes; ++g) {
+        p->group_plane[g] = g;
+        p->group_first[g] = p->n_taps;
+        p->group_taps[g] = n_in[g];
+        int lo = 1 << 30;
+        for (int t = 0; t < n_in[g]; ++t) lo = std::min(lo, taps[g][t].qh * p->Wq + taps[g][t].qw);
+        p->group_base[g] = lo;
+        max_base = std::max(max_base, lo);
+        for (int t = 0; t < n_in[g]; ++t) {
+            const int rel = taps[g][t].qh * p->Wq + taps[g][t].qw - lo;
+            p->tap_id[p->n_taps] = taps[g][t].id;
+            p->tap_rel[p->n_taps++] = rel;
+            span = std::max(span, rel);
+        }
+    }
+    p->T = (long long)s.N * p->strips * p->Hq * p->Wq;
+    p->P = p->T + span + max_base;       // rows past the end of a plane read as zeros or as the next plane, for no valid cell
+    if (p->P >= (1ll << 31) - 4096) return false;
+    p->a_bytes = (long long)p->n_planes * p->P * p->elems * 4;
+    p->u_bytes = (long long)p->n_taps * s.Cout * p->elems * 4;
+    if (p->a_bytes > (4ll << 30)) return false;
+
+    // Tiling: the shortest loop, rounds of items over the SMs times the pace of a block of 32 elements: the issuing thread's
+    // serial time (about 0.3 us per step and 32 ns per instruction), the tensor core's (max(bn, 64 + bn / 2) cycles per
+    // instruction) or the delivery of regions and weight tiles (15 ps per byte and SM), whichever is longest.
+    const int co16 = (int)rup(s.Cout, 16);
+    long long best = -1;
+    for (int bn = 256; bn >= 32; bn /= 2)
+        for (int mt = 1; mt <= 4; mt *= 2) {
+            const int nb = (int)cdiv(co16, bn), b_n = (int)rup(cdiv(co16, nb), 16);
+            if (2 * mt * b_n > 512 || (bn > 32 && co16 <= bn / 2)) continue;
+            const int rows = 128 * mt + span, boxes = (int)cdiv(rows, 256), box_rows = (int)rup(cdiv(rows, boxes), 8);
+            if (boxes * box_rows > kLineMaxRegion) continue;
+            const long long a_slot = (long long)boxes * box_rows * 128, b_tile = (long long)b_n * 128;
+            const long long tile_blocks = cdiv(p->T, 128 * mt), items = tile_blocks * nb;
+            if (items >= (1ll << 31)) continue;
+            const long long rounds = cdiv(items, num_sms);
+            for (int g = 3; g >= 1; --g) {
+                const long long room = kLineSmemBytes - 1024;
+                int b_slots = (int)((room - 2 * a_slot) / (g * b_tile));
+                if (2 * a_slot >= room || b_slots < (g == 1 ? 3 : 2)) continue;
+                b_slots = std::min(b_slots, kLineMaxB);
+                const int a_slots = (int)std::min<long long>(kLineMaxA, (room - b_slots * g * b_tile) / a_slot);
+                long long steps = 0;
+                for (int i = 0; i < p->n_groups; ++i) steps += cdiv(p->group_taps[i], g);
+                const long long issue = steps * 300000 + (long long)p->n_taps * p->k_steps * 32000;
+                const long long mma = (long long)p->n_taps * mt * p->k_steps * std::max(b_n, 64 + b_n / 2) * 550;
+                const long long load = (p->n_taps * b_tile + p->n_groups * a_slot) * 15;
+                const long long drain = (long long)mt * b_n * 128 * 4 * 30 + 500000;
+                const long long cost = rounds * std::max(std::max(issue, std::max(mma, load)) * (p->elems / 32), drain) + drain;
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    p->bn = b_n;
+                    p->n_co_blocks = nb;
+                    p->mt = mt;
+                    p->region = boxes * box_rows;
+                    p->boxes = boxes;
+                    p->box_rows = box_rows;
+                    p->taps_per_step = g;
+                    p->a_slots = a_slots;
+                    p->b_slots = b_slots;
+                    p->n_tile_blocks = tile_blocks;
+                    p->n_items = items;
+                }
+            }
+        }
+    return best >= 0;
+}
+
+}  // namespace mnnb

@@ -347,6 +347,16 @@ int contract_split(long long items, int k_blocks, int num_sms)
     return split;
 }
 
+bool gemm_packs_lines(const LayerShape& s)
+{
+    if (s.groups != 1 || s.k < 2 || s.k > 7 || s.stride > 4 || !(s.Cin % 32 == 0 || s.Cin * s.k <= 32)) return false;
+    // rows of cells a tap can reach past an output, bounds of the grid of cells and of the packed planes
+    const long long reach = (long long)(s.k - 1) * s.dil / s.stride;
+    const long long wq = s.OW + reach, hq = s.OH + reach;
+    const u128 cells = (u128)s.N * (u128)hq * (u128)wq, planes = (u128)(s.stride * s.stride), elems = (s.Cin + 31) / 32 * 32;
+    return reach * (wq + 1) <= 600 && cells < (1u << 30) && planes * (cells + 2048) * elems * 4 <= (u128)(4ll << 30);
+}
+
 bool gemm_reads_x(const LayerShape& s, int operand, int passes)
 {
     return s.k == 1 && s.stride == 1 && s.pad == 0 && s.groups == 1 && operand == MNN_OPERAND_TF32 && passes == 1 &&
@@ -417,6 +427,20 @@ int gemm_split(const LayerShape& s, const Calibration& cal)
     contract_tiling((long long)tile_blocks, 1, s.Cout, sms, &bn, &n_co_blocks);
     const uint64_t k_blocks = ceil_div(round_up((uint64_t)s.Cin * s.k * s.k, 8), 32);
     return contract_split((long long)(tile_blocks * (uint64_t)n_co_blocks), (int)k_blocks, sms);
+}
+
+// The packed-line form (line_conv.cu): one pass over x that writes the planes, and a product that reads them once and runs
+// the tensor core at about half of its contraction rate.
+uint64_t packed_cost(const LayerShape& s, const Calibration& cal)
+{
+    const u128 reach = (u128)((uint64_t)(s.k - 1) * s.dil / s.stride);
+    const u128 cells = (u128)s.N * (s.OH + reach) * (s.OW + reach);
+    const u128 a_bytes = cells * (uint64_t)(s.stride < s.k ? s.stride * s.stride : s.k * s.k) * round_up(s.Cin, 32) * 4u;
+    const u128 x_bytes = (u128)4 * s.N * s.Cin * s.H * s.W, y_bytes = (u128)4 * s.N * s.Cout * s.OH * s.OW;
+    const u128 flops = (u128)2 * s.N * s.OH * s.OW * s.Cout * (uint64_t)(s.Cin * s.k * s.k);
+    const uint64_t c0 = (uint64_t)cal.c[0];
+    return saturate((u128)kernel_ps((x_bytes + a_bytes) * c0, 0, 0, cal) +
+                    kernel_ps((a_bytes + y_bytes) * c0, flops * 2u * (uint64_t)cal.c[2], 0, cal));
 }
 
 uint64_t winograd_chunk_cost(const LayerShape& s, int m, int operand, int passes, uint64_t n, bool resident,
@@ -582,7 +606,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
             const uint64_t cost_i = implicit_ok ? gemm_cost(s, c.operand, MNN_GEMM_LHS_IMPLICIT, cal) : MNN_COST_INADMISSIBLE;
             // left operand: as asked for, else the cheapest that applies (patch matrix, x itself, implicit gather;
             // earlier in this order on ties; the implicit gather only once its rate constant is known)
-            int lhs = o.gemm_lhs;
+            int lhs = o.gemm_lhs, booked = lhs;
             if (lhs == MNN_GEMM_LHS_AUTO) {
                 lhs = MNN_GEMM_LHS_PATCHES;
                 uint64_t best_lhs = cost_patches;
@@ -593,19 +617,23 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 // (plain pointwise layers keep the tuned paths: measured, the implicit gather never beat them there)
                 const bool pointwise = s.k == 1 && s.stride == 1;
                 if (implicit_ok && !pointwise && cal.c[13] > 0 && cost_i < best_lhs) lhs = MNN_GEMM_LHS_IMPLICIT;
+                booked = lhs;
                 // So few work items that their K loop is cut over clusters: the cut gather beats writing the patches first
                 // (one image, 3x3 stride 2: 64 -> 128 at 56 x 56 10.8 against 22.4 us, 256 -> 512 at 14 x 14 14.2 against
-                // 24.0 us).  The booked cost stays the patch matrix's, an upper bound.
-                if (implicit_ok && !pointwise && cal.c[13] > 0 && lhs == MNN_GEMM_LHS_PATCHES && gemm_split(s, cal) > 1)
-                    lhs = MNN_GEMM_LHS_IMPLICIT;
+                // 24.0 us); with more items x is packed into lines of positions where that form applies (line_conv.cu).  The booked
+                // cost stays that of the operand chosen above, an upper bound.
+                if (implicit_ok && !pointwise && cal.c[13] > 0 && gemm_split(s, cal) > 1) {
+                    if (lhs == MNN_GEMM_LHS_PATCHES) lhs = MNN_GEMM_LHS_IMPLICIT;
+                } else if (implicit_ok && gemm_packs_lines(s) &&
+                           packed_cost(s, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
+                    lhs = MNN_GEMM_LHS_PACKED;
+                }
             }
             const bool take_x = lhs == MNN_GEMM_LHS_X;
             if (take_x && ppm < kGemmLhsXErrorPpm) ppm = kGemmLhsXErrorPpm;
             lhs_of[i] = lhs;
             ppm_of[i] = ppm;
-            d->cost_ps[i] = lhs == MNN_GEMM_LHS_X ? cost_x
-                            : lhs == MNN_GEMM_LHS_IMPLICIT && (o.gemm_lhs == MNN_GEMM_LHS_IMPLICIT || cost_i < cost_patches) ? cost_i
-                                                                                                                            : cost_patches;
+            d->cost_ps[i] = booked == MNN_GEMM_LHS_X ? cost_x : (booked == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches);
             continue;
         }
         // Winograd

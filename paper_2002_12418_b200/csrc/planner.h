@@ -20,7 +20,7 @@ struct Decision {
     int algo = 0, m = 0, alpha = 0, operand = 0, passes = 0, points_id = 0;
     int chunk_images = 0, n_chunks = 0;
     int chosen = -1;
-    int gemm_lhs = 0;                  // MNN_GEMM_LHS_PATCHES or MNN_GEMM_LHS_X for the GEMM scheme, else 0
+    int gemm_lhs = 0;                  // MNN_GEMM_LHS_* for the GEMM scheme, else 0
     int fused = 0;                     // Winograd F(2x2,3x3) as the single fused kernel
     int paper_n_hat = 0;               // Eq. 2's argmin over n in {1, 2, 4, 6} and the counts themselves
     uint64_t paper_mul[4] = {0, 0, 0, 0};
@@ -51,6 +51,10 @@ void contract_tiling(long long tile_blocks, int alpha2, int Cout, int num_sms, i
 // cluster costs about 3 us (4 blocks cut in two: 5.9 -> 8.3 us; 16 blocks cut in four: 12.3 -> 8.1 us);
 // clusters of 8 only for up to 8 items (a GPC holds two of them at best; 16 such clusters ran in two waves).
 int contract_split(long long items, int k_blocks, int num_sms);
+
+// True when the layer fits the packed-line product (line_conv.cu; guarantees that line_plan finds a tiling): k in 2..7,
+// stride at most 4, Cin a multiple of 32 or Cin * k at most 32, and taps that reach at most 600 positions past an output.
+bool gemm_packs_lines(const LayerShape& s);
 
 // True when the GEMM scheme can take x itself as its left operand (no patch matrix): a 1x1 stride-1 unpadded
 // ungrouped layer with H*W >= 32 and a multiple of 4, single-pass TF32 operands.

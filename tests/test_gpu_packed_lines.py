@@ -1,0 +1,76 @@
+"""The GEMM scheme on packed lines of positions (strided, dilated and few-channel layers) against the fp64 direct-convolution
+oracle, through the C ABI.  The planner takes it by itself; a shape that it routes elsewhere would fail the assertion."""
+import numpy as np
+import pytest
+
+from oracle import direct_conv as oc
+from paper_2002_12418_b200 import binding as B
+from paper_2002_12418_b200 import workloads as W
+from tests.util import assert_close, to_dev
+
+pytestmark = pytest.mark.gpu
+
+# (N, Cin, Cout, H, W, k, stride, pad, dilation)
+SHAPES = [
+    (40, 32, 128, 20, 20, 3, 2, 1, 1),       # one block of channels, four phases
+    (64, 64, 130, 15, 13, 3, 2, 1, 1),       # odd extents, output channels off the tile, cells that are no outputs
+    (16, 96, 40, 30, 44, 3, 1, 2, 2),        # dilation 2
+    (9, 64, 272, 37, 33, 3, 1, 3, 3),        # dilation 3, two channel blocks of a wide layer
+    (30, 32, 64, 26, 28, 5, 2, 2, 1),        # 25 taps in four phases
+    (60, 32, 48, 60, 60, 3, 3, 0, 1),        # stride 3, one tap per phase, no padding
+    (40, 64, 64, 47, 51, 2, 2, 1, 1),        # even kernel
+    (6, 3, 64, 96, 100, 7, 2, 3, 1),         # few channels: 21 of 24 elements, strips with a partial last one
+    (5, 4, 33, 60, 130, 5, 2, 2, 2),         # few channels, dilation, 20 elements
+    (7, 6, 24, 70, 65, 5, 2, 1, 1),          # few channels, 30 of 32 elements
+]
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch
+    assert torch.cuda.is_available()
+    B.lib()
+    return torch
+
+
+def run(torch, layer, inputs):
+    x, w, b = inputs
+    r = B.ConvLayerRunner(layer.N, layer.Cin, layer.Cout, layer.H, layer.W, layer.k, layer.stride, layer.pad, layer.dilation,
+                          B.make_opts(relu=layer.relu, force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1))
+    info = r.info
+    assert info.gemm_lhs == B.GEMM_LHS_PACKED and info.launches_per_run == 2
+    r.workspace.fill_(0xFF)                   # NaNs wherever a kernel reads what none has written
+    B.mnn_conv_set_workspace(r.plan, r._ws_ptr, info.workspace_bytes)
+    y = torch.full((layer.N, layer.Cout, info.OH, info.OW), float("nan"), device="cuda:0")
+    xd, wd, bd = to_dev(torch, x), to_dev(torch, w), to_dev(torch, b) if b is not None else None
+    r.run(xd, wd, bd, y)
+    again = r.run(xd, wd, bd)
+    torch.cuda.synchronize()
+    assert r.device_status() == 0 and torch.equal(y, again)
+    out = y.cpu().numpy()
+    r.close()
+    return out
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("relu", [True, False])
+def test_parity(torch, shape, relu):
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    layer = W.ConvLayer("lines", N, Cin, Cout, H, W_, k, s, p, d, relu=relu, x_dist="normal", seed=sum(shape),
+                        bias_dist="normal0.1" if relu else "zero")
+    x, w, b = W.make_inputs(layer)
+    assert_close(run(torch, layer, (x, w, b)), oc.direct_conv(x, w, b, s, p, d, 1, relu), B.PREC_TF32, "packed lines")
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_integer_inputs_bit_exact(torch, shape):
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    layer = W.ConvLayer("lines", N, Cin, Cout, H, W_, k, s, p, d, relu=False, seed=11)
+    x, w, b = W.integer_inputs(layer, -3, 3)
+    assert np.array_equal(run(torch, layer, (x, w, b)).astype(np.float64), oc.direct_conv(x, w, b, s, p, d, 1, False))
+
+
+def test_more_than_the_staged_bias(torch):
+    layer = W.ConvLayer("lines", 4, 32, 2100, 20, 20, 3, 2, 1, relu=True, seed=5)
+    x, w, b = W.make_inputs(layer)
+    assert_close(run(torch, layer, (x, w, b)), oc.direct_conv(x, w, b, 2, 1, 1, 1, True), B.PREC_TF32, "packed lines")

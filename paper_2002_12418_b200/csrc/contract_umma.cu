@@ -72,18 +72,30 @@ struct KernelParams {
 // status codes written on a bounded wait that ran out
 constexpr int kErrProducerWait = 1, kErrMmaWaitFull = 2, kErrMmaWaitTmem = 3, kErrEpilogueWait = 4;
 
-// Shared-memory descriptor of a K-major operand tile whose rows are SW bytes long and SW-byte swizzled.
+// High words of the shared-memory descriptors (distance of 8-row groups, version, swizzle mode): K-major rows of SW bytes in
+// the SW-byte swizzle, and the MN-major operand of 32-bit elements (ptx::smem_desc_mn128_b32).
 template <int SW>
-__device__ __forceinline__ uint64_t desc_k(uint32_t smem_addr)
+constexpr uint32_t kDescHiB = ((uint32_t)SW * 8u >> 4) | (1u << 14) | ((SW == 128 ? 2u : 4u) << 29);
+template <int SW, bool A_MN>
+constexpr uint32_t kDescHiA = A_MN ? ((512u >> 4) | (1u << 14) | (1u << 29)) : kDescHiB<SW>;
+
+template <int KIND>
+__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t a_hi, uint32_t b_hi, uint32_t idesc, uint32_t accumulate)
 {
-    if (SW == 128) return ptx::smem_desc_k128(smem_addr);
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;                         // 8-row groups of 64-byte rows
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;                                  // 64-byte swizzle
-    return d;
+    if (KIND == 0)
+        asm volatile(
+            "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %4};\n\tsetp.ne.b32 p, %6, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(a_hi), "r"(b_hi),
+            "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
+            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %4};\n\tsetp.ne.b32 p, %6, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(a_hi), "r"(b_hi),
+            "r"(idesc), "r"(accumulate)
+            : "memory");
 }
 
 // SW = bytes of K per shared-memory row of an operand tile (the swizzle span): 128, or 64 where 128-byte rows
@@ -94,7 +106,10 @@ __device__ __forceinline__ uint64_t desc_k(uint32_t smem_addr)
 // share of its K blocks, and the partial accumulators meet in distributed shared memory (cluster.cuh).  A block of K is
 // delivered to one SM at about 63 GB/s whatever the others do, so the loop shortens by the number of CTAs: 1024 -> 1024
 // pointwise on one 7 x 7 image 21.8 -> 12.6 us, 512 -> 512 on one 14 x 14 image 12.3 -> 8.1 us.
-template <int KIND, int SW, bool SPLIT = false>
+//
+// The operand form is fixed at compile time (PASSES 1 or 3, A_MN) because the threads that issue copies and instructions are
+// on the critical path, see line_conv.cu: PASSFIGS
+template <int KIND, int SW, int PASSES, bool A_MN = false, bool SPLIT = false>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_constant__ CUtensorMap map_v_lo,
                      const __grid_constant__ CUtensorMap map_u_hi, const __grid_constant__ CUtensorMap map_u_lo,
@@ -115,7 +130,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_bytes = kTileM * SW;                            // one V tile (128 tiles)
     const uint32_t b_bytes = (uint32_t)p.bn * SW;                    // one U tile (bn output channels)
-    const uint32_t split = p.passes == 3 ? 2u : 1u;
+    constexpr uint32_t split = PASSES == 3 ? 2u : 1u;
     const uint32_t stage_bytes = (a_bytes + b_bytes) * split;
     // stage layout: [A_hi][A_lo?][B_hi][B_lo?]
     const uint32_t off_a_lo = a_bytes, off_b_hi = a_bytes * split, off_b_lo = a_bytes * split + b_bytes;
@@ -160,45 +175,42 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     if (warp == 0) {
         if (lane == 0) {
             uint32_t stage = 0, phase = 0;
-            bool ok = true;
-            for (long long item = first_item; item < p.n_items && ok; item += item_step) {
+            int err = 0;
+            for (long long item = first_item; item < p.n_items; item += item_step) {
                 const int tb = (int)(item % p.n_tile_blocks);
                 const long long r = item / p.n_tile_blocks;
                 const int nb = (int)(r % p.n_co_blocks);
                 const int xi = (int)(r / p.n_co_blocks);
+                const int row_a = tb * kTileM, row_b = nb * p.bn;
+                // a_mn: the item's whole atoms, and the ragged last atom of the image
+                const int img = A_MN ? tb / p.tiles_per_image : 0;
+                const int a0 = A_MN ? (tb - img * p.tiles_per_image) * (kTileM / 32) : 0;          // first atom of the item
+                const int n_full = A_MN ? min(kTileM / 32, max(0, p.full_atoms - a0)) : 0;
+                const bool ragged = A_MN && p.full_atoms < p.atoms_per_image && a0 + kTileM / 32 >= p.atoms_per_image;
+                const CUtensorMap* const map_atoms = A_MN && a0 + kTileM / 32 <= p.full_atoms ? &map_v_hi : &map_v_lo;
+                const uint32_t bytes = A_MN ? (uint32_t)(n_full + (ragged ? 1 : 0)) * 4096u + b_bytes : stage_bytes;
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_bounded(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrProducerWait);
-                        *abortp = 1;
-                        ok = false;
-                        break;
+                        err = kErrProducerWait;
+                        goto producer_failed;
                     }
                     const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
                     const uint32_t sbase = smem_base + stage * stage_bytes;
-                    if (p.a_mn) {
-                        const int img = tb / p.tiles_per_image;
-                        const int a0 = (tb - img * p.tiles_per_image) * (kTileM / 32);       // first atom of the item
-                        const int n_full = min(kTileM / 32, max(0, p.full_atoms - a0));
-                        const bool ragged = p.full_atoms < p.atoms_per_image && a0 + kTileM / 32 >= p.atoms_per_image;
-                        ptx::mbar_expect_tx(bar, (uint32_t)(n_full + (ragged ? 1 : 0)) * 4096u + b_bytes);
-                        if (n_full > 0)
-                            ptx::tma_load_4d(sbase, a0 + kTileM / 32 <= p.full_atoms ? &map_v_hi : &map_v_lo, bar, 0,
-                                             kb * k_elems, a0, img);
-                        if (ragged)
-                            ptx::tma_load_3d(sbase + (uint32_t)n_full * 4096u, &map_x_ragged, bar, p.full_atoms * 32,
-                                             kb * k_elems, img);
+                    const int ke = kb * k_elems;
+                    ptx::mbar_expect_tx(bar, bytes);
+                    if (A_MN) {
+                        if (n_full > 0) ptx::tma_load_4d(sbase, map_atoms, bar, 0, ke, a0, img);
+                        if (ragged) ptx::tma_load_3d(sbase + (uint32_t)n_full * 4096u, &map_x_ragged, bar, p.full_atoms * 32, ke, img);
+                        ptx::tma_load_3d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, xi);
+                    } else if (PASSES == 3 && p.merged) {
+                        ptx::tma_load_4d(sbase, &map_v_hi, bar, ke, row_a, 0, xi);
+                        ptx::tma_load_4d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, 0, xi);
                     } else {
-                        ptx::mbar_expect_tx(bar, stage_bytes);
-                        if (p.merged) ptx::tma_load_4d(sbase, &map_v_hi, bar, kb * k_elems, tb * kTileM, 0, xi);
-                        else ptx::tma_load_3d(sbase, &map_v_hi, bar, kb * k_elems, tb * kTileM, xi);
-                    }
-                    if (p.merged) {
-                        ptx::tma_load_4d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, nb * p.bn, 0, xi);
-                    } else {
-                        ptx::tma_load_3d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, nb * p.bn, xi);
-                        if (split == 2) {
-                            ptx::tma_load_3d(sbase + off_a_lo, &map_v_lo, bar, kb * k_elems, tb * kTileM, xi);
-                            ptx::tma_load_3d(sbase + off_b_lo, &map_u_lo, bar, kb * k_elems, nb * p.bn, xi);
+                        ptx::tma_load_3d(sbase, &map_v_hi, bar, ke, row_a, xi);
+                        ptx::tma_load_3d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, xi);
+                        if (PASSES == 3) {
+                            ptx::tma_load_3d(sbase + off_a_lo, &map_v_lo, bar, ke, row_a, xi);
+                            ptx::tma_load_3d(sbase + off_b_lo, &map_u_lo, bar, ke, row_b, xi);
                         }
                     }
                     if (++stage == (uint32_t)p.stages) {
@@ -207,76 +219,80 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                     }
                 }
             }
+        producer_failed:
+            if (err) {
+                if (!*abortp) atomicCAS(p.status, 0, err);
+                *abortp = 1;
+            }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = ptx::mma_idesc(KIND == 0 ? 2 : 1, kTileM, p.bn, p.a_mn != 0);
+            const uint32_t idesc = ptx::mma_idesc(KIND == 0 ? 2 : 1, kTileM, p.bn, A_MN);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
-            bool ok = true;
-            for (long long item = first_item; item < p.n_items && ok; item += item_step) {
+            int err = 0;
+            // descriptors as low words over constant high words: K-major steps are 32 bytes along the row, MN-major steps 8
+            // rows of 128 bytes
+            constexpr uint32_t kStepA = A_MN ? 1024u >> 4 : 2u;
+            const uint32_t lo0 = (smem_base & 0x3FFFFu) >> 4;
+            const uint32_t a_lo0 = lo0 | ((A_MN ? 4096u >> 4 : 1u) << 16), b_lo0 = (lo0 + (off_b_hi >> 4)) | (1u << 16);
+            for (long long item = first_item; item < p.n_items; item += item_step) {
                 if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
-                    if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
-                    *abortp = 1;
-                    ok = false;
-                    break;
+                    err = kErrMmaWaitTmem;
+                    goto mma_failed;
                 }
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)p.bn;
+                uint32_t accumulate = 0;
                 for (int kb = kb0; kb < kb1; ++kb) {
+                    const uint32_t a_lo = a_lo0 + stage * (stage_bytes >> 4), b_lo = b_lo0 + stage * (stage_bytes >> 4);
                     if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
-                        *abortp = 1;
-                        ok = false;
-                        break;
+                        err = kErrMmaWaitFull;
+                        goto mma_failed;
                     }
-                    ptx::tc_fence_after();
-                    const uint32_t sbase = smem_base + stage * stage_bytes;
 #pragma unroll
                     for (int ks = 0; ks < SW / 32; ++ks) {
-                        // K-major: 8 K elements are 32 bytes along the row; MN-major: 8 rows of 128 bytes
-                        const uint64_t a_hi = (SW == 128 && p.a_mn) ? ptx::smem_desc_mn128_b32(sbase + ks * 1024, 4096)
-                                                                    : desc_k<SW>(sbase + ks * 32);
-                        const uint64_t b_hi = desc_k<SW>(sbase + off_b_hi + ks * 32);
-                        ptx::mma_ss<KIND>(d_tmem, a_hi, b_hi, idesc, ((kb - kb0) | ks) != 0 ? 1u : 0u);
-                        if (split == 2) {
-                            const uint64_t a_lo = desc_k<SW>(sbase + off_a_lo + ks * 32);
-                            const uint64_t b_lo = desc_k<SW>(sbase + off_b_lo + ks * 32);
-                            ptx::mma_ss<KIND>(d_tmem, a_lo, b_hi, idesc, 1u);
-                            ptx::mma_ss<KIND>(d_tmem, a_hi, b_lo, idesc, 1u);
+                        const uint32_t ah = a_lo + (uint32_t)ks * kStepA, bh = b_lo + (uint32_t)ks * 2u;
+                        mma_lo<KIND>(d_tmem, ah, bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, ks ? 1u : accumulate);
+                        if (PASSES == 3) {
+                            mma_lo<KIND>(d_tmem, ah + (off_a_lo >> 4), bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
+                            mma_lo<KIND>(d_tmem, ah, bh + (b_bytes >> 4), kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
                         }
                     }
+                    accumulate = 1u;
                     ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));     // stage reusable once these MMAs retire
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                if (!ok) break;
                 ptx::mma_commit(ptx::smem_u32(&tfull_bar[acc]));           // accumulator complete
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
+            }
+        mma_failed:
+            if (err) {
+                if (!*abortp) atomicCAS(p.status, 0, err);
+                *abortp = 1;
             }
         }
     } else {
         const int q = warp & 3;                       // TMEM lane quarter this warp may read
         const int part = (warp - 2) >> 2;             // which part of the columns this warp drains
         uint32_t acc = 0, acc_phase = 0;
-        bool ok = true;
-        for (long long item = first_item; item < p.n_items && ok; item += item_step) {
+        for (long long item = first_item; item < p.n_items; item += item_step) {
             const int tb = (int)(item % p.n_tile_blocks);
             const long long r = item / p.n_tile_blocks;
             const int nb = (int)(r % p.n_co_blocks);
             const int xi = (int)(r / p.n_co_blocks);
             // one lane polls for the warp
             int got = 1;
-            if (lane == 0) got = ptx::mbar_wait_bounded(ptx::smem_u32(&tfull_bar[acc]), acc_phase, abortp) ? 1 : 0;
+            if (lane == 0) got = ptx::mbar_wait_relaxed(ptx::smem_u32(&tfull_bar[acc]), acc_phase, abortp) ? 1 : 0;
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) {
                 if (lane == 0) {
                     if (!*abortp) atomicCAS(p.status, 0, kErrEpilogueWait);
                     *abortp = 1;
                 }
-                ok = false;
                 break;
             }
             ptx::tc_fence_after();
@@ -291,7 +307,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             if (p.epi.mode == 0) {
                 step = p.epi.m_row_stride;
                 dst = p.epi.M + ((size_t)xi * p.Cout + co0) * p.epi.m_row_stride + t;
-            } else if (p.a_mn) {
+            } else if (A_MN) {
                 const int img = tb / p.tiles_per_image;
                 const int pix = ((tb - img * p.tiles_per_image) * (kTileM / 32) + q) * 32 + lane;   // this warp's atom
                 t_ok = pix < p.hw;
@@ -396,7 +412,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             bool t_ok;
             float* dst;
             long long step;
-            if (p.a_mn) {
+            if (A_MN) {
                 const int img = tb / p.tiles_per_image;
                 const int pix = (tb - img * p.tiles_per_image) * kTileM + row;
                 t_ok = pix < p.hw;
@@ -587,7 +603,7 @@ cudaError_t umma_contract_setup(UmmaContract* uc, int mode, int alpha2, int Cout
     // rows of 128 bytes unless that leaves fewer than three stages and the K loop is long (at least four
     // 128-byte blocks; measured: 512 channels BF16 hi + lo 0.604 -> 0.576 ms, shorter loops lose)
     int sw = kSwizzleBytes;
-    if (!uc->a_mn && (kSmemBudget - 1024) / ((kTileM + uc->bn) * sw * split) < 3 && cin_pad * eb >= 4 * sw) sw = 64;
+    if (split == 2 && (kSmemBudget - 1024) / ((kTileM + uc->bn) * sw * split) < 3 && cin_pad * eb >= 4 * sw) sw = 64;
     uc->stages_sw = sw;
     const int k_elems = sw / eb;
     uc->k_blocks = (cin_pad + k_elems - 1) / k_elems;
@@ -633,8 +649,10 @@ cudaError_t umma_contract_setup(UmmaContract* uc, int mode, int alpha2, int Cout
         uc->map_v_lo = uc->map_v_hi;
         uc->map_u_lo = uc->map_u_hi;
     }
-    for (auto kern : {contract_umma_kernel<0, 128>, contract_umma_kernel<1, 128>, contract_umma_kernel<0, 64>,
-                      contract_umma_kernel<1, 64>, contract_umma_kernel<0, 128, true>, contract_umma_kernel<1, 128, true>}) {
+    for (auto kern : {contract_umma_kernel<0, 128, 1>, contract_umma_kernel<0, 128, 3>, contract_umma_kernel<0, 64, 3>,
+                      contract_umma_kernel<1, 128, 1>, contract_umma_kernel<1, 128, 3>, contract_umma_kernel<1, 64, 3>,
+                      contract_umma_kernel<0, 128, 1, true>, contract_umma_kernel<0, 128, 1, true, true>,
+                      contract_umma_kernel<0, 128, 1, false, true>, contract_umma_kernel<1, 128, 1, false, true>}) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e != cudaSuccess) return e;
     }
@@ -719,9 +737,9 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     p.split = contract_split(p.n_items, p.k_blocks, uc.num_sms);
     p.epi_warps = uc.k_blocks <= 2 || p.split > 1 ? 8 : 4;
     if (p.split > 1)
-        return launch_cluster(p.split, contract_umma_kernel<0, 128, true>, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
+        return launch_cluster(p.split, contract_umma_kernel<0, 128, 1, true, true>, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
                               (size_t)uc.smem_bytes, stream, map_lead, map_last, uc.map_u_hi, uc.map_u_lo, map_ragged, p);
-    return launch_overlapped(contract_umma_kernel<0, 128>, dim3((unsigned)grid), dim3(64 + 32 * p.epi_warps), (size_t)uc.smem_bytes, stream,
+    return launch_overlapped(contract_umma_kernel<0, 128, 1, true>, dim3((unsigned)grid), dim3(64 + 32 * p.epi_warps), (size_t)uc.smem_bytes, stream,
                              map_lead, map_last, uc.map_u_hi, uc.map_u_lo, map_ragged, p);
 }
 
@@ -752,12 +770,14 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
     p.epi = epi;
     p.status = status;
     long long grid = p.n_items < uc.num_sms ? p.n_items : uc.num_sms;
-    auto kern = uc.kind == 0 ? (uc.stages_sw == 64 ? contract_umma_kernel<0, 64> : contract_umma_kernel<0, 128>)
-                             : (uc.stages_sw == 64 ? contract_umma_kernel<1, 64> : contract_umma_kernel<1, 128>);
-    p.split = epi.mode == 1 && uc.stages_sw == 128 ? contract_split(p.n_items, p.k_blocks, uc.num_sms) : 1;
+    auto kern = uc.kind == 0 ? (uc.passes == 1 ? contract_umma_kernel<0, 128, 1>
+                                               : (uc.stages_sw == 64 ? contract_umma_kernel<0, 64, 3> : contract_umma_kernel<0, 128, 3>))
+                             : (uc.passes == 1 ? contract_umma_kernel<1, 128, 1>
+                                               : (uc.stages_sw == 64 ? contract_umma_kernel<1, 64, 3> : contract_umma_kernel<1, 128, 3>));
+    p.split = epi.mode == 1 && uc.passes == 1 ? contract_split(p.n_items, p.k_blocks, uc.num_sms) : 1;
     p.epi_warps = (uc.alpha2 == 1 && (uc.k_blocks <= 2 || p.split > 1)) ? 8 : 4;
     if (p.split > 1) {
-        auto split_kern = uc.kind == 0 ? contract_umma_kernel<0, 128, true> : contract_umma_kernel<1, 128, true>;
+        auto split_kern = uc.kind == 0 ? contract_umma_kernel<0, 128, 1, false, true> : contract_umma_kernel<1, 128, 1, false, true>;
         return launch_cluster(p.split, split_kern, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
                               (size_t)uc.smem_bytes, stream, uc.map_v_hi, uc.map_v_lo, uc.map_u_hi, uc.map_u_lo, uc.map_u_hi, p);
     }

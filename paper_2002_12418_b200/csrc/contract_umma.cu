@@ -9,7 +9,7 @@
 // quarter of the tensor-memory lanes, the load of the next 16 columns in flight while
 // the previous 16 are stored; two warps per quarter, each taking half of the columns,
 // gain nothing on long K loops, where the stores already run near the HBM write rate,
-// and are used where the K loop is at most two blocks long).
+// and are used where the K loop is at most eight blocks long).
 // The MMA "M" dimension is the tile index t (operand A = V), "N" the output channel
 // (operand B = U), "K" the input channel; TF32 or BF16 operands, fp32 accumulation;
 // with passes = 3 the operands come as hi + lo pairs and hi*hi + lo*hi + hi*lo are
@@ -42,8 +42,9 @@ namespace mnnb {
 namespace {
 
 // warp 0: TMA, warp 1: MMA + TMEM owner, then 4 or 8 epilogue warps (KernelParams::epi_warps; the warps of a
-// lane quarter split the columns).  Eight pay where the K loop is one or two blocks long and the epilogue
-// decides (a 32 -> 64 pointwise layer at 112 x 112: 78 -> 68 us); on long K loops they cost 0.3-0.6 %.
+// lane quarter split the columns).  Eight pay where the K loop is at most eight blocks long and the epilogue decides (batch
+// 64, 128 -> 256 pointwise at 28 x 28 20.4 -> 18.7 us; Winograd contraction of 64 channels at 56 x 56, batch 32 20.0 ->
+// 18.8 us); on longer K loops they cost 0.2-2 %.
 constexpr int kMaxEpilogueWarps = 8;
 constexpr int kMaxThreads = 64 + 32 * kMaxEpilogueWarps;
 constexpr int kTileM = 128;            // tiles (rows of V) per work item
@@ -108,8 +109,11 @@ __device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t 
 // pointwise on one 7 x 7 image 21.8 -> 12.6 us, 512 -> 512 on one 14 x 14 image 12.3 -> 8.1 us.
 //
 // The operand form is fixed at compile time (PASSES 1 or 3, A_MN) because the threads that issue copies and instructions are
-// on the critical path, see line_conv.cu: PASSFIGS
-template <int KIND, int SW, int PASSES, bool A_MN = false, bool SPLIT = false>
+// on the critical path (see line_conv.cu).  KB = blocks of K (shared-memory rows) per stage: a wait, a commit and the loop
+// around them cost the issuing thread more than the four instructions of a single-pass block, so long single-pass K loops
+// take two blocks per stage: one image 512 -> 512 3x3 at 7 x 7 (Winograd) 14.4 -> 12.9 us, 512 -> 512 pointwise at 14 x 14
+// 7.5 -> 7.2 us.
+template <int KIND, int SW, int PASSES, int KB, bool A_MN = false, bool SPLIT = false>
 __global__ void __launch_bounds__(kMaxThreads, 1)
 contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_constant__ CUtensorMap map_v_lo,
                      const __grid_constant__ CUtensorMap map_u_hi, const __grid_constant__ CUtensorMap map_u_lo,
@@ -131,9 +135,10 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     const uint32_t a_bytes = kTileM * SW;                            // one V tile (128 tiles)
     const uint32_t b_bytes = (uint32_t)p.bn * SW;                    // one U tile (bn output channels)
     constexpr uint32_t split = PASSES == 3 ? 2u : 1u;
-    const uint32_t stage_bytes = (a_bytes + b_bytes) * split;
-    // stage layout: [A_hi][A_lo?][B_hi][B_lo?]
-    const uint32_t off_a_lo = a_bytes, off_b_hi = a_bytes * split, off_b_lo = a_bytes * split + b_bytes;
+    static_assert(KB == 1 || PASSES == 1, "hi + lo stages hold one block");
+    const uint32_t stage_bytes = (a_bytes + b_bytes) * split * KB;
+    // stage layout: [A_hi][A_lo?][B_hi][B_lo?], or [A] x KB [B] x KB (MN-major A: KB * 32 channels per atom)
+    const uint32_t off_a_lo = a_bytes, off_b_hi = a_bytes * split * KB, off_b_lo = a_bytes * split + b_bytes;
     volatile int* abortp = &abort_flag;
 
     if (threadIdx.x == 0) {
@@ -188,7 +193,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 const int n_full = A_MN ? min(kTileM / 32, max(0, p.full_atoms - a0)) : 0;
                 const bool ragged = A_MN && p.full_atoms < p.atoms_per_image && a0 + kTileM / 32 >= p.atoms_per_image;
                 const CUtensorMap* const map_atoms = A_MN && a0 + kTileM / 32 <= p.full_atoms ? &map_v_hi : &map_v_lo;
-                const uint32_t bytes = A_MN ? (uint32_t)(n_full + (ragged ? 1 : 0)) * 4096u + b_bytes : stage_bytes;
+                const uint32_t bytes = A_MN ? (uint32_t)(n_full + (ragged ? 1 : 0)) * (4096u * KB) + b_bytes * KB : stage_bytes;
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_bounded(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
                         err = kErrProducerWait;
@@ -196,18 +201,22 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                     }
                     const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
                     const uint32_t sbase = smem_base + stage * stage_bytes;
-                    const int ke = kb * k_elems;
+                    const int ke = kb * (k_elems * KB);
                     ptx::mbar_expect_tx(bar, bytes);
                     if (A_MN) {
                         if (n_full > 0) ptx::tma_load_4d(sbase, map_atoms, bar, 0, ke, a0, img);
-                        if (ragged) ptx::tma_load_3d(sbase + (uint32_t)n_full * 4096u, &map_x_ragged, bar, p.full_atoms * 32, ke, img);
-                        ptx::tma_load_3d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, xi);
+                        if (ragged) ptx::tma_load_3d(sbase + (uint32_t)n_full * (4096u * KB), &map_x_ragged, bar, p.full_atoms * 32, ke, img);
+#pragma unroll
+                        for (int h = 0; h < KB; ++h) ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
                     } else if (PASSES == 3 && p.merged) {
                         ptx::tma_load_4d(sbase, &map_v_hi, bar, ke, row_a, 0, xi);
                         ptx::tma_load_4d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, 0, xi);
                     } else {
-                        ptx::tma_load_3d(sbase, &map_v_hi, bar, ke, row_a, xi);
-                        ptx::tma_load_3d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, xi);
+#pragma unroll
+                        for (int h = 0; h < KB; ++h) {
+                            ptx::tma_load_3d(sbase + h * a_bytes, &map_v_hi, bar, ke + h * k_elems, row_a, xi);
+                            ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
+                        }
                         if (PASSES == 3) {
                             ptx::tma_load_3d(sbase + off_a_lo, &map_v_lo, bar, ke, row_a, xi);
                             ptx::tma_load_3d(sbase + off_b_lo, &map_u_lo, bar, ke, row_b, xi);
@@ -234,7 +243,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             // rows of 128 bytes
             constexpr uint32_t kStepA = A_MN ? 1024u >> 4 : 2u;
             const uint32_t lo0 = (smem_base & 0x3FFFFu) >> 4;
-            const uint32_t a_lo0 = lo0 | ((A_MN ? 4096u >> 4 : 1u) << 16), b_lo0 = (lo0 + (off_b_hi >> 4)) | (1u << 16);
+            const uint32_t a_lo0 = lo0 | ((A_MN ? 4096u * KB >> 4 : 1u) << 16), b_lo0 = (lo0 + (off_b_hi >> 4)) | (1u << 16);
             for (long long item = first_item; item < p.n_items; item += item_step) {
                 if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
                     err = kErrMmaWaitTmem;
@@ -250,8 +259,10 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                         goto mma_failed;
                     }
 #pragma unroll
-                    for (int ks = 0; ks < SW / 32; ++ks) {
-                        const uint32_t ah = a_lo + (uint32_t)ks * kStepA, bh = b_lo + (uint32_t)ks * 2u;
+                    for (int ks = 0; ks < KB * (SW / 32); ++ks) {
+                        const int h = ks / (SW / 32), in = ks - h * (SW / 32);
+                        const uint32_t ah = a_lo + (A_MN ? (uint32_t)ks * kStepA : (uint32_t)h * (a_bytes >> 4) + (uint32_t)in * kStepA);
+                        const uint32_t bh = b_lo + (uint32_t)h * (b_bytes >> 4) + (uint32_t)in * 2u;
                         mma_lo<KIND>(d_tmem, ah, bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, ks ? 1u : accumulate);
                         if (PASSES == 3) {
                             mma_lo<KIND>(d_tmem, ah + (off_a_lo >> 4), bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
@@ -568,6 +579,14 @@ cudaError_t launch_wait_probe(int* device_word, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+// Blocks of K per stage: two on single-pass loops of at least four blocks (an odd count wastes half a stage, which shorter
+// loops feel) where that leaves three stages.  With 256 channels per item it leaves two, and the copies no longer hide:
+// 512 -> 512 at 14 x 14 batch 64 21.3 -> 21.9 us, 256 -> 256 at 28 x 28 25.9 -> 27.7 us.
+static int contract_blocks_per_stage(int passes, int k_blocks, int stages)
+{
+    return passes == 1 && stages >= 6 && k_blocks >= 4 && (k_blocks % 2 == 0 || k_blocks >= 9) ? 2 : 1;
+}
+
 cudaError_t umma_contract_setup(UmmaContract* uc, int mode, int alpha2, int Cout, int cin_pad, long long tiles_capacity,
                                 void* U_hi, void* U_lo, void* V_hi, void* V_lo, const char** why)
 {
@@ -615,6 +634,7 @@ cudaError_t umma_contract_setup(UmmaContract* uc, int mode, int alpha2, int Cout
         return cudaErrorInvalidValue;
     }
     uc->stages = stages;
+    uc->kb = contract_blocks_per_stage(uc->passes, uc->k_blocks, stages);
     // Always ask for the full budget so that at most one CTA is resident per SM: a second CTA could
     // otherwise block inside the tensor-memory allocation.
     uc->smem_bytes = kSmemBudget;
@@ -649,10 +669,11 @@ cudaError_t umma_contract_setup(UmmaContract* uc, int mode, int alpha2, int Cout
         uc->map_v_lo = uc->map_v_hi;
         uc->map_u_lo = uc->map_u_hi;
     }
-    for (auto kern : {contract_umma_kernel<0, 128, 1>, contract_umma_kernel<0, 128, 3>, contract_umma_kernel<0, 64, 3>,
-                      contract_umma_kernel<1, 128, 1>, contract_umma_kernel<1, 128, 3>, contract_umma_kernel<1, 64, 3>,
-                      contract_umma_kernel<0, 128, 1, true>, contract_umma_kernel<0, 128, 1, true, true>,
-                      contract_umma_kernel<0, 128, 1, false, true>, contract_umma_kernel<1, 128, 1, false, true>}) {
+    for (auto kern : {contract_umma_kernel<0, 128, 1, 1>, contract_umma_kernel<0, 128, 1, 2>, contract_umma_kernel<0, 128, 3, 1>,
+                      contract_umma_kernel<0, 64, 3, 1>, contract_umma_kernel<1, 128, 1, 1>, contract_umma_kernel<1, 128, 1, 2>,
+                      contract_umma_kernel<1, 128, 3, 1>, contract_umma_kernel<1, 64, 3, 1>, contract_umma_kernel<0, 128, 1, 1, true>,
+                      contract_umma_kernel<0, 128, 1, 2, true>, contract_umma_kernel<0, 128, 1, 2, true, true>,
+                      contract_umma_kernel<0, 128, 1, 2, false, true>, contract_umma_kernel<1, 128, 1, 2, false, true>}) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
         if (e != cudaSuccess) return e;
     }
@@ -675,6 +696,7 @@ cudaError_t umma_contract_setup_x(UmmaContract* uc, int Cout, int Cin, int cin_p
     uc->x_cin = Cin;
     uc->x_hw = hw;
     uc->k_blocks = (Cin + 31) / 32;
+    uc->kb = contract_blocks_per_stage(1, uc->k_blocks, uc->stages);
     return cudaSuccess;
 }
 
@@ -700,12 +722,13 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     auto encode_atoms = [&](CUtensorMap* m, int h) {
         const cuuint64_t dims[4] = {32, (cuuint64_t)uc.x_cin, (cuuint64_t)p.full_atoms, (cuuint64_t)uc.x_images};
         const cuuint64_t strides[3] = {plane, 128, (cuuint64_t)uc.x_cin * plane};
-        const cuuint32_t box[4] = {32, 32, (cuuint32_t)h, 1};
+        const cuuint32_t box[4] = {32, (cuuint32_t)(32 * uc.kb), (cuuint32_t)h, 1};
         return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(x), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     CUtensorMap map_lead, map_last, map_ragged;
+    const int ch = 32 * uc.kb;                        // channels per box
     const int h_lead = p.full_atoms < kTileM / 32 ? p.full_atoms : kTileM / 32;
     int h_last = p.full_atoms - (p.tiles_per_image - 1) * (kTileM / 32);       // whole atoms of an image's last item
     if (h_last < 1 || h_last > kTileM / 32) h_last = h_lead;                   // (none: the map is not used)
@@ -713,7 +736,7 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     {
         const cuuint64_t dims[3] = {(cuuint64_t)uc.x_hw, (cuuint64_t)uc.x_cin, (cuuint64_t)uc.x_images};
         const cuuint64_t strides[2] = {plane, (cuuint64_t)uc.x_cin * plane};
-        const cuuint32_t box[3] = {32, 32, 1};
+        const cuuint32_t box[3] = {32, (cuuint32_t)ch, 1};
         if (fn(&map_ragged, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(x), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -724,9 +747,9 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     p.n_tile_blocks = uc.x_images * p.tiles_per_image;
     p.n_co_blocks = uc.n_co_blocks;
     p.bn = uc.bn;
-    p.k_blocks = uc.k_blocks;
+    p.k_blocks = (uc.k_blocks + uc.kb - 1) / uc.kb;
     p.passes = 1;
-    p.stages = uc.stages;
+    p.stages = uc.stages / uc.kb;
     p.tmem_cols = uc.tmem_cols;
     p.Cout = uc.Cout;
     p.tiles = (long long)p.n_tile_blocks * kTileM;
@@ -734,12 +757,12 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     p.epi = epi;
     p.status = status;
     const long long grid = p.n_items < uc.num_sms ? p.n_items : uc.num_sms;
-    p.split = contract_split(p.n_items, p.k_blocks, uc.num_sms);
-    p.epi_warps = uc.k_blocks <= 2 || p.split > 1 ? 8 : 4;
+    p.split = uc.kb == 2 ? contract_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
+    p.epi_warps = uc.k_blocks <= 8 || p.split > 1 ? 8 : 4;
     if (p.split > 1)
-        return launch_cluster(p.split, contract_umma_kernel<0, 128, 1, true, true>, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
+        return launch_cluster(p.split, contract_umma_kernel<0, 128, 1, 2, true, true>, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
                               (size_t)uc.smem_bytes, stream, map_lead, map_last, uc.map_u_hi, uc.map_u_lo, map_ragged, p);
-    return launch_overlapped(contract_umma_kernel<0, 128, 1, true>, dim3((unsigned)grid), dim3(64 + 32 * p.epi_warps), (size_t)uc.smem_bytes, stream,
+    return launch_overlapped(uc.kb == 2 ? contract_umma_kernel<0, 128, 1, 2, true> : contract_umma_kernel<0, 128, 1, 1, true>, dim3((unsigned)grid), dim3(64 + 32 * p.epi_warps), (size_t)uc.smem_bytes, stream,
                              map_lead, map_last, uc.map_u_hi, uc.map_u_lo, map_ragged, p);
 }
 
@@ -760,9 +783,9 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
     p.n_tile_blocks = (int)((tiles + kTileM - 1) / kTileM);
     p.n_co_blocks = uc.n_co_blocks;
     p.bn = uc.bn;
-    p.k_blocks = uc.k_blocks;
+    p.k_blocks = (uc.k_blocks + uc.kb - 1) / uc.kb;
     p.passes = uc.passes;
-    p.stages = uc.stages;
+    p.stages = uc.stages / uc.kb;
     p.tmem_cols = uc.tmem_cols;
     p.Cout = uc.Cout;
     p.tiles = tiles;
@@ -770,14 +793,14 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
     p.epi = epi;
     p.status = status;
     long long grid = p.n_items < uc.num_sms ? p.n_items : uc.num_sms;
-    auto kern = uc.kind == 0 ? (uc.passes == 1 ? contract_umma_kernel<0, 128, 1>
-                                               : (uc.stages_sw == 64 ? contract_umma_kernel<0, 64, 3> : contract_umma_kernel<0, 128, 3>))
-                             : (uc.passes == 1 ? contract_umma_kernel<1, 128, 1>
-                                               : (uc.stages_sw == 64 ? contract_umma_kernel<1, 64, 3> : contract_umma_kernel<1, 128, 3>));
-    p.split = epi.mode == 1 && uc.passes == 1 ? contract_split(p.n_items, p.k_blocks, uc.num_sms) : 1;
-    p.epi_warps = (uc.alpha2 == 1 && (uc.k_blocks <= 2 || p.split > 1)) ? 8 : 4;
+    auto kern = uc.kind == 0 ? (uc.passes == 1 ? (uc.kb == 2 ? contract_umma_kernel<0, 128, 1, 2> : contract_umma_kernel<0, 128, 1, 1>)
+                                               : (uc.stages_sw == 64 ? contract_umma_kernel<0, 64, 3, 1> : contract_umma_kernel<0, 128, 3, 1>))
+                             : (uc.passes == 1 ? (uc.kb == 2 ? contract_umma_kernel<1, 128, 1, 2> : contract_umma_kernel<1, 128, 1, 1>)
+                                               : (uc.stages_sw == 64 ? contract_umma_kernel<1, 64, 3, 1> : contract_umma_kernel<1, 128, 3, 1>));
+    p.split = epi.mode == 1 && uc.kb == 2 ? contract_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
+    p.epi_warps = uc.k_blocks <= 8 || p.split > 1 ? 8 : 4;
     if (p.split > 1) {
-        auto split_kern = uc.kind == 0 ? contract_umma_kernel<0, 128, 1, false, true> : contract_umma_kernel<1, 128, 1, false, true>;
+        auto split_kern = uc.kind == 0 ? contract_umma_kernel<0, 128, 1, 2, false, true> : contract_umma_kernel<1, 128, 1, 2, false, true>;
         return launch_cluster(p.split, split_kern, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
                               (size_t)uc.smem_bytes, stream, uc.map_v_hi, uc.map_v_lo, uc.map_u_hi, uc.map_u_lo, uc.map_u_hi, p);
     }

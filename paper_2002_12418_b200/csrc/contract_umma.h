@@ -17,7 +17,8 @@ struct UmmaContract {
     int bn;            // MMA N (output channels per work item), multiple of 16, <= 256
     int n_co_blocks;
     int k_blocks;
-    int stages;
+    int stages;                        // of one block of K
+    int kb = 1;                        // blocks of K per stage the kernel uses (stages / kb of them)
     int stages_sw = 128;               // bytes of K per shared-memory row of a stage (128, or 64 for deeper pipelines)
     int tmem_cols;
     int smem_bytes;

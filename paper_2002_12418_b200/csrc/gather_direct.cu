@@ -120,8 +120,9 @@ __global__ void __launch_bounds__(256) gather_kernel(const float* __restrict__ x
 
 // 1 x 1, stride 1, no padding: the gather is a transposition of each image from [channel][pixel] to
 // [pixel][channel] with rounding.  A CTA moves a 64 x 64 block through shared memory: 128-bit loads along
-// the pixels, 128-bit (fp32 containers) or 64-bit (bf16) stores along the channels.  Needs H * W % 4 == 0.
-template <int MODE>
+// the pixels (32-bit where H * W is not a multiple of 4: 7 x 7 planes, 1024 channels batch 64 18.6 -> 4.3 us against the
+// element-wise gather), 128-bit (fp32 containers) or 64-bit (bf16) stores along the channels.
+template <int MODE, bool VEC>
 __global__ void __launch_bounds__(256) gather_1x1_kernel(const float* __restrict__ x, void* V_hi, void* V_lo, int Cin, int hw,
                                                          int k_pad)
 {
@@ -130,7 +131,21 @@ __global__ void __launch_bounds__(256) gather_1x1_kernel(const float* __restrict
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int p0 = blockIdx.x * 64, c0 = blockIdx.y * 64, n = blockIdx.z;
     const float* xn = x + (size_t)n * Cin * hw;
-    {
+    if (!VEC) {
+        const int pl = threadIdx.x & 31, cr = threadIdx.x >> 5;            // 32 pixels x 8 channels per step
+        float v[2][8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int c = c0 + cr + 8 * i, px = p0 + pl + 32 * h;
+                v[h][i] = c < Cin && px < hw ? __ldg(xn + (size_t)c * hw + px) : 0.0f;
+            }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) tile[cr + 8 * i][pl + 32 * h] = v[h][i];
+    } else {
         const int pv = (threadIdx.x & 15) * 4, cr = threadIdx.x >> 4;      // 16 vectors of 4 pixels x 16 channels
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -984,14 +999,16 @@ cudaError_t launch_gather(const float* x, void* V_hi, void* V_lo, const GatherGe
     const long long T = (long long)g.N * g.OH * g.OW;
     if (T <= 0) return cudaSuccess;
     const int hw = g.H * g.W;
-    if (g.k == 1 && g.stride == 1 && g.pad == 0 && hw % 4 == 0 && g.N <= 65535 && (g.k_pad + 63) / 64 <= 65535) {
+    if (g.k == 1 && g.stride == 1 && g.pad == 0 && g.N <= 65535 && (g.k_pad + 63) / 64 <= 65535) {
         const dim3 grid((unsigned)((hw + 63) / 64), (unsigned)((g.k_pad + 63) / 64), (unsigned)g.N);
+        auto launch = [&](auto kern) { return launch_overlapped(kern, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad); };
+        const bool vec = hw % 4 == 0;
         switch (mode) {
-            case STORE_TF32: return launch_overlapped(gather_1x1_kernel<STORE_TF32>, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad);
-            case STORE_BF16: return launch_overlapped(gather_1x1_kernel<STORE_BF16>, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad);
-            case STORE_TF32_SPLIT: return launch_overlapped(gather_1x1_kernel<STORE_TF32_SPLIT>, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad);
-            case STORE_BF16_SPLIT: return launch_overlapped(gather_1x1_kernel<STORE_BF16_SPLIT>, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad);
-            default: return launch_overlapped(gather_1x1_kernel<STORE_FP32>, grid, dim3(256), 0, stream, x, V_hi, V_lo, g.Cin, hw, g.k_pad);
+            case STORE_TF32: return launch(vec ? gather_1x1_kernel<STORE_TF32, true> : gather_1x1_kernel<STORE_TF32, false>);
+            case STORE_BF16: return launch(vec ? gather_1x1_kernel<STORE_BF16, true> : gather_1x1_kernel<STORE_BF16, false>);
+            case STORE_TF32_SPLIT: return launch(vec ? gather_1x1_kernel<STORE_TF32_SPLIT, true> : gather_1x1_kernel<STORE_TF32_SPLIT, false>);
+            case STORE_BF16_SPLIT: return launch(vec ? gather_1x1_kernel<STORE_BF16_SPLIT, true> : gather_1x1_kernel<STORE_BF16_SPLIT, false>);
+            default: return launch(vec ? gather_1x1_kernel<STORE_FP32, true> : gather_1x1_kernel<STORE_FP32, false>);
         }
     }
     {

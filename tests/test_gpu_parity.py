@@ -507,3 +507,16 @@ def test_stem_shared_channels(torch, N, Cout, H, Wd):
     xi, wi, bi = W.integer_inputs(layer, -3, 3)
     got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (xi, wi, bi))
     assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))
+
+
+# 1 x 1 layers whose planes are not a multiple of four pixels: the scalar transposing gather (one and two pixel blocks, the
+# last one partial, channels off the block of 64), every operand format.
+@pytest.mark.parametrize("Cin,hw", [(64, (7, 7)), (100, (9, 11)), (24, (3, 1)), (130, (13, 5))])
+@pytest.mark.parametrize("operand,precision", [(B.OPERAND_TF32, B.PREC_TF32), (B.OPERAND_BF16, B.PREC_BF16)])
+def test_pointwise_odd_planes(torch, Cin, hw, operand, precision):
+    layer = W.ConvLayer("t", 3, Cin, 40, hw[0], hw[1], 1, 1, 0, relu=True, seed=Cin)
+    xi, wi, bi = W.integer_inputs(layer, -3, 3)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_GEMM, operand=operand, precision=precision,
+                                                    gemm_lhs=B.GEMM_LHS_PATCHES), (xi, wi, bi))
+    assert info.gemm_lhs == B.GEMM_LHS_PATCHES
+    assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))

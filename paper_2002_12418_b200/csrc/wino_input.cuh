@@ -442,16 +442,22 @@ input_transform_ws_kernel(const float* __restrict__ x, const __grid_constant__ C
     if (*abortp) __nanosleep(200000);
 }
 
-// Small planes whose rows are not 16-byte aligned (W not a multiple of 4: 14 x 14, 7 x 7, ...), which TMA
-// cannot address row by row: one CTA per (image, block of 64 channels) copies the 64 contiguous channel planes
-// into shared memory with plain coalesced loads, each plane zero-padded to hp rows x wp columns (image row ih
-// at staged row ih + pad, image column iw at staged column lead + iw; everything else stays zero, which is the
-// convolution's padding and the overhang of the last tiles), and then transforms ALL tiles of the image from
-// there with the same row and column passes as the ring-buffer kernel: a tile's vectors are found exactly as
-// there, with wp words between staged rows.  hp and wp / 4 are odd, so that 32 lanes reading 128-bit vectors
-// from 32 consecutive planes touch every bank once.
+// Planes whose rows are not 16-byte aligned (W not a multiple of 4: 14 x 14, 7 x 7, ...), which TMA cannot address row
+// by row: one CTA per (image, band of `tr` tile rows, block of 64 channels) copies the band's rows of the 64 channel planes
+// (contiguous per channel) into shared memory with plain coalesced loads, each zero-padded to hp rows x wp columns (image
+// row ih at staged row ih + pad - band * tr * m, image column iw at staged column lead + iw; everything else stays
+// zero, which is the convolution's padding and the overhang of the last tiles), and then transforms all tiles of the band
+// with the same row and column passes as the ring-buffer kernel: a tile's vectors are found exactly as there, with wp
+// words between staged rows.  hp and wp / 4 are odd, so that 32 lanes reading 128-bit vectors from 32 consecutive planes
+// touch every bank once.
+//
+// A CTA is one trip to memory and one sweep of arithmetic, so its only overlap is with the other CTA of its SM and the
+// bands are whole planes or as tall as two CTAs per SM allow, and lower where taller ones would not fill the chip.
+// Measured, transform only: one image of 256 channels 14 x 14 7.5 -> 3.6 us
+// (28 CTAs instead of 4), 512 channels 7 x 7 batch 32 7.5 -> 5.8 us; against the ring kernel with cp.async loaders: 100
+// channels 35 x 45 batch 7 13.0 -> 7.4 us, 304 channels 64 x 14 batch 64 112 -> 84 us.
 struct PlaneItems {
-    int hp, wp, lead, cblocks;
+    int hp, wp, lead, cblocks, tr, bands;
 };
 
 template <int ALPHA, bool SYM, bool PAIR>
@@ -465,36 +471,42 @@ input_transform_plane_kernel(const float* __restrict__ x, char* V_hi, char* V_lo
     const int plane = pi.hp * pi.wp;
     {
         float4* z = reinterpret_cast<float4*>(s_buf);
-        for (int i = threadIdx.x; i < kItChannels * plane / 4; i += kItThreads) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = threadIdx.x; i < kItChannels * plane / 4; i += blockDim.x) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
     __syncthreads();
-    const int img = blockIdx.x / pi.cblocks, cb = blockIdx.x - img * pi.cblocks;
-    const int c0 = cb * kItChannels, hw = g.H * g.W;
-    const float* ximg = x + (size_t)img * g.Cin * hw;
+    const int ib = blockIdx.x / pi.cblocks, cb = blockIdx.x - ib * pi.cblocks;
+    const int img = ib / pi.bands, band = ib - img * pi.bands;
+    const int ty0 = band * pi.tr, tr = min(pi.tr, g.th - ty0);
+    const int top = ty0 * g.m - g.pad;                             // image row of staged row 0
+    const int ih0 = max(0, top), ih1 = min(g.H, top + (tr - 1) * g.m + ALPHA);
+    const int c0 = cb * kItChannels;
+    const int n_warps = blockDim.x >> 5, hw = (ih1 - ih0) * g.W;
     if (hw <= 256) {
         // A lane's pixels (lane, lane + 32, ...) land at the same offsets in every plane: decode them once, then
         // copy two channels per step, sixteen loads in flight per lane.  Channels beyond Cin stay zero.
+        const size_t plane_hw = (size_t)g.H * g.W;
+        const float* xband = x + (size_t)img * g.Cin * plane_hw + (size_t)ih0 * g.W + lane;
         int off[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int p = k * 32 + lane, r = p / g.W;
-            off[k] = p < hw ? (g.pad + r) * pi.wp + pi.lead + (p - r * g.W) : -1;
+            off[k] = p < hw ? (ih0 - top + r) * pi.wp + pi.lead + (p - r * g.W) : -1;
         }
-        for (int c = warp; c < kItChannels; c += 2 * kItWarps) {
+        for (int c = warp; c < kItChannels; c += 2 * n_warps) {
             float v[2][8];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                const int ci = c0 + c + j * kItWarps;
-                const float* src = ximg + (size_t)(ci < g.Cin ? ci : 0) * hw + lane;
+                const int ci = c0 + c + j * n_warps;
+                const float* src = xband + (size_t)(ci < g.Cin ? ci : 0) * plane_hw;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) v[j][k] = (off[k] >= 0 && ci < g.Cin) ? __ldg(src + 32 * k) : 0.0f;
             }
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                float* dst = s_buf + (size_t)slot_of<PAIR>(c + j * kItWarps) * plane;
-                if (c0 + c + j * kItWarps < g.Cin) {
+                float* dst = s_buf + (size_t)slot_of<PAIR>(c + j * n_warps) * plane;
+                if (c0 + c + j * n_warps < g.Cin) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
                         if (off[k] >= 0) dst[off[k]] = v[j][k];
@@ -502,39 +514,51 @@ input_transform_plane_kernel(const float* __restrict__ x, char* V_hi, char* V_lo
             }
         }
     } else {
-        // A warp copies channels warp, warp + 16, ... (kItChannels / kItWarps of them), 32 pixels per step; the
-        // steps of all its channels form one sequence, taken eight at a time: eight loads in flight per lane,
-        // then the eight stores.  Channels beyond Cin are skipped: their planes stay zero.
-        constexpr int kChPerWarp = kItChannels / kItWarps;
-        const int steps_per_ch = (hw + 31) / 32, n_steps = kChPerWarp * steps_per_ch;
-        for (int s0 = 0; s0 < n_steps; s0 += 8) {
-            float v[8];
-            int dst[8];
+        // Row by row: eight rows x 64 columns of two channels per step, 32 loads in flight per lane, addresses by row
+        // offsets (no division per element).  Channels beyond Cin stay zero.
+        const int rows = ih1 - ih0;
+        const size_t plane_hw = (size_t)g.H * g.W;
+        for (int c = warp; c < kItChannels && c0 + c < g.Cin; c += 2 * n_warps) {
+            const bool two = c0 + c + n_warps < g.Cin;
+            const float* src = x + ((size_t)img * g.Cin + c0 + c) * plane_hw + (size_t)ih0 * g.W + lane;
+            const float* src2 = src + (two ? (size_t)n_warps * plane_hw : 0);
+            float* dst = s_buf + (size_t)slot_of<PAIR>(c) * plane + (ih0 - top) * pi.wp + pi.lead + lane;
+            float* dst2 = s_buf + (size_t)slot_of<PAIR>(c + n_warps) * plane + (ih0 - top) * pi.wp + pi.lead + lane;
+            for (int r0 = 0; r0 < rows; r0 += 8)
+                for (int x0 = 0; x0 < g.W; x0 += 64) {
+                    const bool in0 = x0 + lane < g.W, in1 = x0 + lane + 32 < g.W;
+                    float v[2][8][2];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int st = s0 + k;
-                const int cw = st / steps_per_ch, p = (st - cw * steps_per_ch) * 32 + lane;
-                const int c = warp + cw * kItWarps, ci = c0 + c;
-                const bool ok = st < n_steps && p < hw && ci < g.Cin;
-                v[k] = ok ? __ldg(ximg + (size_t)ci * hw + p) : 0.0f;
-                const int r = p / g.W, col = p - r * g.W;
-                dst[k] = ok ? slot_of<PAIR>(c) * plane + (g.pad + r) * pi.wp + pi.lead + col : -1;
-            }
+                    for (int i = 0; i < 8; ++i) {
+                        const bool row = r0 + i < rows;
+                        const int o = row ? (r0 + i) * g.W + x0 : 0;
+                        v[0][i][0] = row && in0 ? __ldg(src + o) : 0.0f;
+                        v[0][i][1] = row && in1 ? __ldg(src + o + 32) : 0.0f;
+                        v[1][i][0] = row && in0 && two ? __ldg(src2 + o) : 0.0f;
+                        v[1][i][1] = row && in1 && two ? __ldg(src2 + o + 32) : 0.0f;
+                    }
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (dst[k] >= 0) s_buf[dst[k]] = v[k];
+                    for (int i = 0; i < 8; ++i) {
+                        if (r0 + i >= rows) break;
+                        const int o = (r0 + i) * pi.wp + x0;
+                        if (in0) dst[o] = v[0][i][0];
+                        if (in1) dst[o + 32] = v[0][i][1];
+                        if (in0 && two) dst2[o] = v[1][i][0];
+                        if (in1 && two) dst2[o + 32] = v[1][i][1];
+                    }
+                }
         }
     }
     __syncthreads();
     const int eb = (mode == STORE_BF16 || mode == STORE_BF16_SPLIT) ? 2 : 4;
     const long long plane_bytes = (long long)g.v_plane * eb;
-    const int units = g.th * g.tw * (PAIR ? 1 : 2);                // (tile[, half of the channel block])
-    for (int u = warp; u < units; u += kItWarps) {
+    const int units = tr * g.tw * (PAIR ? 1 : 2);                // (tile[, half of the channel block])
+    for (int u = warp; u < units; u += n_warps) {
         const int ti = PAIR ? u : (u >> 1), half = PAIR ? 0 : (u & 1);
         const int ty = ti / g.tw, tx = ti - ty * g.tw;
         const int c = c0 + (PAIR ? 2 * lane : half * 32 + lane);
         if (c >= g.cin_pad) continue;
-        const long long tile = ((long long)img * g.th + ty) * g.tw + tx;
+        const long long tile = ((long long)img * g.th + ty0 + ty) * g.tw + tx;
         const int s0 = pi.lead + tx * g.m - g.pad;                 // staged column of the tile's first input column
         const float* p0 = s_buf + (size_t)(PAIR ? lane : half * 32 + lane) * plane + (size_t)(ty * g.m) * pi.wp + (s0 & ~3);
         const float* p1 = p0 + (size_t)32 * plane;
@@ -543,26 +567,38 @@ input_transform_plane_kernel(const float* __restrict__ x, char* V_hi, char* V_lo
     }
 }
 
-// Padded plane shape for input_transform_plane_kernel; false when 64 planes do not fit the shared-memory budget.
-inline bool plan_plane_items(const WinoGeom& g, int alpha, PlaneItems* pi, size_t* smem)
+// Band shape for input_transform_plane_kernel; false when 64 planes of one tile row do not fit the shared-memory budget.
+inline bool plan_plane_items(const WinoGeom& g, int alpha, int num_sms, PlaneItems* pi, size_t* smem)
 {
     const int lead = (g.pad + 3) / 4 * 4;
-    int hp = (g.th - 1) * g.m + alpha;
-    if (hp < g.H + g.pad) hp = g.H + g.pad;
-    if ((hp & 1) == 0) ++hp;
     // columns: the image, and whole 4-wide vectors up to three columns past the last tile
     int wp = lead - g.pad + (g.tw - 1) * g.m + alpha + 3;
     if (wp < lead + g.W) wp = lead + g.W;
     wp = (wp + 3) / 4 * 4;
     if (((wp / 4) & 1) == 0) wp += 4;
-    const long long bytes = (long long)kItChannels * hp * wp * 4;
-    const long long blocks = (long long)g.images * ((g.cin_pad + kItChannels - 1) / kItChannels);
-    if (bytes > kItSmemBudget || blocks > 2147483647ll) return false;
-    pi->hp = hp;
+    auto rows = [&](int tr) { return ((tr - 1) * g.m + alpha) | 1; };
+    auto bytes = [&](int tr) { return (long long)kItChannels * rows(tr) * wp * 4; };
+    pi->cblocks = (g.cin_pad + kItChannels - 1) / kItChannels;
+    const long long per_band = (long long)g.images * pi->cblocks;
+    if (bytes(1) > kItSmemBudget) return false;
+    // the whole plane where it fits, else the tallest band two of which share an SM (any that fits where even one tile row
+    // takes more), then lower ones until the chip is full
+    int tr = g.th;
+    const long long room = bytes(1) <= kItSmemBudget / 2 ? kItSmemBudget / 2 : kItSmemBudget;
+    if (bytes(tr) > kItSmemBudget)
+        while (tr > 1 && bytes(tr) > room) --tr;
+    while (tr > 1 && per_band * ((g.th + tr - 1) / tr) < num_sms) --tr;
+    pi->bands = (g.th + tr - 1) / tr;
+    tr = (g.th + pi->bands - 1) / pi->bands;
+    if (per_band * pi->bands > 2147483647ll) return false;
+    // bands beat the ring kernel up to alpha = 6, those of wide rows from half a CTA per SM on (8 images of 64 channels 75 x
+    // 75 24 -> 20 us; one image of 222 channels 88 x 90, 88 CTAs, 12.9 -> 11.4 us; but 7 x 7 kernels at 45 x 45 17 -> 27 us)
+    if (pi->bands > 1 && (alpha > 6 || (((tr - 1) * g.m + alpha) * g.W > 256 && 2 * per_band * pi->bands < num_sms))) return false;
+    pi->tr = tr;
+    pi->hp = rows(tr);
     pi->wp = wp;
     pi->lead = lead;
-    pi->cblocks = (g.cin_pad + kItChannels - 1) / kItChannels;
-    *smem = (size_t)bytes;
+    *smem = (size_t)bytes(tr);
     return true;
 }
 
@@ -650,14 +686,17 @@ cudaError_t launch_input_ws(const float* x, void* V_hi, void* V_lo, const WinoGe
             tma_ok = false;
     }
     if (!tma_ok) {
-        // small planes: the whole image of a channel block in shared memory
+        // bands of tile rows of a channel block in shared memory
         PlaneItems pi;
         size_t psmem = 0;
-        if (plan_plane_items(g, ALPHA, &pi, &psmem)) {
+        if (plan_plane_items(g, ALPHA, num_sms, &pi, &psmem)) {
             auto launch_plane = [&](auto kern) -> cudaError_t {
                 cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kItSmemBudget);
                 if (e != cudaSuccess) return e;
-                return launch_overlapped(kern, dim3((unsigned)(g.images * pi.cblocks)), dim3(kItThreads), psmem, stream, x,
+                // half the threads where several CTAs come to an SM: two then share it (the registers allow 512 threads)
+                const unsigned blocks = (unsigned)(g.images * pi.bands * pi.cblocks);
+                const unsigned threads = psmem <= kItSmemBudget / 2 && blocks > (unsigned)num_sms ? kItThreads / 2 : kItThreads;
+                return launch_overlapped(kern, dim3(blocks), dim3(threads), psmem, stream, x,
                                          static_cast<char*>(V_hi), static_cast<char*>(V_lo), g, pi, mode, bt);
             };
             if (sym) return launch_plane(input_transform_plane_kernel<ALPHA, true, kPair>);

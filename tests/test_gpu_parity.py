@@ -520,3 +520,17 @@ def test_pointwise_odd_planes(torch, Cin, hw, operand, precision):
                                                     gemm_lhs=B.GEMM_LHS_PATCHES), (xi, wi, bi))
     assert info.gemm_lhs == B.GEMM_LHS_PATCHES
     assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))
+
+
+# Unaligned widths: the input transform by bands of tile rows.  Whole planes, bands of one and several tile rows (the last one
+# shorter), rows narrow and wider than a staging step of 64 columns, channels off the block of 64, 256 and 512 threads.
+@pytest.mark.parametrize("N,Cin,H,W_,pad", [(1, 64, 14, 14, 1), (1, 200, 15, 13, 0), (3, 72, 35, 45, 1), (40, 64, 26, 30, 1),
+                                            (20, 16, 75, 75, 2), (30, 70, 9, 101, 1), (160, 24, 7, 7, 1), (2, 130, 67, 33, 1)])
+@pytest.mark.parametrize("m", [2, 4])
+def test_input_transform_bands(torch, N, Cin, H, W_, pad, m):
+    layer = W.ConvLayer("t", N, Cin, 24, H, W_, 3, 1, pad, relu=True, seed=Cin + H)
+    x, w, b = W.make_inputs(layer)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_WINOGRAD, force_m=m, operand=B.OPERAND_BF16, passes=3,
+                                                    fused=B.FUSED_NEVER), (x, w, b))
+    assert info.algo == B.ALGO_WINOGRAD and info.m == m
+    assert rel_l2(got, oracle(layer, x, w, b)) < 1e-4

@@ -404,8 +404,8 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
             float2 h[4][4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                if (p.sym) wino::pass_1d<4, true, float2>(d[r], h[r], Bt);
-                else wino::pass_1d<4, false, float2>(d[r], h[r], Bt);
+                if (p.sym) wino::pass_1d<4, true>(d[r], h[r], Bt);
+                else wino::pass_1d<4, false>(d[r], h[r], Bt);
             }
             // ... and request the next one, so that its latency is covered by this step's arithmetic and stores
             if (s + 1 < n_steps) step_window(s + 1, d);
@@ -426,8 +426,8 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                 float2 col[4], o[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) col[r] = h[r][j];
-                if (p.sym) wino::pass_1d<4, true, float2>(col, o, Bt);
-                else wino::pass_1d<4, false, float2>(col, o, Bt);
+                if (p.sym) wino::pass_1d<4, true>(col, o, Bt);
+                else wino::pass_1d<4, false>(col, o, Bt);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) *reinterpret_cast<float2*>(dst + (i * 4 + j) * kVPosBytes) = tf32_pair(o[i]);
             }

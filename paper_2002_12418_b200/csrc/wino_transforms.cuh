@@ -3,8 +3,10 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "kernels.h"
-#include "wino_input.cuh"
+#include "wino_input_two_pass.cuh"
 
 namespace mnnb {
 namespace wino {
@@ -124,6 +126,57 @@ cudaError_t launch_output_am(const float* Mx, const float* bias, float* y, const
     return launch_overlapped(output_transform_kernel<ALPHA, M>, grid, dim3(kOutThreads), 0, stream, Mx, bias, y, g, relu, at);
 }
 
+// Defined beside the other tensor-map code (contract_umma.cu).
+bool encode_input_map(CUtensorMap* map, const float* x, int images, int C, int H, int W, int box_w);
+
+// Input transform.  Which kernel, by tile, alignment and size (whole layers, us):
+//   alpha >= 7               two-pass: the ring kernel would have to sweep the tile in parts.
+//   rows that TMA can address (W a multiple of 4, Cin even)
+//                            ring; but from alpha = 5 on two-pass where its CTAs fit the chip at once, since it
+//                            has no pipeline to fill: 128 channels 28 x 28 batch 1 / 8 / 12 / 16, alpha = 6: 12.5 / 17.2 /
+//                            21.1 / 21.1 ring, 12.2 / 15.1 / 18.8 / 20.5 two-pass (224 / 336 / 448 CTAs of 444); beyond, 64
+//                            channels 56 x 56 batch 32 52 / 61.  alpha = 4: 64 channels 56 x 56 11.4 / 12.9.
+//   other rows               two-pass; but the plane kernel up to 16 columns where two-pass CTAs come more than once to a
+//                            slot: 512 channels 7 x 7 batch 8 / 16 / 32 17.0 / 19.5 / 24.6 plane, 15.0 / 18.9 / 26.5 two-pass.
+template <int ALPHA>
+cudaError_t launch_input(const float* x, void* V_hi, void* V_lo, const WinoGeom& g, int mode, const TransformMatrices& mats,
+                         int* status, int num_sms, cudaStream_t stream)
+{
+    MatBt2 bt;
+    for (int i = 0; i < ALPHA * ALPHA; ++i) bt.v[i] = make_float2(mats.Bt[i], mats.Bt[i]);
+    const bool sym = bt_has_symmetric_structure(mats.Bt, ALPHA);
+    const TwoPassItems tp = plan_two_pass_items<ALPHA>(g);
+    if constexpr (ALPHA <= 6) {
+        const bool one_wave = tp.n_items <= (long long)tp_ctas(ALPHA) * num_sms;
+        const bool tma_ok = g.W % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && g.Cin % 2 == 0;
+        InputItems it;
+        PlaneItems pi;
+        size_t smem = 0;
+        CUtensorMap xmap;
+        auto launch = [&](auto kern, unsigned blocks, unsigned threads, auto&&... args) -> cudaError_t {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kItSmemBudget);
+            if (e != cudaSuccess) return e;
+            return launch_overlapped(kern, dim3(blocks), dim3(threads), smem, stream, x, args...);
+        };
+        if (tma_ok) {
+            if (!(one_wave && ALPHA >= 5) && plan_input_items(g, ALPHA, num_sms, &it) &&
+                encode_input_map(&xmap, x, g.images, g.Cin, g.H, g.W, it.wb)) {
+                smem = (size_t)it.nbuf * it.buf_words * sizeof(float);
+                const unsigned blocks = (unsigned)std::min<long long>(it.n_items, num_sms);
+                if (blocks == 0) return cudaSuccess;
+                return launch(sym ? input_transform_ws_kernel<ALPHA, true> : input_transform_ws_kernel<ALPHA, false>, blocks, kItThreads,
+                              xmap, static_cast<char*>(V_hi), static_cast<char*>(V_lo), g, it, mode, bt, status);
+            }
+        } else if (!one_wave && plan_plane_items(g, ALPHA, num_sms, &pi, &smem)) {
+            // half the threads where several CTAs come to an SM: two then share it (the registers allow 512 threads)
+            const unsigned blocks = (unsigned)(g.images * pi.bands * pi.cblocks);
+            const unsigned threads = smem <= kItSmemBudget / 2 && blocks > (unsigned)num_sms ? kItThreads / 2 : kItThreads;
+            return launch(sym ? input_transform_plane_kernel<ALPHA, true> : input_transform_plane_kernel<ALPHA, false>, blocks, threads,
+                          static_cast<char*>(V_hi), static_cast<char*>(V_lo), g, pi, mode, bt);
+        }
+    }
+    return launch_input_two_pass<ALPHA>(x, V_hi, V_lo, g, tp, mode, sym, bt, num_sms, stream);
+}
 
 }  // namespace wino
 }  // namespace mnnb
@@ -134,7 +187,7 @@ cudaError_t launch_output_am(const float* Mx, const float* bias, float* y, const
 #define MNNB_INPUT_ARGS const float *x, void *V_hi, void *V_lo, const WinoGeom &g, int mode, const TransformMatrices &mats, int *status, int num_sms, cudaStream_t stream
 #define MNNB_OUTPUT_ARGS const float *Mx, const float *bias, float *y, const WinoGeom &g, int relu, const TransformMatrices &mats, cudaStream_t stream
 #define MNNB_DEFINE_INPUT(A) \
-    namespace mnnb { cudaError_t MNNB_INPUT_FN(A)(MNNB_INPUT_ARGS) { return wino::launch_input_ws<A>(x, V_hi, V_lo, g, mode, mats, status, num_sms, stream); } }
+    namespace mnnb { cudaError_t MNNB_INPUT_FN(A)(MNNB_INPUT_ARGS) { return wino::launch_input<A>(x, V_hi, V_lo, g, mode, mats, status, num_sms, stream); } }
 #define MNNB_DEFINE_OUTPUT(A, MM) \
     namespace mnnb { cudaError_t MNNB_OUTPUT_FN(A, MM)(MNNB_OUTPUT_ARGS) { return wino::launch_output_am<A, MM>(Mx, bias, y, g, relu, mats, stream); } }
 #define MNNB_DECLARE_INPUT(A) namespace mnnb { cudaError_t MNNB_INPUT_FN(A)(MNNB_INPUT_ARGS); }

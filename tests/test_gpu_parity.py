@@ -534,3 +534,20 @@ def test_input_transform_bands(torch, N, Cin, H, W_, pad, m):
                                                     fused=B.FUSED_NEVER), (x, w, b))
     assert info.algo == B.ALGO_WINOGRAD and info.m == m
     assert rel_l2(got, oracle(layer, x, w, b)) < 1e-4
+
+
+# Input transform by two passes through shared memory: tile rows cut into segments (ragged last one), channels off the
+# block of 32, more items than CTAs fit the chip (the next item's loads in flight), single tiles; every operand format.
+@pytest.mark.parametrize("N,Cin,H,W_,k,m", [
+    (2, 33, 19, 45, 7, 4), (1, 5, 9, 150, 5, 6), (3, 64, 13, 31, 7, 6), (70, 96, 9, 37, 5, 4), (1, 7, 41, 30, 2, 6), (9, 40, 97, 131, 3, 4),
+    (1, 16, 2, 3, 5, 2), (2, 34, 57, 64, 3, 4)])
+@pytest.mark.parametrize("operand,passes", [(B.OPERAND_BF16, 3), (B.OPERAND_TF32, 3), (B.OPERAND_BF16, 1), (B.OPERAND_TF32, 1)])
+def test_input_transform_two_pass(torch, N, Cin, H, W_, k, m, operand, passes):
+    layer = W.ConvLayer("t", N, Cin, 24, H, W_, k, 1, k // 2, relu=True, seed=Cin + H)
+    x, w, b = W.make_inputs(layer)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_WINOGRAD, force_m=m, operand=operand, passes=passes,
+                                                    fused=B.FUSED_NEVER), (x, w, b))
+    assert info.algo == B.ALGO_WINOGRAD and info.m == m
+    # three times the error expected of operands rounded to this format, amplified by these transforms, and fp32 arithmetic
+    bound = 3e-6 * B.mnn_accuracy_ppm(m, k, info.points_id, operand, passes) + 2e-5
+    if bound < 0.1: assert rel_l2(got, oracle(layer, x, w, b)) < bound

@@ -11,8 +11,8 @@
 // address, and an input element crosses from L2 once per region instead of k * k times.
 //
 // What bounds it: the serial time of the issuing thread and then the tensor core's TF32 rate (3 x 3 dilation 2, 256 channels
-// 28 x 28, batch 16: 34 us product, 436 TFLOP/s); on few-channel layers the bytes of the packed planes.  Measured, both
-// launches, against the implicit gather / the patch matrix: that layer 40 us (86 / 107); 64 -> 128 3x3 stride 2 at 56 x 56
+// 28 x 28, batch 16: 31 us product, 475 TFLOP/s); on few-channel layers the bytes of the packed planes.  Measured, both
+// launches, against the implicit gather / the patch matrix: that layer 37 us (86 / 107); 64 -> 128 3x3 stride 2 at 56 x 56
 // batch 32 27 us (45 / 66); 128 -> 256 at 28 x 28 26 us (45 / 56); 256 -> 512 at 14 x 14 38 us (79 / 68); 3 -> 64 7x7
 // stride 2 at 224 x 224 batch 32 70 us (247 / 156).
 #include "line_conv.h"

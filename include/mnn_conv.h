@@ -95,8 +95,8 @@ enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_ST
  *              dilation: producer warps of the GEMM kernel gather the patches into the
  *              shared-memory operand tile themselves (single-pass TF32 operands, rounded
  *              to nearest).  AUTO = the planner takes the cheapest that applies; it may also report
- *              PACKED (not an option value): x is re-laid into lines of positions, rounded to nearest,
- *              and every kernel tap reads them at a shifted start.  Asking
+ *              PACKED (not an option value): x is re-laid into lines of positions, rounded to nearest
+ *              (TF32 or BF16), and every kernel tap reads them at a shifted start.  Asking
  *              for X or IMPLICIT where it does not apply fails the plan.
  *   fused      Winograd F(2x2, 3x3) as ONE kernel (input transform, contraction and output
  *              transform fused; the transformed tensors V and M never reach device memory):

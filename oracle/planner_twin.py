@@ -176,24 +176,85 @@ def gemm_may_read_x(L: Layer, operand: int, passes: int) -> bool:
             and passes == 1 and L.H * L.W >= 32 and (L.H * L.W) % 4 == 0)
 
 
-def packs_lines(L: Layer) -> bool:
-    """x packed into lines of positions: k in 2..7, stride <= 4, Cin a multiple of 32 or Cin * k <= 32, taps reaching at most
-    600 positions past an output, packed planes of at most 4 GiB."""
-    if L.groups != 1 or not 2 <= L.k <= 7 or L.stride > 4 or not (L.Cin % 32 == 0 or L.Cin * L.k <= 32):
+def packs_lines(L: Layer, operand: int) -> bool:
+    """x packed into lines of positions: k in 2..7, stride <= 4, Cin a multiple of 32 or Cin * k <= 32 (BF16: a multiple of
+    64), taps reaching at most 600 positions past an output, packed planes of at most 4 GiB."""
+    if operand == OPERAND_BF16:
+        channels = L.Cin % 64 == 0
+    else:
+        channels = L.Cin % 32 == 0 or L.Cin * L.k <= 32
+    if L.groups != 1 or not 2 <= L.k <= 7 or L.stride > 4 or not channels:
         return False
     reach = (L.k - 1) * L.dil // L.stride
     wq, hq = L.OW + reach, L.OH + reach
     cells = L.N * hq * wq
     return (reach * (wq + 1) <= 600 and cells < 2 ** 30
-            and L.stride ** 2 * (cells + 2048) * (cdiv(L.Cin, 32) * 32) * 4 <= 4 << 30)
+            and L.stride ** 2 * (cells + 2048) * (cdiv(L.Cin, 32) * 32) * _bytes_of(operand) <= 4 << 30)
 
 
-def packed_cost(L: Layer, c) -> int:
-    """Packed lines: a pass from x to the packed planes, and a product that reads them, at half the contraction's tensor rate."""
+def bf16_lines(L: Layer, sms: int):
+    """(bytes of the packed planes, estimated time of the product in ps) of the BF16 packed-line form, or None: the geometry
+    of the cells and the cheapest tiling (output channels bn, mt tiles of 128 cells, g taps per step) that fits."""
+    s, offs = L.stride, {}
+    for a in range(L.k):
+        for b in range(L.k):
+            offs.setdefault((a * L.dil % s, b * L.dil % s), []).append((a * L.dil // s, b * L.dil // s))
+    if len(offs) > 16:
+        return None
+    qs = [q for group in offs.values() for q in group]
+
+    def pitch(size, out, phases, reach):
+        lead = min(cdiv(L.pad - r, s) if r < L.pad else 0 for r in phases)
+        end = max((size - 1 + L.pad - r) // s + 1 if size - 1 + L.pad - r >= 0 else 0 for r in phases)
+        return max(out, min(out + reach, max(end, out + reach - lead)))
+
+    hq = pitch(L.H, L.OH, [r for r, _ in offs], max(q[0] for q in qs))
+    wq = pitch(L.W, L.OW, [r for _, r in offs], max(q[1] for q in qs))
+    rows = [[qh * wq + qw for qh, qw in group] for group in offs.values()]
+    span, base = max(max(r) - min(r) for r in rows), max(min(r) for r in rows)
+    cells, taps = L.N * hq * wq, L.k * L.k
+    positions = cells + span + base
+    a_bytes = len(rows) * positions * L.Cin * 2
+    if positions >= (1 << 31) - 4096 or a_bytes > 4 << 30:
+        return None
+    co16, room, best = cdiv(L.Cout, 16) * 16, 207 * 1024, None
+    for bn in (256, 128, 64, 32):
+        for mt in (1, 2, 4):
+            nb = cdiv(co16, bn)
+            n = cdiv(cdiv(co16, nb), 16) * 16
+            boxes = cdiv(128 * mt + span, 256)
+            region = boxes * (cdiv(cdiv(128 * mt + span, boxes), 8) * 8)
+            if 2 * mt * n > 512 or (bn > 32 and co16 <= bn // 2) or region > 1024:
+                continue
+            a_slot, b_tile = region * 128, n * 128
+            rounds = cdiv(cdiv(cells, 128 * mt) * nb, sms)
+            for g in (3, 2, 1):
+                if 2 * a_slot >= room or (room - 2 * a_slot) // (g * b_tile) < (3 if g == 1 else 2):
+                    continue
+                issue = sum(cdiv(len(r), g) for r in rows) * 194000 + taps * 4 * 45000
+                mma = taps * mt * 4 * (212 * n + 15000)
+                load = (taps * b_tile + len(rows) * a_slot) * 63 // 5
+                drain = mt * n * 512 * 28 + 1087000
+                item = max(issue, mma, load) * (L.Cin // 64) + 285000 + mt * 363000
+                cost = rounds * max(item, drain) + drain
+                if best is None or cost * (100 + 3 * mt) < best[0]:
+                    best = (cost * (100 + 3 * mt), cost)
+    return None if best is None else (a_bytes, best[1])
+
+
+def packed_cost(L: Layer, operand: int, c) -> int:
+    """Packed lines: a pass from x to the packed planes, and a product that reads them: in TF32 at half the contraction's tensor
+    rate, in BF16 by the estimate of its tiling."""
+    x, y = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW
+    if operand == OPERAND_BF16:
+        lines = bf16_lines(L, c[7] if c[7] > 0 else 148)
+        if lines is None:
+            return INADMISSIBLE
+        a, product = lines
+        return sat(kernel_ps(c, mem_as=(x + a) * c[0] * 4 // 3) + kernel_ps(c, mem_as=(a + y) * c[0], tensor_as=product * 10 ** 6))
     reach = (L.k - 1) * L.dil // L.stride
     planes = min(L.stride, L.k) ** 2
     a = L.N * (L.OH + reach) * (L.OW + reach) * planes * cdiv(L.Cin, 32) * 32 * 4
-    x, y = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW
     flops = 2 * L.N * L.OH * L.OW * L.Cout * L.Cin * L.k * L.k
     return sat(kernel_ps(c, mem_as=(x + a) * c[0]) + kernel_ps(c, mem_as=(a + y) * c[0], tensor_as=flops * 2 * c[2]))
 
@@ -392,16 +453,15 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 costs_of = lhs
                 # items so few that their K loop is cut over clusters: the implicit gather instead of patches; else packed
                 # lines where they apply.  Booked at the cost of the operand chosen above.
-                if implicit_ok:
-                    sms = c[7] if c[7] > 0 else 148
-                    blocks = cdiv(L.N * L.OH * L.OW, 128)
-                    _, co_blocks = contraction_tiling(blocks, 1, L.Cout, sms)
-                    cut = cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1
-                    if cut and not (L.k == 1 and L.stride == 1) and c[13] > 0:
-                        if lhs == LHS_PATCHES:
-                            lhs = LHS_IMPLICIT
-                    elif packs_lines(L) and packed_cost(L, c) < costs[lhs]:
-                        lhs = LHS_PACKED
+                sms = c[7] if c[7] > 0 else 148
+                blocks = cdiv(L.N * L.OH * L.OW, 128)
+                _, co_blocks = contraction_tiling(blocks, 1, L.Cout, sms)
+                cut = cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1
+                if implicit_ok and cut and not (L.k == 1 and L.stride == 1) and c[13] > 0:
+                    if lhs == LHS_PATCHES:
+                        lhs = LHS_IMPLICIT
+                elif packs_lines(L, operand) and packed_cost(L, operand, c) < costs[lhs]:
+                    lhs = LHS_PACKED
                 costs[lhs] = costs[costs_of]
             if lhs == LHS_X:
                 p = max(p, LHS_X_ERROR_PPM)
@@ -435,6 +495,11 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
     for i in range(N_CANDIDATES):
         if ch.cost_ps[i] != INADMISSIBLE and (best < 0 or ch.cost_ps[i] < ch.cost_ps[best]):
             best = i
+    # BF16 class: packed lines in BF16 take over from a scheme that is neither faster nor expected to be more accurate
+    if best not in (-1, 2) and side.get(2, {}).get("lhs") == LHS_PACKED and side[2]["ppm"] <= side.get(best, {}).get("ppm", 0):
+        cost = packed_cost(L, OPERAND_BF16, c)
+        if cost < ch.cost_ps[best]:
+            ch.cost_ps[2], best = cost, 2
     if best < 0:
         return ch
     algo, m, operand, passes = _candidates()[best]

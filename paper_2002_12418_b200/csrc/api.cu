@@ -287,7 +287,7 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
         p->d.error_ppm = accuracy_ppm(1, 1, 0, p->d.operand, p->d.passes);
     }
     if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
-        const LineShape ls = {N, Cin, Cout, H, W, k, stride, dilation, pad, s.OH, s.OW};
+        const LineShape ls = {N, Cin, Cout, H, W, k, stride, dilation, pad, s.OH, s.OW, p->d.operand == MNN_OPERAND_BF16};
         p->packed = line_plan(ls, 148, &p->lc.p);
         if (!p->packed) {
             fail(MNN_EUNSUPPORTED, "no tiling of the packed-line product fits this layer");

@@ -3,7 +3,7 @@
 //
 //     y[co][cell] = sum over (element block, tap) of  A[plane][cell + shift(tap)][element] * U[tap][co][element]
 //
-// Two launches.  The pack kernel transposes x into planes of positions, rounded to TF32.  The product kernel is the
+// Two launches.  The pack kernel transposes x into planes of positions, rounded to TF32 or BF16.  The product kernel is the
 // persistent pipeline of contract_umma.cu (TMA producer, one MMA thread, epilogue warps, two accumulators) with two rings: a
 // region of 128 * mt + span consecutive positions x 32 elements is staged once per (element block, plane), and one weight
 // tile per tap.  A row of the region is 128 bytes in the 128-byte swizzle, whose pattern depends on the address alone and
@@ -15,7 +15,14 @@
 // launches, against the implicit gather / the patch matrix: that layer 37 us (86 / 107); 64 -> 128 3x3 stride 2 at 56 x 56
 // batch 32 27 us (45 / 66); 128 -> 256 at 28 x 28 26 us (45 / 56); 256 -> 512 at 14 x 14 38 us (79 / 68); 3 -> 64 7x7
 // stride 2 at 224 x 224 batch 32 70 us (247 / 156).
+//
+// BF16 operands (the BF16 accuracy class) halve the planes and the instructions: 256 channels 56 x 56 batch 64 product 303 ->
+// 176 us (1.35 PFLOP/s), layer 248 us against 431 in the Winograd scheme; 64 channels 56 x 56 batch 64 50 us against 103.
 #include "line_conv.h"
+
+#include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "contract_umma.h"
 #include "umma.cuh"
@@ -45,18 +52,23 @@ struct LineParams {
 // word, so that an instruction costs the issuing thread one addition per operand.
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 
+template <bool BF16>
 __device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile(
-        "{\n\t"
-        ".reg .b64 da, db;\n\t"
-        ".reg .pred p;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n\t"
-        "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate)
-        : "memory");
+#define MNNB_LINE_MMA(KIND)                                                                                                \
+    asm volatile(                                                                                                          \
+        "{\n\t"                                                                                                            \
+        ".reg .b64 da, db;\n\t"                                                                                            \
+        ".reg .pred p;\n\t"                                                                                                \
+        "mov.b64 da, {%1, %3};\n\t"                                                                                        \
+        "mov.b64 db, {%2, %3};\n\t"                                                                                        \
+        "setp.ne.b32 p, %5, 0;\n\t"                                                                                        \
+        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %4, p;\n\t"                                                 \
+        "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate)                                 \
+        : "memory")
+    if (BF16) MNNB_LINE_MMA("f16");
+    else MNNB_LINE_MMA("tf32");
+#undef MNNB_LINE_MMA
 }
 
 // MT = tiles of 128 cells per item, KS = tensor-core steps per block of elements, G = weight tiles per step (slot, barrier and
@@ -64,7 +76,7 @@ __device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t 
 // path: measured with the clock, a step spent about 225 cycles in a wait that was ready, 93 in the commit, 220 in loop
 // control and 58 per instruction.  Dilation-2 layer above, product only: 66 us with run-time loop bounds, 43.5 unrolled,
 // 38 with up to three taps per step; 256 -> 512 stride 2: 36 -> 31 us with the failure checks out of the loop conditions.
-template <int MT, int KS, int G>
+template <int MT, int KS, int G, bool BF16>
 __global__ void __launch_bounds__(line_threads(MT), 1)
 line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ LineParams p)
 {
@@ -77,6 +89,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     volatile int* abortp = &abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kBlockElems = BF16 ? 64 : 32;
     const uint32_t a_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_slot_bytes = (uint32_t)p.region * 128u, b_tile_bytes = (uint32_t)p.bn * 128u, b_slot_bytes = G * b_tile_bytes;
     const uint32_t b_base = a_base + (uint32_t)p.a_slots * a_slot_bytes;
@@ -132,7 +145,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         ptx::mbar_expect_tx(abar, a_slot_bytes);
                         const int row0 = (int)(tb * 128u * (unsigned)MT) + p.group_base[g];
                         for (int b = 0; b < p.boxes; ++b)
-                            ptx::tma_load_3d(a_base + as * a_slot_bytes + (uint32_t)(b * p.box_rows) * 128u, &map_a, abar, eb * 32,
+                            ptx::tma_load_3d(a_base + as * a_slot_bytes + (uint32_t)(b * p.box_rows) * 128u, &map_a, abar, eb * kBlockElems,
                                              row0 + b * p.box_rows, p.group_plane[g]);
                         if (++as == (uint32_t)p.a_slots) {
                             as = 0;
@@ -150,7 +163,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 #pragma unroll
                             for (int j = 0; j < G; ++j)
                                 if (j < n)
-                                    ptx::tma_load_3d(b_base + bs * b_slot_bytes + j * b_tile_bytes, &map_u, bbar, eb * 32, (int)nb * p.bn, t + j);
+                                    ptx::tma_load_3d(b_base + bs * b_slot_bytes + j * b_tile_bytes, &map_u, bbar, eb * kBlockElems, (int)nb * p.bn, t + j);
                             if (++bs == (uint32_t)p.b_slots) {
                                 bs = 0;
                                 b_phase ^= 1u;
@@ -167,7 +180,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         // ------------------------------ MMA issue: one thread per tile of 128 cells ------------------------------
         if (lane == 0) {
             const uint32_t tile = (uint32_t)warp - 1u;
-            const uint32_t idesc = ptx::mma_idesc(2, 128, p.bn);
+            const uint32_t idesc = ptx::mma_idesc(BF16 ? 1 : 2, 128, p.bn);
             uint32_t as = 0, a_phase = 0, bs = 0, b_phase = 0, acc = 0, acc_phase = 0;
             int err = 0;
             const uint32_t a_lo_base = (1u << 16) | (((a_base & 0x3FFFFu) >> 4) + tile * 1024u), b_lo_base = (1u << 16) | ((b_base & 0x3FFFFu) >> 4);
@@ -202,7 +215,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                                 if (j < n) {
 #pragma unroll
                                     for (int ks = 0; ks < KS; ++ks)
-                                        mma_lo(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), idesc,
+                                        mma_lo<BF16>(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), idesc,
                                                (j | ks) ? 1u : accumulate);
                                 }
                             accumulate = 1u;
@@ -319,7 +332,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // ---------------------------------------------------------------------------
 struct PackParams {
     const float* x;
-    float* A;
+    void* A;
     long long P, T;
     int Cin, H, W, k, stride, dil, pad, strips, Hq, Wq, elems, n_planes;
     int phase_h[kLineMaxPlanes], phase_w[kLineMaxPlanes];
@@ -335,6 +348,7 @@ __device__ __forceinline__ float tf32_rn(float v)
 // 32 positions x 64 channels of one plane per CTA, transposed through shared memory: lanes run over positions while x is
 // read and over channels while A is written.  The planes of a position block are neighbours in the grid, so that the phases
 // of a stride share the sectors of x in L2.
+template <bool BF16>
 __global__ void __launch_bounds__(256) line_pack_kernel(const __grid_constant__ PackParams p)
 {
     __shared__ float tile[64][33];
@@ -357,18 +371,24 @@ __global__ void __launch_bounds__(256) line_pack_kernel(const __grid_constant__ 
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = ok && c0 + warp + 8 * e < p.Cin ? __ldg(src + (size_t)(8 * e) * plane) : 0.0f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tile[warp + 8 * e][lane] = tf32_rn(v[e]);
+        for (int e = 0; e < 8; ++e) tile[warp + 8 * e][lane] = BF16 ? v[e] : tf32_rn(v[e]);
     }
     __syncthreads();
-    // 16 lanes write the 64 channels of a position as 128-bit pieces
+    // 16 lanes write the 64 channels of a position, four each
     const int cv = (threadIdx.x & 15) * 4;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int pl = (threadIdx.x >> 4) + 16 * h;
         const long long pos = p0 + pl;
         if (pos >= p.P || c0 + cv >= p.elems) continue;
-        *reinterpret_cast<float4*>(p.A + ((long long)z * p.P + pos) * p.elems + c0 + cv) =
-            make_float4(tile[cv][pl], tile[cv + 1][pl], tile[cv + 2][pl], tile[cv + 3][pl]);
+        const long long at = ((long long)z * p.P + pos) * p.elems + c0 + cv;
+        if (BF16) {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(tile[cv][pl], tile[cv + 1][pl]), hi = __floats2bfloat162_rn(tile[cv + 2][pl], tile[cv + 3][pl]);
+            *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.A) + at) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        } else {
+            *reinterpret_cast<float4*>(static_cast<float*>(p.A) + at) = make_float4(tile[cv][pl], tile[cv + 1][pl], tile[cv + 2][pl], tile[cv + 3][pl]);
+        }
     }
 }
 
@@ -410,7 +430,7 @@ __global__ void __launch_bounds__(256) line_pack_few_kernel(const __grid_constan
         *reinterpret_cast<float4*>(&tile[warp][lane][4 * q]) =
             make_float4(tf32_rn(v[4 * q]), tf32_rn(v[4 * q + 1]), tf32_rn(v[4 * q + 2]), tf32_rn(v[4 * q + 3]));
     __syncwarp();
-    float* dst = p.A + ((long long)z * p.P + p0) * 32;
+    float* dst = static_cast<float*>(p.A) + ((long long)z * p.P + p0) * 32;
     const int piece = lane & 7;
     if (piece < USED / 4)
 #pragma unroll
@@ -422,8 +442,8 @@ __global__ void __launch_bounds__(256) line_pack_few_kernel(const __grid_constan
 
 struct WeightParams {
     const float* w;
-    float* U;
-    int Cout, Cin, k, elems, few, n_taps;
+    void* U;
+    int Cout, Cin, k, elems, few, bf16, n_taps;
     int tap_id[kLineMaxTaps];
 };
 
@@ -441,22 +461,25 @@ __global__ void __launch_bounds__(256) line_weights_kernel(const __grid_constant
     } else {
         v = p.w[((size_t)co * p.Cin + e) * p.k * p.k + tap];
     }
-    p.U[gid] = tf32_rn(v);
+    if (p.bf16) static_cast<__nv_bfloat16*>(p.U)[gid] = __float2bfloat16_rn(v);
+    else static_cast<float*>(p.U)[gid] = tf32_rn(v);
 }
 
 typedef void (*LineKernel)(CUtensorMap, CUtensorMap, LineParams);
 
-template <int MT, int KS>
-LineKernel line_kernel_g(int g)
+template <int KS, bool BF16>
+LineKernel line_kernel_of(const LinePlan& p)
 {
-    return g == 3 ? line_gemm_kernel<MT, KS, 3> : g == 2 ? line_gemm_kernel<MT, KS, 2> : line_gemm_kernel<MT, KS, 1>;
+    auto by_g = [&](auto mt) -> LineKernel {
+        constexpr int MT = decltype(mt)::value;
+        return p.taps_per_step == 3 ? line_gemm_kernel<MT, KS, 3, BF16> : p.taps_per_step == 2 ? line_gemm_kernel<MT, KS, 2, BF16> : line_gemm_kernel<MT, KS, 1, BF16>;
+    };
+    return p.mt == 4 ? by_g(std::integral_constant<int, 4>()) : p.mt == 2 ? by_g(std::integral_constant<int, 2>()) : by_g(std::integral_constant<int, 1>());
 }
 
 LineKernel line_kernel(const LinePlan& p)
 {
-    if (p.k_steps == 4)
-        return p.mt == 4 ? line_kernel_g<4, 4>(p.taps_per_step) : p.mt == 2 ? line_kernel_g<2, 4>(p.taps_per_step) : line_kernel_g<1, 4>(p.taps_per_step);
-    return p.mt == 4 ? line_kernel_g<4, 3>(p.taps_per_step) : p.mt == 2 ? line_kernel_g<2, 3>(p.taps_per_step) : line_kernel_g<1, 3>(p.taps_per_step);
+    return p.s.bf16 ? line_kernel_of<4, true>(p) : p.k_steps == 4 ? line_kernel_of<4, false>(p) : line_kernel_of<3, false>(p);
 }
 
 }  // namespace
@@ -469,8 +492,9 @@ cudaError_t line_setup(LineConv* lc, void* A, void* U, const char** why)
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lc->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (!encode_operand_map_sw(&lc->map_a, A, 4, p.elems, p.P, p.n_planes, p.P * p.elems, p.box_rows, 128) ||
-        !encode_operand_map_sw(&lc->map_u, U, 4, p.elems, p.s.Cout, p.n_taps, (long long)p.s.Cout * p.elems, p.bn, 128)) {
+    const int eb = p.s.bf16 ? 2 : 4;
+    if (!encode_operand_map_sw(&lc->map_a, A, eb, p.elems, p.P, p.n_planes, p.P * p.elems, p.box_rows, 128) ||
+        !encode_operand_map_sw(&lc->map_u, U, eb, p.elems, p.s.Cout, p.n_taps, (long long)p.s.Cout * p.elems, p.bn, 128)) {
         *why = "cuTensorMapEncodeTiled failed or is unavailable";
         return cudaErrorInvalidValue;
     }
@@ -484,10 +508,10 @@ cudaError_t launch_line_weights(const LinePlan& lp, const float* w, void* U, cud
 {
     WeightParams p = {};
     p.w = w;
-    p.U = static_cast<float*>(U);
-    p.Cout = lp.s.Cout; p.Cin = lp.s.Cin; p.k = lp.s.k; p.elems = lp.elems; p.few = lp.few; p.n_taps = lp.n_taps;
+    p.U = U;
+    p.Cout = lp.s.Cout; p.Cin = lp.s.Cin; p.k = lp.s.k; p.elems = lp.elems; p.few = lp.few; p.bf16 = lp.s.bf16; p.n_taps = lp.n_taps;
     for (int i = 0; i < lp.n_taps; ++i) p.tap_id[i] = lp.tap_id[i];
-    const long long total = lp.u_bytes / 4;
+    const long long total = (long long)lp.n_taps * lp.s.Cout * lp.elems;
     line_weights_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(p);
     return cudaGetLastError();
 }
@@ -497,7 +521,7 @@ cudaError_t launch_line_pack(const LinePlan& lp, const float* x, void* A, cudaSt
     PackParams p = {};
     const LineShape& s = lp.s;
     p.x = x;
-    p.A = static_cast<float*>(A);
+    p.A = A;
     p.P = lp.P; p.T = lp.T;
     p.Cin = s.Cin; p.H = s.H; p.W = s.W; p.k = s.k; p.stride = s.stride; p.dil = s.dil; p.pad = s.pad; p.strips = lp.strips; p.Hq = lp.Hq; p.Wq = lp.Wq;
     p.elems = lp.elems; p.n_planes = lp.n_planes;
@@ -510,7 +534,7 @@ cudaError_t launch_line_pack(const LinePlan& lp, const float* x, void* A, cudaSt
                                  dim3(256), 0, stream, p);
     const long long gx = (lp.P + 31) / 32 * lp.n_planes;
     if (gx > 2147483647ll || (lp.elems + 63) / 64 > 65535) return cudaErrorInvalidValue;
-    return launch_overlapped(line_pack_kernel, dim3((unsigned)gx, (unsigned)((lp.elems + 63) / 64)), dim3(256), 0, stream, p);
+    return launch_overlapped(s.bf16 ? line_pack_kernel<true> : line_pack_kernel<false>, dim3((unsigned)gx, (unsigned)((lp.elems + 63) / 64)), dim3(256), 0, stream, p);
 }
 
 cudaError_t launch_line_gemm(const LineConv& lc, const float* bias, float* y, int relu, int* status, cudaStream_t stream)
@@ -521,7 +545,7 @@ cudaError_t launch_line_gemm(const LineConv& lc, const float* bias, float* y, in
     p.bias = bias; p.y = y; p.status = status;
     p.T = lp.T;
     p.n_items = (unsigned)lp.n_items; p.n_tile_blocks = (unsigned)lp.n_tile_blocks;
-    p.Cout = lp.s.Cout; p.bn = lp.bn; p.blocks = lp.elems / 32; p.n_groups = lp.n_groups;
+    p.Cout = lp.s.Cout; p.bn = lp.bn; p.blocks = lp.blocks; p.n_groups = lp.n_groups;
     p.region = lp.region; p.boxes = lp.boxes; p.box_rows = lp.box_rows; p.a_slots = lp.a_slots; p.b_slots = lp.b_slots;
     p.tmem_cols = 32;
     while (p.tmem_cols < 2 * lp.mt * lp.bn) p.tmem_cols *= 2;

@@ -16,9 +16,9 @@ struct LineConv {
 
 // Tensor maps over the packed planes A (a_bytes, 16-byte aligned) and the weights U (u_bytes, 16-byte aligned).
 cudaError_t line_setup(LineConv* lc, void* A, void* U, const char** why);
-// U [tap][Cout][elems], TF32-rounded.
+// U [tap][Cout][elems], rounded to the operand type.
 cudaError_t launch_line_weights(const LinePlan& p, const float* w, void* U, cudaStream_t stream);
-// x into A, TF32-rounded.
+// x into A, rounded to the operand type.
 cudaError_t launch_line_pack(const LinePlan& p, const float* x, void* A, cudaStream_t stream);
 // y = act(conv + bias) from A and U.
 cudaError_t launch_line_gemm(const LineConv& lc, const float* bias, float* y, int relu, int* status, cudaStream_t stream);

@@ -24,10 +24,12 @@ bool line_plan(const LineShape& s, int num_sms, LinePlan* p)
 {
     std::memset(p, 0, sizeof(*p));
     p->s = s;
-    p->few = s.Cin % 32 != 0;
-    if (p->few && s.Cin * s.k > 32) return false;
+    const int block = s.bf16 ? 64 : 32, eb = s.bf16 ? 2 : 4;
+    p->few = s.Cin % block != 0;
+    if (p->few && (s.bf16 || s.Cin * s.k > 32)) return false;
     if (s.k > 7 || s.stride > 4) return false;
     p->elems = p->few ? 32 : s.Cin;
+    p->blocks = p->elems / block;
     p->k_steps = p->few && s.Cin * s.k <= 24 ? 3 : 4;
 
     // phases and taps, grouped by phase
@@ -88,14 +90,14 @@ bool line_plan(const LineShape& s, int num_sms, LinePlan* p)
     p->T = (long long)s.N * p->strips * p->Hq * p->Wq;
     p->P = p->T + span + max_base;       // rows past the end of a plane read as zeros or as the next plane, for no valid cell
     if (p->P >= (1ll << 31) - 4096) return false;
-    p->a_bytes = (long long)p->n_planes * p->P * p->elems * 4;
-    p->u_bytes = (long long)p->n_taps * s.Cout * p->elems * 4;
+    p->a_bytes = (long long)p->n_planes * p->P * p->elems * eb;
+    p->u_bytes = (long long)p->n_taps * s.Cout * p->elems * eb;
     if (p->a_bytes > (4ll << 30)) return false;
 
-    // Tiling: the shortest loop, rounds of items over the SMs times the pace of a block of 32 elements: an issuing thread's
+    // Tiling: the shortest loop, rounds of items over the SMs times the pace of a block of 128 bytes: an issuing thread's
     // serial time (0.2 us per step and 45 ns per instruction; each tile of cells has a thread of its own), the tensor core's
     // (15 ns + 0.21 ns per output channel and instruction) or the delivery of regions and weight tiles (12.6 ps per byte and
-    // SM), whichever is longest; then what an item costs besides or its drain, and the fill.  Fitted to 690 measured
+    // SM), whichever is longest; then what an item costs besides or its drain.  Fitted to 690 measured
     // products (20 layers, every tiling) to 8 %; the choice is within 5 % of the best of most, 11 % at worst, with 3 % held
     // against each further tile of an item.
     // Two tiles of 128 channels rather than one of 256: half the weight bytes and two issuing threads (256 channels 28 x 28
@@ -124,7 +126,7 @@ bool line_plan(const LineShape& s, int num_sms, LinePlan* p)
                 const long long mma = (long long)p->n_taps * mt * p->k_steps * (212 * b_n + 15000);
                 const long long load = (p->n_taps * b_tile + p->n_groups * a_slot) * 63 / 5;
                 const long long drain = (long long)mt * b_n * 128 * 4 * 28 + 1087000;
-                const long long cost = rounds * std::max(std::max(issue, std::max(mma, load)) * (p->elems / 32) + 285000 + mt * 363000, drain) + drain + 2420000;
+                const long long cost = rounds * std::max(std::max(issue, std::max(mma, load)) * p->blocks + 285000 + mt * 363000, drain) + drain;
                 if (best < 0 || cost * (100 + 3 * mt) < best) {
                     best = cost * (100 + 3 * mt);
                     p->bn = b_n;
@@ -138,6 +140,7 @@ bool line_plan(const LineShape& s, int num_sms, LinePlan* p)
                     p->b_slots = b_slots;
                     p->n_tile_blocks = tile_blocks;
                     p->n_items = items;
+                    p->loop_ps = cost;
                 }
             }
         }

@@ -1,7 +1,7 @@
 // Geometry and tiling of the packed-line convolution (line_conv.cu).  Host only, integers only.
 //
-// x is re-laid ("packed") into planes of positions, a position being one 128-byte row per block of 32 operand elements:
-//     A [plane][position][elements]           elements = input channels, padded to a multiple of 32
+// x is re-laid ("packed") into planes of positions, a position being one 128-byte row per block of 32 TF32 or 64 BF16 operand elements:
+//     A [plane][position][elements]           elements = input channels, a multiple of 32 (TF32) or 64 (BF16)
 // A position is a cell (n, i, j) of a grid of N x Hq x Wq cells, a cell an output position, a plane one of the input phases
 // of the stride.  Kernel tap (a, b) reads, for every cell, the cell `shift` positions further on in its phase's plane, so a
 // tap is a change of the operand's start row and nothing is gathered.  Rows and images share their zero padding: the cells
@@ -21,13 +21,14 @@ constexpr int kLineMaxRegion = 1024;     // positions staged at a time
 
 struct LineShape {
     int N, Cin, Cout, H, W, k, stride, dil, pad, OH, OW;
+    int bf16;                            // operand elements: BF16 (not in the few-channel form), else TF32
 };
 
 struct LinePlan {
     LineShape s;
     int few;                             // the few-channel form
-    int elems;                           // elements per position (multiple of 32)
-    int k_steps;                         // tensor-core steps of 8 elements in the last block of 32 (3 for few channels of at most 24 elements, else 4)
+    int elems, blocks;                   // elements per position, in blocks of 128 bytes
+    int k_steps;                         // tensor-core steps of 32 bytes in a block (3 for few channels of at most 24 elements, else 4)
     int n_planes, phase_h[kLineMaxPlanes], phase_w[kLineMaxPlanes];
     int strips, Hq, Wq;                  // strips: 1 unless few
     long long T, P;                      // cells; positions per plane in memory
@@ -41,6 +42,7 @@ struct LinePlan {
     int taps_per_step;                   // weight tiles that share a slot and a barrier
     int a_slots, b_slots;
     long long n_tile_blocks, n_items, a_bytes, u_bytes;
+    long long loop_ps;                   // estimated time of the product without its launch and fill
 };
 
 // Fills *p; false where the form does not apply (channels not a multiple of 32 and not few, region or phases too large).

@@ -10,6 +10,8 @@
 // reproduced bit for bit from the nine layer integers and the constant record.
 #include "planner.h"
 
+#include "line_plan.h"
+
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -347,14 +349,15 @@ int contract_split(long long items, int k_blocks, int num_sms)
     return split;
 }
 
-bool gemm_packs_lines(const LayerShape& s)
+bool gemm_packs_lines(const LayerShape& s, int operand)
 {
-    if (s.groups != 1 || s.k < 2 || s.k > 7 || s.stride > 4 || !(s.Cin % 32 == 0 || s.Cin * s.k <= 32)) return false;
+    const int block = operand == MNN_OPERAND_BF16 ? 64 : 32;      // channels per 128 bytes
+    if (s.groups != 1 || s.k < 2 || s.k > 7 || s.stride > 4 || !(s.Cin % block == 0 || (block == 32 && s.Cin * s.k <= 32))) return false;
     // rows of cells a tap can reach past an output, bounds of the grid of cells and of the packed planes
     const long long reach = (long long)(s.k - 1) * s.dil / s.stride;
     const long long wq = s.OW + reach, hq = s.OH + reach;
-    const u128 cells = (u128)s.N * (u128)hq * (u128)wq, planes = (u128)(s.stride * s.stride), elems = (s.Cin + 31) / 32 * 32;
-    return reach * (wq + 1) <= 600 && cells < (1u << 30) && planes * (cells + 2048) * elems * 4 <= (u128)(4ll << 30);
+    const u128 cells = (u128)s.N * (u128)hq * (u128)wq, planes = (u128)(s.stride * s.stride), a_bytes = operand_bytes(operand) * (u128)((s.Cin + 31) / 32 * 32);
+    return reach * (wq + 1) <= 600 && cells < (1u << 30) && planes * (cells + 2048) * a_bytes <= (u128)(4ll << 30);
 }
 
 bool gemm_reads_x(const LayerShape& s, int operand, int passes)
@@ -429,16 +432,26 @@ int gemm_split(const LayerShape& s, const Calibration& cal)
     return contract_split((long long)(tile_blocks * (uint64_t)n_co_blocks), (int)k_blocks, sms);
 }
 
-// The packed-line form (line_conv.cu): one pass over x that writes the planes, and a product that reads them once and runs
-// the tensor core at about half of its contraction rate.
-uint64_t packed_cost(const LayerShape& s, const Calibration& cal)
+// The packed-line form (line_conv.cu): one pass over x that writes the planes, at three quarters of the copy rate, and a
+// product that reads them once.  In TF32 the product is charged half of the contraction's tensor rate, an upper bound that
+// only chooses between the left operands of the GEMM scheme; in BF16, where it competes with the other schemes, the time that
+// its tiling was chosen by.
+uint64_t packed_cost(const LayerShape& s, int operand, const Calibration& cal)
 {
+    const uint64_t c0 = (uint64_t)cal.c[0];
+    const u128 x_bytes = (u128)4 * s.N * s.Cin * s.H * s.W, y_bytes = (u128)4 * s.N * s.Cout * s.OH * s.OW;
+    if (operand == MNN_OPERAND_BF16) {
+        const LineShape ls = {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.stride, s.dil, s.pad, s.OH, s.OW, 1};
+        LinePlan p;
+        if (!line_plan(ls, cal.c[7] > 0 ? (int)cal.c[7] : 148, &p)) return MNN_COST_INADMISSIBLE;
+        const u128 a_bytes = (u128)p.a_bytes;
+        return saturate((u128)kernel_ps((x_bytes + a_bytes) * c0 * 4u / 3u, 0, 0, cal) +
+                        kernel_ps((a_bytes + y_bytes) * c0, (u128)p.loop_ps * 1000000u, 0, cal));
+    }
     const u128 reach = (u128)((uint64_t)(s.k - 1) * s.dil / s.stride);
     const u128 cells = (u128)s.N * (s.OH + reach) * (s.OW + reach);
     const u128 a_bytes = cells * (uint64_t)(s.stride < s.k ? s.stride * s.stride : s.k * s.k) * round_up(s.Cin, 32) * 4u;
-    const u128 x_bytes = (u128)4 * s.N * s.Cin * s.H * s.W, y_bytes = (u128)4 * s.N * s.Cout * s.OH * s.OW;
     const u128 flops = (u128)2 * s.N * s.OH * s.OW * s.Cout * (uint64_t)(s.Cin * s.k * s.k);
-    const uint64_t c0 = (uint64_t)cal.c[0];
     return saturate((u128)kernel_ps((x_bytes + a_bytes) * c0, 0, 0, cal) +
                     kernel_ps((a_bytes + y_bytes) * c0, flops * 2u * (uint64_t)cal.c[2], 0, cal));
 }
@@ -624,8 +637,8 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 // cost stays that of the operand chosen above, an upper bound.
                 if (implicit_ok && !pointwise && cal.c[13] > 0 && gemm_split(s, cal) > 1) {
                     if (lhs == MNN_GEMM_LHS_PATCHES) lhs = MNN_GEMM_LHS_IMPLICIT;
-                } else if (implicit_ok && gemm_packs_lines(s) &&
-                           packed_cost(s, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
+                } else if (gemm_packs_lines(s, c.operand) &&
+                           packed_cost(s, c.operand, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
                     lhs = MNN_GEMM_LHS_PACKED;
                 }
             }
@@ -663,6 +676,16 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     int best = -1;
     for (int i = 0; i < MNN_N_CANDIDATES; ++i)
         if (d->cost_ps[i] != MNN_COST_INADMISSIBLE && (best < 0 || d->cost_ps[i] < d->cost_ps[best])) best = i;
+    // BF16 class: packed lines in BF16, booked above at the cost of the patch matrix, take over from a scheme that is neither
+    // faster by this estimate nor expected to be more accurate (3x3 256 channels 56 x 56 batch 64: 257 us, Winograd with m =
+    // 4 and TF32 operands 431; 64 channels 50 / 103; but 512 channels 7 x 7 batch 32 26 / 19).
+    if (best >= 0 && best != 2 && lhs_of[2] == MNN_GEMM_LHS_PACKED && ppm_of[2] <= ppm_of[best]) {
+        const uint64_t cost = packed_cost(s, MNN_OPERAND_BF16, cal);
+        if (cost < d->cost_ps[best]) {
+            d->cost_ps[2] = cost;
+            best = 2;
+        }
+    }
 
     // A forced combination outside the candidate list (other m, fp32 checking contraction).
     const bool off_list = o.force_algo == MNN_ALGO_WINOGRAD && o.force_m != 0 &&

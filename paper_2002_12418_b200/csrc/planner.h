@@ -52,9 +52,10 @@ void contract_tiling(long long tile_blocks, int alpha2, int Cout, int num_sms, i
 // clusters of 8 only for up to 8 items (a GPC holds two of them at best; 16 such clusters ran in two waves).
 int contract_split(long long items, int k_blocks, int num_sms);
 
-// True when the layer fits the packed-line product (line_conv.cu; guarantees that line_plan finds a tiling): k in 2..7,
-// stride at most 4, Cin a multiple of 32 or Cin * k at most 32, and taps that reach at most 600 positions past an output.
-bool gemm_packs_lines(const LayerShape& s);
+// True when the layer fits the packed-line product with this operand type (line_conv.cu; guarantees that line_plan finds a
+// tiling): k in 2..7, stride at most 4, Cin a multiple of 32 or Cin * k at most 32 (BF16: Cin a multiple of 64), and taps
+// that reach at most 600 positions past an output.
+bool gemm_packs_lines(const LayerShape& s, int operand);
 
 // True when the GEMM scheme can take x itself as its left operand (no patch matrix): a 1x1 stride-1 unpadded
 // ungrouped layer with H*W >= 32 and a multiple of 4, single-pass TF32 operands.

@@ -74,3 +74,31 @@ def test_more_than_the_staged_bias(torch):
     layer = W.ConvLayer("lines", 4, 32, 2100, 20, 20, 3, 2, 1, relu=True, seed=5)
     x, w, b = W.make_inputs(layer)
     assert_close(run(torch, layer, (x, w, b)), oc.direct_conv(x, w, b, 2, 1, 1, 1, True), B.PREC_TF32, "packed lines")
+
+
+# BF16 operands: blocks of 64 channels; one and several blocks, phases, ragged channel tiles, one and two tiles of cells per
+# item, and a layer that leaves the Winograd scheme for this form by itself.  Integers are exact in BF16.
+@pytest.mark.parametrize("shape,auto", [((20, 64, 40, 17, 19, 3, 1, 1, 1), False), ((90, 64, 130, 15, 13, 3, 2, 1, 1), False),
+                                        ((6, 192, 272, 37, 33, 3, 1, 3, 3), False), ((30, 128, 48, 26, 28, 5, 2, 2, 1), False),
+                                        ((40, 64, 64, 47, 51, 2, 2, 1, 1), False), ((64, 64, 64, 56, 56, 3, 1, 1, 1), True)])
+def test_bf16(torch, shape, auto):
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    layer = W.ConvLayer("lines", N, Cin, Cout, H, W_, k, s, p, d, relu=True, seed=sum(shape))
+    r = B.ConvLayerRunner(N, Cin, Cout, H, W_, k, s, p, d,
+                          B.make_opts(relu=True, precision=B.PREC_BF16, **({} if auto else dict(force_algo=B.ALGO_GEMM, operand=B.OPERAND_BF16))))
+    assert (r.info.algo, r.info.gemm_lhs, r.info.operand) == (B.ALGO_GEMM, B.GEMM_LHS_PACKED, B.OPERAND_BF16)
+    r.workspace.fill_(0xFF)                   # NaNs wherever a kernel reads what none has written
+    B.mnn_conv_set_workspace(r.plan, r._ws_ptr, r.info.workspace_bytes)
+    for exact in (True, False):
+        x, w, b = W.integer_inputs(layer, -3, 3) if exact else W.make_inputs(layer)
+        wd = to_dev(torch, w)
+        r.prepare(wd)
+        got = r.run(to_dev(torch, x), wd, to_dev(torch, b))
+        torch.cuda.synchronize()
+        assert r.device_status() == 0
+        ref = oc.direct_conv(x, w, b, s, p, d, 1, True)
+        if exact:
+            assert np.array_equal(got.cpu().numpy().astype(np.float64), ref)
+        else:
+            assert_close(got.cpu().numpy(), ref, B.PREC_BF16, "packed lines in BF16")
+    r.close()

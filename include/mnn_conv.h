@@ -291,7 +291,7 @@ MNN_API int mnn_strassen_rule(long long m, long long n, long long k);
  * consts[2] attoseconds per TF32 tensor flop  consts[3] attoseconds per BF16 tensor flop
  * consts[4] attoseconds per fp32 ALU flop     consts[5] picoseconds of fixed cost per kernel (launch, ramp-up, tail)
  * consts[6] L2 bytes usable for one chunk     consts[7] number of SMs
- * consts[8] attoseconds per flop of the direct kernel
+ * consts[8] attoseconds per flop of the direct kernel on layers too small to fill the chip
  * consts[9] attoseconds per flop of the direct kernel for layers with at most 4 input channels
  *            (measured on 3 -> 32, 3x3, stride 2, padding 1, which has a kernel of its own; the other shapes
  *            with at most 4 input channels are booked at twice this figure)

@@ -134,8 +134,14 @@ def direct_cost(L: Layer, c) -> int:
     # within 48 KiB), which has its own kernel; the other few-channel shapes run at half that rate
     fast = (L.Cin == 3 and L.k == 3 and L.stride == 2 and L.pad == 1 and L.dil == 1 and L.H % 2 == 0 and L.W % 4 == 0
             and 27 * (cdiv(L.Cout, 32) * 32) * 4 <= 48 * 1024)
-    rate = (c[9] if fast else 2 * c[9]) if few_channels else c[8]
-    return kernel_ps(c, mem_as=traffic * c[0], alu_as=flops * rate)
+    if few_channels:
+        return kernel_ps(c, mem_as=traffic * c[0], alu_as=flops * (c[9] if fast else 2 * c[9]))
+    # c[8] is the rate of layers too small to fill the chip; for k > 1 the lesser of that and 13.3 ns per patch element plus the
+    # arithmetic at three tenths of it
+    alu = flops * c[8]
+    if L.k > 1:
+        alu = min(alu, cpg * L.k * L.k * 13300000000 + flops * c[8] * 3 // 10)
+    return kernel_ps(c, mem_as=traffic * c[0], alu_as=alu)
 
 
 # ---------------------------------------------------------------------------------------

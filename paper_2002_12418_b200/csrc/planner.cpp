@@ -12,6 +12,7 @@
 
 #include "line_plan.h"
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -53,7 +54,7 @@ Calibration default_calibration()
     c.c[5] = 3530000;     // ps of fixed cost per kernel: launch, ramp-up and tail (the t_schedule of Eq. 5)
     c.c[6] = 80ll << 20;  // L2 bytes one chunk's V + M may occupy
     c.c[7] = 148;         // SMs
-    c.c[8] = 571000;      // as per flop of the direct kernel (~3.5 TFLOP/s)
+    c.c[8] = 571000;      // as per flop of the direct kernel on layers too small to fill the chip (~1.8 TFLOP/s; 13 on large ones)
     c.c[9] = 31000;       // as per flop of the 3 -> Cout 3x3 stride-2 kernel (~32 TFLOP/s); other Cin <= 4 shapes: twice that
     c.c[10] = 23000000;   // as per byte of U delivered to one SM by the fused kernel's weight stream (~43 GB/s per SM)
     c.c[11] = 6000000;    // ps per 32-channel block of a fused work item (64 MMAs of 128 x 32 x 8 at ~90 ns each)
@@ -315,8 +316,15 @@ uint64_t direct_cost(const LayerShape& s, const Calibration& cal)
     // pixels per thread); the other few-channel shapes run the one-pixel kernel at half that rate
     const bool pixel_blocks = s.Cin == 3 && s.k == 3 && s.stride == 2 && s.pad == 1 && s.dil == 1 && s.H % 2 == 0 &&
                               s.W % 4 == 0 && (long long)27 * ((s.Cout + 31) / 32 * 32) * 4 <= 48 * 1024;
-    const uint64_t rate = (uint64_t)(stem ? (pixel_blocks ? cal.c[9] : 2 * cal.c[9]) : cal.c[8]);
-    return kernel_ps((u128)(x_bytes + y_bytes + w_bytes) * (uint64_t)cal.c[0], 0, (u128)flops * rate, cal);
+    if (stem) return kernel_ps((u128)(x_bytes + y_bytes + w_bytes) * (uint64_t)cal.c[0], 0, (u128)flops * (uint64_t)(pixel_blocks ? cal.c[9] : 2 * cal.c[9]), cal);
+    // consts[8] is the rate of layers too small to fill the chip.  For k > 1, where it overstates those with short patches, the
+    // lesser of that and what the tile kernel spends on a patch (13.3 ns per element: trips to memory, whatever the size) plus
+    // its arithmetic at three tenths of the constant.  One image: 24 -> 40 at 33 x 31 (216 elements) 7.0 us, the patch
+    // matrix 14.1; 32 -> 32 at 28 x 28 (288) 6.8 us, Winograd 9.2; 64 -> 64 at 28 x 28 (576) 13.6 us, Winograd 8.7.
+    const uint64_t patch = (uint64_t)(s.Cin / s.groups) * s.k * s.k;
+    u128 alu = (u128)flops * (uint64_t)cal.c[8];
+    if (s.k > 1) alu = std::min(alu, (u128)patch * 13300000000ull + (u128)flops * (uint64_t)cal.c[8] * 3u / 10u);
+    return kernel_ps((u128)(x_bytes + y_bytes + w_bytes) * (uint64_t)cal.c[0], 0, alu, cal);
 }
 
 }  // namespace

@@ -478,9 +478,9 @@ uint64_t winograd_chunk_cost(const LayerShape& s, int m, int operand, int passes
     const uint64_t y_bytes = 4ull * n * s.Cout * s.OH * s.OW;
     const uint64_t cV = (uint64_t)(resident ? cal.c[1] : cal.c[0]);
     const uint64_t c0 = (uint64_t)cal.c[0], cA = (uint64_t)cal.c[4];
-    // from alpha = 8 on a lane of the input transform holds one channel instead of a packed pair (twice the ALU
-    // time) and does the tile in sweeps of columns; measured against the pair form: x 2 at alpha = 8, x 2.25 at
-    // alpha = 10, x 4 at alpha = 12 (quarters: 8, 9, 16)
+    // larger tiles cost the input transform more per multiply-add: x 2 at alpha = 8, x 2.25 at alpha = 10, x 4 at alpha = 12
+    // (quarters: 8, 9, 16), measured on a form that did them in sweeps of columns; the two-pass kernel needs less, so this is
+    // an upper bound
     const u128 tile_channels_in = (u128)n * tiles_img * (uint64_t)s.Cin, tile_channels_out = (u128)n * tiles_img * (uint64_t)s.Cout;
     const u128 in_alu = (alpha >= 12 ? 16u : (alpha >= 10 ? 9u : (alpha >= 8 ? 8u : 4u))) * alpha * a2 * tile_channels_in * cA;
     const uint64_t in = kernel_ps((u128)x_bytes * c0 + (u128)v_bytes * cV, 0, in_alu, cal);

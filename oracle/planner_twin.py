@@ -192,9 +192,11 @@ def packs_lines(L: Layer, operand: int) -> bool:
     if L.groups != 1 or not 2 <= L.k <= 7 or L.stride > 4 or not channels:
         return False
     reach = (L.k - 1) * L.dil // L.stride
-    wq, hq = L.OW + reach, L.OH + reach
+    row, hq = L.OW + reach, L.OH + reach
+    strips = cdiv(L.OW, 16)                                # few channels: strips of equal width
+    wq = max(row, strips * cdiv(L.OW, strips)) if L.Cin % 32 else row
     cells = L.N * hq * wq
-    return (reach * (wq + 1) <= 600 and cells < 2 ** 30
+    return (reach * (row + 1) <= 600 and cells < 2 ** 30
             and L.stride ** 2 * (cells + 2048) * (cdiv(L.Cin, 32) * 32) * _bytes_of(operand) <= 4 << 30)
 
 

@@ -363,9 +363,11 @@ bool gemm_packs_lines(const LayerShape& s, int operand)
     if (s.groups != 1 || s.k < 2 || s.k > 7 || s.stride > 4 || !(s.Cin % block == 0 || (block == 32 && s.Cin * s.k <= 32))) return false;
     // rows of cells a tap can reach past an output, bounds of the grid of cells and of the packed planes
     const long long reach = (long long)(s.k - 1) * s.dil / s.stride;
-    const long long wq = s.OW + reach, hq = s.OH + reach;
+    const long long few_strips = (s.OW + 15) / 16;                 // few channels: strips of equal width, together up to strips - 1 columns wider
+    const long long row = s.OW + reach, hq = s.OH + reach;
+    const long long wq = s.Cin % block ? std::max(row, few_strips * ((s.OW + few_strips - 1) / few_strips)) : row;
     const u128 cells = (u128)s.N * (u128)hq * (u128)wq, planes = (u128)(s.stride * s.stride), a_bytes = operand_bytes(operand) * (u128)((s.Cin + 31) / 32 * 32);
-    return reach * (wq + 1) <= 600 && cells < (1u << 30) && planes * (cells + 2048) * a_bytes <= (u128)(4ll << 30);
+    return reach * (row + 1) <= 600 && cells < (1u << 30) && planes * (cells + 2048) * a_bytes <= (u128)(4ll << 30);
 }
 
 bool gemm_reads_x(const LayerShape& s, int operand, int passes)

@@ -302,6 +302,21 @@ def test_first_minimum_wins_ties_and_inadmissible_is_never_chosen():
     assert ch.algo == T.ALGO_DIRECT and all(c == T.INADMISSIBLE for c in ch.cost_ps[1:])
 
 
+# Few-channel packed lines cut a row into equal strips, together up to strips - 1 columns wider than the row: just below the
+# 4 GiB bound of the packed planes the tiling must not find fewer bytes than the choice counted (the plan would fail).
+@pytest.mark.parametrize("Cin,k,OW", [(3, 2, 49), (3, 2, 113), (4, 3, 113), (10, 3, 49)])
+def test_every_layer_near_the_packed_bound_plans(Cin, k, OW):
+    strips = -(-OW // 16)
+    at_bound = (4 << 30) // (128 * (OW + k - 1) * max(OW + k - 1, strips * -(-OW // strips)))
+    seen = set()
+    for N in range(at_bound - 8, int(at_bound * 1.08), max(1, at_bound // 200)):
+        layer = W.ConvLayer("near", N, Cin, 64, OW + k - 1, OW + k - 1, k, 1, 0, relu=False)
+        info = compare(layer, dict(force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1),
+                       dict(force_algo=T.ALGO_GEMM, operand=T.OPERAND_TF32, passes=1), B.mnn_get_calibration())
+        seen.add(info.gemm_lhs == B.GEMM_LHS_PACKED)
+    assert seen == {True, False}
+
+
 def test_routing_rules():
     t = ppm_table()
     for l in all_layers():

@@ -335,54 +335,66 @@ __global__ void __launch_bounds__(kTileThreads) direct_tile_kernel(const float* 
     const long long plane = (long long)g.H * g.W;
     const float* xb = x + (n * g.Cin + (long long)grp * cpg) * plane + (long long)ih0 * g.W + iw0;
     const float* wb = w + (size_t)(grp * opg + co0) * K;
+    // A tap outside the image adds its weight times zero, which is nothing if the weight is finite.  Where that, or the input,
+    // left a sum that is no number, the CTA goes over its patches again and passes such taps over.
     float acc[TCO];
+    for (bool careful = false;; careful = true) {
 #pragma unroll
-    for (int j = 0; j < TCO; ++j) acc[j] = 0.0f;
-
-    for (int k0 = 0; k0 < K; k0 += kTileChunk) {
-        const int kn = min(kTileChunk, K - k0);
-        if (k0) __syncthreads();
-        for (int i = threadIdx.x; i < kn; i += kTileThreads) {
-            const int kk = k0 + i, ci = kk / k2, e = kk - ci * k2, a = e / g.k, b = e - a * g.k;
-            s_off[i] = ((ci * plane + (long long)a * g.dil * g.W + b * g.dil) << 8) | (a << 4) | b;
-        }
-        // eight elements x four channels per warp and step
-        constexpr int kLc = 4, kLe = 8;
-        const int le = lane % kLe, lc = lane / kLe;
-        for (int e0 = warp * kLe; e0 < kn; e0 += 8 * kLe)
-#pragma unroll
-            for (int c = 0; c < TCO; c += kLc)
-                if (e0 + le < kn) s_w[(e0 + le) * kRow + c + lc] = c + lc < n_co ? __ldg(wb + (size_t)(c + lc) * K + k0 + e0 + le) : 0.0f;
-        __syncthreads();
-        const int i0 = kn * slice / kw, i1 = kn * (slice + 1) / kw;
-        int i = i0;
-        auto load = [&](int idx) {
-            const long long o = s_off[idx];
-            const bool ok = ((rows_in >> ((unsigned)o >> 4 & 15u)) & (cols_in >> ((unsigned)o & 15u)) & 1u) != 0;
-            return ok ? __ldg(xb + (o >> 8)) : 0.0f;
-        };
-        auto fma_row = [&](float v, int idx) {
-            const float* wr = s_w + idx * kRow;
-#pragma unroll
-            for (int q = 0; q < TCO / 4; ++q) {
-                const float4 w4 = *reinterpret_cast<const float4*>(wr + 4 * q);
-                acc[4 * q] = fmaf(w4.x, v, acc[4 * q]);
-                acc[4 * q + 1] = fmaf(w4.y, v, acc[4 * q + 1]);
-                acc[4 * q + 2] = fmaf(w4.z, v, acc[4 * q + 2]);
-                acc[4 * q + 3] = fmaf(w4.w, v, acc[4 * q + 3]);
+        for (int j = 0; j < TCO; ++j) acc[j] = 0.0f;
+        for (int k0 = 0; k0 < K; k0 += kTileChunk) {
+            const int kn = min(kTileChunk, K - k0);
+            if (k0) __syncthreads();
+            for (int i = threadIdx.x; i < kn; i += kTileThreads) {
+                const int kk = k0 + i, ci = kk / k2, e = kk - ci * k2, a = e / g.k, b = e - a * g.k;
+                s_off[i] = ((ci * plane + (long long)a * g.dil * g.W + b * g.dil) << 8) | (a << 4) | b;
             }
-        };
-        for (; i + 8 <= i1; i += 8) {
-            float v[8];
+            // eight elements x four channels per warp and step
+            constexpr int kLc = 4, kLe = 8;
+            const int le = lane % kLe, lc = lane / kLe;
+            for (int e0 = warp * kLe; e0 < kn; e0 += 8 * kLe)
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = load(i + u);
+                for (int c = 0; c < TCO; c += kLc)
+                    if (e0 + le < kn) s_w[(e0 + le) * kRow + c + lc] = c + lc < n_co ? __ldg(wb + (size_t)(c + lc) * K + k0 + e0 + le) : 0.0f;
+            __syncthreads();
+            const int i0 = kn * slice / kw, i1 = kn * (slice + 1) / kw;
+            int i = i0;
+            auto inside = [&](long long o) { return ((rows_in >> ((unsigned)o >> 4 & 15u)) & (cols_in >> ((unsigned)o & 15u)) & 1u) != 0; };
+            auto load = [&](int idx) {
+                const long long o = s_off[idx];
+                return inside(o) ? __ldg(xb + (o >> 8)) : 0.0f;
+            };
+            auto fma_row = [&](float v, int idx) {
+                const float* wr = s_w + idx * kRow;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) fma_row(v[u], i + u);
+                for (int q = 0; q < TCO / 4; ++q) {
+                    const float4 w4 = *reinterpret_cast<const float4*>(wr + 4 * q);
+                    acc[4 * q] = fmaf(w4.x, v, acc[4 * q]);
+                    acc[4 * q + 1] = fmaf(w4.y, v, acc[4 * q + 1]);
+                    acc[4 * q + 2] = fmaf(w4.z, v, acc[4 * q + 2]);
+                    acc[4 * q + 3] = fmaf(w4.w, v, acc[4 * q + 3]);
+                }
+            };
+            if (careful) {
+#pragma unroll 1
+                for (; i < i1; ++i)
+                    if (inside(s_off[i])) fma_row(load(i), i);
+                continue;
+            }
+            for (; i + 8 <= i1; i += 8) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = load(i + u);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) fma_row(v[u], i + u);
+            }
+            for (; i < i1; ++i) fma_row(load(i), i);
         }
-        for (; i < i1; ++i) fma_row(load(i), i);
+        int nan = 0;
+#pragma unroll
+        for (int j = 0; j < TCO; ++j) nan |= acc[j] != acc[j];
+        if (!__syncthreads_or(nan) || careful) break;
     }
     if (kw > 1) {
-        __syncthreads();
         float* red = s_w;                                           // [warp][TCO][32]
 #pragma unroll
         for (int j = 0; j < TCO; ++j) red[(warp * TCO + j) * 32 + lane] = acc[j];

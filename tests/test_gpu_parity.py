@@ -487,6 +487,23 @@ def test_direct_tiles(torch, N, Cin, Cout, H, W_, k, stride, dil, groups):
     assert np.array_equal(goti.astype(np.float64), oracle(layer, xi, wi, bi))
 
 
+# A tap outside the image is no term of the sum: an infinite weight reaches the outputs whose tap lies inside and no others.
+@pytest.mark.parametrize("N,Cin,Cout,H,W_,k,groups", [(1, 12, 24, 9, 10, 3, 2), (2, 130, 5, 12, 10, 3, 1), (40, 16, 48, 33, 30, 3, 2),
+                                                      (1, 20, 12, 14, 14, 5, 4)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_direct_weights_that_are_not_finite(torch, N, Cin, Cout, H, W_, k, groups, bad):
+    layer = W.ConvLayer("t", N, Cin, Cout, H, W_, k, 1, k // 2, groups=groups, relu=False, seed=Cin)
+    x, w, b = W.integer_inputs(layer)
+    w[1, 0, 0, 0] = bad                       # the upper left tap: outside for the first k / 2 rows and columns
+    w[2, -1, k - 1, k // 2] = bad             # the lower middle tap
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (x, w, b))
+    assert info.algo == B.ALGO_DIRECT
+    want = oracle(layer, x, w, b)
+    assert np.isfinite(want[:, 1, :k // 2]).all() and not np.isfinite(want[:, 1, k // 2:, k // 2:]).any()
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
+    assert np.array_equal(np.where(np.isfinite(want), got.astype(np.float64), 0.0), np.where(np.isfinite(want), want, 0.0))
+
+
 # Depthwise planes cut into bands of 4, 8, 16 and 32 rows (fewer planes, shorter bands), the last band partial, and 7 x 7
 # planes held whole at odd width; the 3 -> Cout stride-2 kernel with its output channels shared out (few images, Cout off
 # the chunk of 16).

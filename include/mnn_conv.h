@@ -96,8 +96,10 @@ enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_ST
  *              shared-memory operand tile themselves (single-pass TF32 operands, rounded
  *              to nearest).  AUTO = the planner takes the cheapest that applies; it may also report
  *              PACKED (not an option value): x is re-laid into lines of positions, rounded to nearest
- *              (TF32 or BF16), and every kernel tap reads them at a shifted start.  Asking
- *              for X or IMPLICIT where it does not apply fails the plan.
+ *              (TF32 or BF16), and every kernel tap reads them at a shifted start.  The lines are about
+ *              as large as x (in the operand format) and lie in the workspace, up to 4 GiB, where
+ *              IMPLICIT needs room for the weights only: ask for that where workspace is short.
+ *              Asking for X or IMPLICIT where it does not apply fails the plan.
  *   fused      Winograd F(2x2, 3x3) as ONE kernel (input transform, contraction and output
  *              transform fused; the transformed tensors V and M never reach device memory):
  *              0 = the planner weighs it against the other candidates, 1 = never,
@@ -252,7 +254,9 @@ MNN_API void mnn_conv_destroy(mnn_conv_plan_t plan);
  * Limits and rules:
  *   - plans whose info.workspace_bytes exceed MNN_STATIC_WORKSPACE_BYTES are
  *     rejected with MNN_EWORKSPACE (nothing is launched); plan with a smaller
- *     batch, or a smaller tile size, to fit.
+ *     batch, or a smaller tile size, to fit.  A plan that the planner put on packed
+ *     lines (info.gemm_lhs PACKED) and that does not fit runs here as it would be
+ *     planned without them, and is rejected only if that does not fit either.
  *   - the first call on each device looks up the array's device address (with
  *     that device current); make that first call outside any stream capture.
  *     The current device must be the device of `stream` in every call.

@@ -49,6 +49,7 @@ struct mnn_conv_plan_s {
     LayerShape s;
     mnn_conv_opts o;
     Decision d;
+    Decision d_unpacked;             // where d takes packed lines: the decision without them (mnn_conv_run_static)
     int store_mode = STORE_TF32;
     int cin_pad = 0;                 // row length of U and V (Winograd: padded Cin; GEMM: padded Cin*k*k)
     long long chunk_tiles = 0;       // capacity of V / M in tiles (or GEMM columns)
@@ -170,6 +171,38 @@ void layout_workspace(mnn_conv_plan_t p)
     p->workspace_bytes = off;
 }
 
+LineShape line_shape(mnn_conv_plan_t p)
+{
+    const LayerShape& s = p->s;
+    return {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.stride, s.dil, s.pad, s.OH, s.OW, p->d.operand == MNN_OPERAND_BF16};
+}
+
+// Form, transform matrices and workspace layout of the decision in p->d (square layers).
+int realise_decision(mnn_conv_plan_t p, const char** why)
+{
+    p->packed = p->fused = p->gemm_x = p->gemm_implicit = false;
+    if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
+        p->packed = line_plan(line_shape(p), 148, &p->lc.p);
+        if (!p->packed) {
+            *why = "no tiling of the packed-line product fits this layer";
+            return MNN_EUNSUPPORTED;
+        }
+    }
+    if (p->d.algo == MNN_ALGO_WINOGRAD) {
+        WinogradMatrices wm;
+        if (!generate_winograd(p->d.m, p->s.k, p->d.points_id, &wm) || p->d.alpha > 12 || p->d.m > 6 || p->s.k > 7) {
+            *why = "no transform matrices for this (m, k, points)";
+            return MNN_EUNSUPPORTED;
+        }
+        std::memset(&p->mats, 0, sizeof(p->mats));
+        std::memcpy(p->mats.At, wm.At32.data(), wm.At32.size() * sizeof(float));
+        std::memcpy(p->mats.G, wm.G32.data(), wm.G32.size() * sizeof(float));
+        std::memcpy(p->mats.Bt, wm.Bt32.data(), wm.Bt32.size() * sizeof(float));
+    }
+    layout_workspace(p);
+    return MNN_OK;
+}
+
 bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; }
 
 // Brackets one launch with events when profiling is on.
@@ -274,40 +307,21 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
     const char* why = "";
     mnn_conv_opts o_plan = o;
     if (p->strassen) o_plan.passes = 1;      // the candidate list holds single-pass GEMMs; the pass count is set below
-    int rc = plan_layer(s, o_plan, current_calibration(), &p->d, &why);
-    if (rc != MNN_OK) {
-        fail(rc, why);
-        delete p;
-        return nullptr;
-    }
-    if (p->strassen) {
+    const Calibration cal = current_calibration();
+    int rc = plan_layer(s, o_plan, cal, true, &p->d, &why);
+    if (rc == MNN_OK && p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) rc = plan_layer(s, o_plan, cal, false, &p->d_unpacked, &why);
+    if (rc == MNN_OK && p->strassen) {
         p->d.passes = o.passes;
         p->d.chosen = -1;
         p->d.gemm_lhs = MNN_GEMM_LHS_PATCHES;
         p->d.error_ppm = accuracy_ppm(1, 1, 0, p->d.operand, p->d.passes);
     }
-    if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
-        const LineShape ls = {N, Cin, Cout, H, W, k, stride, dilation, pad, s.OH, s.OW, p->d.operand == MNN_OPERAND_BF16};
-        p->packed = line_plan(ls, 148, &p->lc.p);
-        if (!p->packed) {
-            fail(MNN_EUNSUPPORTED, "no tiling of the packed-line product fits this layer");
-            delete p;
-            return nullptr;
-        }
+    if (rc == MNN_OK) rc = realise_decision(p, &why);
+    if (rc != MNN_OK) {
+        fail(rc, why);
+        delete p;
+        return nullptr;
     }
-    if (p->d.algo == MNN_ALGO_WINOGRAD) {
-        WinogradMatrices wm;
-        if (!generate_winograd(p->d.m, k, p->d.points_id, &wm) || p->d.alpha > 12 || p->d.m > 6 || k > 7) {
-            fail(MNN_EUNSUPPORTED, "no transform matrices for this (m, k, points)");
-            delete p;
-            return nullptr;
-        }
-        std::memset(&p->mats, 0, sizeof(p->mats));
-        std::memcpy(p->mats.At, wm.At32.data(), wm.At32.size() * sizeof(float));
-        std::memcpy(p->mats.G, wm.G32.data(), wm.G32.size() * sizeof(float));
-        std::memcpy(p->mats.Bt, wm.Bt32.data(), wm.Bt32.size() * sizeof(float));
-    }
-    layout_workspace(p);
     return p;
 }
 
@@ -1144,14 +1158,21 @@ extern "C" int mnn_conv_run_static(mnn_conv_plan_t p, const float* x, const floa
 {
     if (!p) return fail(MNN_EINVAL, "NULL plan");
     if (!x || !w || !y) return fail(MNN_EINVAL, "NULL tensor pointer");
-    if (p->workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES)
-        return fail(MNN_EWORKSPACE, "this plan needs " + std::to_string(p->workspace_bytes) +
-                                        " workspace bytes; the built-in workspace holds " +
-                                        std::to_string((long long)MNN_STATIC_WORKSPACE_BYTES));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // A private copy of the host-side plan whose workspace is the built-in array: the caller's
     // plan (its own workspace, prepared weights, profiling state) is left untouched.
     mnn_conv_plan_s local = *p;
+    if (p->packed && p->workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES) {
+        // packed planes do not fit: the layer as it is planned without them (the implicit gather stores none)
+        const char* why = "";
+        local.d = p->d_unpacked;
+        const int rc = realise_decision(&local, &why);
+        if (rc != MNN_OK) return fail(rc, why);
+    }
+    if (local.workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES)
+        return fail(MNN_EWORKSPACE, "this plan needs " + std::to_string(local.workspace_bytes) +
+                                        " workspace bytes; the built-in workspace holds " +
+                                        std::to_string((long long)MNN_STATIC_WORKSPACE_BYTES));
     local.profiling = false;
     local.events.clear();
     local.event_stage.clear();

@@ -569,7 +569,7 @@ void winograd_chunking(const LayerShape& s, int m, int operand, int passes, cons
     *cost_ps = best_cost;
 }
 
-int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, Decision* d, const char** err)
+int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, bool packed_lines, Decision* d, const char** err)
 {
     static const int kM[3] = {2, 4, 6};
     for (int i = 0; i < MNN_N_CANDIDATES; ++i) d->cost_ps[i] = MNN_COST_INADMISSIBLE;
@@ -647,7 +647,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 // cost stays that of the operand chosen above, an upper bound.
                 if (implicit_ok && !pointwise && cal.c[13] > 0 && gemm_split(s, cal) > 1) {
                     if (lhs == MNN_GEMM_LHS_PATCHES) lhs = MNN_GEMM_LHS_IMPLICIT;
-                } else if (gemm_packs_lines(s, c.operand) &&
+                } else if (packed_lines && gemm_packs_lines(s, c.operand) &&
                            packed_cost(s, c.operand, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
                     lhs = MNN_GEMM_LHS_PACKED;
                 }

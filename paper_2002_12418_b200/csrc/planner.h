@@ -75,11 +75,13 @@ int best_points(int m, int k, int operand, int passes, long long* ppm_out);
 void winograd_chunking(const LayerShape& s, int m, int operand, int passes, const Calibration& cal,
                        int* chunk_images, int* n_chunks, uint64_t* cost_ps);
 
-// Fills *d.  Returns MNN_OK or an mnn_status with *err set to a static reason.
 // True when the layer's shape admits the fused Winograd F(2x2, 3x3) kernel.
 bool fused_shape_ok(const LayerShape& s);
 
-int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, Decision* d, const char** err);
+// Fills *d.  Returns MNN_OK or an mnn_status with *err set to a static reason.  packed_lines = false keeps the GEMM scheme from
+// packed lines, the one left operand chosen by itself whose workspace can far exceed the patch matrix's or the implicit
+// gather's.
+int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, bool packed_lines, Decision* d, const char** err);
 
 // True when the Winograd kernels exist for (m, k).
 bool winograd_supported(int m, int k);

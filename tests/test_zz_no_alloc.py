@@ -70,6 +70,31 @@ def test_static_workspace_run_matches_workspace_run_twice():
     _both_ways(torch, e, B.make_opts(relu=1, fused=B.FUSED_ONLY))
 
 
+# Layers planned on packed lines whose planes do not fit the built-in array, but whose implicit gather or patch matrix does:
+# they run as the plan that asks for that operand, bit for bit.
+@pytest.mark.parametrize("shape,lhs", [((12, 3, 64, 160, 160, 3, 1, 1, 1), B.GEMM_LHS_IMPLICIT), ((8, 64, 48, 140, 137, 3, 2, 1, 1), B.GEMM_LHS_IMPLICIT),
+                                       ((8, 64, 24, 150, 120, 3, 1, 2, 2), B.GEMM_LHS_IMPLICIT), ((12, 4, 128, 224, 224, 3, 2, 1, 1), B.GEMM_LHS_PATCHES)])
+def test_static_workspace_where_the_packed_planes_do_not_fit(shape, lhs):
+    import torch
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    layer = W.ConvLayer("planes", N, Cin, Cout, H, W_, k, s, p, d, relu=True, seed=sum(shape))
+    x, w, b = W.make_inputs(layer)
+    xd, wd, bd = to_dev(torch, x), to_dev(torch, w), to_dev(torch, b)
+    gemm = dict(relu=1, force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1)
+    plan = B.mnn_conv_plan_ex(*shape, B.make_opts(**gemm))
+    info = B.mnn_conv_plan_query(plan)
+    assert info.gemm_lhs == B.GEMM_LHS_PACKED and info.workspace_bytes > B.STATIC_WORKSPACE_BYTES
+    y = torch.full((N, Cout, info.OH, info.OW), float("nan"), device="cuda:0")
+    B.mnn_conv_run_static(plan, xd.data_ptr(), wd.data_ptr(), bd.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    B.mnn_conv_destroy(plan)
+    r = B.ConvLayerRunner(*shape, B.make_opts(gemm_lhs=lhs, **gemm))
+    y_ref = r.run(xd, wd, bd)
+    torch.cuda.synchronize()
+    assert r.device_status() == 0 and torch.equal(y, y_ref)
+    r.close()
+    assert_close(y.cpu().numpy(), oc.direct_conv(x, w, b, s, p, d, 1, True), B.PREC_TF32, "packed planes that do not fit")
+
+
 def test_static_workspace_rejects_plans_that_do_not_fit():
     import torch
     big = W.ConvLayer("big", 32, 256, 256, 56, 56, 3, 1, 1, seed=1)

@@ -310,6 +310,58 @@ def gemm_cost(L: Layer, operand: int, lhs, c) -> int:
     return sat(gather + contract)
 
 
+def staged_gather(L: Layer):
+    """(time in ps of a CTA's serial loads, CTAs) of the gather staged through shared memory, or (0, 0) where it does not
+    serve: output positions in segments of at most 64 columns, at most 64 positions per CTA (128 / 256 for short rows of V), a
+    slab of at most 64 groups of four patch elements whose input region fits 9216 floats; half a microsecond per step of
+    region rows (eight warps), 0.2 us for each further 32 columns."""
+    if L.k == 1:
+        return 0, 0
+    groups, k2 = cdiv(L.Cin * L.k * L.k, 8) * 2, L.k * L.k
+    width = cdiv(L.OW, cdiv(L.OW, 64))
+    rows = max(1, min((256 if groups <= 16 else 128 if groups <= 32 else 64) // width, L.OH))
+    rh = (rows - 1) * L.stride + (L.k - 1) * L.dil + 1
+    rw = (width - 1) * L.stride + (L.k - 1) * L.dil + 1
+
+    def channels(q):
+        return (4 * q + k2 - 2) // k2 + 1
+    fitting = [q for q in {min(q, groups) for q in range(8, 65, 8)} if channels(q) * rh * rw <= 9216]
+    if not fitting:
+        return 0, 0
+    slab, lanes = max(fitting), 32
+    while lanes > 1 and lanes // 2 >= rw:
+        lanes //= 2
+    return (cdiv(channels(slab) * rh, 8 * (32 // lanes)) * (300000 + 200000 * cdiv(rw, lanes)),
+            L.N * cdiv(L.OH, rows) * cdiv(L.OW, width) * cdiv(groups, slab))
+
+
+def patch_operand_time(L: Layer, lhs, c):
+    """Time in ps of the TF32 GEMM scheme over patches that are written first (LHS_PATCHES) or gathered by producer warps
+    (LHS_IMPLICIT), the K loop cut over clusters; chooses between the two where the loop is cut."""
+    sms = c[7] if c[7] > 0 else 148
+    Kp, T = cdiv(L.Cin * L.k * L.k, 8) * 8, L.N * L.OH * L.OW
+    bn, co_blocks = contraction_tiling(cdiv(T, 128), 1, L.Cout, sms)
+    items = cdiv(T, 128) * co_blocks
+    rounds, split = cdiv(items, sms), cluster_split(items, cdiv(Kp, 32), sms)
+    x, y, v, u = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW, T * Kp * 4, L.Cout * Kp * 4
+    drain = 128 * bn * 4 * 45
+    if lhs == LHS_IMPLICIT:
+        gather = 128 * 32 * c[13] * 5 // 8 // 10 ** 6
+        block = max(gather * 15 // 8 if L.Cin % 32 else gather * 2 if L.stride >= 4 else gather, bn * 128 * 16)
+        fixed, traffic = 3000000 if split > 1 else 0, x + u + y
+    else:
+        serial, ctas = staged_gather(L)
+        moved = (x + v) * c[0] // 10 ** 6
+        if serial:
+            fixed = 5500000 + max(serial, serial * cdiv(ctas, 4 * sms) * 3 // 4) + moved * 6 // 5
+        else:
+            fixed = max(5500000, moved * 5)
+        block = max((128 * 128 + bn * 128) * 16, 2 * 128 * bn * 32 * c[2] * sms // 10 ** 6) * 3 // 5
+        traffic = v + u + y
+    item = max(cdiv(cdiv(Kp, 32), split) * block, drain + 500000)
+    return fixed + kernel_ps(c, mem_as=traffic * c[0], tensor_as=(rounds * item + drain // 2) * 10 ** 6)
+
+
 # ---------------------------------------------------------------------------------------
 # Winograd F(m x m, k x k) as three kernels (Eq. 6), chunked over the batch.
 # ---------------------------------------------------------------------------------------
@@ -459,14 +511,14 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 if implicit_ok and not (L.k == 1 and L.stride == 1) and c[13] > 0 and costs[LHS_IMPLICIT] < costs[lhs]:
                     lhs = LHS_IMPLICIT
                 costs_of = lhs
-                # items so few that their K loop is cut over clusters: the implicit gather instead of patches; else packed
-                # lines where they apply.  Booked at the cost of the operand chosen above.
+                # items so few that their K loop is cut over clusters: the implicit gather instead of patches where that takes
+                # less; else packed lines where they apply.  Booked at the cost of the operand chosen above.
                 sms = c[7] if c[7] > 0 else 148
                 blocks = cdiv(L.N * L.OH * L.OW, 128)
                 _, co_blocks = contraction_tiling(blocks, 1, L.Cout, sms)
                 cut = cluster_split(blocks * co_blocks, cdiv(cdiv(L.Cin * L.k * L.k, 8) * 8, 32), sms) > 1
                 if implicit_ok and cut and not (L.k == 1 and L.stride == 1) and c[13] > 0:
-                    if lhs == LHS_PATCHES:
+                    if lhs == LHS_PATCHES and patch_operand_time(L, LHS_IMPLICIT, c) < patch_operand_time(L, LHS_PATCHES, c):
                         lhs = LHS_IMPLICIT
                 elif packs_lines(L, operand) and packed_cost(L, operand, c) < costs[lhs]:
                     lhs = LHS_PACKED

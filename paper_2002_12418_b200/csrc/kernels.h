@@ -106,6 +106,8 @@ struct GatherGeom {
     int N, Cin, H, W, OH, OW, k, stride, pad, dil, k_pad;
 };
 cudaError_t launch_gather(const float* x, void* V_hi, void* V_lo, const GatherGeom& g, int mode, cudaStream_t stream);
+// The gather staged through shared memory: time in ps of a CTA's serial loads, and its CTAs; 0 where another gather serves.
+long long staged_gather_ps(const GatherGeom& g, long long* ctas);
 
 // Epilogue of a contraction: 0 = write M[xi][co][t]; 1 = write y[n][co][pix] = act(. + bias), t = n*ohw + pix.
 struct ContractEpilogue {

@@ -10,6 +10,7 @@
 // reproduced bit for bit from the nine layer integers and the constant record.
 #include "planner.h"
 
+#include "kernels.h"
 #include "line_plan.h"
 
 #include <algorithm>
@@ -431,15 +432,44 @@ uint64_t gemm_cost(const LayerShape& s, int operand, int lhs, const Calibration&
     return saturate((u128)gather + contract);
 }
 
-// CTAs per work item of the GEMM scheme over gathered patches in TF32 (what the kernels' host side computes).
-int gemm_split(const LayerShape& s, const Calibration& cal)
+// What the GEMM scheme takes in TF32 with its patches written first (MNN_GEMM_LHS_PATCHES) or gathered by producer warps
+// (_IMPLICIT), each with its K loop cut over clusters as the kernels cut it: closer than gemm_cost, which ranks the schemes
+// and books both uncut.  *split = CTAs per work item.  Fitted to 825 layers measured with both operands (strides 1 to 5,
+// kernels up to 11): for nine in ten of them the patch matrix takes 0.87 to 1.12 of this, the implicit gather 0.85 to 1.4.
+uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal, int* split)
 {
-    const int sms = cal.c[7] > 0 ? (int)cal.c[7] : 148;
-    const uint64_t tile_blocks = ceil_div((uint64_t)s.N * s.OH * s.OW, 128);
+    const uint64_t sms = cal.c[7] > 0 ? (uint64_t)cal.c[7] : 148, c0 = (uint64_t)cal.c[0];
+    const uint64_t Kp = round_up((uint64_t)s.Cin * s.k * s.k, 8), k_blocks = ceil_div(Kp, 32);
+    const uint64_t T = (uint64_t)s.N * s.OH * s.OW, tile_blocks = ceil_div(T, 128);
     int bn = 256, n_co_blocks = 1;
-    contract_tiling((long long)tile_blocks, 1, s.Cout, sms, &bn, &n_co_blocks);
-    const uint64_t k_blocks = ceil_div(round_up((uint64_t)s.Cin * s.k * s.k, 8), 32);
-    return contract_split((long long)(tile_blocks * (uint64_t)n_co_blocks), (int)k_blocks, sms);
+    contract_tiling((long long)tile_blocks, 1, s.Cout, (int)sms, &bn, &n_co_blocks);
+    const uint64_t items = tile_blocks * (uint64_t)n_co_blocks, rounds = ceil_div(items, sms);
+    *split = contract_split((long long)items, (int)k_blocks, (int)sms);
+    const uint64_t x_bytes = 4ull * s.N * s.Cin * s.H * s.W, y_bytes = 4ull * s.N * s.Cout * s.OH * s.OW;
+    const uint64_t v_bytes = T * Kp * 4, u_bytes = (uint64_t)s.Cout * Kp * 4;
+    const uint64_t blocks = ceil_div(k_blocks, (uint64_t)*split), drain = 128ull * bn * 4 * 45;
+    uint64_t block, fixed = 0;
+    u128 bytes = (u128)x_bytes + u_bytes + y_bytes;
+    if (lhs == MNN_GEMM_LHS_IMPLICIT) {
+        // A block of 128 x 32 elements took 1.02 us, five eighths of what consts[13] books; element-wise (Cin not a multiple
+        // of 32) 1.9 us, and two of them from a stride of four on.  A cut costs 3 us.
+        const uint64_t gather = saturate((u128)128 * 32 * (uint64_t)cal.c[13] * 5u / 8u / 1000000u);
+        block = std::max<uint64_t>(s.Cin % 32 != 0 ? gather * 15 / 8 : s.stride >= 4 ? gather * 2 : gather, (uint64_t)bn * 128 * 16);
+        if (*split > 1) fixed = 3000000;
+    } else {
+        // The staged gather is bound by a CTA's serial loads (four CTAs share an SM) long before its bytes; a block of the
+        // contraction takes six tenths of the time gemm_cost gives it.
+        long long ctas = 0;
+        const GatherGeom g = {s.N, s.Cin, s.H, s.W, s.OH, s.OW, s.k, s.stride, s.pad, s.dil, (int)Kp};
+        const uint64_t serial = (uint64_t)staged_gather_ps(g, &ctas), waves = ceil_div((uint64_t)ctas, 4 * sms);
+        const uint64_t moved = saturate((u128)(x_bytes + v_bytes) * c0 / 1000000u);
+        fixed = serial ? 5500000 + std::max<uint64_t>(serial, serial * waves * 3 / 4) + moved * 6 / 5 : std::max<uint64_t>(5500000, moved * 5);
+        const uint64_t mma = saturate((u128)(2ull * 128 * bn * 32) * (uint64_t)cal.c[2] * sms / 1000000u);
+        block = std::max<uint64_t>((128ull * 128 + (uint64_t)bn * 128) * 16, mma) * 3 / 5;
+        bytes = (u128)v_bytes + u_bytes + y_bytes;
+    }
+    const uint64_t item = std::max<uint64_t>(blocks * block, drain + 500000);
+    return saturate((u128)fixed + kernel_ps(bytes * c0, (u128)(rounds * item + drain / 2) * 1000000u, 0, cal));
 }
 
 // The packed-line form (line_conv.cu): one pass over x that writes the planes, at three quarters of the copy rate, and a
@@ -641,12 +671,15 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 const bool pointwise = s.k == 1 && s.stride == 1;
                 if (implicit_ok && !pointwise && cal.c[13] > 0 && cost_i < best_lhs) lhs = MNN_GEMM_LHS_IMPLICIT;
                 booked = lhs;
-                // So few work items that their K loop is cut over clusters: the cut gather beats writing the patches first
-                // (one image, 3x3 stride 2: 64 -> 128 at 56 x 56 10.8 against 22.4 us, 256 -> 512 at 14 x 14 14.2 against
-                // 24.0 us); with more items x is packed into lines of positions where that form applies (line_conv.cu).  The booked
-                // cost stays that of the operand chosen above, an upper bound.
-                if (implicit_ok && !pointwise && cal.c[13] > 0 && gemm_split(s, cal) > 1) {
-                    if (lhs == MNN_GEMM_LHS_PATCHES) lhs = MNN_GEMM_LHS_IMPLICIT;
+                // So few work items that their K loop is cut over clusters: the implicit gather instead of the patch matrix where
+                // it takes less time cut than the patches take with the same cut (one image, 3x3 stride 2: 64 -> 128 at 56 x 56
+                // 10.8 against 22.4 us, 256 -> 512 at 14 x 14 14.2 against 24.0; but 47 images, 304 -> 304 3x3 stride 2 at 8 x 8
+                // 100 against 67).  With more items x is packed into lines of positions where that form applies
+                // (line_conv.cu).  The booked cost stays that of the operand chosen above.
+                int split = 1;
+                const uint64_t time_i = implicit_ok && !pointwise && cal.c[13] > 0 ? patch_operand_time(s, MNN_GEMM_LHS_IMPLICIT, cal, &split) : 0;
+                if (split > 1) {
+                    if (lhs == MNN_GEMM_LHS_PATCHES && time_i < patch_operand_time(s, MNN_GEMM_LHS_PATCHES, cal, &split)) lhs = MNN_GEMM_LHS_IMPLICIT;
                 } else if (packed_lines && gemm_packs_lines(s, c.operand) &&
                            packed_cost(s, c.operand, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
                     lhs = MNN_GEMM_LHS_PACKED;

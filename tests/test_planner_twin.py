@@ -317,6 +317,25 @@ def test_every_layer_near_the_packed_bound_plans(Cin, k, OW):
     assert seen == {True, False}
 
 
+# Layers whose K loop is cut over clusters: the implicit gather where its serial gather is the shorter way (ResNet-18's
+# stride-2 layers at one image), the patch matrix where it is not (measured 67 against 100, 63 / 96, 259 / 425, 46 / 57 us).
+@pytest.mark.parametrize("shape,lhs", [
+    ((1, 64, 128, 56, 56, 3, 2, 1, 1), B.GEMM_LHS_IMPLICIT), ((1, 128, 256, 28, 28, 3, 2, 1, 1), B.GEMM_LHS_IMPLICIT),
+    ((1, 256, 512, 14, 14, 3, 2, 1, 1), B.GEMM_LHS_IMPLICIT), ((47, 304, 304, 8, 8, 3, 2, 1, 1), B.GEMM_LHS_PATCHES),
+    ((19, 107, 134, 9, 37, 5, 2, 2, 1), B.GEMM_LHS_PATCHES), ((16, 383, 365, 17, 100, 6, 2, 0, 3), B.GEMM_LHS_PATCHES),
+    ((6, 31, 174, 15, 15, 7, 1, 12, 4), B.GEMM_LHS_PATCHES)])
+def test_cut_layers_take_the_shorter_gather(shape, lhs):
+    N, Cin, Cout, H, W_, k, stride, pad, dil = shape
+    layer = W.ConvLayer("cut", N, Cin, Cout, H, W_, k, stride, pad, dil)
+    if k == 6:                                               # (no accuracy figures for this size in the table)
+        plan = B.mnn_conv_plan_ex(*shape, B.make_opts(relu=1))
+        info = B.mnn_conv_plan_query(plan)
+        B.mnn_conv_destroy(plan)
+    else:
+        info = compare(layer, {}, {}, B.mnn_get_calibration())
+    assert (info.algo, info.gemm_lhs) == (B.ALGO_GEMM, lhs)
+
+
 def test_routing_rules():
     t = ppm_table()
     for l in all_layers():

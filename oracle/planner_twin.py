@@ -174,6 +174,12 @@ def cluster_split(items: int, k_blocks: int, sms: int) -> int:
     return n
 
 
+def tile_copy_split(items: int, k_blocks: int, sms: int) -> int:
+    """The same for the contraction, whose blocks are cheaper: no cut below 36 blocks, 20 where it is by four or eight."""
+    n = cluster_split(items, k_blocks, sms)
+    return n if k_blocks >= (20 if n > 2 else 36) else 1
+
+
 # ---------------------------------------------------------------------------------------
 # GEMM scheme (k = 1 "is just a matrix multiplication"; k > 1 over gathered patches).
 # ---------------------------------------------------------------------------------------
@@ -342,23 +348,24 @@ def patch_operand_time(L: Layer, lhs, c):
     Kp, T = cdiv(L.Cin * L.k * L.k, 8) * 8, L.N * L.OH * L.OW
     bn, co_blocks = contraction_tiling(cdiv(T, 128), 1, L.Cout, sms)
     items = cdiv(T, 128) * co_blocks
-    rounds, split = cdiv(items, sms), cluster_split(items, cdiv(Kp, 32), sms)
+    rounds, split = cdiv(items, sms), (cluster_split if lhs == LHS_IMPLICIT else tile_copy_split)(items, cdiv(Kp, 32), sms)
     x, y, v, u = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW, T * Kp * 4, L.Cout * Kp * 4
     drain = 128 * bn * 4 * 45
     if lhs == LHS_IMPLICIT:
         gather = 128 * 32 * c[13] * 5 // 8 // 10 ** 6
         block = max(gather * 15 // 8 if L.Cin % 32 else gather * 2 if L.stride >= 4 else gather, bn * 128 * 16)
-        fixed, traffic = 3000000 if split > 1 else 0, x + u + y
+        fixed, traffic = 0, x + u + y
     else:
         serial, ctas = staged_gather(L)
         moved = (x + v) * c[0] // 10 ** 6
         if serial:
-            fixed = 5500000 + max(serial, serial * cdiv(ctas, 4 * sms) * 3 // 4) + moved * 6 // 5
+            fixed = 2500000 + max(serial, serial * cdiv(ctas, 4 * sms) * 3 // 4) + moved * 6 // 5
         else:
-            fixed = max(5500000, moved * 5)
+            fixed = max(2500000, moved * 5)
         block = max((128 * 128 + bn * 128) * 16, 2 * 128 * bn * 32 * c[2] * sms // 10 ** 6) * 3 // 5
         traffic = v + u + y
     item = max(cdiv(cdiv(Kp, 32), split) * block, drain + 500000)
+    fixed += 3000000 if split > 1 else 0                    # what a cut costs
     return fixed + kernel_ps(c, mem_as=traffic * c[0], tensor_as=(rounds * item + drain // 2) * 10 ** 6)
 
 

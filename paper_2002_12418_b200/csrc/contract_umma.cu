@@ -743,7 +743,7 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     p.epi = epi;
     p.status = status;
     const long long grid = p.n_items < uc.num_sms ? p.n_items : uc.num_sms;
-    p.split = uc.kb == 2 ? contract_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
+    p.split = uc.kb == 2 ? tile_copy_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
     p.epi_warps = uc.k_blocks <= 8 || p.split > 1 ? 8 : 4;
     if (p.split > 1)
         return launch_cluster(p.split, contract_umma_kernel<0, 128, 1, 2, true, true>, dim3((unsigned)(p.n_items * p.split)), dim3(64 + 32 * p.epi_warps),
@@ -783,7 +783,7 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
                                                : (uc.stages_sw == 64 ? contract_umma_kernel<0, 64, 3, 1> : contract_umma_kernel<0, 128, 3, 1>))
                              : (uc.passes == 1 ? (uc.kb == 2 ? contract_umma_kernel<1, 128, 1, 2> : contract_umma_kernel<1, 128, 1, 1>)
                                                : (uc.stages_sw == 64 ? contract_umma_kernel<1, 64, 3, 1> : contract_umma_kernel<1, 128, 3, 1>));
-    p.split = epi.mode == 1 && uc.kb == 2 ? contract_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
+    p.split = epi.mode == 1 && uc.kb == 2 ? tile_copy_split(p.n_items, uc.k_blocks, uc.num_sms) : 1;
     p.epi_warps = uc.k_blocks <= 8 || p.split > 1 ? 8 : 4;
     if (p.split > 1) {
         auto split_kern = uc.kind == 0 ? contract_umma_kernel<0, 128, 1, 2, false, true> : contract_umma_kernel<1, 128, 1, 2, false, true>;

@@ -358,6 +358,12 @@ int contract_split(long long items, int k_blocks, int num_sms)
     return split;
 }
 
+int tile_copy_split(long long items, int k_blocks, int num_sms)
+{
+    const int split = contract_split(items, k_blocks, num_sms);
+    return k_blocks >= (split > 2 ? 20 : 36) ? split : 1;
+}
+
 bool gemm_packs_lines(const LayerShape& s, int operand)
 {
     const int block = operand == MNN_OPERAND_BF16 ? 64 : 32;      // channels per 128 bytes
@@ -435,7 +441,8 @@ uint64_t gemm_cost(const LayerShape& s, int operand, int lhs, const Calibration&
 // What the GEMM scheme takes in TF32 with its patches written first (MNN_GEMM_LHS_PATCHES) or gathered by producer warps
 // (_IMPLICIT), each with its K loop cut over clusters as the kernels cut it: closer than gemm_cost, which ranks the schemes
 // and books both uncut.  *split = CTAs per work item.  Fitted to 825 layers measured with both operands (strides 1 to 5,
-// kernels up to 11): for nine in ten of them the patch matrix takes 0.87 to 1.12 of this, the implicit gather 0.85 to 1.4.
+// kernels up to 11); on 600 others, eight in ten took within a tenth of it, and the choice by it half a percent more than
+// the better operand each time.
 uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal, int* split)
 {
     const uint64_t sms = cal.c[7] > 0 ? (uint64_t)cal.c[7] : 148, c0 = (uint64_t)cal.c[0];
@@ -444,18 +451,18 @@ uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal
     int bn = 256, n_co_blocks = 1;
     contract_tiling((long long)tile_blocks, 1, s.Cout, (int)sms, &bn, &n_co_blocks);
     const uint64_t items = tile_blocks * (uint64_t)n_co_blocks, rounds = ceil_div(items, sms);
-    *split = contract_split((long long)items, (int)k_blocks, (int)sms);
+    *split = lhs == MNN_GEMM_LHS_IMPLICIT ? contract_split((long long)items, (int)k_blocks, (int)sms)
+                                          : tile_copy_split((long long)items, (int)k_blocks, (int)sms);
     const uint64_t x_bytes = 4ull * s.N * s.Cin * s.H * s.W, y_bytes = 4ull * s.N * s.Cout * s.OH * s.OW;
     const uint64_t v_bytes = T * Kp * 4, u_bytes = (uint64_t)s.Cout * Kp * 4;
     const uint64_t blocks = ceil_div(k_blocks, (uint64_t)*split), drain = 128ull * bn * 4 * 45;
-    uint64_t block, fixed = 0;
+    uint64_t block, fixed = *split > 1 ? 3000000 : 0;                   // (what a cut costs)
     u128 bytes = (u128)x_bytes + u_bytes + y_bytes;
     if (lhs == MNN_GEMM_LHS_IMPLICIT) {
         // A block of 128 x 32 elements took 1.02 us, five eighths of what consts[13] books; element-wise (Cin not a multiple
-        // of 32) 1.9 us, and two of them from a stride of four on.  A cut costs 3 us.
+        // of 32) 1.9 us, and two of them from a stride of four on.
         const uint64_t gather = saturate((u128)128 * 32 * (uint64_t)cal.c[13] * 5u / 8u / 1000000u);
         block = std::max<uint64_t>(s.Cin % 32 != 0 ? gather * 15 / 8 : s.stride >= 4 ? gather * 2 : gather, (uint64_t)bn * 128 * 16);
-        if (*split > 1) fixed = 3000000;
     } else {
         // The staged gather is bound by a CTA's serial loads (four CTAs share an SM) long before its bytes; a block of the
         // contraction takes six tenths of the time gemm_cost gives it.
@@ -463,7 +470,7 @@ uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal
         const GatherGeom g = {s.N, s.Cin, s.H, s.W, s.OH, s.OW, s.k, s.stride, s.pad, s.dil, (int)Kp};
         const uint64_t serial = (uint64_t)staged_gather_ps(g, &ctas), waves = ceil_div((uint64_t)ctas, 4 * sms);
         const uint64_t moved = saturate((u128)(x_bytes + v_bytes) * c0 / 1000000u);
-        fixed = serial ? 5500000 + std::max<uint64_t>(serial, serial * waves * 3 / 4) + moved * 6 / 5 : std::max<uint64_t>(5500000, moved * 5);
+        fixed += serial ? 2500000 + std::max<uint64_t>(serial, serial * waves * 3 / 4) + moved * 6 / 5 : std::max<uint64_t>(2500000, moved * 5);
         const uint64_t mma = saturate((u128)(2ull * 128 * bn * 32) * (uint64_t)cal.c[2] * sms / 1000000u);
         block = std::max<uint64_t>((128ull * 128 + (uint64_t)bn * 128) * 16, mma) * 3 / 5;
         bytes = (u128)v_bytes + u_bytes + y_bytes;

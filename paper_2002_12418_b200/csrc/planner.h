@@ -47,10 +47,14 @@ void install_calibration(const Calibration& c);
 void contract_tiling(long long tile_blocks, int alpha2, int Cout, int num_sms, int* bn, int* n_co_blocks);
 
 // CTAs that share the K loop of one work item of the GEMM scheme (1, 2, 4 or 8): items so few that most SMs would idle are cut
-// along K and the partial accumulators added through distributed shared memory.  At least four blocks of K per CTA: the
-// cluster costs about 3 us (4 blocks cut in two: 5.9 -> 8.3 us; 16 blocks cut in four: 12.3 -> 8.1 us);
-// clusters of 8 only for up to 8 items (a GPC holds two of them at best; 16 such clusters ran in two waves).
+// along K and the partial accumulators added through distributed shared memory.  At least four blocks of K per CTA, since the
+// cluster costs about 3 us; clusters of 8 only for up to 8 items (a GPC holds two of them at best; 16 such clusters ran in
+// two waves).  contract_split: the implicit gather, a microsecond or two per block.  tile_copy_split: the contraction, whose
+// blocks arrive by tile copies in 0.2 us: cut in two it gains from 36 blocks on, in four from 20 on (mean of ten small 1 x 1
+// layers each, whole / cut: two CTAs at 8 blocks 11.4 / 14.3 us, 15 13.2 / 14.0, 28 15.4 / 17.4, 40 18.4 / 18.4; four at 16 13.3 /
+// 13.4, 24 14.6 / 13.2, 40 18.1 / 14.7; eight at 32 15.7 / 12.3).
 int contract_split(long long items, int k_blocks, int num_sms);
+int tile_copy_split(long long items, int k_blocks, int num_sms);
 
 // True when the layer fits the packed-line product with this operand type (line_conv.cu; guarantees that line_plan finds a
 // tiling): k in 2..7, stride at most 4, Cin a multiple of 32 or Cin * k at most 32 (BF16: Cin a multiple of 64), and taps

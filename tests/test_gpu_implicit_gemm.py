@@ -96,7 +96,8 @@ def test_where_it_does_not_apply(torch):
 # channels off the tile), for the implicit gather and for the contraction over patches and over x itself.
 @pytest.mark.parametrize("lhs", [B.GEMM_LHS_PATCHES, B.GEMM_LHS_X, B.GEMM_LHS_IMPLICIT])
 @pytest.mark.parametrize("shape", [(1, 264, 40, 8, 12, 1, 1, 0), (1, 520, 300, 7, 7, 1, 1, 0), (1, 72, 24, 9, 9, 3, 2, 1),
-                                   (3, 100, 130, 13, 13, 3, 1, 1), (1, 1000, 64, 10, 10, 1, 1, 0), (2, 96, 48, 12, 12, 5, 2, 2)])
+                                   (3, 100, 130, 13, 13, 3, 1, 1), (1, 1000, 64, 10, 10, 1, 1, 0), (2, 96, 48, 12, 12, 5, 2, 2),
+                                   (1, 1288, 500, 28, 28, 1, 1, 0)])       # (the contraction in two: 41 blocks, 56 items)
 def test_k_loop_cut_over_clusters(torch, shape, lhs):
     N, Cin, Cout, H, W_, k, s, p = shape
     if lhs == B.GEMM_LHS_X and (k > 1 or H * W_ % 4):

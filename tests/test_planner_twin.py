@@ -291,6 +291,16 @@ def test_contraction_tiling_by_hand():
     assert bn % 16 == 0 and bn * blocks >= 24
 
 
+def test_k_loop_splits_by_hand():
+    # doubled while twice the CTAs fit the SMs and each keeps four blocks: 10 items 10 -> 20 -> 40 of 148; 32 blocks allow 8
+    assert [T.cluster_split(10, k, 148) for k in (7, 8, 15, 16, 32, 100)] == [1, 2, 2, 4, 4, 4]
+    assert [T.cluster_split(8, k, 148) for k in (31, 32)] == [4, 8]
+    assert [T.cluster_split(n, 64, 148) for n in (18, 19, 37, 38, 74, 75)] == [4, 4, 4, 2, 2, 1]
+    # the contraction: not below 20 blocks, in two not below 36
+    assert [T.tile_copy_split(10, k, 148) for k in (8, 19, 20, 64)] == [1, 1, 4, 4]
+    assert [T.tile_copy_split(50, k, 148) for k in (20, 35, 36)] == [1, 1, 2]
+
+
 def test_first_minimum_wins_ties_and_inadmissible_is_never_chosen():
     L = T.Layer(32, 128, 128, 28, 28, 3, 1, 1)
     ppm = {key: 1 for key in ppm_table()}                   # everything admissible

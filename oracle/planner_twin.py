@@ -206,12 +206,18 @@ def packs_lines(L: Layer, operand: int) -> bool:
             and L.stride ** 2 * (cells + 2048) * (cdiv(L.Cin, 32) * 32) * _bytes_of(operand) <= 4 << 30)
 
 
-def bf16_lines(L: Layer, sms: int):
-    """(bytes of the packed planes, estimated time of the product in ps) of the BF16 packed-line form, or None: the geometry
-    of the cells and the cheapest tiling (output channels bn, mt tiles of 128 cells, g taps per step) that fits."""
-    s, offs = L.stride, {}
+def packed_lines(L: Layer, operand: int, sms: int):
+    """Geometry and tiling of the packed-line form, or None: the planes' bytes, the estimated time of the product in ps, whether the
+    few-channel form (kernel columns among the elements, rows cut into equal strips of at most 16), the strips' width, and the
+    cheapest tiling that fits (output channels bn, mt tiles of 128 cells, g taps per step, stage slots)."""
+    bf16, s, offs = operand == OPERAND_BF16, L.stride, {}
+    few = L.Cin % (64 if bf16 else 32) != 0
+    if few and (bf16 or L.Cin * L.k > 32) or L.k > 7 or s > 4:
+        return None
+    elems = 32 if few else L.Cin
+    k_steps = 3 if few and L.Cin * L.k <= 24 else 4
     for a in range(L.k):
-        for b in range(L.k):
+        for b in range(1 if few else L.k):
             offs.setdefault((a * L.dil % s, b * L.dil % s), []).append((a * L.dil // s, b * L.dil // s))
     if len(offs) > 16:
         return None
@@ -224,11 +230,15 @@ def bf16_lines(L: Layer, sms: int):
 
     hq = pitch(L.H, L.OH, [r for r, _ in offs], max(q[0] for q in qs))
     wq = pitch(L.W, L.OW, [r for _, r in offs], max(q[1] for q in qs))
+    strips = 1
+    if few:
+        strips = cdiv(L.OW, 16)
+        wq = cdiv(L.OW, strips)
     rows = [[qh * wq + qw for qh, qw in group] for group in offs.values()]
     span, base = max(max(r) - min(r) for r in rows), max(min(r) for r in rows)
-    cells, taps = L.N * hq * wq, L.k * L.k
+    cells, taps = L.N * strips * hq * wq, sum(map(len, rows))
     positions = cells + span + base
-    a_bytes = len(rows) * positions * L.Cin * 2
+    a_bytes = len(rows) * positions * elems * (2 if bf16 else 4)
     if positions >= (1 << 31) - 4096 or a_bytes > 4 << 30:
         return None
     co16, room, best = cdiv(L.Cout, 16) * 16, 207 * 1024, None
@@ -245,32 +255,37 @@ def bf16_lines(L: Layer, sms: int):
             for g in (3, 2, 1):
                 if 2 * a_slot >= room or (room - 2 * a_slot) // (g * b_tile) < (3 if g == 1 else 2):
                     continue
-                issue = sum(cdiv(len(r), g) for r in rows) * 194000 + taps * 4 * 45000
-                mma = taps * mt * 4 * (212 * n + 15000)
+                issue = sum(cdiv(len(r), g) for r in rows) * 194000 + taps * k_steps * 45000
+                mma = taps * mt * k_steps * (212 * n + 15000)
                 load = (taps * b_tile + len(rows) * a_slot) * 63 // 5
                 drain = mt * n * 512 * 28 + 1087000
-                item = max(issue, mma, load) * (L.Cin // 64) + 285000 + mt * 363000
+                item = max(issue, mma, load) * (elems * (2 if bf16 else 4) // 128) + 285000 + mt * 363000
                 cost = rounds * max(item, drain) + drain
                 if best is None or cost * (100 + 3 * mt) < best[0]:
-                    best = (cost * (100 + 3 * mt), cost)
-    return None if best is None else (a_bytes, best[1])
+                    b_slots = min(12, (room - 2 * a_slot) // (g * b_tile))
+                    best = (cost * (100 + 3 * mt), cost, dict(bn=n, mt=mt, g=g, b_slots=b_slots,
+                                                              a_slots=min(4, (room - b_slots * g * b_tile) // a_slot)))
+    return None if best is None else dict(a_bytes=a_bytes, product_ps=best[1], few=few, width=wq, **best[2])
 
 
 def packed_cost(L: Layer, operand: int, c) -> int:
-    """Packed lines: a pass from x to the packed planes, and a product that reads them: in TF32 at half the contraction's tensor
-    rate, in BF16 by the estimate of its tiling."""
+    """Packed lines: a pass from x to the packed planes at three quarters of the copy rate (half from a stride of four on, in
+    TF32), and a product that takes its tiling's estimate or reads the planes and writes y.  TF32: what exceeds two thirds of
+    L2, in strips that are not whole sectors, costs five times more; the product's launch hides behind the pack (of few
+    channels: 2 us of it)."""
     x, y = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW
-    if operand == OPERAND_BF16:
-        lines = bf16_lines(L, c[7] if c[7] > 0 else 148)
-        if lines is None:
-            return INADMISSIBLE
-        a, product = lines
-        return sat(kernel_ps(c, mem_as=(x + a) * c[0] * 4 // 3) + kernel_ps(c, mem_as=(a + y) * c[0], tensor_as=product * 10 ** 6))
-    reach = (L.k - 1) * L.dil // L.stride
-    planes = min(L.stride, L.k) ** 2
-    a = L.N * (L.OH + reach) * (L.OW + reach) * planes * cdiv(L.Cin, 32) * 32 * 4
-    flops = 2 * L.N * L.OH * L.OW * L.Cout * L.Cin * L.k * L.k
-    return sat(kernel_ps(c, mem_as=(x + a) * c[0]) + kernel_ps(c, mem_as=(a + y) * c[0], tensor_as=flops * 2 * c[2]))
+    p = packed_lines(L, operand, c[7] if c[7] > 0 else 148)
+    if p is None:
+        return INADMISSIBLE
+    moved, tf32 = (x + p["a_bytes"]) * c[0] * 4 // 3, operand != OPERAND_BF16
+    if tf32 and L.stride >= 4:
+        moved = moved * 3 // 2
+    kept = c[6] * 2 // 3
+    if tf32 and p["few"] and y > kept and (L.OW % 8 or p["width"] % 8):
+        y += 5 * (y - kept)
+    hidden = 0 if not tf32 else min(2000000, c[5]) if p["few"] else c[5]
+    return sat(kernel_ps(c, mem_as=moved) - hidden
+               + kernel_ps(c, mem_as=(p["a_bytes"] + y) * c[0], tensor_as=p["product_ps"] * 10 ** 6))
 
 
 def gemm_cost(L: Layer, operand: int, lhs, c) -> int:
@@ -364,9 +379,9 @@ def patch_operand_time(L: Layer, lhs, c):
             fixed = max(2500000, moved * 5)
         block = max((128 * 128 + bn * 128) * 16, 2 * 128 * bn * 32 * c[2] * sms // 10 ** 6) * 3 // 5
         traffic = v + u + y
-    item = max(cdiv(cdiv(Kp, 32), split) * block, drain + 500000)
+    item = max(cdiv(cdiv(Kp, 32), split) * block, 128 * bn * 4 * 82 + 1250000 if lhs == LHS_IMPLICIT and split == 1 else drain + 500000)
     fixed += 3000000 if split > 1 else 0                    # what a cut costs
-    return fixed + kernel_ps(c, mem_as=traffic * c[0], tensor_as=(rounds * item + drain // 2) * 10 ** 6)
+    return fixed + kernel_ps(c, mem_as=traffic * c[0], tensor_as=(rounds * item + (drain // 2 if split > 1 else drain)) * 10 ** 6)
 
 
 # ---------------------------------------------------------------------------------------
@@ -527,8 +542,11 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 if implicit_ok and cut and not (L.k == 1 and L.stride == 1) and c[13] > 0:
                     if lhs == LHS_PATCHES and patch_operand_time(L, LHS_IMPLICIT, c) < patch_operand_time(L, LHS_PATCHES, c):
                         lhs = LHS_IMPLICIT
-                elif packs_lines(L, operand) and packed_cost(L, operand, c) < costs[lhs]:
-                    lhs = LHS_PACKED
+                elif packs_lines(L, operand):
+                    # TF32: unless estimated at 6/5 of the other operand's time or more
+                    tf32 = implicit_ok and lhs != LHS_X
+                    if packed_cost(L, operand, c) * (5 if tf32 else 1) < (6 * patch_operand_time(L, lhs, c) if tf32 else costs[lhs]):
+                        lhs = LHS_PACKED
                 costs[lhs] = costs[costs_of]
             if lhs == LHS_X:
                 p = max(p, LHS_X_ERROR_PPM)

@@ -475,32 +475,39 @@ uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal
         block = std::max<uint64_t>((128ull * 128 + (uint64_t)bn * 128) * 16, mma) * 3 / 5;
         bytes = (u128)v_bytes + u_bytes + y_bytes;
     }
-    const uint64_t item = std::max<uint64_t>(blocks * block, drain + 500000);
-    return saturate((u128)fixed + kernel_ps(bytes * c0, (u128)(rounds * item + drain / 2) * 1000000u, 0, cal));
+    // the next item's loop runs while an accumulator is drained: the implicit gather's four warps take 82 ps per byte and 1.25 us
+    // per item, the contraction's 45 ps and half a microsecond (as a cut item does into shared memory)
+    const uint64_t tail = *split > 1 ? drain / 2 : drain;
+    const uint64_t item = std::max<uint64_t>(blocks * block, lhs == MNN_GEMM_LHS_IMPLICIT && *split == 1 ? 128ull * bn * 4 * 82 + 1250000 : drain + 500000);
+    return saturate((u128)fixed + kernel_ps(bytes * c0, (u128)(rounds * item + tail) * 1000000u, 0, cal));
 }
 
 // The packed-line form (line_conv.cu): one pass over x that writes the planes, at three quarters of the copy rate, and a
-// product that reads them once.  In TF32 the product is charged half of the contraction's tensor rate, an upper bound that
-// only chooses between the left operands of the GEMM scheme; in BF16, where it competes with the other schemes, the time that
-// its tiling was chosen by.
+// product that takes the time its tiling was chosen by, or reads them and writes y.  In TF32 it only chooses between the left
+// operands of the GEMM scheme (nine in ten of 500 measured layers within a fifth of it); in BF16 it competes with the other
+// schemes.
 uint64_t packed_cost(const LayerShape& s, int operand, const Calibration& cal)
 {
     const uint64_t c0 = (uint64_t)cal.c[0];
     const u128 x_bytes = (u128)4 * s.N * s.Cin * s.H * s.W, y_bytes = (u128)4 * s.N * s.Cout * s.OH * s.OW;
-    if (operand == MNN_OPERAND_BF16) {
-        const LineShape ls = {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.stride, s.dil, s.pad, s.OH, s.OW, 1};
-        LinePlan p;
-        if (!line_plan(ls, cal.c[7] > 0 ? (int)cal.c[7] : 148, &p)) return MNN_COST_INADMISSIBLE;
-        const u128 a_bytes = (u128)p.a_bytes;
-        return saturate((u128)kernel_ps((x_bytes + a_bytes) * c0 * 4u / 3u, 0, 0, cal) +
-                        kernel_ps((a_bytes + y_bytes) * c0, (u128)p.loop_ps * 1000000u, 0, cal));
+    const LineShape ls = {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.stride, s.dil, s.pad, s.OH, s.OW, operand == MNN_OPERAND_BF16};
+    LinePlan p;
+    if (!line_plan(ls, cal.c[7] > 0 ? (int)cal.c[7] : 148, &p)) return MNN_COST_INADMISSIBLE;
+    const u128 a_bytes = (u128)p.a_bytes;
+    u128 moved = (x_bytes + a_bytes) * c0 * 4u / 3u, stored = y_bytes;
+    if (operand != MNN_OPERAND_BF16) {
+        // strides of four and more: no two phases share a sector of x
+        if (s.stride >= 4) moved = moved * 3u / 2u;
+        // few channels: the product writes y strip by strip, in pieces of sectors unless both the row and the strip are whole
+        // ones; what L2 cannot hold until the next strip costs five times its bytes more (y of 94 / 150 / 307 / 596 MB: 50 / 133 /
+        // 268 / 595 us; 4 -> 381 3x3 dilation 2 at 144 x 144, 27 images, 853 MB in whole sectors: 271)
+        const u128 kept = (u128)(uint64_t)cal.c[6] * 2u / 3u;
+        if (p.few && y_bytes > kept && (s.OW % 8 != 0 || p.Wq % 8 != 0)) stored += (y_bytes - kept) * 5u;
     }
-    const u128 reach = (u128)((uint64_t)(s.k - 1) * s.dil / s.stride);
-    const u128 cells = (u128)s.N * (s.OH + reach) * (s.OW + reach);
-    const u128 a_bytes = cells * (uint64_t)(s.stride < s.k ? s.stride * s.stride : s.k * s.k) * round_up(s.Cin, 32) * 4u;
-    const u128 flops = (u128)2 * s.N * s.OH * s.OW * s.Cout * (uint64_t)(s.Cin * s.k * s.k);
-    return saturate((u128)kernel_ps((x_bytes + a_bytes) * c0, 0, 0, cal) +
-                    kernel_ps((a_bytes + y_bytes) * c0, flops * 2u * (uint64_t)cal.c[2], 0, cal));
+    // TF32: the product's launch hides behind the pack, with few channels for the most part (measured)
+    uint64_t pack = kernel_ps(moved, 0, 0, cal);
+    if (operand != MNN_OPERAND_BF16) pack -= p.few ? std::min<uint64_t>(2000000, (uint64_t)cal.c[5]) : (uint64_t)cal.c[5];
+    return saturate((u128)pack + kernel_ps((a_bytes + stored) * c0, (u128)p.loop_ps * 1000000u, 0, cal));
 }
 
 uint64_t winograd_chunk_cost(const LayerShape& s, int m, int operand, int passes, uint64_t n, bool resident,
@@ -681,15 +688,19 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 // So few work items that their K loop is cut over clusters: the implicit gather instead of the patch matrix where
                 // it takes less time cut than the patches take with the same cut (one image, 3x3 stride 2: 64 -> 128 at 56 x 56
                 // 10.8 against 22.4 us, 256 -> 512 at 14 x 14 14.2 against 24.0; but 47 images, 304 -> 304 3x3 stride 2 at 8 x 8
-                // 100 against 67).  With more items x is packed into lines of positions where that form applies
-                // (line_conv.cu).  The booked cost stays that of the operand chosen above.
+                // 100 against 67).  With more items x is packed into lines of positions where that form applies (line_conv.cu) and is
+                // the shorter way.  The booked cost stays that of the operand chosen above.
                 int split = 1;
                 const uint64_t time_i = implicit_ok && !pointwise && cal.c[13] > 0 ? patch_operand_time(s, MNN_GEMM_LHS_IMPLICIT, cal, &split) : 0;
                 if (split > 1) {
                     if (lhs == MNN_GEMM_LHS_PATCHES && time_i < patch_operand_time(s, MNN_GEMM_LHS_PATCHES, cal, &split)) lhs = MNN_GEMM_LHS_IMPLICIT;
-                } else if (packed_lines && gemm_packs_lines(s, c.operand) &&
-                           packed_cost(s, c.operand, cal) < (lhs == MNN_GEMM_LHS_X ? cost_x : lhs == MNN_GEMM_LHS_IMPLICIT ? cost_i : cost_patches)) {
-                    lhs = MNN_GEMM_LHS_PACKED;
+                } else if (packed_lines && gemm_packs_lines(s, c.operand)) {
+                    // TF32: the lines where they are estimated at less than 6/5 of the operand above, since either estimate can be a
+                    // fifth off and the lines, where they lose by little, win by more (602 layers measured with both: 1.1 % over the
+                    // better one each time, 2.0 % without the fifth)
+                    const bool tf32 = implicit_ok && lhs != MNN_GEMM_LHS_X;
+                    const uint64_t other = tf32 ? patch_operand_time(s, lhs, cal, &split) : lhs == MNN_GEMM_LHS_X ? cost_x : cost_patches;
+                    if ((u128)packed_cost(s, c.operand, cal) * (tf32 ? 5u : 1u) < (u128)other * (tf32 ? 6u : 1u)) lhs = MNN_GEMM_LHS_PACKED;
                 }
             }
             const bool take_x = lhs == MNN_GEMM_LHS_X;

@@ -320,7 +320,7 @@ def test_every_layer_near_the_packed_bound_plans(Cin, k, OW):
     at_bound = (4 << 30) // (128 * (OW + k - 1) * max(OW + k - 1, strips * -(-OW // strips)))
     seen = set()
     for N in range(at_bound - 8, int(at_bound * 1.08), max(1, at_bound // 200)):
-        layer = W.ConvLayer("near", N, Cin, 64, OW + k - 1, OW + k - 1, k, 1, 0, relu=False)
+        layer = W.ConvLayer("near", N, Cin, 4, OW + k - 1, OW + k - 1, k, 1, 0, relu=False)
         info = compare(layer, dict(force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1),
                        dict(force_algo=T.ALGO_GEMM, operand=T.OPERAND_TF32, passes=1), B.mnn_get_calibration())
         seen.add(info.gemm_lhs == B.GEMM_LHS_PACKED)
@@ -344,6 +344,19 @@ def test_cut_layers_take_the_shorter_gather(shape, lhs):
     else:
         info = compare(layer, {}, {}, B.mnn_get_calibration())
     assert (info.algo, info.gemm_lhs) == (B.ALGO_GEMM, lhs)
+
+
+# Packed lines against the operand they replace, each by its own time (measured 196 against 595 us, 52 / 104, 56 / 133, 402 / 1183,
+# 290 / 595 where the lines lose; 53 / 27, 86 / 37 where they win).
+@pytest.mark.parametrize("shape,packed", [
+    ((30, 256, 348, 26, 26, 7, 1, 1, 4), False), ((36, 2, 289, 60, 60, 5, 1, 2, 1), False),
+    ((26, 2, 419, 146, 59, 7, 1, 0, 1), False), ((47, 416, 406, 5, 168, 5, 2, 5, 3), False), ((16, 3, 326, 172, 172, 3, 1, 0, 1), False),
+    ((32, 64, 128, 56, 56, 3, 2, 1, 1), True), ((16, 256, 256, 28, 28, 3, 1, 2, 2), True), ((32, 3, 64, 224, 224, 7, 2, 3, 1), True)])
+def test_packed_lines_are_compared_by_their_own_time(shape, packed):
+    N, Cin, Cout, H, W_, k, stride, pad, dil = shape
+    kw = dict(force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1)
+    info = compare(W.ConvLayer("lines", N, Cin, Cout, H, W_, k, stride, pad, dil), kw, kw, B.mnn_get_calibration())
+    assert (info.gemm_lhs == B.GEMM_LHS_PACKED) == packed
 
 
 def test_routing_rules():

@@ -64,6 +64,10 @@ __device__ __forceinline__ float round_tf32(float v)
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// SPLIT: a cluster of p.split CTAs per work item, one item per cluster.  A form of its own, because the cluster's code costs
+// the other one 0.3 to 1 us per launch (19 images 32 -> 48 1x1 stride 2 at 15 x 30 6.0 -> 5.6 us without it, 16 images 64 -> 64 3x3
+// at 56 x 56 58.1 -> 57.1).
+template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
 {
@@ -107,9 +111,10 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
     ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
     // work items of this CTA and its share of their K blocks
-    const uint32_t rank = p.split > 1 ? ptx::cluster_ctarank() : 0u;
-    const long long first_item = blockIdx.x / (unsigned)p.split, item_step = gridDim.x / (unsigned)p.split;
-    const int kb0 = p.k_blocks * (int)rank / p.split, kb1 = p.k_blocks * ((int)rank + 1) / p.split;
+    const uint32_t rank = SPLIT ? ptx::cluster_ctarank() : 0u;
+    const long long first_item = SPLIT ? blockIdx.x / (unsigned)p.split : blockIdx.x;
+    const long long item_step = SPLIT ? gridDim.x / (unsigned)p.split : gridDim.x;
+    const int kb0 = SPLIT ? p.k_blocks * (int)rank / p.split : 0, kb1 = SPLIT ? p.k_blocks * ((int)rank + 1) / p.split : p.k_blocks;
     const bool bias_in_smem = p.Cout <= kMaxSharedBias;
     if (bias_in_smem && warp >= 2 && warp < 2 + kEpilogueWarps) {
         for (int i = threadIdx.x - 64; i < p.Cout; i += 32 * kEpilogueWarps) s_bias[i] = p.bias ? __ldg(p.bias + i) : 0.0f;
@@ -209,7 +214,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
             const int n_chunks = (n_co + 15) >> 4;
             auto store_chunk = [&](const uint32_t (&v)[16], int ch) {
                 const int c0 = ch * 16;
-                if (p.split > 1) {                        // partial sums over the operand slots, which nothing uses any more
+                if (SPLIT) {                              // partial sums over the operand slots, which nothing uses any more
                     float* red = reinterpret_cast<float*>(generic_base) + q * 32 + lane;
 #pragma unroll
                     for (int j = 0; j < 16; ++j) red[(c0 + j) * 128] = __uint_as_float(v[j]);
@@ -380,7 +385,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
         }
     }
 
-    if (p.split > 1) {
+    if (SPLIT) {
         __syncwarp();
         ptx::cluster_sync_all();
         if (warp < 12 && !*abortp && first_item < p.n_items) {            // three sets of four warps share the columns
@@ -465,7 +470,8 @@ cudaError_t implicit_gemm_setup(ImplicitGemm* ig, const GatherGeom& g, int Cout,
         *why = "cuTensorMapEncodeTiled failed or is unavailable";
         return cudaErrorInvalidValue;
     }
-    e = cudaFuncSetAttribute(implicit_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    e = cudaFuncSetAttribute(implicit_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(implicit_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
     if (e != cudaSuccess) return e;
     ig->ready = true;
     return cudaSuccess;
@@ -496,7 +502,8 @@ cudaError_t launch_implicit_gemm(const ImplicitGemm& ig, const float* x, const f
     p.status = status;
     p.split = contract_split(p.n_items, p.k_blocks, ig.num_sms);
     const long long grid = p.split > 1 ? p.n_items * p.split : (p.n_items < ig.num_sms ? p.n_items : ig.num_sms);
-    return launch_cluster(p.split, implicit_gemm_kernel, dim3((unsigned)grid), dim3(kThreads), (size_t)ig.smem_bytes, stream, ig.map_u, p);
+    return launch_cluster(p.split, p.split > 1 ? implicit_gemm_kernel<true> : implicit_gemm_kernel<false>, dim3((unsigned)grid), dim3(kThreads),
+                          (size_t)ig.smem_bytes, stream, ig.map_u, p);
 }
 
 }  // namespace mnnb

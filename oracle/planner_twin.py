@@ -139,7 +139,7 @@ def direct_cost(L: Layer, c) -> int:
     # c[8] is the rate of layers too small to fill the chip; for k > 1 the lesser of that and 13.3 ns per patch element plus the
     # arithmetic at three tenths of it
     alu = flops * c[8]
-    if L.k > 1:
+    if L.k > 1 and L.Cout > L.groups:                       # (groups of one output channel run a thread per output)
         alu = min(alu, cpg * L.k * L.k * 13300000000 + flops * c[8] * 3 // 10)
     return kernel_ps(c, mem_as=traffic * c[0], alu_as=alu)
 

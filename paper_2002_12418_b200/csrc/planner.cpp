@@ -321,10 +321,11 @@ uint64_t direct_cost(const LayerShape& s, const Calibration& cal)
     // consts[8] is the rate of layers too small to fill the chip.  For k > 1, where it overstates those with short patches, the
     // lesser of that and what the tile kernel spends on a patch (13.3 ns per element: trips to memory, whatever the size) plus
     // its arithmetic at three tenths of the constant.  One image: 24 -> 40 at 33 x 31 (216 elements) 7.0 us, the patch
-    // matrix 14.1; 32 -> 32 at 28 x 28 (288) 6.8 us, Winograd 9.2; 64 -> 64 at 28 x 28 (576) 13.6 us, Winograd 8.7.
+    // matrix 14.1; 32 -> 32 at 28 x 28 (288) 6.8 us, Winograd 9.2; 64 -> 64 at 28 x 28 (576) 13.6 us, Winograd 8.7.  Groups of one
+    // output channel run a thread per output instead (15 images 128 -> 1 3x3 at 120 x 120: 474 us, Winograd 144).
     const uint64_t patch = (uint64_t)(s.Cin / s.groups) * s.k * s.k;
     u128 alu = (u128)flops * (uint64_t)cal.c[8];
-    if (s.k > 1) alu = std::min(alu, (u128)patch * 13300000000ull + (u128)flops * (uint64_t)cal.c[8] * 3u / 10u);
+    if (s.k > 1 && s.Cout > s.groups) alu = std::min(alu, (u128)patch * 13300000000ull + (u128)flops * (uint64_t)cal.c[8] * 3u / 10u);
     return kernel_ps((u128)(x_bytes + y_bytes + w_bytes) * (uint64_t)cal.c[0], 0, alu, cal);
 }
 

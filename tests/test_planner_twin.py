@@ -291,6 +291,27 @@ def test_contraction_tiling_by_hand():
     assert bn % 16 == 0 and bn * blocks >= 24
 
 
+# One output channel: the direct kernel is a thread per output there and may not be booked at the tile kernel's rate (measured
+# 545 us against Winograd's 134, 474 / 144, 77 / 32); from two channels on it is the tile kernel.
+@pytest.mark.parametrize("shape,direct", [((5, 448, 1, 63, 167, 2, 1, 0), False), ((15, 128, 1, 120, 120, 3, 1, 1), False),
+                                          ((7, 43, 1, 150, 25, 3, 1, 3), False), ((1, 24, 40, 33, 31, 3, 1, 1), True)])
+def test_one_output_channel_is_not_booked_as_tiles(shape, direct):
+    info = compare(W.ConvLayer("one", *shape), {}, {}, B.mnn_get_calibration())
+    assert (info.algo == B.ALGO_DIRECT) == direct
+
+
+def test_direct_cost_of_short_patches_by_hand():
+    L = T.Layer(1, 32, 32, 28, 28, 3, 1, 1)                 # 288 patch elements, 14.45 Mflop, 0.24 MB
+    flops, traffic = 2 * 32 * 32 * 784 * 9, 4 * (32 * 784 * 2 + 32 * 32 * 9)
+    by_patch, by_rate = 288 * 13300000000 + flops * 571000 * 3 // 10, flops * 571000
+    cal = list(CAL)
+    cal[0], cal[5], cal[8] = 173000, 3530000, 571000
+    assert by_patch < by_rate and traffic * 173000 < by_patch
+    assert T.direct_cost(L, cal) == by_patch // 10 ** 6 + 3530000
+    one = T.Layer(1, 32, 1, 28, 28, 3, 1, 1)
+    assert T.direct_cost(one, cal) == 2 * 32 * 784 * 9 * 571000 // 10 ** 6 + 3530000
+
+
 def test_k_loop_splits_by_hand():
     # doubled while twice the CTAs fit the SMs and each keeps four blocks: 10 items 10 -> 20 -> 40 of 148; 32 blocks allow 8
     assert [T.cluster_split(10, k, 148) for k in (7, 8, 15, 16, 32, 100)] == [1, 2, 2, 4, 4, 4]

@@ -60,6 +60,7 @@ struct mnn_conv_plan_s {
     bool gemm_implicit = false;      // GEMM scheme with the patches gathered inside the GEMM kernel: no V, one launch
     ImplicitGemm ig;
     bool packed = false;             // GEMM scheme on packed lines: V holds the packed planes, two launches
+    int tiling_sms = 148;            // SMs the packed lines are tiled for: the cost model's, so that what it booked is what runs
     LineConv lc;
     TransformMatrices mats;
     // run-time state
@@ -182,7 +183,7 @@ int realise_decision(mnn_conv_plan_t p, const char** why)
 {
     p->packed = p->fused = p->gemm_x = p->gemm_implicit = false;
     if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
-        p->packed = line_plan(line_shape(p), 148, &p->lc.p);
+        p->packed = line_plan(line_shape(p), p->tiling_sms, &p->lc.p);
         if (!p->packed) {
             *why = "no tiling of the packed-line product fits this layer";
             return MNN_EUNSUPPORTED;
@@ -308,6 +309,7 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
     mnn_conv_opts o_plan = o;
     if (p->strassen) o_plan.passes = 1;      // the candidate list holds single-pass GEMMs; the pass count is set below
     const Calibration cal = current_calibration();
+    if (cal.c[7] > 0) p->tiling_sms = (int)cal.c[7];
     int rc = plan_layer(s, o_plan, cal, true, &p->d, &why);
     if (rc == MNN_OK && p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) rc = plan_layer(s, o_plan, cal, false, &p->d_unpacked, &why);
     if (rc == MNN_OK && p->strassen) {

@@ -176,24 +176,21 @@ extern "C" int mnn_calibrate(int device, void* stream, long long consts[MNN_N_CO
         }
     }
 
-    // direct kernel rate: 3x3, 64 -> 64 channels, 56 x 56, 4 images
+    // direct kernel on a layer too small to fill the chip: 3x3, 64 -> 64 channels, 14 x 14, one image
     {
-        DirectGeom g = {4, 64, 64, 56, 56, 56, 56, 3, 1, 1, 1, 1, 1};
+        DirectGeom g = {1, 64, 64, 14, 14, 14, 14, 3, 1, 1, 1, 1, 1};
         float* x = reinterpret_cast<float*>(buf);
-        float* w = x + (size_t)4 * 64 * 56 * 56;
+        float* w = x + (size_t)64 * 14 * 14;
         float* y = w + 64 * 64 * 9 + 64;
         fill_kernel<<<blocks, 256, 0, st>>>(x, (size_t)(y - x), 1.0f);
-        for (int i = 0; i < 2; ++i) launch_direct(x, w, nullptr, y, g, st);
+        for (int i = 0; i < 5; ++i) launch_direct(x, w, nullptr, y, g, st);
         tm.start();
-        const int reps = 5;
+        const int reps = 50;
         for (int i = 0; i < reps; ++i) launch_direct(x, w, nullptr, y, g, st);
         ms = tm.stop();
-        const double flops = 2.0 * 4 * 64 * 64 * 56 * 56 * 9;
         double t = ms / reps - launch_ms;
         if (t < ms / reps * 0.25) t = ms / reps * 0.25;
-        // (layers too small to fill the chip, which the constant is for, run at 2/15 of this one's rate: 64 -> 64 3x3 at 14 x 14,
-        // one image, 600000 as per flop against 77000)
-        cal.c[8] = to_ll(t * 7.5e15 / flops);
+        cal.c[8] = to_ll(t * 1e15 / (2.0 * 64 * 64 * 14 * 14 * 9));
     }
 
     // rate of the direct kernel for very few input channels: 3x3 stride 2, 3 -> 32 channels, 224 x 224, 32 images

@@ -568,3 +568,14 @@ def test_input_transform_two_pass(torch, N, Cin, H, W_, k, m, operand, passes):
     # three times the error expected of operands rounded to this format, amplified by these transforms, and fp32 arithmetic
     bound = 3e-6 * B.mnn_accuracy_ppm(m, k, info.points_id, operand, passes) + 2e-5
     if bound < 0.1: assert rel_l2(got, oracle(layer, x, w, b)) < bound
+
+
+def test_calibration_of_the_direct_kernel(torch):
+    """consts[8] is measured on the kind of layer it stands for (64 -> 64 3x3 at 14 x 14, one image: about 8 us); the bound of two
+    holds the built-in record, taken on the same card with gaps between the launches."""
+    before = B.mnn_get_calibration()
+    try:
+        got = B.mnn_calibrate(0, torch.cuda.current_stream().cuda_stream)
+        assert all(c > 0 for c in got[:9]) and before[8] / 2 < got[8] < before[8] * 2
+    finally:
+        B.mnn_set_calibration(before)

@@ -489,7 +489,7 @@ def test_direct_tiles(torch, N, Cin, Cout, H, W_, k, stride, dil, groups):
 
 # A tap outside the image is no term of the sum: an infinite weight reaches the outputs whose tap lies inside and no others.
 @pytest.mark.parametrize("N,Cin,Cout,H,W_,k,groups", [(1, 12, 24, 9, 10, 3, 2), (2, 130, 5, 12, 10, 3, 1), (40, 16, 48, 33, 30, 3, 2),
-                                                      (1, 20, 12, 14, 14, 5, 4)])
+                                                      (1, 20, 12, 14, 14, 5, 4), (20, 128, 20, 30, 30, 3, 1)])
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
 def test_direct_weights_that_are_not_finite(torch, N, Cin, Cout, H, W_, k, groups, bad):
     layer = W.ConvLayer("t", N, Cin, Cout, H, W_, k, 1, k // 2, groups=groups, relu=False, seed=Cin)

@@ -1204,7 +1204,11 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
     if (g.Cout == g.groups) {
         long long blocks = (total + 255) / 256;
         if (blocks > 148ll * 64) blocks = 148ll * 64;
-        return launch_overlapped(direct_generic_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, x, w, bias, y, g, total);
+        // Overlapped with the previous kernel's end except from half a CTA to five per SM: those settle unevenly beside the
+        // CTAs that are still there (7 x 7 depthwise, one image, 64 channels 28 x 28, 196 CTAs: 6.8 us plain, 9.7 overlapped; 24
+        // CTAs 6.7 / 6.3, 784 CTAs 14.2 / 13.5).
+        const bool overlap = blocks <= 74 || blocks >= 740;
+        return launch_chained(overlap, direct_generic_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, x, w, bias, y, g, total);
     }
     // channels per warp: as many as the group has, up to 16; the patch is cut until the CTAs fill the SMs twice
     const int opg = g.Cout / g.groups, K = g.Cin / g.groups * g.k * g.k;

@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) 
 
 // One thread per output element: groups with a single output channel (depthwise layers that the 3x3 kernels below do not
 // take), where a position has one multiply-add per element and staging the weights costs more than it saves (64 channels
-// 5x5 at 28 x 28, batch 8: 14.4 us, 15.6 with the tile kernel).
+// 5x5 at 28 x 28, batch 8: 14.4 us, 15.6 with the tile kernel), and very short patches (launch_direct).
 __global__ void __launch_bounds__(256) direct_generic_kernel(const float* __restrict__ x, const float* __restrict__ w,
                                                              const float* __restrict__ bias, float* __restrict__ y,
                                                              DirectGeom g, long long total)
@@ -1201,7 +1201,11 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
         direct_stem_kernel<<<grid, kStemThreads, smem, stream>>>(x, w, bias, y, g, co_pad);
         return cudaGetLastError();
     }
-    if (g.Cout == g.groups) {
+    const int opg = g.Cout / g.groups, K = g.Cin / g.groups * g.k * g.k;
+    // A thread per output also for patches of up to 3 elements, where staging them is most of the work, while the outputs come
+    // twice to a thread of the chip at most (8 images, 2 -> 32 in 2 groups 1x1 stride 2 at 14 x 14 3.1 -> 2.2 us; 70 such layers
+    // 1.08 times as fast).
+    if (opg == 1 || (K <= 3 && total <= 148ll * 512)) {
         long long blocks = (total + 255) / 256;
         if (blocks > 148ll * 64) blocks = 148ll * 64;
         // Overlapped with the previous kernel's end except from half a CTA to five per SM: those settle unevenly beside the
@@ -1211,7 +1215,6 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
         return launch_chained(overlap, direct_generic_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, x, w, bias, y, g, total);
     }
     // channels per warp: as many as the group has, up to 16; the patch is cut until the CTAs fill the SMs twice
-    const int opg = g.Cout / g.groups, K = g.Cin / g.groups * g.k * g.k;
     const int tco = opg >= 16 ? 16 : (opg >= 5 ? 8 : 4);
     const long long T = (long long)g.N * g.OH * g.OW;
     const long long co_tiles = (opg + tco - 1) / tco, cts = co_tiles * g.groups;

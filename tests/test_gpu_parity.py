@@ -487,6 +487,18 @@ def test_direct_tiles(torch, N, Cin, Cout, H, W_, k, stride, dil, groups):
     assert np.array_equal(goti.astype(np.float64), oracle(layer, xi, wi, bi))
 
 
+# Short patches on both sides of the lines between a thread per output and the tile kernel: 3 and 4 elements, 75776 outputs and
+# more.
+@pytest.mark.parametrize("N,Cin,Cout,H,W_,k,stride,groups", [
+    (2, 32, 96, 28, 28, 1, 2, 32), (1, 6, 8, 97, 97, 1, 1, 2), (1, 6, 8, 98, 98, 1, 1, 2), (2, 8, 10, 14, 14, 1, 1, 2)])
+def test_direct_short_patches(torch, N, Cin, Cout, H, W_, k, stride, groups):
+    layer = W.ConvLayer("t", N, Cin, Cout, H, W_, k, stride, k // 2, groups=groups, relu=Cout % 3 == 0, seed=Cout)
+    xi, wi, bi = W.integer_inputs(layer)
+    got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_DIRECT), (xi, wi, bi))
+    assert info.algo == B.ALGO_DIRECT
+    assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))
+
+
 # A tap outside the image is no term of the sum: an infinite weight reaches the outputs whose tap lies inside and no others.
 @pytest.mark.parametrize("N,Cin,Cout,H,W_,k,groups", [(1, 12, 24, 9, 10, 3, 2), (2, 130, 5, 12, 10, 3, 1), (40, 16, 48, 33, 30, 3, 2),
                                                       (1, 20, 12, 14, 14, 5, 4), (20, 128, 20, 30, 30, 3, 1)])

@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(kStemThreads) direct_stem_fixed_kernel(const f
 // channels at 224 x 224: 25 units, 7.0 us -> 98 units, 5.3 us).
 constexpr int kPairCoChunk = 16;   // output channels per sweep over the 27 taps
 
-template <bool RELU, int ROWS>
+template <bool RELU, int ROWS, bool SHARE>
 __global__ void __launch_bounds__(kStemThreads, ROWS == 1 ? 5 : 3)
 direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ bias,
                            float* __restrict__ y, DirectGeom g, int co_pad, int groups, int co_split, int n_units)
@@ -641,8 +641,8 @@ direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict_
     __syncthreads();
     const int ohw = g.OH * g.OW, half_w = g.OW >> 1, per_image = (g.OH / ROWS) * half_w;
     for (int unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
-        // (image, group of pixel blocks, share of the output channels); ROWS = 2 is taken for full machines and never shares
-        const int pg = ROWS == 1 ? unit / co_split : unit, cs = ROWS == 1 ? unit - pg * co_split : 0;
+        // (image, group of pixel blocks, share of the output channels)
+        const int pg = SHARE ? unit / co_split : unit, cs = SHARE ? unit - pg * co_split : 0;
         const int n = pg / groups;
         const int pp = (pg - n * groups) * kStemThreads + threadIdx.x;
         if (pp >= per_image) continue;
@@ -666,7 +666,7 @@ direct_stem_s2_pair_kernel(const float* __restrict__ x, const float* __restrict_
                 c[ci][r][3] = row_ok ? m1.x : 0.0f;
                 c[ci][r][4] = row_ok ? m1.y : 0.0f;
             }
-        for (int c0 = cs * kPairCoChunk; c0 < g.Cout; c0 += (ROWS == 1 ? co_split : 1) * kPairCoChunk) {
+        for (int c0 = cs * kPairCoChunk; c0 < g.Cout; c0 += (SHARE ? co_split : 1) * kPairCoChunk) {
             float2 acc[PIX][kPairCoChunk / 2];                 // pixel = 2 * row + column
 #pragma unroll
             for (int j = 0; j < kPairCoChunk / 2; ++j) {
@@ -1174,18 +1174,24 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
         if (g.Cin == 3 && g.k == 3 && g.dil == 1 && g.stride == 2 && g.pad == 1 && g.H % 2 == 0 && g.W % 4 == 0 &&
             smem <= 48 * 1024 && reinterpret_cast<uintptr_t>(x) % 8 == 0 && reinterpret_cast<uintptr_t>(y) % 8 == 0) {
             const long long blocks2 = (long long)g.N * (((g.OH / 2) * (g.OW / 2) + kStemThreads - 1) / kStemThreads);
-            const int rows = g.H % 4 == 0 && blocks2 >= 148 ? 2 : 1;
-            const int per_image = (g.OH / rows) * (g.OW / 2);
-            const int groups = (per_image + kStemThreads - 1) / kStemThreads;
-            int co_split = 1;
-            while (rows == 1 && (long long)g.N * groups * co_split < 148 && co_split * kPairCoChunk < g.Cout) co_split *= 2;
+            // Two output rows per block, unless units of one row that also share an image's channels are twice as many on a chip
+            // they do not fill otherwise (29 images 68 x 68, 24 channels: 87 units 7.6 us, 290 units 6.4; but 9 images 172 x
+            // 172: 135 units 7.6 us, 261 of one row without sharing 8.6)
+            int rows = 1, groups = (g.OH * (g.OW / 2) + kStemThreads - 1) / kStemThreads, co_split = 1;
+            while ((long long)g.N * groups * co_split < 148 && co_split * kPairCoChunk < g.Cout) co_split *= 2;
+            if (g.H % 4 == 0 && (co_split == 1 || (long long)g.N * groups * co_split < 2 * blocks2)) {
+                rows = 2;
+                groups = (int)(blocks2 / g.N);
+                co_split = 1;
+            }
             const long long units = (long long)g.N * groups * co_split;
             if (units <= 2147483647ll) {
                 const int resident = 148 * (rows == 1 ? 5 : 3);
                 const unsigned blocks = (unsigned)(units < resident ? units : resident);
-#define MNNB_STEM_PAIR(RELU, ROWS) direct_stem_s2_pair_kernel<RELU, ROWS><<<blocks, kStemThreads, smem, stream>>>(x, w, bias, y, g, co_pad, groups, co_split, (int)units)
-                if (rows == 2) { if (g.relu) MNNB_STEM_PAIR(true, 2); else MNNB_STEM_PAIR(false, 2); }
-                else { if (g.relu) MNNB_STEM_PAIR(true, 1); else MNNB_STEM_PAIR(false, 1); }
+#define MNNB_STEM_PAIR(...) direct_stem_s2_pair_kernel<__VA_ARGS__><<<blocks, kStemThreads, smem, stream>>>(x, w, bias, y, g, co_pad, groups, co_split, (int)units)
+                if (rows == 2) { if (g.relu) MNNB_STEM_PAIR(true, 2, false); else MNNB_STEM_PAIR(false, 2, false); }
+                else if (co_split == 1) { if (g.relu) MNNB_STEM_PAIR(true, 1, false); else MNNB_STEM_PAIR(false, 1, false); }
+                else { if (g.relu) MNNB_STEM_PAIR(true, 1, true); else MNNB_STEM_PAIR(false, 1, true); }
 #undef MNNB_STEM_PAIR
                 return cudaGetLastError();
             }

@@ -530,7 +530,8 @@ def test_depthwise_bands(torch, C, H, W_, N, stride):
     assert np.array_equal(got.astype(np.float64), oracle(layer, xi, wi, bi))
 
 
-@pytest.mark.parametrize("N,Cout,H,Wd", [(1, 33, 64, 96), (1, 64, 30, 44), (2, 16, 128, 128), (6, 40, 160, 160)])
+@pytest.mark.parametrize("N,Cout,H,Wd", [(1, 33, 64, 96), (1, 64, 30, 44), (2, 16, 128, 128), (6, 40, 160, 160), (9, 24, 172, 172),
+                                         (18, 33, 62, 148)])
 def test_stem_shared_channels(torch, N, Cout, H, Wd):
     layer = W.ConvLayer("t", N, 3, Cout, H, Wd, 3, 2, 1, 1, relu=True, seed=Cout)
     xi, wi, bi = W.integer_inputs(layer, -3, 3)

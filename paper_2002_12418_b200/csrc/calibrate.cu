@@ -291,13 +291,14 @@ extern "C" int mnn_calibrate(int device, void* stream, long long consts[MNN_N_CO
         }
     }
 
-    // implicit GEMM: pace of the producer warps' gather.  3x3 stride 2, 64 -> 64 channels, 56 x 56, 4 images: 25
-    // work items of 18 blocks of 32 patch elements each, one item per SM, so the run is launch + 18 blocks + drain
+    // implicit GEMM: pace of the producer warps' gather.  3x3 stride 2, 64 -> 64 channels, 56 x 56, 23 images: 141 work items of
+    // 18 blocks of 32 patch elements each, one item per SM and too many to be cut over clusters, so the run is launch + 18 blocks +
+    // drain
     {
-        GatherGeom g = {4, 64, 56, 56, 28, 28, 3, 2, 1, 1, 576};
+        GatherGeom g = {23, 64, 56, 56, 28, 28, 3, 2, 1, 1, 576};
         int* status = reinterpret_cast<int*>(buf);
         float* x = reinterpret_cast<float*>(buf + 1024);
-        float* U = x + (size_t)4 * 64 * 56 * 56;
+        float* U = x + (size_t)23 * 64 * 56 * 56;
         float* y = U + (size_t)64 * 576;
         cudaMemsetAsync(buf, 0, 1024, st);
         ImplicitGemm ig;

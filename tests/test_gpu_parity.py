@@ -583,12 +583,16 @@ def test_input_transform_two_pass(torch, N, Cin, H, W_, k, m, operand, passes):
     if bound < 0.1: assert rel_l2(got, oracle(layer, x, w, b)) < bound
 
 
-def test_calibration_of_the_direct_kernel(torch):
-    """consts[8] is measured on the kind of layer it stands for (64 -> 64 3x3 at 14 x 14, one image: about 8 us); the bound of two
-    holds the built-in record, taken on the same card with gaps between the launches."""
+def test_calibration_of_direct_and_gather(torch):
+    """consts[8] is measured on the kind of layer it stands for (64 -> 64 3x3 at 14 x 14, one image: about 8 us), consts[13], the
+    implicit gather's pace, on a layer whose K loop is not cut (a block of 128 x 32 elements in 1 us, 250e6 as per element; a cut one
+    gives 160e6).  Within a factor of two of the built-in record; a host that is busy while the launch cost is
+    measured distorts both, so the middle one of five calibrations counts."""
     before = B.mnn_get_calibration()
     try:
-        got = B.mnn_calibrate(0, torch.cuda.current_stream().cuda_stream)
-        assert all(c > 0 for c in got[:9]) and before[8] / 2 < got[8] < before[8] * 2
+        runs = [B.mnn_calibrate(0, torch.cuda.current_stream().cuda_stream) for _ in range(5)]
     finally:
         B.mnn_set_calibration(before)
+    got = [sorted(r[i] for r in runs)[2] for i in range(len(before))]
+    assert all(c > 0 for c in got[:9]) and before[8] / 2 < got[8] < before[8] * 2
+    assert before[13] / 2 < got[13] < before[13] * 2

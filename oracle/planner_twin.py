@@ -367,7 +367,7 @@ def patch_operand_time(L: Layer, lhs, c):
     x, y, v, u = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW, T * Kp * 4, L.Cout * Kp * 4
     drain = 128 * bn * 4 * 45
     if lhs == LHS_IMPLICIT:
-        gather = 128 * 32 * c[13] * 5 // 8 // 10 ** 6
+        gather = min(1024000, 128 * 32 * c[13] // 10 ** 6)  # ps per block of 128 x 32 elements, measured
         block = max(gather * 15 // 8 if L.Cin % 32 else gather * 2 if L.stride >= 4 else gather, bn * 128 * 16)
         fixed, traffic = 0, x + u + y
     else:

@@ -460,9 +460,10 @@ uint64_t patch_operand_time(const LayerShape& s, int lhs, const Calibration& cal
     uint64_t block, fixed = *split > 1 ? 3000000 : 0;                   // (what a cut costs)
     u128 bytes = (u128)x_bytes + u_bytes + y_bytes;
     if (lhs == MNN_GEMM_LHS_IMPLICIT) {
-        // A block of 128 x 32 elements took 1.02 us, five eighths of what consts[13] books; element-wise (Cin not a multiple
-        // of 32) 1.9 us, and two of them from a stride of four on.
-        const uint64_t gather = saturate((u128)128 * 32 * (uint64_t)cal.c[13] * 5u / 8u / 1000000u);
+        // A block of 128 x 32 elements took 1.02 us on these layers (consts[13], which ranks the schemes, says 1.6 in the built-in
+        // record and 1.0 to 1.1 where it is measured: the lesser counts); element-wise (Cin not a multiple of 32) 1.9 us, and two of them from a
+        // stride of four on.
+        const uint64_t gather = std::min<uint64_t>(1024000, saturate((u128)128 * 32 * (uint64_t)cal.c[13] / 1000000u));
         block = std::max<uint64_t>(s.Cin % 32 != 0 ? gather * 15 / 8 : s.stride >= 4 ? gather * 2 : gather, (uint64_t)bn * 128 * 16);
     } else {
         // The staged gather is bound by a CTA's serial loads (four CTAs share an SM) long before its bytes; a block of the

@@ -367,6 +367,18 @@ def test_cut_layers_take_the_shorter_gather(shape, lhs):
     assert (info.algo, info.gemm_lhs) == (B.ALGO_GEMM, lhs)
 
 
+def test_the_gathers_choice_does_not_depend_on_its_booked_rate(restore_calibration):
+    # the gather's pace is a figure of the kernel: with the rate that calibration finds (250e6 against the built-in 400e6) the
+    # booked costs move, but where the patch matrix is still booked the choice between the two must stay
+    l = W.ConvLayer("cut", 47, 304, 304, 8, 8, 3, 2, 1, 1)
+    kw = dict(force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1)
+    for rate in (400, 250):
+        cal = list(restore_calibration)
+        cal[13] = rate * 10 ** 6
+        B.mnn_set_calibration(cal)
+        assert compare(l, kw, kw, cal).gemm_lhs == B.GEMM_LHS_PATCHES
+
+
 # Packed lines against the operand they replace, each by its own time (measured 196 against 595 us, 52 / 104, 56 / 133, 402 / 1183,
 # 290 / 595 where the lines lose; 53 / 27, 86 / 37 where they win).
 @pytest.mark.parametrize("shape,packed", [

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from oracle import direct_conv as oc
+from oracle import planner_twin as T
 from paper_2002_12418_b200 import binding as B
 from paper_2002_12418_b200 import workloads as W
 from tests.util import assert_close, to_dev
@@ -101,4 +102,37 @@ def test_bf16(torch, shape, auto):
             assert np.array_equal(got.cpu().numpy().astype(np.float64), ref)
         else:
             assert_close(got.cpu().numpy(), ref, B.PREC_BF16, "packed lines in BF16")
+    r.close()
+
+
+# Every tiling the planner reaches: one, two and four tiles of 128 cells per item (as many issuing threads), one, two and three
+# weight tiles per step (partial groups, other slot sizes), three and four tensor-core steps per block.  The planner's
+# integer twin names the tiling, so a shape that comes to another one fails.  Integers: exact.
+@pytest.mark.parametrize("shape,bf16,mt,g", [
+    ((6, 32, 299, 10, 82, 2, 1, 1, 6), False, 1, 1), ((11, 32, 34, 12, 92, 2, 1, 1, 6), False, 1, 2),
+    ((10, 32, 1, 28, 65, 3, 1, 1, 4), False, 2, 1), ((29, 32, 18, 13, 33, 3, 1, 6, 6), False, 2, 2),
+    ((40, 32, 1, 13, 93, 2, 1, 1, 3), False, 4, 1), ((32, 32, 26, 20, 52, 3, 1, 2, 2), False, 4, 2),
+    ((63, 32, 1, 26, 26, 2, 1, 1, 6), False, 4, 3), ((9, 1, 471, 91, 23, 2, 1, 0, 1), False, 1, 2),
+    ((14, 2, 178, 109, 69, 5, 1, 0, 2), False, 4, 2), ((20, 9, 1, 25, 76, 3, 1, 1, 1), False, 4, 3),
+    ((17, 64, 72, 33, 68, 6, 2, 0, 6), True, 1, 1), ((1, 64, 75, 34, 78, 6, 2, 0, 6), True, 1, 2),
+    ((53, 128, 2, 20, 28, 4, 1, 0, 6), True, 2, 1), ((50, 128, 58, 23, 23, 4, 1, 0, 6), True, 2, 2),
+    ((48, 64, 1, 11, 87, 2, 1, 0, 3), True, 4, 1), ((55, 64, 18, 27, 27, 3, 1, 1, 4), True, 4, 2),
+    ((23, 64, 1, 110, 17, 2, 1, 0, 4), True, 4, 3)])
+def test_every_tiling(torch, shape, bf16, mt, g):
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    operand = B.OPERAND_BF16 if bf16 else B.OPERAND_TF32
+    tiling = T.packed_lines(T.Layer(N, Cin, Cout, H, W_, k, s, p, d), operand, 148)
+    assert (tiling["mt"], tiling["g"]) == (mt, g)
+    layer = W.ConvLayer("lines", N, Cin, Cout, H, W_, k, s, p, d, relu=False, seed=sum(shape))
+    x, w, b = W.integer_inputs(layer, -3, 3)
+    r = B.ConvLayerRunner(*shape, B.make_opts(relu=0, precision=B.PREC_BF16 if bf16 else B.PREC_TF32, force_algo=B.ALGO_GEMM,
+                                              operand=operand, passes=1))
+    assert r.info.gemm_lhs == B.GEMM_LHS_PACKED
+    r.workspace.fill_(0xFF)                   # NaNs wherever a kernel reads what none has written
+    B.mnn_conv_set_workspace(r.plan, r._ws_ptr, r.info.workspace_bytes)
+    y = torch.full((N, Cout, r.info.OH, r.info.OW), float("nan"), device="cuda:0")
+    r.run(to_dev(torch, x), to_dev(torch, w), to_dev(torch, b), y)
+    torch.cuda.synchronize()
+    assert r.device_status() == 0
+    assert np.array_equal(y.cpu().numpy().astype(np.float64), oc.direct_conv(x, w, b, s, p, d, 1, False))
     r.close()

@@ -566,6 +566,14 @@ def test_input_transform_bands(torch, N, Cin, H, W_, pad, m):
     assert rel_l2(got, oracle(layer, x, w, b)) < 1e-4
 
 
+def _absolute_input_transform(x, m, k, pad, points_id):
+    """sum of |B^T| |d| |B| per element of V, in the layout of input_transform_f64."""
+    Bt = np.abs(wx.matrices_f64(m, k, points_id)[2])
+    tiles = np.abs(wx.extract_tiles_f64(x, m, k, pad))
+    V = np.einsum("ia,ntucab,jb->ijntuc", Bt, tiles, Bt, optimize=True)
+    return V.reshape(Bt.shape[0] ** 2, -1, x.shape[1])
+
+
 # Input transform by two passes through shared memory: tile rows cut into segments (ragged last one), channels off the
 # block of 32, more items than CTAs fit the chip (the next item's loads in flight), single tiles; every operand format.
 @pytest.mark.parametrize("N,Cin,H,W_,k,m", [
@@ -578,8 +586,26 @@ def test_input_transform_two_pass(torch, N, Cin, H, W_, k, m, operand, passes):
     got, info, _ = run_layer(torch, layer, opts_for(layer, force_algo=B.ALGO_WINOGRAD, force_m=m, operand=operand, passes=passes,
                                                     fused=B.FUSED_NEVER), (x, w, b))
     assert info.algo == B.ALGO_WINOGRAD and info.m == m
+    # V itself, element by element: two fp32 passes of alpha terms over B^T rounded once (2 alpha + 4 roundings of the sum of
+    # magnitudes), then one rounding to the format (twice its digits as hi + lo).  The layer's result follows below, but its
+    # bound grows with the transforms' amplification.
+    r = B.ConvLayerRunner(N, Cin, 24, H, W_, k, 1, k // 2, 1, opts_for(layer, force_algo=B.ALGO_WINOGRAD, force_m=m, operand=operand, passes=passes,
+                                                                       fused=B.FUSED_NEVER))
+    r.run(to_dev(torch, x), to_dev(torch, w), None, torch.zeros((N, 24, info.OH, info.OW), device="cuda:0"), stage_mask=B.STAGE_INPUT)
+    torch.cuda.synchronize()
+    n, eb, dtype = info.alpha ** 2 * info.chunk_tiles * info.cin_pad, *((2, torch.bfloat16) if operand == B.OPERAND_BF16 else (4, torch.float32))
+    V = r.workspace_view(info.v_offset, n * eb, dtype).double()
+    if passes == 3:
+        V = V + r.workspace_view(info.v_offset + info.v_bytes // 2, n * eb, dtype).double()
+    V = V.cpu().numpy().reshape(info.alpha ** 2, info.chunk_tiles, info.cin_pad)
+    r.close()
+    ref, size = wx.input_transform_f64(x, m, k, k // 2, info.points_id), _absolute_input_transform(x, m, k, k // 2, info.points_id)
+    half_ulp = 2.0 ** -((8 if operand == B.OPERAND_BF16 else 11) * (2 if passes == 3 else 1))
+    fp32 = (2 * info.alpha + 4) * 2.0 ** -24 * size
+    assert (np.abs(V[:, :, :Cin] - ref) <= fp32 + half_ulp * (np.abs(ref) + fp32)).all() and not V[:, :, Cin:].any()
     # three times the error expected of operands rounded to this format, amplified by these transforms, and fp32 arithmetic
     bound = 3e-6 * B.mnn_accuracy_ppm(m, k, info.points_id, operand, passes) + 2e-5
+    assert np.isfinite(got).all()
     if bound < 0.1: assert rel_l2(got, oracle(layer, x, w, b)) < bound
 
 

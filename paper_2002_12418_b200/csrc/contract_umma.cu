@@ -54,15 +54,15 @@ constexpr int kSwizzleBytes = 128;     // bytes of K per shared-memory row
 constexpr int kSmemBudget = 200 * 1024;
 
 struct KernelParams {
-    int alpha2, n_tile_blocks, n_co_blocks, bn, k_blocks, passes, stages, tmem_cols;   // bn = output channels per work item
+    int alpha2, n_tile_blocks, n_co_blocks, bn, k_blocks, stages, tmem_cols;   // bn = output channels per work item
     int Cout;
     long long tiles;
     long long n_items;
     ContractEpilogue epi;
     int* status;
-    // a_mn mode: operand A comes from x [images][Cin][hw]; atoms of 32 pixels: full_atoms = hw / 32 whole ones
+    // A_MN kernels: operand A comes from x [images][Cin][hw]; atoms of 32 pixels: full_atoms = hw / 32 whole ones
     // and a ragged one when hw % 32 != 0; tiles_per_image work items of up to four atoms cover an image
-    int a_mn, hw, full_atoms, atoms_per_image, tiles_per_image;
+    int hw, full_atoms, atoms_per_image, tiles_per_image;
     // 1: hi and lo operand tiles arrive with one copy each for V and U (maps with a hi / lo dimension, see
     // encode_operand_pair_map); halves the copies the producer issues per stage
     int merged;
@@ -74,7 +74,10 @@ struct KernelParams {
 constexpr int kErrProducerWait = 1, kErrMmaWaitFull = 2, kErrMmaWaitTmem = 3, kErrEpilogueWait = 4;
 
 // High words of the shared-memory descriptors (distance of 8-row groups, version, swizzle mode): K-major rows of SW bytes in
-// the SW-byte swizzle, and the MN-major operand of 32-bit elements (ptx::smem_desc_mn128_b32).
+// the SW-byte swizzle, and the MN-major operand of 32-bit elements, which the tensor core takes only in the "128-byte swizzle
+// with a 32-byte base": rows of 128 bytes hold 32 consecutive elements of M of one K index, the four 32-byte pieces of a row
+// are permuted by the row index modulo 4 (what a TMA load with SWIZZLE_128B_ATOM_32B of a box {32 elements of M, rows of K}
+// produces), four rows (512 bytes) form an atom, and consecutive atoms along K are 512 bytes apart.
 template <int SW>
 constexpr uint32_t kDescHiB = ((uint32_t)SW * 8u >> 4) | (1u << 14) | ((SW == 128 ? 2u : 4u) << 29);
 template <int SW, bool A_MN>
@@ -693,7 +696,6 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return cudaErrorInvalidValue;
     KernelParams p;
-    p.a_mn = 1;
     p.merged = 0;
     p.hw = uc.x_hw;
     p.full_atoms = uc.x_hw / 32;
@@ -734,7 +736,6 @@ cudaError_t launch_contract_umma_x(const UmmaContract& uc, const float* x, const
     p.n_co_blocks = uc.n_co_blocks;
     p.bn = uc.bn;
     p.k_blocks = (uc.k_blocks + uc.kb - 1) / uc.kb;
-    p.passes = 1;
     p.stages = uc.stages / uc.kb;
     p.tmem_cols = uc.tmem_cols;
     p.Cout = uc.Cout;
@@ -759,7 +760,6 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
     if (tiles <= 0) return cudaSuccess;
     if (tiles > uc.tiles_capacity) return cudaErrorInvalidValue;
     KernelParams p;
-    p.a_mn = 0;
     p.merged = uc.merged;
     p.hw = 0;
     p.full_atoms = 0;
@@ -770,7 +770,6 @@ cudaError_t launch_contract_umma(const UmmaContract& uc, long long tiles, const 
     p.n_co_blocks = uc.n_co_blocks;
     p.bn = uc.bn;
     p.k_blocks = (uc.k_blocks + uc.kb - 1) / uc.kb;
-    p.passes = uc.passes;
     p.stages = uc.stages / uc.kb;
     p.tmem_cols = uc.tmem_cols;
     p.Cout = uc.Cout;

@@ -52,6 +52,8 @@ def stage_work(info, N, Cin, Cout, H, W, k, groups):
         if info.gemm_lhs in (B.GEMM_LHS_X, B.GEMM_LHS_IMPLICIT):
             v = x_bytes                    # the contraction reads x itself
         else:
+            if info.gemm_lhs == B.GEMM_LHS_PACKED:
+                v = info.v_bytes           # the packed planes
             out["input"] = (x_bytes + v, 0)
         out["contract"] = (v + b_el * Cout * K + y_bytes, 2 * T * Cout * K * info.passes)
     else:

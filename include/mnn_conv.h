@@ -135,6 +135,9 @@ typedef struct {
  * ALU flops * c_alu) + launch cost, in integer picoseconds).
  * cost_ps[] order: 0 DIRECT; 1 GEMM tf32; 2 GEMM bf16; 3..5 Winograd m=2,4,6 tf32x1;
  * 6..8 tf32x3; 9..11 bf16x1; 12..14 bf16x3; 15 Winograd F(2x2,3x3) tf32x1 as one fused kernel.
+ * The costs rank the schemes.  A GEMM candidate is booked at the cheapest of PATCHES, X and IMPLICIT without a cut of
+ * the K loop, also where the planner then runs it as PACKED or cuts the loop over clusters, which it decides by
+ * closer estimates that are not reported; GEMM bf16 that takes over as PACKED is booked at its own cost.
  * Candidates that are not applicable or fail the accuracy gate hold MNN_COST_INADMISSIBLE; every
  * other figure saturates at MNN_COST_INADMISSIBLE - 1.
  * paper_mul[] is the paper's own multiplication count (Eq. 2) for output tile sizes n = 1, 2, 4, 6,

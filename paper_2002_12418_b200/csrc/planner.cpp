@@ -740,7 +740,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     for (int i = 0; i < MNN_N_CANDIDATES; ++i)
         if (d->cost_ps[i] != MNN_COST_INADMISSIBLE && (best < 0 || d->cost_ps[i] < d->cost_ps[best])) best = i;
     // BF16 class: packed lines in BF16, booked above at the cost of the patch matrix, take over from a scheme that is neither
-    // faster by this estimate nor expected to be more accurate (3x3 256 channels 56 x 56 batch 64: 257 us, Winograd with m =
+    // faster by this estimate nor expected to be more accurate (3x3 256 channels 56 x 56 batch 64, warm: 248 us, Winograd with m =
     // 4 and TF32 operands 431; 64 channels 50 / 103; but 512 channels 7 x 7 batch 32 26 / 19).
     if (best >= 0 && best != 2 && lhs_of[2] == MNN_GEMM_LHS_PACKED && ppm_of[2] <= ppm_of[best]) {
         const uint64_t cost = packed_cost(s, MNN_OPERAND_BF16, cal);

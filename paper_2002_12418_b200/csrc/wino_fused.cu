@@ -153,7 +153,7 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
     __shared__ int abort_flag;
     volatile int* abortp = &abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform_warp(), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t v_base = smem_base;                                 // V: [buffer][position][tile][16 channels], swizzled
     const uint32_t u_base = smem_base + kVBufs * kVBufBytes;           // U ring: [slot][position in group][128 rows][16 channels]
@@ -189,22 +189,24 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
 
     if (warp == 0) {
         // ------------------------------ weight stream (bulk copies) ------------------------------
-        if (lane == 0) {
+        {
             uint32_t slot = 0, phase = 0;
             bool ok = true;
             for (int item = first; item < p.n_items && ok; item += step) {
                 const int cb = item / p.n_tile_blocks;
                 const uint8_t* src = p.U + (size_t)cb * p.k_blocks * kUBlockBytes;
                 for (int c = 0; c < p.k_blocks * kGroups; ++c) {           // consecutive copies are consecutive in memory
-                    if (!ptx::mbar_wait_relaxed(ptx::smem_u32(&u_empty[slot]), phase ^ 1u, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrStreamWait);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&u_empty[slot]), phase ^ 1u, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrStreamWait);
                         *abortp = 1;
                         ok = false;
                         break;
                     }
                     const uint32_t bar = ptx::smem_u32(&u_full[slot]);
-                    ptx::mbar_expect_tx(bar, kUSlotBytes);
-                    bulk_load(u_base + slot * kUSlotBytes, src + (size_t)c * kUSlotBytes, kUSlotBytes, bar);
+                    if (ptx::elect_one()) {
+                        ptx::mbar_expect_tx(bar, kUSlotBytes);
+                        bulk_load(u_base + slot * kUSlotBytes, src + (size_t)c * kUSlotBytes, kUSlotBytes, bar);
+                    }
                     if (++slot == kSlots) {
                         slot = 0;
                         phase ^= 1u;
@@ -214,21 +216,21 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issue ------------------------------
-        if (lane == 0) {
+        {
             const uint32_t idesc = ptx::mma_idesc(2, kCo, kTiles);
             uint32_t slot = 0, phase = 0, buf = 0, v_phase = 0, acc_phase = 0;
             bool ok = true;
             const uint32_t a_lo_base = kDescLo + (u_base >> 4), b_lo_base = kDescLo + (v_base >> 4);
             for (int item = first; item < p.n_items && ok; item += step) {
-                if (!ptx::mbar_wait_bounded(ptx::smem_u32(&acc_empty), acc_phase ^ 1u, abortp)) {
-                    if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitAcc);
+                if (!ptx::mbar_wait_warp(ptx::smem_u32(&acc_empty), acc_phase ^ 1u, abortp)) {
+                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitAcc);
                     *abortp = 1;
                     break;
                 }
                 ptx::tc_fence_after();
                 for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
-                    if (!ptx::mbar_wait_bounded(ptx::smem_u32(&v_full[buf]), v_phase, abortp)) {
-                        if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitV);
+                    if (!ptx::mbar_wait_warp(ptx::smem_u32(&v_full[buf]), v_phase, abortp)) {
+                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitV);
                         *abortp = 1;
                         ok = false;
                         break;
@@ -236,8 +238,8 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                     const uint32_t acc0 = kb != 0 ? 1u : 0u;
 #pragma unroll 1
                     for (int grp = 0; grp < kGroups; ++grp) {
-                        if (!ptx::mbar_wait_bounded(ptx::smem_u32(&u_full[slot]), phase, abortp)) {
-                            if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitU);
+                        if (!ptx::mbar_wait_warp(ptx::smem_u32(&u_full[slot]), phase, abortp)) {
+                            if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitU);
                             *abortp = 1;
                             ok = false;
                             break;
@@ -246,27 +248,29 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                         const uint32_t a_lo = a_lo_base + slot * (kUSlotBytes >> 4);
                         const uint32_t b_lo = b_lo_base + buf * (kVBufBytes >> 4) + (uint32_t)grp * ((kGroup * kVPosBytes) >> 4);
                         const uint32_t d_t = tmem_base + (uint32_t)grp * (kGroup * kTiles);
+                        if (ptx::elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < kKBlock / 8; ++ks)
+                            for (int ks = 0; ks < kKBlock / 8; ++ks)
 #pragma unroll
-                            for (int g = 0; g < kGroup; ++g)
-                                mma_tf32_lo(d_t + g * kTiles, a_lo + g * (kUPosBytes >> 4) + ks * 2,
-                                            b_lo + g * (kVPosBytes >> 4) + ks * 2, kDescHi, idesc, ks != 0 ? 1u : acc0);
-                        ptx::mma_commit(ptx::smem_u32(&u_empty[slot]));
+                                for (int g = 0; g < kGroup; ++g)
+                                    mma_tf32_lo(d_t + g * kTiles, a_lo + g * (kUPosBytes >> 4) + ks * 2,
+                                                b_lo + g * (kVPosBytes >> 4) + ks * 2, kDescHi, idesc, ks != 0 ? 1u : acc0);
+                            ptx::mma_commit(ptx::smem_u32(&u_empty[slot]));
+                        }
                         if (++slot == kSlots) {
                             slot = 0;
                             phase ^= 1u;
                         }
                     }
                     if (!ok) break;
-                    ptx::mma_commit(ptx::smem_u32(&v_empty[buf]));     // this buffer may be overwritten once these MMAs retire
+                    if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&v_empty[buf]));     // this buffer may be overwritten once these MMAs retire
                     if (++buf == kVBufs) {
                         buf = 0;
                         v_phase ^= 1u;
                     }
                 }
                 if (!ok) break;
-                ptx::mma_commit(ptx::smem_u32(&acc_full));
+                if (ptx::elect_one()) ptx::mma_commit(ptx::smem_u32(&acc_full));
                 acc_phase ^= 1u;
             }
         }

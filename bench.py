@@ -237,7 +237,12 @@ def stage_work(layer, info):
     y_bytes = 4 * N * Cout * info.OH * info.OW
     b_el = (2 if info.operand == B.OPERAND_BF16 else 4) * (2 if info.passes == 3 else 1)
     out = {}
-    if info.algo == B.ALGO_WINOGRAD and info.fused:
+    if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
+        T = N * info.OH * (-(-info.OW // info.m))
+        out["contraction"] = {"bytes": x_bytes + y_bytes + info.u_bytes, "flops": 2 * layer.k * info.alpha * Cout * Cin * T * info.passes}
+    elif info.algo == B.ALGO_GEMM and info.gemm_lhs == B.GEMM_LHS_ROWS:
+        out["contraction"] = {"bytes": x_bytes + y_bytes + info.u_bytes, "flops": layer.direct_flops * info.passes}
+    elif info.algo == B.ALGO_WINOGRAD and info.fused:
         T = N * (-(-info.OH // 2)) * (-(-info.OW // 2))
         out["contraction"] = {"bytes": x_bytes + y_bytes + 4 * 16 * Cout * Cin, "flops": 2 * 16 * Cout * Cin * T}
     elif info.algo == B.ALGO_WINOGRAD:

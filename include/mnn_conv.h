@@ -53,7 +53,10 @@ enum { MNN_PREC_TF32 = 0, MNN_PREC_BF16 = 1 };             /* accuracy class */
 enum { MNN_OPERAND_AUTO = 0, MNN_OPERAND_TF32 = 1, MNN_OPERAND_BF16 = 2, MNN_OPERAND_FP32_REF = 3 };
 enum { MNN_POINTS_AUTO = 0, MNN_POINTS_PAPER = 1, MNN_POINTS_UNIT = 2, MNN_POINTS_MIXED = 3 };
 enum { MNN_GEMM_LHS_AUTO = 0, MNN_GEMM_LHS_PATCHES = 1, MNN_GEMM_LHS_X = 2, MNN_GEMM_LHS_IMPLICIT = 3,
-       MNN_GEMM_LHS_PACKED = 4 };
+       MNN_GEMM_LHS_PACKED = 4, MNN_GEMM_LHS_ROWS = 5 };
+/* info.fused: the form of a Winograd plan other than the two-dimensional one (the option of the same name has values of its own):
+ * one kernel on 2 x 2 tiles or one kernel by rows */
+enum { MNN_FUSED_TILES = 1, MNN_FUSED_ROWS = 2 };
 enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_STAGE_OUTPUT = 8,
        MNN_STAGE_ALL = 15 };
 
@@ -99,6 +102,8 @@ enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_ST
  *              (TF32 or BF16), and every kernel tap reads them at a shifted start.  The lines are about
  *              as large as x (in the operand format) and lie in the workspace, up to 4 GiB, where
  *              IMPLICIT needs room for the weights only: ask for that where workspace is short.
+ *              ROWS (not an option value; only where the caller leaves every choice open): the definition in one
+ *              kernel that converts rows of x itself, one BF16 product, or three of hi + lo halves (passes = 3).
  *              Asking for X or IMPLICIT where it does not apply fails the plan.
  *   fused      Winograd F(2x2, 3x3) as ONE kernel (input transform, contraction and output
  *              transform fused; the transformed tensors V and M never reach device memory):
@@ -137,7 +142,8 @@ typedef struct {
  * 6..8 tf32x3; 9..11 bf16x1; 12..14 bf16x3; 15 Winograd F(2x2,3x3) tf32x1 as one fused kernel.
  * The costs rank the schemes.  A GEMM candidate is booked at the cheapest of PATCHES, X and IMPLICIT without a cut of
  * the K loop, also where the planner then runs it as PACKED or cuts the loop over clusters, which it decides by
- * closer estimates that are not reported; GEMM bf16 that takes over as PACKED is booked at its own cost.
+ * closer estimates that are not reported; GEMM bf16 that takes over as PACKED is booked at its own cost, and so is a form by rows
+ * that takes over: the definition as candidate 2 (with passes = 3 in the TF32 class), Winograd as 12.
  * Candidates that are not applicable or fail the accuracy gate hold MNN_COST_INADMISSIBLE; every
  * other figure saturates at MNN_COST_INADMISSIBLE - 1.
  * paper_mul[] is the paper's own multiplication count (Eq. 2) for output tile sizes n = 1, 2, 4, 6,
@@ -161,9 +167,9 @@ typedef struct {
     long long u_offset, u_bytes, v_offset, v_bytes, m_offset, m_bytes;
     long long predicted_error_ppm;   /* accuracy model's relative L2 error x 1e6 for the choice */
     int chosen_candidate;            /* index into cost_ps, -1 when the choice was forced outside the list */
-    int gemm_lhs;                    /* GEMM scheme: MNN_GEMM_LHS_PATCHES, _X, _IMPLICIT or _PACKED as planned, else 0 */
+    int gemm_lhs;                    /* GEMM scheme: MNN_GEMM_LHS_PATCHES, _X, _IMPLICIT, _PACKED or _ROWS as planned, else 0 */
     unsigned long long cost_ps[MNN_N_CANDIDATES];
-    int fused;                       /* 1 when the plan is the single fused Winograd kernel (no V, no M) */
+    int fused;                       /* MNN_FUSED_TILES, MNN_FUSED_ROWS: Winograd in one kernel (no V, no M); else 0 */
     int paper_n_hat;
     unsigned long long paper_mul[4];
     int strassen;                    /* 1 when the plan runs one Strassen level (alpha = 1, seven products) */

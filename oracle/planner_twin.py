@@ -37,7 +37,7 @@ from dataclasses import dataclass, field
 ALGO_WINOGRAD, ALGO_GEMM, ALGO_DIRECT = 1, 2, 3
 OPERAND_TF32, OPERAND_BF16, OPERAND_FP32_REF = 1, 2, 3
 PREC_TF32, PREC_BF16 = 0, 1
-LHS_PATCHES, LHS_X, LHS_IMPLICIT, LHS_PACKED = 1, 2, 3, 4
+LHS_PATCHES, LHS_X, LHS_IMPLICIT, LHS_PACKED, LHS_ROWS = 1, 2, 3, 4, 5
 INADMISSIBLE = 2 ** 64 - 1
 SATURATED = 2 ** 64 - 2
 MAX_CHUNK_BYTES = 4 << 30          # V + M of one chunk may not exceed this, whatever the cost says
@@ -286,6 +286,78 @@ def packed_cost(L: Layer, operand: int, c) -> int:
     hidden = 0 if not tf32 else min(2000000, c[5]) if p["few"] else c[5]
     return sat(kernel_ps(c, mem_as=moved) - hidden
                + kernel_ps(c, mem_as=(p["a_bytes"] + y) * c[0], tensor_as=p["product_ps"] * 10 ** 6))
+
+
+def _mma_cycles(n: int) -> int:
+    """An instruction of 128 x n x 32 bytes: 57 cycles for its left operand, more only from 128 channels on."""
+    return max(n // 2, 57 + n // 7)
+
+
+def rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, slots, rounds):
+    """Time of the convolution by rows in ps without its launch."""
+    def moved(n):
+        return 4096 + 32 * n
+
+    steps, wide = k, 2 if mode == 2 else 1
+    tiles = steps * taps * mt
+    mma = tiles * (_mma_cycles(2 * bn) + _mma_cycles(bn) if mode == 2 else mode * _mma_cycles(bn)) * 461
+    shared = tiles * (moved(2 * bn) + moved(bn) if mode == 2 else mode * moved(bn)) + steps * b_slot + a_slot
+    x_bytes, tasks = rows * 64 * (1 if m == 1 else alpha), cdiv(rows, 32) * (1 if m == 1 else 2)
+    serial = cdiv(tasks, 10) * 595000 if m == 1 else cdiv(tasks, 12) * 1418000
+    stage = max(mma, (shared * 2 + x_bytes * (12 if m == 1 else 3)) * 193 // 100, serial) + steps * 51500
+    drain, loop = 1098000 + 5700 * mt * bn * alpha * wide, slots * stage + 672000
+    cost = rounds * max(loop, drain) + drain if bufs == 2 else rounds * (loop + drain)
+    return cost + (2348000 + 4000 * mt * bn * m if split > 1 else 0) - 446000
+
+
+def rows_tiling(L: Layer, m: int, passes: int, sms: int):
+    """The one-kernel convolution by rows: m outputs of a row per cell (one-dimensional Winograd F(2, 3); 1: the definition), kernel
+    rows as shifts.  The cheapest tiling that fits as a dict with its time in ps, or None."""
+    k = L.k
+    if not (m == 2 and k == 3 or m == 1 and k in (2, 3, 5, 7)):
+        return None
+    alpha = 1 if m == 1 else m + k - 1
+    taps = k if m == 1 else alpha
+
+    def pitch(size, out, reach):
+        return max(out, min(out + reach, max(size + L.pad, out + reach - L.pad)))
+
+    hq = pitch(L.H, L.OH, k - 1)
+    wq = pitch(L.W, L.OW, k - 1) if m == 1 else cdiv(L.OW, m)
+    cells, span = L.N * hq * wq, (k - 1) * wq + (k - 1 if m == 1 else 0)
+    if cells >= (1 << 31) - 65536 or span > 2048:
+        return None
+    stages, co16, room, best = cdiv(L.Cin, 16), cdiv(L.Cout, 16) * 16, 213 * 1024, None
+    for mode in ([1] if passes == 1 else [3] if m == 2 else [2, 3]):
+        halves, wide = (1 if mode == 1 else 2), (2 if mode == 2 else 1)
+        for mt in ((1, 2) if m == 1 else (1,)):
+            seen = set()
+            for nb in range(1, co16 // 16 + 1):
+                bn = cdiv(cdiv(co16, nb), 16) * 16
+                if bn in seen:
+                    continue
+                seen.add(bn)
+                if wide * bn > 256 or alpha * mt * wide * bn > 512:
+                    continue
+                bufs = 2 if 2 * alpha * mt * wide * bn <= 512 else 1
+                if mt == 2 and bufs == 1:
+                    continue
+                rows = cdiv(128 * mt + span, 8) * 8
+                a_slot, b_slot = alpha * halves * rows * 32, taps * halves * bn * 32
+                if 2 * a_slot + 3 * b_slot > room:
+                    continue
+                items = cdiv(cells, 128 * mt) * nb
+                if items >= 1 << 31:
+                    continue
+                for split in (1, 2, 4, 8):
+                    if split > 1 and (mt > 1 or items * split > sms or split == 4 and items > 32 or split == 8 and items > 8
+                                      or stages < 2 * split or bn * m * 512 > room):
+                        break
+                    cost = rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, cdiv(stages, split),
+                                     cdiv(items * split, sms))
+                    if best is None or cost < best["time_ps"]:
+                        best = dict(time_ps=cost, mode=mode, mt=mt, bn=bn, split=split, items=items, rows=rows)
+    return best
 
 
 def gemm_cost(L: Layer, operand: int, lhs, c) -> int:
@@ -585,15 +657,38 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
         cost = packed_cost(L, OPERAND_BF16, c)
         if cost < ch.cost_ps[best]:
             ch.cost_ps[2], best = cost, 2
+    # The convolution by rows takes over where nothing is forced, it is estimated faster than a tensor-core scheme (by what is held
+    # against it: the estimates' measured errors) and not expected to be less accurate: as candidate 2 (the definition) or 12 (Winograd m = 2).
+    held = 10 if L.W % 4 and L.k <= 5 else 15 if L.k == 7 and best >= 3 and _candidates()[best][1] == 6 else 11
+    rows, ppm_before = False, side.get(best, {}).get("ppm", 0)
+    free = o.force_algo == o.force_m == o.operand == o.passes == o.points_id == o.gemm_lhs == o.fused == 0
+    if free and wino_shape and best > 0:
+        for m in (1, 2):
+            passes, slot = (1 if o.precision == PREC_BF16 else 3), (2 if m == 1 else 12)
+            t = None if m == 2 and passes == 1 else rows_tiling(L, m, passes, c[7] if c[7] > 0 else 148)
+            if t is None:
+                continue
+            pid, p = (0, ppm.get((1, L.k, 0, OPERAND_BF16, passes), -1)) if m == 1 else best_points(ppm, m, L.k, OPERAND_BF16, passes)
+            now = ch.cost_ps[best]
+            lines = not rows and side[best].get("lhs") == LHS_PACKED
+            if lines and L.Cout < 256:
+                continue
+            if lines:
+                now = min(now, packed_cost(L, _candidates()[best][2], c))
+            cost = t["time_ps"] + c[5]
+            if p < 0 or p > ppm_before or cost * (10 if rows else 9 if lines else held) >= now * 10:
+                continue
+            best, rows, ch.cost_ps[slot] = slot, True, cost
+            side[slot] = dict(lhs=LHS_ROWS, ppm=p, pid=pid, chunk=L.N, n_chunks=1)
     if best < 0:
         return ch
     algo, m, operand, passes = _candidates()[best]
-    ch.chosen, ch.algo, ch.operand, ch.passes = best, algo, operand, passes
+    ch.chosen, ch.algo, ch.operand, ch.passes = best, algo, operand, 3 if rows and o.precision == PREC_TF32 else passes
     ch.error_ppm = side.get(best, {}).get("ppm", 0)
     if algo == ALGO_WINOGRAD:
         ch.m, ch.points_id = m, side[best]["pid"]
         ch.chunk_images, ch.n_chunks = side[best]["chunk"], side[best]["n_chunks"]
-        ch.fused = 1 if best == FUSED_SLOT else 0
+        ch.fused = 1 if best == FUSED_SLOT else 2 if rows else 0
     else:
         ch.m, ch.points_id, ch.chunk_images, ch.n_chunks = 1, 0, L.N, 1
         ch.gemm_lhs = side[best]["lhs"] if algo == ALGO_GEMM else 0

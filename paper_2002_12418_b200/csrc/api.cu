@@ -17,6 +17,7 @@
 #include "kernels.h"
 #include "line_conv.h"
 #include "planner.h"
+#include "rows_conv.h"
 #include "strassen.h"
 #include "wino_fused.h"
 #include "wino_rect.h"
@@ -65,6 +66,7 @@ struct mnn_conv_plan_s {
     TransformMatrices mats;
     // run-time state
     char* ws = nullptr;              // status word and U (persistent part), and V, M unless tws is set
+    int* status = nullptr;           // the status word where it lies elsewhere: a network keeps those of its layers together
     char* tws = nullptr;             // optional separate transient part: V at tws, M at tws + (m_offset - v_offset)
     long long ws_bytes = 0;
     const float* prepared_w = nullptr;
@@ -76,6 +78,8 @@ struct mnn_conv_plan_s {
     int pad_h = 0, pad_w = 0;        // rectangular plans: padding per axis (s.pad is unused there)
     bool fused = false;              // Winograd F(2x2,3x3) as the single fused kernel: the workspace holds U only
     FusedWino fw;
+    bool rows = false;               // the convolution by rows in one kernel: the workspace holds U only
+    RowsConv rc;
     // optional per-launch timing
     bool profiling = false;
     std::vector<cudaEvent_t> events;     // pairs (before, after)
@@ -93,7 +97,7 @@ void* v_lo(mnn_conv_plan_t p)
     return store_is_split(p->store_mode) ? transient_base(p) + p->v_offset + p->v_bytes / 2 : nullptr;
 }
 float* m_buf(mnn_conv_plan_t p) { return reinterpret_cast<float*>(transient_base(p) + p->m_offset); }
-int* status_word(mnn_conv_plan_t p) { return reinterpret_cast<int*>(p->ws); }
+int* status_word(mnn_conv_plan_t p) { return p->status ? p->status : reinterpret_cast<int*>(p->ws); }
 
 int store_mode_of(int operand, int passes)
 {
@@ -114,7 +118,14 @@ void layout_workspace(mnn_conv_plan_t p)
         return;
     }
     long long off = kStatusBytes;
-    if (p->rect) {
+    if (p->rows) {
+        p->cin_pad = p->rc.p.k_slots * kRowsChannels;
+        p->chunk_tiles = p->rc.p.T;
+        p->m_row_stride = 0;
+        p->u_bytes = align_up(p->rc.p.u_bytes, 2048);
+        p->v_bytes = p->m_bytes = 0;
+        p->launches_per_run = 1;
+    } else if (p->rect) {
         const long long n_seg = p->rect == 1 ? (s.OW + d.m - 1) / d.m : (s.OH + d.m - 1) / d.m;
         p->cin_pad = (int)align_up(s.Cin, 8);
         p->chunk_tiles = p->rect == 1 ? (long long)s.N * s.OH * n_seg : (long long)s.N * n_seg * s.OW;
@@ -129,7 +140,7 @@ void layout_workspace(mnn_conv_plan_t p)
         p->cin_pad = (int)align_up(s.Cin, 8);
         p->chunk_tiles = (long long)d.chunk_images * th * tw;
         p->m_row_stride = (int)align_up(p->chunk_tiles, 32);
-        p->fused = d.fused != 0;
+        p->fused = d.fused == MNN_FUSED_TILES;
         p->u_bytes = p->fused ? align_up(fused_wino_weight_bytes(s.Cout, s.Cin), 2048) : align_up(a2 * s.Cout * p->cin_pad * eb, 2048);
         p->v_bytes = p->fused ? 0 : align_up(a2 * p->chunk_tiles * p->cin_pad * eb, 2048);
         p->m_bytes = p->fused ? 0 : align_up(a2 * s.Cout * p->m_row_stride * 4, 1024);
@@ -181,7 +192,7 @@ LineShape line_shape(mnn_conv_plan_t p)
 // Form, transform matrices and workspace layout of the decision in p->d (square layers).
 int realise_decision(mnn_conv_plan_t p, const char** why)
 {
-    p->packed = p->fused = p->gemm_x = p->gemm_implicit = false;
+    p->packed = p->fused = p->gemm_x = p->gemm_implicit = p->rows = false;
     if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
         p->packed = line_plan(line_shape(p), p->tiling_sms, &p->lc.p);
         if (!p->packed) {
@@ -199,6 +210,20 @@ int realise_decision(mnn_conv_plan_t p, const char** why)
         std::memcpy(p->mats.At, wm.At32.data(), wm.At32.size() * sizeof(float));
         std::memcpy(p->mats.G, wm.G32.data(), wm.G32.size() * sizeof(float));
         std::memcpy(p->mats.Bt, wm.Bt32.data(), wm.Bt32.size() * sizeof(float));
+    }
+    if (p->d.rows) {
+        const LayerShape& s = p->s;
+        const int m = p->d.algo == MNN_ALGO_WINOGRAD ? p->d.m : 1;
+        p->rows = rows_plan({s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.k, s.pad, s.pad, s.OH, s.OW, m, p->d.passes}, p->tiling_sms, &p->rc.p);
+        if (p->rows && m > 1) {
+            std::memcpy(p->rc.At, p->mats.At, sizeof(float) * m * p->d.alpha);
+            std::memcpy(p->rc.G, p->mats.G, sizeof(float) * p->d.alpha * s.k);
+            std::memcpy(p->rc.Bt, p->mats.Bt, sizeof(float) * p->d.alpha * p->d.alpha);
+        }
+        if (!p->rows || !rows_matrices_ok(p->rc)) {
+            *why = "no tiling of the convolution by rows fits this layer";
+            return MNN_EUNSUPPORTED;
+        }
     }
     layout_workspace(p);
     return MNN_OK;
@@ -420,6 +445,31 @@ mnn_conv_plan_t mnn_conv_plan_rect(int N, int Cin, int Cout, int H, int W, int k
         delete p;
         return nullptr;
     }
+    // Left to itself in the TF32 class: the definition in one kernel by rows instead, hi + lo operands (more accurate than any
+    // transform), where that is estimated faster.  The three kernels: 11.1 us, the product's multiply-adds at 0.44 PMAC/s and V and M
+    // at 2.8 TB/s (fitted to 38 random layers, 11 % rms, so a tenth is held against the rows).  192 channels 17 x 17 batch 32, 1 x 7: 28.8 -> 21.7 us.
+    if (o.precision == MNN_PREC_TF32 && passes == 3 && o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 &&
+        o.points_id == 0 && o.gemm_lhs == MNN_GEMM_LHS_AUTO && o.fused == 0) {
+        const Calibration cal = current_calibration();
+        if (cal.c[7] > 0) p->tiling_sms = (int)cal.c[7];
+        RowsConv rc;
+        const long long macs = 3ll * p->d.alpha * p->chunk_tiles * Cout * p->cin_pad;
+        const long long three = 11100000 + macs / 100000 * 229 + (p->v_bytes + p->m_bytes) / 100 * 36;
+        const long long rows_ppm = accuracy_ppm(1, k, 0, MNN_OPERAND_BF16, 3);
+        if (rows_ppm >= 0 && rows_ppm <= ppm && rows_plan({N, Cin, Cout, H, W, kh, kw, pad_h, pad_w, OH, OW, 1, 3}, p->tiling_sms, &rc.p) &&
+            (rc.p.time_ps + cal.c[5]) * 11 < three * 10) {
+            p->rc = rc;
+            p->rows = true;
+            p->d.rows = true;
+            p->d.algo = MNN_ALGO_GEMM;
+            p->d.m = 1;
+            p->d.alpha = k;
+            p->d.points_id = 0;
+            p->d.gemm_lhs = MNN_GEMM_LHS_ROWS;
+            p->d.error_ppm = rows_ppm;
+            layout_workspace(p);
+        }
+    }
     return p;
 }
 
@@ -465,7 +515,7 @@ int mnn_conv_plan_query(mnn_conv_plan_t p, mnn_conv_info* info)
     info->chosen_candidate = p->d.chosen;
     info->gemm_lhs = p->d.algo == MNN_ALGO_GEMM ? p->d.gemm_lhs : 0;
     for (int i = 0; i < MNN_N_CANDIDATES; ++i) info->cost_ps[i] = p->d.cost_ps[i];
-    info->fused = p->fused ? 1 : 0;
+    info->fused = p->d.algo == MNN_ALGO_WINOGRAD ? p->d.fused : 0;
     info->strassen = p->strassen ? 1 : 0;
     info->rect = p->rect;
     if (p->strassen) info->predicted_error_ppm = 3 * p->d.error_ppm;
@@ -493,6 +543,7 @@ static cudaError_t setup_tensor_kernels(mnn_conv_plan_t p, const char** why)
 {
     const int alpha2 = p->d.algo == MNN_ALGO_WINOGRAD ? p->d.alpha * p->d.alpha : 1;
     if (p->packed) return line_setup(&p->lc, v_hi(p), u_hi(p), why);
+    if (p->rows) return rows_setup(&p->rc);
     if (p->fused) return fused_wino_setup(&p->fw, p->s.Cout, p->s.Cin, u_hi(p), why);
     if (p->rect)
         return umma_contract_setup(&p->uc, p->store_mode, p->d.alpha, p->s.Cout, p->cin_pad, p->chunk_tiles, u_hi(p), u_lo(p),
@@ -565,7 +616,7 @@ static int set_workspace_split(mnn_conv_plan_t p, void* persistent, long long pe
     p->ws = static_cast<char*>(workspace);
     p->tws = static_cast<char*>(transient);
     p->ws_bytes = bytes;
-    cudaError_t e = cudaMemset(p->ws, 0, kStatusBytes);
+    cudaError_t e = p->status ? cudaMemset(p->status, 0, sizeof(int)) : cudaMemset(p->ws, 0, kStatusBytes);
     if (e != cudaSuccess) return fail_cuda(e, "clearing the status word");
     if (p->d.operand != MNN_OPERAND_FP32_REF) {
         const char* why = "";
@@ -584,11 +635,11 @@ static int check_run_args(mnn_conv_plan_t p, const float* x, const float* w, con
     if ((mask & ~(unsigned)MNN_STAGE_ALL) || mask == 0) return fail(MNN_EINVAL, "bad stage mask");
     if (p->workspace_bytes > 0 && !p->ws) return fail(MNN_EWORKSPACE, "call mnn_conv_set_workspace first");
     const bool direct = p->d.algo == MNN_ALGO_DIRECT;
-    const bool one_kernel = p->gemm_x || p->gemm_implicit || p->fused;       // x in, y out in the contraction stage
+    const bool one_kernel = p->gemm_x || p->gemm_implicit || p->fused || p->rows;       // x in, y out in the contraction stage
     const bool need_x = direct || (!one_kernel && (mask & MNN_STAGE_INPUT)) || (one_kernel && (mask & MNN_STAGE_CONTRACT));
     const bool need_w = direct || (mask & MNN_STAGE_WEIGHT);
-    const bool need_y = direct || (!p->fused && (mask & MNN_STAGE_OUTPUT)) ||
-                        (((p->d.algo == MNN_ALGO_GEMM && !p->strassen) || p->fused) && (mask & MNN_STAGE_CONTRACT));
+    const bool need_y = direct || (!p->fused && !p->rows && (mask & MNN_STAGE_OUTPUT)) ||
+                        (((p->d.algo == MNN_ALGO_GEMM && !p->strassen) || p->fused || p->rows) && (mask & MNN_STAGE_CONTRACT));
     if ((need_x && !x) || (need_w && !w) || (need_y && !y)) return fail(MNN_EINVAL, "NULL tensor pointer");
     if ((x && !aligned16(x)) || (w && !aligned16(w)) || (y && !aligned16(y)))
         return fail(MNN_EALIGN, "x, w and y must be 16-byte aligned");
@@ -629,7 +680,9 @@ static int do_weights(mnn_conv_plan_t p, const float* w, cudaStream_t st)
 {
     cudaError_t e;
     LaunchTimer lt(p, st, 0);
-    if (p->packed)
+    if (p->rows)
+        e = launch_rows_weights(p->rc, w, u_hi(p), st);
+    else if (p->packed)
         e = launch_line_weights(p->lc.p, w, u_hi(p), st);
     else if (p->gemm_implicit)
         e = launch_implicit_weights(w, u_hi(p), p->s.Cout, p->s.Cin, p->s.k, p->cin_pad, st);
@@ -689,6 +742,14 @@ int mnn_conv_run_stages(mnn_conv_plan_t p, const float* x, const float* w, const
     }
     const bool reference = d.operand == MNN_OPERAND_FP32_REF;
 
+    if (p->rows) {
+        // one kernel, booked as the contraction stage
+        if (!(mask & MNN_STAGE_CONTRACT)) return MNN_OK;
+        LaunchTimer lt(p, st, 2);
+        e = launch_rows_conv(p->rc, x, u_hi(p), bias, y, s.relu, status_word(p), st);
+        if (e != cudaSuccess) return fail_cuda(e, "convolution by rows");
+        return MNN_OK;
+    }
     if (p->rect) {
         const RectGeom g = rect_geom(p);
         if (reference) return fail(MNN_EUNSUPPORTED, "rectangular kernels run on the tensor-core contraction only");
@@ -984,7 +1045,8 @@ mnn_net_t mnn_net_plan(int N, int H, int W, int n_layers, const mnn_layer_desc* 
     }
     net->N = N; net->H = H; net->W = W;
     int c = layers[0].Cin, h = H, w = W;
-    long long off = 0;
+    long long off = kStatusBytes;                  // the status words of all layers
+    static_assert(MNN_NET_MAX_LAYERS * sizeof(int) <= kStatusBytes, "a word per layer");
     for (int i = 0; i < n_layers; ++i) {
         const mnn_layer_desc& L = layers[i];
         if (L.Cin != c) {
@@ -1004,9 +1066,9 @@ mnn_net_t mnn_net_plan(int N, int H, int W, int n_layers, const mnn_layer_desc* 
             return nullptr;
         }
         net->plans.push_back(p);
-        // virtual walk: the persistent part (status word + U) gets its own place, the transient part
+        // virtual walk: the persistent part (U) gets its own place, the transient part
         // (V + M) only counts towards the maximum, the output towards the activation buffers
-        const long long persistent = p->workspace_bytes > 0 ? align_up(p->v_offset, 1024) : 0;
+        const long long persistent = p->workspace_bytes > 0 ? align_up(p->v_offset - kStatusBytes, 1024) : 0;
         const long long transient = p->workspace_bytes > 0 ? p->workspace_bytes - p->v_offset : 0;
         net->persistent_offset.push_back(off);
         off += persistent;
@@ -1018,7 +1080,7 @@ mnn_net_t mnn_net_plan(int N, int H, int W, int n_layers, const mnn_layer_desc* 
         }
         c = L.Cout; h = p->s.OH; w = p->s.OW;
     }
-    net->persistent_bytes = off;
+    net->persistent_bytes = net->sum_of_layer_workspaces > 0 ? off : 0;
     net->transient_bytes = align_up(net->transient_bytes, 1024);
     net->activation_bytes = align_up(net->activation_bytes, 1024);
     net->transient_offset = net->persistent_bytes;
@@ -1061,7 +1123,9 @@ int mnn_net_set_workspace(mnn_net_t net, void* workspace, long long bytes)
     for (size_t i = 0; i < net->plans.size(); ++i) {
         mnn_conv_plan_t p = net->plans[i];
         if (p->workspace_bytes == 0) continue;
-        int rc = set_workspace_split(p, base + net->persistent_offset[i], align_up(p->v_offset, 1024),
+        // (the plan's own layout begins with a status word, which lies at the head of the network's workspace instead)
+        p->status = reinterpret_cast<int*>(base) + i;
+        int rc = set_workspace_split(p, base + net->persistent_offset[i] - kStatusBytes, align_up(p->v_offset, 1024),
                                      base + net->transient_offset, net->transient_bytes);
         if (rc != MNN_OK) return rc;
     }

@@ -12,6 +12,7 @@
 
 #include "kernels.h"
 #include "line_plan.h"
+#include "rows_plan.h"
 
 #include <algorithm>
 #include <cmath>
@@ -618,6 +619,7 @@ void winograd_chunking(const LayerShape& s, int m, int operand, int passes, cons
 int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, bool packed_lines, Decision* d, const char** err)
 {
     static const int kM[3] = {2, 4, 6};
+    d->rows = false;
     for (int i = 0; i < MNN_N_CANDIDATES; ++i) d->cost_ps[i] = MNN_COST_INADMISSIBLE;
 
     const uint64_t tol_ppm = o.precision == MNN_PREC_BF16 ? 10000 : 1000;
@@ -750,6 +752,43 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
         }
     }
 
+    // The convolution by rows, one kernel, where the planner is free and it is estimated faster than a tensor-core scheme that is not
+    // expected to be more accurate; a tenth is held against it, nothing on rows that are no multiple of 16 bytes (Winograd
+    // there measured 1.0 to 1.4 times its estimate, k <= 5), half against F(6, 7) (measured at 0.65 to 0.9 of its estimate); packed lines, of
+    // all layers with cold inputs, take a tenth more than theirs (256 channels 56 x 56 batch 64 BF16: 249 us, by rows 218): rows of Winograd F(2, 3) in hi + lo BF16 (booked as candidate 12), or the definition (as
+    // candidate 2), with hi + lo operands in the TF32 class.  One image, 3x3: 64 channels 56 x 56 13.1 -> 8.5 us, 128 channels
+    // 28 x 28 12.2 -> 8.6, 256 channels 14 x 14 11.3 -> 9.1.
+    const unsigned held = s.W % 4 != 0 && s.k <= 5 ? 10 : s.k == 7 && best >= 3 && cands[best].m == 6 ? 15 : 11;
+    const long long ppm_before = best >= 0 ? ppm_of[best] : 0;      // what the forms below may not exceed
+    const bool free_choice = o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 && o.points_id == 0 &&
+                             o.chunk_images == 0 && o.gemm_lhs == MNN_GEMM_LHS_AUTO && o.fused == 0;
+    if (free_choice && wino_shape_ok && best > 0) {
+        const int sms = cal.c[7] > 0 ? (int)cal.c[7] : 148;
+        for (int m = 1; m <= 2; ++m) {
+            const int passes = o.precision == MNN_PREC_BF16 ? 1 : 3, slot = m == 1 ? 2 : 12;
+            const RowsShape rs = {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.k, s.pad, s.pad, s.OH, s.OW, m, passes};
+            RowsPlan rp;
+            if ((m == 2 && passes == 1) || !rows_plan(rs, sms, &rp)) continue;
+            long long ppm = 0;
+            const int pid = m == 1 ? 0 : best_points(m, s.k, MNN_OPERAND_BF16, passes, &ppm);
+            if (m == 1) ppm = accuracy_ppm(1, s.k, 0, MNN_OPERAND_BF16, passes);
+            uint64_t now = d->cost_ps[best];
+            const bool lines = !d->rows && lhs_of[best] == MNN_GEMM_LHS_PACKED;
+            if (lines && s.Cout < 256) continue;      // (64 channels 56 x 56 batch 64: 50 us in lines, 51 by rows)
+            if (lines) now = std::min(now, packed_cost(s, cands[best].operand, cal));
+            const uint64_t cost = (uint64_t)rp.time_ps + (uint64_t)cal.c[5];
+            if (ppm < 0 || ppm > ppm_before || (u128)cost * (d->rows ? 10u : lines ? 9u : held) >= (u128)now * 10u) continue;
+            best = slot;
+            d->rows = true;
+            d->cost_ps[slot] = cost;
+            ppm_of[slot] = ppm;
+            pts_of[slot] = pid;
+            lhs_of[slot] = m == 1 ? MNN_GEMM_LHS_ROWS : 0;
+            chunk_of[slot] = s.N;
+            nch_of[slot] = 1;
+        }
+    }
+
     // A forced combination outside the candidate list (other m, fp32 checking contraction).
     const bool off_list = o.force_algo == MNN_ALGO_WINOGRAD && o.force_m != 0 &&
                           (o.operand == MNN_OPERAND_FP32_REF || !(o.force_m == 2 || o.force_m == 4 || o.force_m == 6));
@@ -804,7 +843,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     d->chosen = best;
     d->algo = c.algo;
     d->operand = c.operand;
-    d->passes = c.passes;
+    d->passes = d->rows && o.precision == MNN_PREC_TF32 ? 3 : c.passes;
     d->error_ppm = ppm_of[best];
     if (c.algo == MNN_ALGO_WINOGRAD) {
         d->m = c.m;
@@ -812,7 +851,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
         d->points_id = pts_of[best];
         d->chunk_images = chunk_of[best];
         d->n_chunks = nch_of[best];
-        d->fused = best == 15 ? 1 : 0;
+        d->fused = best == 15 ? MNN_FUSED_TILES : d->rows ? MNN_FUSED_ROWS : 0;
         if (o.chunk_images > 0 && !d->fused) {
             d->chunk_images = o.chunk_images < s.N ? o.chunk_images : s.N;
             d->n_chunks = (s.N + d->chunk_images - 1) / d->chunk_images;

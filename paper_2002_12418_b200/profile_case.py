@@ -30,7 +30,10 @@ def stage_work(info, N, Cin, Cout, H, W, k, groups):
     y_bytes = 4 * N * Cout * info.OH * info.OW
     b_el = (2 if info.operand == B.OPERAND_BF16 else 4) * (2 if info.passes == 3 else 1)
     out = {}
-    if info.algo == B.ALGO_WINOGRAD and info.fused:
+    if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
+        T = N * info.OH * (-(-info.OW // info.m))          # one-dimensional tiles; the kernel's rows shift
+        out["contract"] = (x_bytes + y_bytes + info.u_bytes, 2 * k * info.alpha * Cout * Cin * T * info.passes)
+    elif info.algo == B.ALGO_WINOGRAD and info.fused:
         T = N * (-(-info.OH // 2)) * (-(-info.OW // 2))
         out["contract"] = (x_bytes + y_bytes + 4 * 16 * Cout * Cin, 2 * 16 * Cout * Cin * T)
     elif info.algo == B.ALGO_WINOGRAD:
@@ -49,7 +52,7 @@ def stage_work(info, N, Cin, Cout, H, W, k, groups):
     elif info.algo == B.ALGO_GEMM:
         K, T = Cin * k * k, N * info.OH * info.OW
         v = b_el * T * K
-        if info.gemm_lhs in (B.GEMM_LHS_X, B.GEMM_LHS_IMPLICIT):
+        if info.gemm_lhs in (B.GEMM_LHS_X, B.GEMM_LHS_IMPLICIT, B.GEMM_LHS_ROWS):
             v = x_bytes                    # the contraction reads x itself
         else:
             if info.gemm_lhs == B.GEMM_LHS_PACKED:

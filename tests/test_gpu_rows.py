@@ -1,0 +1,117 @@
+"""The convolution by rows in one kernel (rows_conv.cu) on the GPU, as the planner chooses it, against the fp64 oracle: last tiles
+and channel blocks that are not full, padded channels, odd rows, paddings other than the one that keeps the size, every kernel size,
+clusters, both accuracy classes; integer inputs bit for bit; repeated runs; NaN."""
+import numpy as np
+import pytest
+
+from oracle import direct_conv as oc
+from paper_2002_12418_b200 import binding as B
+from paper_2002_12418_b200 import workloads as W
+from tests.util import rel_l2, to_dev
+
+pytestmark = pytest.mark.gpu
+
+# hi + lo BF16 operands leave 2^-17 of each factor and drop lo * lo: 3 * 2^-17 of a product at most, half of that as a 2-norm over
+# many; F(2, 3) enlarges it by the norms of its matrices; one BF16 product 2 * 2^-9.
+BOUND = {"rows1": 2.3e-5, "rows2": 3e-5, "bf16": 4e-3}
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch
+    assert torch.cuda.is_available()
+    B.lib()
+    return torch
+
+
+def form(info):
+    if info.algo == B.ALGO_GEMM and info.gemm_lhs == B.GEMM_LHS_ROWS:
+        return "rows1" if info.passes == 3 else "bf16"
+    return "rows2" if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS else None
+
+
+def run(torch, shape, x, w, b, relu, cls=B.PREC_TF32, repeats=1):
+    N, Cin, Cout, H, W_, k, pad = shape
+    r = B.ConvLayerRunner(N, Cin, Cout, H, W_, k, 1, pad, 1, B.make_opts(relu=relu, precision=cls))
+    info = r.info
+    xd, wd, bd = to_dev(torch, x), to_dev(torch, w), to_dev(torch, b) if b is not None else None
+    ys = []
+    for _ in range(repeats):
+        y = torch.full((N, Cout, info.OH, info.OW), float("nan"), device="cuda:0")
+        r.run(xd, wd, bd, y)
+        ys.append(y)
+    torch.cuda.synchronize()
+    assert r.device_status() == 0
+    r.close()
+    assert all(torch.equal(ys[0], y) for y in ys[1:])
+    return ys[0].cpu().numpy(), info
+
+
+# (N, Cin, Cout, H, W, k, pad), one per kernel size, way of issuing the three products, tiles per item and CTAs per item
+SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "rows1"), ((1, 200, 130, 8, 6, 2, 1), "rows1"), ((1, 256, 8, 26, 29, 2, 1), "rows1"),
+          ((17, 16, 17, 33, 39, 2, 1), "rows1"), 
+          ((1, 64, 100, 11, 10, 3, 1), "rows1"), ((9, 130, 1, 22, 30, 3, 2), "rows1"), ((1, 130, 64, 5, 17, 3, 1), "rows1"), ((2, 256, 33, 8, 9, 3, 0), "rows1"),
+          ((17, 64, 1, 25, 40, 3, 2), "rows1"), ((5, 16, 100, 6, 29, 3, 1), "rows1"), ((1, 256, 130, 11, 5, 3, 0), "rows1"),
+          ((17, 16, 8, 30, 38, 3, 1), "rows1"), ((7, 100, 72, 35, 45, 3, 1), "rows1"),
+          ((1, 16, 200, 8, 10, 5, 2), "rows1"), ((9, 64, 1, 38, 18, 5, 2), "rows1"), ((5, 130, 1, 12, 33, 5, 4), "rows1"), ((17, 24, 1, 36, 29, 5, 2), "rows1"),
+          ((17, 16, 33, 36, 20, 5, 0), "rows1"), ((1, 16, 33, 31, 8, 7, 3), "rows1"), ((5, 64, 1, 34, 20, 7, 3), "rows1"), ((2, 256, 1, 5, 34, 7, 6), "rows1"),
+          ((17, 17, 1, 25, 37, 7, 6), "rows1"),
+          ((2, 100, 33, 34, 6, 2, 1), "bf16"), ((1, 33, 100, 23, 9, 3, 1), "bf16"), ((1, 130, 33, 15, 11, 3, 1), "bf16"), ((3, 256, 8, 19, 9, 3, 0), "bf16"),
+          ((9, 130, 1, 28, 29, 3, 1), "bf16"), ((2, 17, 100, 27, 7, 5, 0), "bf16"), ((1, 256, 1, 39, 35, 5, 4), "bf16"), ((17, 130, 1, 34, 36, 5, 4), "bf16"),
+          ((1, 24, 72, 6, 13, 7, 3), "bf16"), ((1, 256, 64, 15, 12, 7, 0), "bf16"),
+          ((32, 64, 64, 56, 56, 3, 1), "rows2"), ((17, 17, 17, 29, 37, 3, 1), "rows2"), ((17, 130, 1, 39, 30, 3, 0), "rows2"), ((17, 256, 1, 9, 33, 3, 1), "rows2"),
+          ((1, 256, 8, 37, 30, 3, 0), "rows2")]
+
+
+@pytest.mark.parametrize("shape,expected", SHAPES)
+def test_against_the_oracle(torch, shape, expected):
+    N, Cin, Cout, H, W_, k, pad = shape
+    layer = W.ConvLayer("rows", N, Cin, Cout, H, W_, k, 1, pad, relu=True, seed=sum(shape))
+    x, w, b = W.make_inputs(layer)
+    cls = B.PREC_BF16 if expected == "bf16" else B.PREC_TF32
+    got, info = run(torch, shape, x, w, b, True, cls, repeats=3)
+    assert form(info) == expected
+    assert rel_l2(got, oc.direct_conv(x, w, b, 1, pad, 1, 1, True)) <= BOUND[expected]
+
+
+# 1 x k and k x 1 kernels left to the plan take the same kernel: every kernel size, one tile and two per item, clusters, odd paddings.
+@pytest.mark.parametrize("N,Cin,Cout,H,W_,kh,kw,ph,pw", [
+    (9, 82, 82, 25, 17, 1, 3, 0, 1), (32, 192, 192, 17, 17, 1, 7, 0, 3), (32, 192, 192, 17, 17, 7, 1, 3, 0), (1, 33, 33, 31, 34, 1, 7, 2, 5),
+    (6, 36, 211, 31, 24, 5, 1, 2, 3), (4, 50, 203, 20, 18, 3, 1, 0, 1), (35, 112, 58, 14, 27, 1, 5, 0, 2), (3, 40, 17, 12, 33, 1, 2, 0, 1), (3, 40, 17, 33, 12, 2, 1, 1, 0)])
+def test_line_kernels(torch, N, Cin, Cout, H, W_, kh, kw, ph, pw):
+    rng = np.random.Generator(np.random.PCG64(N + Cin + kh))
+    x = np.maximum(rng.standard_normal((N, Cin, H, W_), dtype=np.float32), 0)
+    w = (rng.standard_normal((Cout, Cin, kh, kw)) * np.sqrt(2.0 / (Cin * kh * kw))).astype(np.float32)
+    b = (rng.standard_normal((Cout,)) * 0.1).astype(np.float32)
+    r = B.ConvLayerRunner(N, Cin, Cout, H, W_, max(kh, kw), plan=B.mnn_conv_plan_rect(N, Cin, Cout, H, W_, kh, kw, ph, pw, B.make_opts(relu=1)))
+    assert form(r.info) == "rows1"
+    y = r.run(to_dev(torch, x), to_dev(torch, w), to_dev(torch, b))
+    torch.cuda.synchronize()
+    assert r.device_status() == 0
+    r.close()
+    assert rel_l2(y.cpu().numpy(), oc.direct_conv_rect(x, w, b, ph, pw, True)) <= BOUND["rows1"]
+
+
+# Small integers are exact in BF16 and in fp32 sums: the definition bit for bit.
+@pytest.mark.parametrize("shape", [(5, 16, 100, 6, 29, 3, 1), (2, 256, 33, 8, 9, 3, 0), (17, 24, 1, 36, 29, 5, 2)])
+def test_integers_bit_for_bit(torch, shape):
+    N, Cin, Cout, H, W_, k, pad = shape
+    rng = np.random.Generator(np.random.PCG64(7))
+    x, w, b = (rng.integers(-3, 4, size=s).astype(np.float32) for s in ((N, Cin, H, W_), (Cout, Cin, k, k), (Cout,)))
+    got, info = run(torch, shape, x, w, b, False)
+    assert form(info) == "rows1"
+    assert np.array_equal(got.astype(np.float64), oc.direct_conv(x, w, b, 1, pad, 1, 1, False))
+
+
+# What is no number stays where its windows reach, without ReLU too.
+def test_not_a_number_reaches_its_windows_only(torch):
+    shape = (1, 64, 100, 11, 10, 3, 1)
+    N, Cin, Cout, H, W_, k, pad = shape
+    x, w, _ = W.make_inputs(W.ConvLayer("nan", N, Cin, Cout, H, W_, k, 1, pad, seed=5))
+    clean, _ = run(torch, shape, x, w, None, False)
+    x[0, 7, 4, 5] = np.nan
+    got, info = run(torch, shape, x, w, None, False)
+    assert form(info) == "rows1"
+    near = np.zeros((H, W_), dtype=bool)
+    near[3:6, 4:7] = True
+    assert np.isnan(got[..., near]).all() and np.array_equal(got[..., ~near], clean[..., ~near])

@@ -334,6 +334,17 @@ def mnn_net_destroy(net) -> None:
     lib().mnn_net_destroy(net)
 
 
+def _raw_stream(device):
+    """A callable that returns the handle of torch's current stream on `device`: torch's own lookup of the handle where the device
+    is named by its index, without the Stream object that torch.cuda.current_stream builds."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or device.index is None:
+        return lambda: torch.cuda.current_stream(device).cuda_stream
+    index = device.index
+    return lambda: raw(index)
+
+
 class NetRunner:
     """A network plan plus its torch-owned workspace; ``run`` is one mnn_net_run on torch's current stream."""
 
@@ -341,6 +352,7 @@ class NetRunner:
         import torch
         self.torch = torch
         self.device = torch.device(device)
+        self.stream = _raw_stream(self.device)
         self.net = mnn_net_plan(N, H, W, layers, precision)
         self.info = mnn_net_query(self.net)
         with torch.cuda.device(self.device):
@@ -348,9 +360,6 @@ class NetRunner:
         self._ws_ptr = (self.workspace.data_ptr() + 1023) // 1024 * 1024
         mnn_net_set_workspace(self.net, self._ws_ptr, self.info.workspace_bytes)
         self._keep = None
-
-    def stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
 
     def prepare(self, ws) -> None:
         mnn_net_prepare(self.net, [w.data_ptr() for w in ws], self.stream())
@@ -391,6 +400,7 @@ class ConvLayerRunner:
         import torch
         self.torch = torch
         self.device = torch.device(device)
+        self.stream = _raw_stream(self.device)
         self.shape = (N, Cin, Cout, H, W, k, stride, pad, dilation)
         if plan is not None:
             self.plan = plan               # e.g. from mnn_conv_plan_rect; owned by the runner from here on
@@ -406,20 +416,17 @@ class ConvLayerRunner:
                 self._ws_ptr = (base + 1023) // 1024 * 1024
                 mnn_conv_set_workspace(self.plan, self._ws_ptr, self.info.workspace_bytes)
 
-    def stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
-
     def prepare(self, w) -> None:
         mnn_conv_prepare_weights(self.plan, w.data_ptr(), self.stream())
 
     def run(self, x, w, bias=None, y=None, stage_mask=None):
-        torch = self.torch
-        N, Cin, Cout = self.shape[0], self.shape[1], self.shape[2]
         if y is None:
-            y = torch.empty((N, Cout, self.info.OH, self.info.OW), dtype=torch.float32, device=self.device)
+            y = self.torch.empty((self.shape[0], self.shape[2], self.info.OH, self.info.OW), dtype=self.torch.float32, device=self.device)
         bp = bias.data_ptr() if bias is not None else None
         if stage_mask is None:
-            mnn_conv_run(self.plan, x.data_ptr(), w.data_ptr(), bp, y.data_ptr(), self.stream())
+            rc = _lib.mnn_conv_run(self.plan, x.data_ptr(), w.data_ptr(), bp, y.data_ptr(), self.stream())
+            if rc != MNN_OK:
+                _check(rc)
         else:
             mnn_conv_run_stages(self.plan, x.data_ptr() if x is not None else None,
                                 w.data_ptr() if w is not None else None, bp, y.data_ptr(), self.stream(), stage_mask)

@@ -237,7 +237,13 @@ def stage_work(layer, info):
     y_bytes = 4 * N * Cout * info.OH * info.OW
     b_el = (2 if info.operand == B.OPERAND_BF16 else 4) * (2 if info.passes == 3 else 1)
     out = {}
-    if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
+    if info.algo == B.ALGO_WINOGRAD and info.fused == B.ROW_WISE:
+        # one-dimensional tiles along the rows (the padded rows between images among them); the product sums over kernel rows too
+        out["input"] = {"bytes": x_bytes + info.v_bytes, "flops": 0}
+        out["contraction"] = {"bytes": info.v_bytes + info.m_bytes + info.u_bytes,
+                              "flops": 2 * layer.k * info.alpha * Cout * Cin * info.chunk_tiles * info.passes}
+        out["output"] = {"bytes": info.m_bytes + y_bytes, "flops": 0}
+    elif info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
         T = N * info.OH * (-(-info.OW // info.m))
         out["contraction"] = {"bytes": x_bytes + y_bytes + info.u_bytes, "flops": 2 * layer.k * info.alpha * Cout * Cin * T * info.passes}
     elif info.algo == B.ALGO_GEMM and info.gemm_lhs == B.GEMM_LHS_ROWS:

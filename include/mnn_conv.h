@@ -55,8 +55,8 @@ enum { MNN_POINTS_AUTO = 0, MNN_POINTS_PAPER = 1, MNN_POINTS_UNIT = 2, MNN_POINT
 enum { MNN_GEMM_LHS_AUTO = 0, MNN_GEMM_LHS_PATCHES = 1, MNN_GEMM_LHS_X = 2, MNN_GEMM_LHS_IMPLICIT = 3,
        MNN_GEMM_LHS_PACKED = 4, MNN_GEMM_LHS_ROWS = 5 };
 /* info.fused: the form of a Winograd plan other than the two-dimensional one (the option of the same name has values of its own):
- * one kernel on 2 x 2 tiles or one kernel by rows */
-enum { MNN_FUSED_TILES = 1, MNN_FUSED_ROWS = 2 };
+ * one kernel on 2 x 2 tiles, one kernel by rows, or three kernels that transform along the rows only */
+enum { MNN_FUSED_TILES = 1, MNN_FUSED_ROWS = 2, MNN_ROW_WISE = 3 };
 enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_STAGE_OUTPUT = 8,
        MNN_STAGE_ALL = 15 };
 
@@ -142,8 +142,8 @@ typedef struct {
  * 6..8 tf32x3; 9..11 bf16x1; 12..14 bf16x3; 15 Winograd F(2x2,3x3) tf32x1 as one fused kernel.
  * The costs rank the schemes.  A GEMM candidate is booked at the cheapest of PATCHES, X and IMPLICIT without a cut of
  * the K loop, also where the planner then runs it as PACKED or cuts the loop over clusters, which it decides by
- * closer estimates that are not reported; GEMM bf16 that takes over as PACKED is booked at its own cost, and so is a form by rows
- * that takes over: the definition as candidate 2 (with passes = 3 in the TF32 class), Winograd as 12.
+ * closer estimates that are not reported; GEMM bf16 that takes over as PACKED is booked at its own cost, and so is a form by rows or row-wise
+ * that takes over: the definition as candidate 2 (with passes = 3 in the TF32 class), Winograd as 12 or 13.
  * Candidates that are not applicable or fail the accuracy gate hold MNN_COST_INADMISSIBLE; every
  * other figure saturates at MNN_COST_INADMISSIBLE - 1.
  * paper_mul[] is the paper's own multiplication count (Eq. 2) for output tile sizes n = 1, 2, 4, 6,
@@ -169,7 +169,8 @@ typedef struct {
     int chosen_candidate;            /* index into cost_ps, -1 when the choice was forced outside the list */
     int gemm_lhs;                    /* GEMM scheme: MNN_GEMM_LHS_PATCHES, _X, _IMPLICIT, _PACKED or _ROWS as planned, else 0 */
     unsigned long long cost_ps[MNN_N_CANDIDATES];
-    int fused;                       /* MNN_FUSED_TILES, MNN_FUSED_ROWS: Winograd in one kernel (no V, no M); else 0 */
+    int fused;                       /* MNN_FUSED_TILES, MNN_FUSED_ROWS: Winograd in one kernel (no V, no M); MNN_ROW_WISE: alpha instead of
+                                        alpha^2 positions, tiles along padded rows; else 0 */
     int paper_n_hat;
     unsigned long long paper_mul[4];
     int strassen;                    /* 1 when the plan runs one Strassen level (alpha = 1, seven products) */

@@ -360,6 +360,44 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
     return best
 
 
+# Row-wise Winograd, hi + lo BF16: F(4, 3), F(4, 5), F(2, 7); parts per million as measured, rounded up.
+ROW_WISE_PPM = {3: 20, 5: 30, 7: 30}
+
+
+def row_wise_tiling(L: Layer, m: int, sms: int):
+    """Three kernels that transform along the rows only: bytes of V and M and the cheapest tiling of the product, or None."""
+    k, alpha, reach = L.k, m + L.k - 1, L.k - 1
+    hq = max(L.OH, min(L.OH + reach, max(L.H + L.pad, L.OH + reach - L.pad)))
+    tiles_w = cdiv(L.OW, m)
+    T, cin_pad = L.N * hq * tiles_w, cdiv(L.Cin, 8) * 8
+    v, mm = 4 * alpha * T * cin_pad, 4 * alpha * L.Cout * (cdiv(T, 32) * 32)
+    if T >= (1 << 31) - 65536 or v + mm > 4 << 30:
+        return None
+    co16, room, best = cdiv(L.Cout, 16) * 16, 207 * 1024, None
+    for mt in (1, 2):
+        for nb in range(cdiv(co16, 256), min(64, co16 // 16) + 1):
+            bn = cdiv(cdiv(co16, nb), 16) * 16
+            need = 128 * mt + reach * tiles_w
+            boxes = cdiv(need, 256)
+            rows = boxes * (cdiv(cdiv(need, boxes), 8) * 8)
+            a_slot, b_slot = 2 * rows * 64, 2 * bn * 64
+            items = cdiv(T, 128 * mt) * nb * alpha
+            if 2 * mt * bn > 512 or 2 * a_slot + 3 * b_slot > room or items >= 1 << 31:
+                continue
+            mma = 6 * mt * k * max(bn // 2, 57 + bn // 7) * 555
+            load = (a_slot + k * b_slot) * 63 // 5
+            drain = mt * bn * 512 * 28 + 1087000
+            cost = cdiv(items, sms) * max(cdiv(cin_pad, 32) * max(mma, load) + 285000, drain) + drain
+            if best is None or cost < best["product_ps"]:
+                best = dict(product_ps=cost, v=v, m=mm, bn=bn, mt=mt)
+    return best
+
+
+def row_wise_cost(L: Layer, t, c) -> int:
+    x, y = 4 * L.N * L.Cin * L.H * L.W, 4 * L.N * L.Cout * L.OH * L.OW
+    return sat(kernel_ps(c, mem_as=(x + t["v"]) * c[0] * 3 // 2) + kernel_ps(c, mem_as=(t["m"] + y) * c[0] * 3 // 2) + t["product_ps"] + c[5])
+
+
 def gemm_cost(L: Layer, operand: int, lhs, c) -> int:
     """lhs: LHS_PATCHES (gather kernel + GEMM), LHS_X / True (the GEMM reads x itself), LHS_IMPLICIT (the patches are
     gathered by producer warps inside the GEMM kernel)."""
@@ -660,7 +698,7 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
     # The convolution by rows takes over where nothing is forced, it is estimated faster than a tensor-core scheme (by what is held
     # against it: the estimates' measured errors) and not expected to be less accurate: as candidate 2 (the definition) or 12 (Winograd m = 2).
     held = 10 if L.W % 4 and L.k <= 5 else 15 if L.k == 7 and best >= 3 and _candidates()[best][1] == 6 else 11
-    rows, ppm_before = False, side.get(best, {}).get("ppm", 0)
+    rows, row_wise, ppm_before = False, False, side.get(best, {}).get("ppm", 0)
     free = o.force_algo == o.force_m == o.operand == o.passes == o.points_id == o.gemm_lhs == o.fused == 0
     if free and wino_shape and best > 0:
         for m in (1, 2):
@@ -680,6 +718,13 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 continue
             best, rows, ch.cost_ps[slot] = slot, True, cost
             side[slot] = dict(lhs=LHS_ROWS, ppm=p, pid=pid, chunk=L.N, n_chunks=1)
+        if o.precision == PREC_TF32 and L.k in ROW_WISE_PPM and ROW_WISE_PPM[L.k] <= ppm_before:
+            m = 2 if L.k == 7 else 4
+            t = row_wise_tiling(L, m, c[7] if c[7] > 0 else 148)
+            if t is not None and row_wise_cost(L, t, c) * (10 if rows else held) < ch.cost_ps[best] * 10:
+                best, rows, row_wise = (12 if m == 2 else 13), False, True
+                ch.cost_ps[best] = row_wise_cost(L, t, c)
+                side[best] = dict(ppm=ROW_WISE_PPM[L.k], pid=best_points(ppm, m, L.k, OPERAND_BF16, 3)[0], chunk=L.N, n_chunks=1)
     if best < 0:
         return ch
     algo, m, operand, passes = _candidates()[best]
@@ -688,7 +733,7 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
     if algo == ALGO_WINOGRAD:
         ch.m, ch.points_id = m, side[best]["pid"]
         ch.chunk_images, ch.n_chunks = side[best]["chunk"], side[best]["n_chunks"]
-        ch.fused = 1 if best == FUSED_SLOT else 2 if rows else 0
+        ch.fused = 1 if best == FUSED_SLOT else 2 if rows else 3 if row_wise else 0
     else:
         ch.m, ch.points_id, ch.chunk_images, ch.n_chunks = 1, 0, L.N, 1
         ch.gemm_lhs = side[best]["lhs"] if algo == ALGO_GEMM else 0

@@ -19,7 +19,7 @@ OPERAND_AUTO, OPERAND_TF32, OPERAND_BF16, OPERAND_FP32_REF = 0, 1, 2, 3
 POINTS_AUTO, POINTS_PAPER, POINTS_UNIT, POINTS_MIXED = 0, 1, 2, 3
 GEMM_LHS_AUTO, GEMM_LHS_PATCHES, GEMM_LHS_X, GEMM_LHS_IMPLICIT, GEMM_LHS_PACKED, GEMM_LHS_ROWS = 0, 1, 2, 3, 4, 5
 FUSED_AUTO, FUSED_NEVER, FUSED_ONLY = 0, 1, 2
-FUSED_TILES, FUSED_BY_ROWS = 1, 2          # values of info.fused
+FUSED_TILES, FUSED_BY_ROWS, ROW_WISE = 1, 2, 3          # values of info.fused
 STAGE_WEIGHT, STAGE_INPUT, STAGE_CONTRACT, STAGE_OUTPUT, STAGE_ALL = 1, 2, 4, 8, 15
 N_CANDIDATES, N_CONSTS = 16, 16
 COST_INADMISSIBLE = 0xFFFFFFFFFFFFFFFF

@@ -16,6 +16,7 @@
 #include "contract_umma.h"
 #include "kernels.h"
 #include "line_conv.h"
+#include "line_wino.h"
 #include "planner.h"
 #include "rows_conv.h"
 #include "strassen.h"
@@ -80,6 +81,8 @@ struct mnn_conv_plan_s {
     FusedWino fw;
     bool rows = false;               // the convolution by rows in one kernel: the workspace holds U only
     RowsConv rc;
+    bool row_wise = false;           // Winograd along the rows only, three kernels (line_wino.cu)
+    LineWino lw;
     // optional per-launch timing
     bool profiling = false;
     std::vector<cudaEvent_t> events;     // pairs (before, after)
@@ -133,6 +136,14 @@ void layout_workspace(mnn_conv_plan_t p)
         p->u_bytes = align_up((long long)d.alpha * s.Cout * p->cin_pad * eb, 2048);
         p->v_bytes = align_up((long long)d.alpha * p->chunk_tiles * p->cin_pad * eb, 2048);
         p->m_bytes = align_up((long long)d.alpha * s.Cout * p->m_row_stride * 4, 1024);
+        p->launches_per_run = 3;
+    } else if (p->row_wise) {
+        p->cin_pad = p->lw.p.cin_pad;
+        p->chunk_tiles = p->lw.p.T;
+        p->m_row_stride = (int)p->lw.p.m_row_stride;
+        p->u_bytes = align_up(p->lw.p.u_bytes, 2048);
+        p->v_bytes = align_up(p->lw.p.v_bytes, 2048);
+        p->m_bytes = align_up(p->lw.p.m_bytes, 1024);
         p->launches_per_run = 3;
     } else if (d.algo == MNN_ALGO_WINOGRAD) {
         const long long a2 = (long long)d.alpha * d.alpha;
@@ -192,7 +203,7 @@ LineShape line_shape(mnn_conv_plan_t p)
 // Form, transform matrices and workspace layout of the decision in p->d (square layers).
 int realise_decision(mnn_conv_plan_t p, const char** why)
 {
-    p->packed = p->fused = p->gemm_x = p->gemm_implicit = p->rows = false;
+    p->packed = p->fused = p->gemm_x = p->gemm_implicit = p->rows = p->row_wise = false;
     if (p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) {
         p->packed = line_plan(line_shape(p), p->tiling_sms, &p->lc.p);
         if (!p->packed) {
@@ -210,6 +221,14 @@ int realise_decision(mnn_conv_plan_t p, const char** why)
         std::memcpy(p->mats.At, wm.At32.data(), wm.At32.size() * sizeof(float));
         std::memcpy(p->mats.G, wm.G32.data(), wm.G32.size() * sizeof(float));
         std::memcpy(p->mats.Bt, wm.Bt32.data(), wm.Bt32.size() * sizeof(float));
+    }
+    if (p->d.fused == MNN_ROW_WISE) {
+        const LayerShape& s = p->s;
+        p->row_wise = line_wino_plan({s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.pad, s.OH, s.OW, p->d.m}, p->tiling_sms, &p->lw.p);
+        if (!p->row_wise) {
+            *why = "no tiling of the row-wise product fits this layer";
+            return MNN_EUNSUPPORTED;
+        }
     }
     if (p->d.rows) {
         const LayerShape& s = p->s;
@@ -544,6 +563,7 @@ static cudaError_t setup_tensor_kernels(mnn_conv_plan_t p, const char** why)
     const int alpha2 = p->d.algo == MNN_ALGO_WINOGRAD ? p->d.alpha * p->d.alpha : 1;
     if (p->packed) return line_setup(&p->lc, v_hi(p), u_hi(p), why);
     if (p->rows) return rows_setup(&p->rc);
+    if (p->row_wise) return line_wino_setup(&p->lw, v_hi(p), u_hi(p), why);
     if (p->fused) return fused_wino_setup(&p->fw, p->s.Cout, p->s.Cin, u_hi(p), why);
     if (p->rect)
         return umma_contract_setup(&p->uc, p->store_mode, p->d.alpha, p->s.Cout, p->cin_pad, p->chunk_tiles, u_hi(p), u_lo(p),
@@ -667,9 +687,10 @@ static RectGeom rect_geom(mnn_conv_plan_t p)
 {
     RectGeom g;
     g.N = p->s.N; g.Cin = p->s.Cin; g.Cout = p->s.Cout; g.H = p->s.H; g.W = p->s.W; g.OH = p->s.OH; g.OW = p->s.OW;
-    g.k = p->s.k; g.along_w = p->rect == 1 ? 1 : 0; g.pad_h = p->pad_h; g.pad_w = p->pad_w;
+    g.k = p->s.k; g.along_w = p->rect == 2 ? 0 : 1; g.pad_h = p->row_wise ? p->s.pad : p->pad_h; g.pad_w = p->row_wise ? p->s.pad : p->pad_w;
     g.m = p->d.m; g.alpha = p->d.alpha;
-    g.n_seg = p->rect == 1 ? (p->s.OW + g.m - 1) / g.m : (p->s.OH + g.m - 1) / g.m;
+    g.n_seg = g.along_w ? (p->s.OW + g.m - 1) / g.m : (p->s.OH + g.m - 1) / g.m;
+    g.lines = p->row_wise ? p->lw.p.Hq : p->s.OH;
     g.cin_pad = p->cin_pad;
     g.tiles = p->chunk_tiles;
     g.m_row_stride = p->m_row_stride;
@@ -682,6 +703,8 @@ static int do_weights(mnn_conv_plan_t p, const float* w, cudaStream_t st)
     LaunchTimer lt(p, st, 0);
     if (p->rows)
         e = launch_rows_weights(p->rc, w, u_hi(p), st);
+    else if (p->row_wise)
+        e = launch_line_wino_weights(p->lw.p, w, u_hi(p), p->mats.G, st);
     else if (p->packed)
         e = launch_line_weights(p->lc.p, w, u_hi(p), st);
     else if (p->gemm_implicit)
@@ -748,6 +771,25 @@ int mnn_conv_run_stages(mnn_conv_plan_t p, const float* x, const float* w, const
         LaunchTimer lt(p, st, 2);
         e = launch_rows_conv(p->rc, x, u_hi(p), bias, y, s.relu, status_word(p), st);
         if (e != cudaSuccess) return fail_cuda(e, "convolution by rows");
+        return MNN_OK;
+    }
+    if (p->row_wise) {
+        const RectGeom g = rect_geom(p);
+        if (mask & MNN_STAGE_INPUT) {
+            LaunchTimer lt(p, st, 1);
+            e = launch_rect_input(x, v_hi(p), static_cast<char*>(v_hi(p)) + p->lw.p.v_bytes / 2, g, p->store_mode, p->mats, st);
+            if (e != cudaSuccess) return fail_cuda(e, "row-wise input transform");
+        }
+        if (mask & MNN_STAGE_CONTRACT) {
+            LaunchTimer lt(p, st, 2);
+            e = launch_line_wino_product(p->lw, m_buf(p), status_word(p), st);
+            if (e != cudaSuccess) return fail_cuda(e, "row-wise product");
+        }
+        if (mask & MNN_STAGE_OUTPUT) {
+            LaunchTimer lt(p, st, 3);
+            e = launch_rect_output(m_buf(p), bias, y, g, s.relu, p->mats, st);
+            if (e != cudaSuccess) return fail_cuda(e, "row-wise output transform");
+        }
         return MNN_OK;
     }
     if (p->rect) {

@@ -12,6 +12,7 @@
 
 #include "kernels.h"
 #include "line_plan.h"
+#include "line_wino.h"
 #include "rows_plan.h"
 
 #include <algorithm>
@@ -571,6 +572,18 @@ uint64_t fused_cost(const LayerShape& s, const Calibration& cal)
                      serial_as, 0, cal);
 }
 
+// Row-wise Winograd with hi + lo BF16 operands, F(4, 3), F(4, 5), F(2, 7): relative L2 error x 1e6 as measured, rounded up; -1 where
+// there is no such form.  (F(4, 7) would have 85, more than the two-dimensional form on hi + lo TF32.)
+long long line_wino_ppm(int k) { return k == 3 ? 20 : k == 5 || k == 7 ? 30 : -1; }
+
+// Its three kernels: passes from x to V and from M to y at measured rates, and the product's own estimate.
+uint64_t line_wino_cost(const LayerShape& s, const LineWinoPlan& p, const Calibration& cal)
+{
+    const u128 x = (u128)4 * s.N * s.Cin * s.H * s.W, y = (u128)4 * s.N * s.Cout * s.OH * s.OW;
+    const u128 in = (x + (u128)p.v_bytes) * (uint64_t)cal.c[0] * 3 / 2, out = ((u128)p.m_bytes + y) * (uint64_t)cal.c[0] * 3 / 2;
+    return saturate((u128)kernel_ps(in, 0, 0, cal) + kernel_ps(out, 0, 0, cal) + (uint64_t)p.product_ps + (uint64_t)cal.c[5]);
+}
+
 }  // namespace
 
 bool fused_shape_ok(const LayerShape& s)
@@ -758,6 +771,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     // all layers with cold inputs, take a tenth more than theirs (256 channels 56 x 56 batch 64 BF16: 249 us, by rows 218): rows of Winograd F(2, 3) in hi + lo BF16 (booked as candidate 12), or the definition (as
     // candidate 2), with hi + lo operands in the TF32 class.  One image, 3x3: 64 channels 56 x 56 13.1 -> 8.5 us, 128 channels
     // 28 x 28 12.2 -> 8.6, 256 channels 14 x 14 11.3 -> 9.1.
+    bool row_wise = false;
     const unsigned held = s.W % 4 != 0 && s.k <= 5 ? 10 : s.k == 7 && best >= 3 && cands[best].m == 6 ? 15 : 11;
     const long long ppm_before = best >= 0 ? ppm_of[best] : 0;      // what the forms below may not exceed
     const bool free_choice = o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 && o.points_id == 0 &&
@@ -786,6 +800,26 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
             lhs_of[slot] = m == 1 ? MNN_GEMM_LHS_ROWS : 0;
             chunk_of[slot] = s.N;
             nch_of[slot] = 1;
+        }
+    }
+
+    if (free_choice && wino_shape_ok && best > 0 && o.precision == MNN_PREC_TF32) {
+        // Row-wise Winograd, hi + lo BF16, m = 4 (booked as candidate 13), or 2 (12) for 7 x 7 kernels, by the same rule.
+        LineWinoPlan lp;
+        const long long ppm = line_wino_ppm(s.k);
+        const int m = s.k == 7 ? 2 : 4, slot = m == 2 ? 12 : 13;
+        if (ppm >= 0 && ppm <= ppm_before && line_wino_plan({s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.pad, s.OH, s.OW, m}, cal.c[7] > 0 ? (int)cal.c[7] : 148, &lp)) {
+            const uint64_t cost = line_wino_cost(s, lp, cal);
+            if ((u128)cost * (d->rows ? 10u : held) < (u128)d->cost_ps[best] * 10u) {
+                best = slot;
+                d->rows = false;
+                row_wise = true;
+                d->cost_ps[slot] = cost;
+                ppm_of[slot] = ppm;
+                pts_of[slot] = best_points(m, s.k, MNN_OPERAND_BF16, 3, nullptr);
+                chunk_of[slot] = s.N;
+                nch_of[slot] = 1;
+            }
         }
     }
 
@@ -851,7 +885,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
         d->points_id = pts_of[best];
         d->chunk_images = chunk_of[best];
         d->n_chunks = nch_of[best];
-        d->fused = best == 15 ? MNN_FUSED_TILES : d->rows ? MNN_FUSED_ROWS : 0;
+        d->fused = best == 15 ? MNN_FUSED_TILES : d->rows ? MNN_FUSED_ROWS : row_wise ? MNN_ROW_WISE : 0;
         if (o.chunk_images > 0 && !d->fused) {
             d->chunk_images = o.chunk_images < s.N ? o.chunk_images : s.N;
             d->n_chunks = (s.N + d->chunk_images - 1) / d->chunk_images;

@@ -21,7 +21,7 @@ struct Decision {
     int chunk_images = 0, n_chunks = 0;
     int chosen = -1;
     int gemm_lhs = 0;                  // MNN_GEMM_LHS_* for the GEMM scheme, else 0
-    int fused = 0;                     // MNN_FUSED_TILES, MNN_FUSED_ROWS: Winograd in one kernel (wino_fused.cu, rows_conv.cu); else 0
+    int fused = 0;                     // MNN_FUSED_TILES, MNN_FUSED_ROWS: Winograd in one kernel (wino_fused.cu, rows_conv.cu); MNN_ROW_WISE (line_wino.cu); else 0
     bool rows = false;                 // the one-kernel convolution by rows (rows_conv.cu), also as a GEMM scheme
     int paper_n_hat = 0;               // Eq. 2's argmin over n in {1, 2, 4, 6} and the counts themselves
     uint64_t paper_mul[4] = {0, 0, 0, 0};

@@ -16,8 +16,9 @@ struct RectGeom {
     int pad_h, pad_w;
     int m, alpha;
     int n_seg;          // tiles per output line: ceil(OW / m) or ceil(OH / m)
+    int lines;          // along_w: lines per image in t, at least OH (row-wise form of square kernels: padded rows too)
     int cin_pad;
-    long long tiles;    // along_w: N * OH * n_seg (t = (n * OH + oh) * n_seg + seg); else N * n_seg * OW (t = (n * n_seg + seg) * OW + ow)
+    long long tiles;    // along_w: N * lines * n_seg (t = (n * lines + oh) * n_seg + seg); else N * n_seg * OW (t = (n * n_seg + seg) * OW + ow)
     long long m_row_stride;
 };
 

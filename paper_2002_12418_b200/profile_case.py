@@ -30,7 +30,11 @@ def stage_work(info, N, Cin, Cout, H, W, k, groups):
     y_bytes = 4 * N * Cout * info.OH * info.OW
     b_el = (2 if info.operand == B.OPERAND_BF16 else 4) * (2 if info.passes == 3 else 1)
     out = {}
-    if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
+    if info.algo == B.ALGO_WINOGRAD and info.fused == B.ROW_WISE:
+        out["input"] = (x_bytes + info.v_bytes, 0)
+        out["contract"] = (info.v_bytes + info.m_bytes + info.u_bytes, 2 * k * info.alpha * Cout * Cin * info.chunk_tiles * info.passes)
+        out["output"] = (info.m_bytes + y_bytes, 0)
+    elif info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS:
         T = N * info.OH * (-(-info.OW // info.m))          # one-dimensional tiles; the kernel's rows shift
         out["contract"] = (x_bytes + y_bytes + info.u_bytes, 2 * k * info.alpha * Cout * Cin * T * info.passes)
     elif info.algo == B.ALGO_WINOGRAD and info.fused:

@@ -1,6 +1,6 @@
-"""The convolution by rows in one kernel (rows_conv.cu) on the GPU, as the planner chooses it, against the fp64 oracle: last tiles
-and channel blocks that are not full, padded channels, odd rows, paddings other than the one that keeps the size, every kernel size,
-clusters, both accuracy classes; integer inputs bit for bit; repeated runs; NaN."""
+"""The convolution by rows in one kernel (rows_conv.cu) and row-wise Winograd (line_wino.cu) on the GPU, as the planner chooses them,
+against the fp64 oracle: last tiles and channel blocks that are not full, padded channels, odd rows, paddings other than the one that
+keeps the size, every kernel size, clusters, both accuracy classes; integer inputs bit for bit; repeated runs; NaN."""
 import numpy as np
 import pytest
 
@@ -12,8 +12,9 @@ from tests.util import rel_l2, to_dev
 pytestmark = pytest.mark.gpu
 
 # hi + lo BF16 operands leave 2^-17 of each factor and drop lo * lo: 3 * 2^-17 of a product at most, half of that as a 2-norm over
-# many; F(2, 3) enlarges it by the norms of its matrices; one BF16 product 2 * 2^-9.
-BOUND = {"rows1": 2.3e-5, "rows2": 3e-5, "bf16": 4e-3}
+# many; F(2, 3) and the row-wise forms enlarge it by the norms of their matrices (2.4e-5 at most in fp64 simulation); one BF16
+# product 2 * 2^-9.
+BOUND = {"rows1": 2.3e-5, "rows2": 3e-5, "wise": 5e-5, "bf16": 4e-3}
 
 
 @pytest.fixture(scope="module")
@@ -27,7 +28,7 @@ def torch():
 def form(info):
     if info.algo == B.ALGO_GEMM and info.gemm_lhs == B.GEMM_LHS_ROWS:
         return "rows1" if info.passes == 3 else "bf16"
-    return "rows2" if info.algo == B.ALGO_WINOGRAD and info.fused == B.FUSED_BY_ROWS else None
+    return {B.FUSED_BY_ROWS: "rows2", B.ROW_WISE: "wise"}.get(info.fused) if info.algo == B.ALGO_WINOGRAD else None
 
 
 def run(torch, shape, x, w, b, relu, cls=B.PREC_TF32, repeats=1):
@@ -60,7 +61,7 @@ SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "row
           ((9, 130, 1, 28, 29, 3, 1), "bf16"), ((2, 17, 100, 27, 7, 5, 0), "bf16"), ((1, 256, 1, 39, 35, 5, 4), "bf16"), ((17, 130, 1, 34, 36, 5, 4), "bf16"),
           ((1, 24, 72, 6, 13, 7, 3), "bf16"), ((1, 256, 64, 15, 12, 7, 0), "bf16"),
           ((32, 64, 64, 56, 56, 3, 1), "rows2"), ((17, 17, 17, 29, 37, 3, 1), "rows2"), ((17, 130, 1, 39, 30, 3, 0), "rows2"), ((17, 256, 1, 9, 33, 3, 1), "rows2"),
-          ((1, 256, 8, 37, 30, 3, 0), "rows2")]
+          ((1, 256, 8, 37, 30, 3, 0), "rows2"), ((17, 256, 1, 33, 31, 5, 2), "wise"), ((17, 256, 1, 18, 9, 7, 3), "wise"), ((17, 130, 1, 33, 38, 7, 0), "wise"), ((64, 128, 128, 28, 28, 5, 2), "wise")]
 
 
 @pytest.mark.parametrize("shape,expected", SHAPES)

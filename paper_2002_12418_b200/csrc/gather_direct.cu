@@ -344,7 +344,6 @@ __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) 
     extern __shared__ __align__(16) unsigned char dt_raw[];
     float* s_w = reinterpret_cast<float*>(dt_raw);                  // [kTileChunk][kRow]; later the partial sums
     long long* s_off = reinterpret_cast<long long*>(dt_raw + sizeof(float) * kTileChunk * kRow);   // offset << 8 | a << 4 | b
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cpg = g.Cin / g.groups, opg = g.Cout / g.groups, k2 = g.k * g.k, K = cpg * k2;
@@ -413,6 +412,10 @@ __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) 
         }
         for (; i < i1; ++i) fma_row(load(i), i);
     }
+    // Only now: let in at the start, the next kernel's blocks took part of this one's time, presumably by settling together on the SMs
+    // that this one's few blocks leave free (19 -> 19 3 x 3 stride 2, 108 x 47, batch 2, passes back to back: 10.4 us there, 6.6 here; in
+    // a graph 9.1 and 6.7; 20 -> 44 in 4 groups, 15 x 15, batch 8: 6.7 and 4.8).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int nan = 0;
     if (kw > 1) {
         __syncthreads();

@@ -8,10 +8,10 @@
 // copies; one issues tcgen05.mma: hi*hi + lo*hi + hi*lo for every (kernel row, position) into one accumulator per position.
 // Eight warps read the accumulators, apply A^T, bias and ReLU and store y.  Neither V nor M exists in memory.
 //
-// What bounds it: an instruction of 128 x N x 16 takes max(N / 2, 57 + N / 7) cycles, the 57 for reading its left operand, so narrow
-// channel blocks cost as much as 96 channels; and what instructions, weights and producers move through shared memory and
-// the L1, one data path (a copy of the x rows into shared memory in place of the producers' loads would pass it twice more).  Bulk
-// copies for the weights because a copy per channel costs its issuing warp 120 cycles.  Measured, one kernel against what ran
+// What bounds it: no memory level is near its rate (256 channels 56 x 56 BF16: tensor pipe 45 % busy, shared-memory banks 37 %, L2 24 %,
+// DRAM 10 %).  An instruction of 128 x N x 16 alone takes max(N / 2, 57 + N / 7) cycles, so narrow channel blocks cost as much as 96
+// channels.  With clocks in each role, which slow it by themselves, the issuing warp spent 112 cycles an instruction at N = 128
+// and 168 at N = 256 (75 and 128 alone) and 630 to 660 a stage waiting; why they are longer there was not separated.  Measured, one kernel against what ran
 // before: one image 64 channels 56 x 56 13.1 -> 8.5 us, 128 channels 28 x 28 12.2 -> 8.6, batch 32 64 channels 51 -> 28 (m = 2),
 // 128 channels 31 -> 23 (m = 2), 7 images 100 -> 72 channels 35 x 45 18.8 -> 13.6, 192 channels 17 x 17 1 x 7 batch 32 28.8 -> 21.7,
 // 256 channels 56 x 56 batch 64 BF16 249 -> 218.  Error against 64 bits 5e-6 (m = 1) and 1e-5 (m = 2) with hi + lo operands.

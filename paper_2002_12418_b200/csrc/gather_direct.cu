@@ -412,9 +412,11 @@ __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) 
         }
         for (; i < i1; ++i) fma_row(load(i), i);
     }
-    // Only now: let in at the start, the next kernel's blocks took part of this one's time, presumably by settling together on the SMs
-    // that this one's few blocks leave free (19 -> 19 3 x 3 stride 2, 108 x 47, batch 2, passes back to back: 10.4 us there, 6.6 here; in
-    // a graph 9.1 and 6.7; 20 -> 44 in 4 groups, 15 x 15, batch 8: 6.7 and 4.8).
+    // Only now: let in at the start, the next kernel's blocks cost strided and small layers much of their time (passes in a graph, start
+    // and here: 19 -> 19 3 x 3 stride 2, 108 x 47, batch 2: 9.1 and 6.7 us; 96 in 3 groups stride 2, 57 x 57, batch 16: 65.8 and 51.9;
+    // 20 -> 44 in 4 groups, 15 x 15, batch 8: 6.1 and 4.8), while larger stride-1 layers lose their overlap of 0.1 to 0.4 us (64 in 8
+    // groups, 56 x 56, batch 8: 23.5 and 23.6; 128 in 32 groups, 28 x 28, batch 16: 22.1 and 22.4).  Why was not separated.
+    // The kernel with a thread per element is the other way round (5 x 5 depthwise 64 channels, 28 x 28, batch 8: 14.0 and 16.7).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int nan = 0;
     if (kw > 1) {

@@ -104,6 +104,8 @@ enum { MNN_STAGE_WEIGHT = 1, MNN_STAGE_INPUT = 2, MNN_STAGE_CONTRACT = 4, MNN_ST
  *              IMPLICIT needs room for the weights only: ask for that where workspace is short.
  *              ROWS (not an option value; only where the caller leaves every choice open): the definition in one
  *              kernel that converts rows of x itself, one BF16 product, or three of hi + lo halves (passes = 3).
+ *              Outputs that the halves leave without a finite value are summed again in fp32, so that an infinity in
+ *              x or w gives what the definition gives.
  *              Asking for X or IMPLICIT where it does not apply fails the plan.
  *   fused      Winograd F(2x2, 3x3) as ONE kernel (input transform, contraction and output
  *              transform fused; the transformed tensors V and M never reach device memory):

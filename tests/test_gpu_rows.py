@@ -116,3 +116,54 @@ def test_not_a_number_reaches_its_windows_only(torch):
     near = np.zeros((H, W_), dtype=bool)
     near[3:6, 4:7] = True
     assert np.isnan(got[..., near]).all() and np.array_equal(got[..., ~near], clean[..., ~near])
+
+
+# Infinite inputs and weights, and inputs that BF16 rounds to infinity, give what the definition gives (with ReLU: fmax(no number, 0)
+# is 0), as the TF32 product does; nothing else changes.  One shape per tiles per item and way of issuing the products, one cluster.
+@pytest.mark.parametrize("relu", [False, True])
+@pytest.mark.parametrize("shape", [(1, 64, 100, 11, 10, 3, 1), (2, 100, 33, 8, 26, 2, 1), (17, 16, 17, 33, 39, 2, 1), (17, 16, 8, 30, 38, 3, 1),
+                                   (2, 256, 33, 8, 9, 3, 0)])
+def test_infinite_and_largest_values(torch, shape, relu):
+    N, Cin, Cout, H, W_, k, pad = shape
+    x, w, b = W.make_inputs(W.ConvLayer("inf", N, Cin, Cout, H, W_, k, 1, pad, seed=6))
+    x[:, 1] *= 0.2                                       # (no product with the largest weight may pass the largest number in one sum and not in the other)
+    clean, info = run(torch, shape, x, w, b, relu)
+    assert form(info) == "rows1"
+    x[0, 7, 4, 5], x[0, 3, 1, 1], x[N - 1, Cin - 1, H - 1, 0] = np.inf, -np.inf, 3.4e38
+    w[2, 5, 0, 0], w[4, 1, 1, 1] = np.inf, 3.4e38
+    got, _ = run(torch, shape, x, w, b, relu)
+    _check_not_finite(got, clean, oc.direct_conv(x, w, b, 1, pad, 1, 1, False), relu, [2, 4])
+
+
+@pytest.mark.parametrize("N,Cin,Cout,H,W_,kh,kw,ph,pw", [(3, 40, 17, 12, 33, 1, 2, 0, 1), (6, 36, 211, 31, 24, 5, 1, 2, 3), (2, 40, 24, 61, 1, 3, 1, 1, 0)])
+def test_infinite_and_largest_values_line_kernels(torch, N, Cin, Cout, H, W_, kh, kw, ph, pw):
+    rng = np.random.Generator(np.random.PCG64(8))
+    x = rng.standard_normal((N, Cin, H, W_), dtype=np.float32)
+    w = (rng.standard_normal((Cout, Cin, kh, kw)) * 0.1).astype(np.float32)
+    outs = []
+    for special in (False, True):
+        if special:
+            x[0, 7, 4, W_ // 2], x[1, 3, 1, 0], x[N - 1, Cin - 1, H - 1, 0] = np.inf, -np.inf, 3.4e38
+        r = B.ConvLayerRunner(N, Cin, Cout, H, W_, max(kh, kw), plan=B.mnn_conv_plan_rect(N, Cin, Cout, H, W_, kh, kw, ph, pw, B.make_opts()))
+        assert form(r.info) == "rows1"
+        y = r.run(to_dev(torch, x), to_dev(torch, w), None)
+        torch.cuda.synchronize()
+        assert r.device_status() == 0
+        outs.append(y.cpu().numpy())
+        r.close()
+    _check_not_finite(outs[1], outs[0], oc.direct_conv_rect(x, w, None, ph, pw, False), False, [])
+
+
+def _check_not_finite(got, clean, ref, relu, touched_channels):
+    """`ref` is the fp64 sum; outputs it leaves at ordinary size are those of the clean run, bit for bit."""
+    fp32 = ref.astype(np.float32)                        # beyond the largest fp32 number: infinite
+    large = ~(np.abs(ref) < 1e30)
+    assert large.any() and np.isinf(fp32).any()
+    want = np.where(np.isnan(fp32), np.float32(0), np.maximum(fp32, np.float32(0))) if relu else fp32
+    same = ~large
+    same[:, touched_channels] = False                    # (a large weight may meet zeros of x only)
+    assert np.array_equal(got[same], clean[same])
+    infinite = large & ~np.isfinite(want)
+    assert np.array_equal(got[infinite], want[infinite], equal_nan=True)
+    finite = large & np.isfinite(want)                   # fp32 sums of at most 2304 terms
+    assert (np.abs(got[finite].astype(np.float64) - want[finite]) <= 2304 * 2.0 ** -23 * 3.4e38).all() and np.isfinite(got[finite]).all()

@@ -186,8 +186,10 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 const int v_row = (rb * 2 + (int)rank) * kRows, u_row = nb * p.bn + (int)rank * (p.bn / 2);
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairProducer);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrPairProducer);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }
@@ -222,8 +224,10 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
             bool ok = true;
             for (long long item = pair; item < p.n_items && ok; item += n_pairs) {
                 if (!ptx::mbar_wait_warp(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
-                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairMmaTmem);
-                    *abortp = 1;
+                    if (lane == 0) {
+                        if (!*abortp) atomicCAS(p.status, 0, kErrPairMmaTmem);
+                        *abortp = 1;
+                    }
                     ok = false;
                     break;
                 }
@@ -231,8 +235,10 @@ contract_pair_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)kPairMaxN;
                 for (int kb = 0; kb < p.k_blocks; ++kb) {
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrPairMmaFull);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrPairMmaFull);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }

@@ -130,8 +130,10 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
                 const int nb = (int)(item / p.n_tile_blocks);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&empty_bar[stage]), phase ^ 1u, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrTmaWait);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrTmaWait);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }
@@ -155,16 +157,20 @@ implicit_gemm_kernel(const __grid_constant__ CUtensorMap map_u, IgParams p)
             bool ok = true;
             for (long long item = first_item; item < p.n_items && ok; item += item_step) {
                 if (!ptx::mbar_wait_warp(ptx::smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, abortp)) {
-                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
-                    *abortp = 1;
+                    if (lane == 0) {
+                        if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitTmem);
+                        *abortp = 1;
+                    }
                     break;
                 }
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)p.bn;
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&full_bar[stage]), phase, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitFull);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }

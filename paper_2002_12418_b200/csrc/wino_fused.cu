@@ -197,8 +197,10 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                 const uint8_t* src = p.U + (size_t)cb * p.k_blocks * kUBlockBytes;
                 for (int c = 0; c < p.k_blocks * kGroups; ++c) {           // consecutive copies are consecutive in memory
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&u_empty[slot]), phase ^ 1u, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrStreamWait);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrStreamWait);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }
@@ -223,15 +225,19 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
             const uint32_t a_lo_base = kDescLo + (u_base >> 4), b_lo_base = kDescLo + (v_base >> 4);
             for (int item = first; item < p.n_items && ok; item += step) {
                 if (!ptx::mbar_wait_warp(ptx::smem_u32(&acc_empty), acc_phase ^ 1u, abortp)) {
-                    if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitAcc);
-                    *abortp = 1;
+                    if (lane == 0) {
+                        if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitAcc);
+                        *abortp = 1;
+                    }
                     break;
                 }
                 ptx::tc_fence_after();
                 for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
                     if (!ptx::mbar_wait_warp(ptx::smem_u32(&v_full[buf]), v_phase, abortp)) {
-                        if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitV);
-                        *abortp = 1;
+                        if (lane == 0) {
+                            if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitV);
+                            *abortp = 1;
+                        }
                         ok = false;
                         break;
                     }
@@ -239,8 +245,10 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
 #pragma unroll 1
                     for (int grp = 0; grp < kGroups; ++grp) {
                         if (!ptx::mbar_wait_warp(ptx::smem_u32(&u_full[slot]), phase, abortp)) {
-                            if (lane == 0 && !*abortp) atomicCAS(p.status, 0, kErrMmaWaitU);
-                            *abortp = 1;
+                            if (lane == 0) {
+                                if (!*abortp) atomicCAS(p.status, 0, kErrMmaWaitU);
+                                *abortp = 1;
+                            }
                             ok = false;
                             break;
                         }

@@ -179,3 +179,16 @@ def test_calibration_record_round_trip_changes_the_plan():
             B.mnn_set_calibration([0] * 16)
     finally:
         B.mnn_set_calibration(base)
+
+
+# A wait that runs out is reported by the thread that then raises the abort flag: a lane that raised it without having reported first
+# could keep every role of its block, which report only while it is down, from writing the status word.
+def test_the_abort_flag_is_raised_only_by_who_has_reported():
+    import glob
+    seen = 0
+    for path in sorted(glob.glob(os.path.join(ROOT, "paper_2002_12418_b200", "csrc", "*.cu*"))):
+        text = open(path).read()
+        for m in re.finditer(r"\*abortp = 1;", text):
+            seen += 1
+            assert re.search(r"if \(!\*abortp( && status)?\)\s+atomicCAS\([^;]*;\s*$", text[:m.start()]), "%s:%d" % (os.path.basename(path), text.count("\n", 0, m.start()) + 1)
+    assert seen >= 30

@@ -352,7 +352,7 @@ class NetRunner:
         import torch
         self.torch = torch
         self.device = torch.device(device)
-        self.stream = _raw_stream(self.device)
+        self._raw_stream = _raw_stream(self.device)
         self.net = mnn_net_plan(N, H, W, layers, precision)
         self.info = mnn_net_query(self.net)
         with torch.cuda.device(self.device):
@@ -360,6 +360,9 @@ class NetRunner:
         self._ws_ptr = (self.workspace.data_ptr() + 1023) // 1024 * 1024
         mnn_net_set_workspace(self.net, self._ws_ptr, self.info.workspace_bytes)
         self._keep = None
+
+    def stream(self) -> int:
+        return self._raw_stream()
 
     def prepare(self, ws) -> None:
         mnn_net_prepare(self.net, [w.data_ptr() for w in ws], self.stream())
@@ -400,7 +403,7 @@ class ConvLayerRunner:
         import torch
         self.torch = torch
         self.device = torch.device(device)
-        self.stream = _raw_stream(self.device)
+        self._raw_stream = _raw_stream(self.device)
         self.shape = (N, Cin, Cout, H, W, k, stride, pad, dilation)
         if plan is not None:
             self.plan = plan               # e.g. from mnn_conv_plan_rect; owned by the runner from here on
@@ -415,6 +418,9 @@ class ConvLayerRunner:
                 base = self.workspace.data_ptr()
                 self._ws_ptr = (base + 1023) // 1024 * 1024
                 mnn_conv_set_workspace(self.plan, self._ws_ptr, self.info.workspace_bytes)
+
+    def stream(self) -> int:
+        return self._raw_stream()
 
     def prepare(self, w) -> None:
         mnn_conv_prepare_weights(self.plan, w.data_ptr(), self.stream())

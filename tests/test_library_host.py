@@ -192,3 +192,38 @@ def test_the_abort_flag_is_raised_only_by_who_has_reported():
             seen += 1
             assert re.search(r"if \(!\*abortp( && status)?\)\s+atomicCAS\([^;]*;\s*$", text[:m.start()]), "%s:%d" % (os.path.basename(path), text.count("\n", 0, m.start()) + 1)
     assert seen >= 30
+
+
+def test_a_subclass_chooses_the_stream_of_its_runs(monkeypatch):
+    import contextlib
+    import types
+    import torch
+
+    class OnStream7:
+        def stream(self):
+            return 7
+
+    class Layer(OnStream7, B.ConvLayerRunner):
+        pass
+
+    class Net(OnStream7, B.NetRunner):
+        pass
+
+    used = []
+    monkeypatch.setattr(torch.cuda, "device", lambda d: contextlib.nullcontext())
+    empty = torch.empty
+    monkeypatch.setattr(torch, "empty", lambda *a, **k: empty(*a, **{**k, "device": "cpu"}))
+    for name in ("mnn_conv_set_workspace", "mnn_net_set_workspace"):
+        monkeypatch.setattr(B, name, lambda *a: None)
+    layer = Layer(1, 8, 8, 9, 9, 3, 1, 1, 1, B.make_opts(force_algo=B.ALGO_GEMM))
+    net = Net(1, 28, 28, [W.ConvLayer("l", 1, 3, 8, 28, 28, 3, 1, 1)])
+    net.bind([empty(8, 3, 3, 3)], [None])
+    fake = types.SimpleNamespace(mnn_conv_run=lambda *a: used.append(a[-1]) or 0, mnn_net_run=lambda *a: used.append(a[-1]) or 0)
+    real = B._lib
+    monkeypatch.setattr(B, "_lib", fake)
+    layer.run(empty(1, 8, 9, 9), empty(8, 8, 3, 3))
+    net.run(empty(1, 3, 28, 28))
+    monkeypatch.setattr(B, "_lib", real)
+    assert used == [7, 7]
+    layer.close()
+    net.close()

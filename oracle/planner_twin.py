@@ -699,11 +699,12 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
     # against it: the estimates' measured errors) and not expected to be less accurate: as candidate 2 (the definition) or 12 (Winograd m = 2).
     held = 10 if L.W % 4 and L.k <= 5 else 15 if L.k == 7 and best >= 3 and _candidates()[best][1] == 6 else 11
     rows, row_wise, ppm_before = False, False, side.get(best, {}).get("ppm", 0)
+    winograd_before = best >= 3              # only then another Winograd form
     free = o.force_algo == o.force_m == o.operand == o.passes == o.points_id == o.gemm_lhs == o.fused == 0
     if free and wino_shape and best > 0:
         for m in (1, 2):
             passes, slot = (1 if o.precision == PREC_BF16 else 3), (2 if m == 1 else 12)
-            t = None if m == 2 and passes == 1 else rows_tiling(L, m, passes, c[7] if c[7] > 0 else 148)
+            t = None if m == 2 and (passes == 1 or not winograd_before) else rows_tiling(L, m, passes, c[7] if c[7] > 0 else 148)
             if t is None:
                 continue
             pid, p = (0, ppm.get((1, L.k, 0, OPERAND_BF16, passes), -1)) if m == 1 else best_points(ppm, m, L.k, OPERAND_BF16, passes)
@@ -718,7 +719,7 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
                 continue
             best, rows, ch.cost_ps[slot] = slot, True, cost
             side[slot] = dict(lhs=LHS_ROWS, ppm=p, pid=pid, chunk=L.N, n_chunks=1)
-        if o.precision == PREC_TF32 and L.k in ROW_WISE_PPM and ROW_WISE_PPM[L.k] <= ppm_before:
+        if winograd_before and o.precision == PREC_TF32 and L.k in ROW_WISE_PPM and ROW_WISE_PPM[L.k] <= ppm_before:
             m = 2 if L.k == 7 else 4
             t = row_wise_tiling(L, m, c[7] if c[7] > 0 else 148)
             if t is not None and row_wise_cost(L, t, c) * (10 if rows else held) < ch.cost_ps[best] * 10:

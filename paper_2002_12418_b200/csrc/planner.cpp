@@ -776,13 +776,15 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     const long long ppm_before = best >= 0 ? ppm_of[best] : 0;      // what the forms below may not exceed
     const bool free_choice = o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 && o.points_id == 0 &&
                              o.chunk_images == 0 && o.gemm_lhs == MNN_GEMM_LHS_AUTO && o.fused == 0;
+    // Winograd takes over from Winograd only: it spreads an infinity over its tiles, which the GEMM scheme keeps to the windows.
+    const bool winograd_before = best >= 3;
     if (free_choice && wino_shape_ok && best > 0) {
         const int sms = cal.c[7] > 0 ? (int)cal.c[7] : 148;
         for (int m = 1; m <= 2; ++m) {
             const int passes = o.precision == MNN_PREC_BF16 ? 1 : 3, slot = m == 1 ? 2 : 12;
             const RowsShape rs = {s.N, s.Cin, s.Cout, s.H, s.W, s.k, s.k, s.pad, s.pad, s.OH, s.OW, m, passes};
             RowsPlan rp;
-            if ((m == 2 && passes == 1) || !rows_plan(rs, sms, &rp)) continue;
+            if ((m == 2 && (passes == 1 || !winograd_before)) || !rows_plan(rs, sms, &rp)) continue;
             long long ppm = 0;
             const int pid = m == 1 ? 0 : best_points(m, s.k, MNN_OPERAND_BF16, passes, &ppm);
             if (m == 1) ppm = accuracy_ppm(1, s.k, 0, MNN_OPERAND_BF16, passes);
@@ -803,7 +805,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
         }
     }
 
-    if (free_choice && wino_shape_ok && best > 0 && o.precision == MNN_PREC_TF32) {
+    if (free_choice && wino_shape_ok && winograd_before && o.precision == MNN_PREC_TF32) {
         // Row-wise Winograd, hi + lo BF16, m = 4 (booked as candidate 13), or 2 (12) for 7 x 7 kernels, by the same rule.
         LineWinoPlan lp;
         const long long ppm = line_wino_ppm(s.k);

@@ -408,6 +408,15 @@ def test_packed_lines_are_compared_by_their_own_time(shape, packed):
     assert (info.gemm_lhs == B.GEMM_LHS_PACKED) == packed
 
 
+# Layers on the GEMM scheme: row-wise Winograd (the first), or F(2, 3) by rows, is estimated faster there, but would spread an infinity
+# over its tiles, and the first would need 47 MB of workspace instead of 6.
+@pytest.mark.parametrize("shape", [(43, 32, 240, 120, 5, 7, 1), (26, 48, 1552, 70, 2, 3, 1), (5, 16, 128, 83, 22, 3, 1), (26, 16, 1408, 12, 12, 3, 0)])
+def test_winograd_by_rows_replaces_winograd_only(shape):
+    N, Cin, Cout, H, W_, k, pad = shape
+    info = compare(W.ConvLayer("gemm", N, Cin, Cout, H, W_, k, 1, pad), {}, {}, B.mnn_get_calibration())
+    assert info.algo == B.ALGO_GEMM and info.workspace_bytes <= B.STATIC_WORKSPACE_BYTES
+
+
 def test_routing_rules():
     t = ppm_table()
     for l in all_layers():

@@ -267,8 +267,9 @@ MNN_API void mnn_conv_destroy(mnn_conv_plan_t plan);
  *   - plans whose info.workspace_bytes exceed MNN_STATIC_WORKSPACE_BYTES are
  *     rejected with MNN_EWORKSPACE (nothing is launched); plan with a smaller
  *     batch, or a smaller tile size, to fit.  A plan that the planner put on packed
- *     lines (info.gemm_lhs PACKED) and that does not fit runs here as it would be
- *     planned without them, and is rejected only if that does not fit either.
+ *     lines or on a form by rows (info.gemm_lhs PACKED or ROWS, info.fused FUSED_ROWS
+ *     or ROW_WISE) and that does not fit runs here as it would be planned without
+ *     them, and is rejected only if that does not fit either.
  *   - the first call on each device looks up the array's device address (with
  *     that device current); make that first call outside any stream capture.
  *     The current device must be the device of `stream` in every call.

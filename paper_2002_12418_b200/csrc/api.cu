@@ -51,7 +51,7 @@ struct mnn_conv_plan_s {
     LayerShape s;
     mnn_conv_opts o;
     Decision d;
-    Decision d_unpacked;             // where d takes packed lines: the decision without them (mnn_conv_run_static)
+    Decision d_static;               // for mnn_conv_run_static, where the workspace of packed lines or of a form by rows does not fit it
     int store_mode = STORE_TF32;
     int cin_pad = 0;                 // row length of U and V (Winograd: padded Cin; GEMM: padded Cin*k*k)
     long long chunk_tiles = 0;       // capacity of V / M in tiles (or GEMM columns)
@@ -248,6 +248,12 @@ int realise_decision(mnn_conv_plan_t p, const char** why)
     return MNN_OK;
 }
 
+// Packed lines or a form by rows that do not fit mnn_conv_run_static's workspace.
+bool exceeds_static_workspace(mnn_conv_plan_t p)
+{
+    return !p->rect && (p->packed || p->rows || p->row_wise) && p->workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES;
+}
+
 bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; }
 
 // Brackets one launch with events when profiling is on.
@@ -354,8 +360,7 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
     if (p->strassen) o_plan.passes = 1;      // the candidate list holds single-pass GEMMs; the pass count is set below
     const Calibration cal = current_calibration();
     if (cal.c[7] > 0) p->tiling_sms = (int)cal.c[7];
-    int rc = plan_layer(s, o_plan, cal, true, &p->d, &why);
-    if (rc == MNN_OK && p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) rc = plan_layer(s, o_plan, cal, false, &p->d_unpacked, &why);
+    int rc = plan_layer(s, o_plan, cal, FORMS_ALL, &p->d, &why);
     if (rc == MNN_OK && p->strassen) {
         p->d.passes = o.passes;
         p->d.chosen = -1;
@@ -363,6 +368,14 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
         p->d.error_ppm = accuracy_ppm(1, 1, 0, p->d.operand, p->d.passes);
     }
     if (rc == MNN_OK) rc = realise_decision(p, &why);
+    if (rc == MNN_OK && exceeds_static_workspace(p)) {
+        mnn_conv_plan_s t = *p;
+        for (int forms = FORMS_NO_ROWS; rc == MNN_OK && forms <= FORMS_PLAIN && exceeds_static_workspace(&t); ++forms) {
+            rc = plan_layer(s, o_plan, cal, forms, &t.d, &why);
+            if (rc == MNN_OK) rc = realise_decision(&t, &why);
+        }
+        p->d_static = t.d;
+    }
     if (rc != MNN_OK) {
         fail(rc, why);
         delete p;
@@ -476,7 +489,7 @@ mnn_conv_plan_t mnn_conv_plan_rect(int N, int Cin, int Cout, int H, int W, int k
         const long long three = 11100000 + macs / 100000 * 229 + (p->v_bytes + p->m_bytes) / 100 * 36;
         const long long rows_ppm = accuracy_ppm(1, k, 0, MNN_OPERAND_BF16, 3);
         if (rows_ppm >= 0 && rows_ppm <= ppm && rows_plan({N, Cin, Cout, H, W, kh, kw, pad_h, pad_w, OH, OW, 1, 3}, p->tiling_sms, &rc.p) &&
-            (rc.p.time_ps + cal.c[5]) * 11 < three * 10) {
+            (rc.p.time_ps + cal.c[5]) * 11 < three * 10) {     // (its workspace, the weights alone, is smaller)
             p->rc = rc;
             p->rows = true;
             p->d.rows = true;
@@ -1270,10 +1283,10 @@ extern "C" int mnn_conv_run_static(mnn_conv_plan_t p, const float* x, const floa
     // A private copy of the host-side plan whose workspace is the built-in array: the caller's
     // plan (its own workspace, prepared weights, profiling state) is left untouched.
     mnn_conv_plan_s local = *p;
-    if (p->packed && p->workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES) {
-        // packed planes do not fit: the layer as it is planned without them (the implicit gather stores none)
+    if (exceeds_static_workspace(p)) {
+        // the layer as it is planned without these forms (the implicit gather stores the weights only, in fewer padded channels)
         const char* why = "";
-        local.d = p->d_unpacked;
+        local.d = p->d_static;
         const int rc = realise_decision(&local, &why);
         if (rc != MNN_OK) return fail(rc, why);
     }

@@ -629,7 +629,7 @@ void winograd_chunking(const LayerShape& s, int m, int operand, int passes, cons
     *cost_ps = best_cost;
 }
 
-int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, bool packed_lines, Decision* d, const char** err)
+int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, int forms, Decision* d, const char** err)
 {
     static const int kM[3] = {2, 4, 6};
     d->rows = false;
@@ -711,7 +711,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
                 const uint64_t time_i = implicit_ok && !pointwise && cal.c[13] > 0 ? patch_operand_time(s, MNN_GEMM_LHS_IMPLICIT, cal, &split) : 0;
                 if (split > 1) {
                     if (lhs == MNN_GEMM_LHS_PATCHES && time_i < patch_operand_time(s, MNN_GEMM_LHS_PATCHES, cal, &split)) lhs = MNN_GEMM_LHS_IMPLICIT;
-                } else if (packed_lines && gemm_packs_lines(s, c.operand)) {
+                } else if (forms != FORMS_PLAIN && gemm_packs_lines(s, c.operand)) {
                     // TF32: the lines where they are estimated at less than 6/5 of the operand above, since either estimate can be a
                     // fifth off and the lines, where they lose by little, win by more (602 layers measured with both: 1.1 % over the
                     // better one each time, 2.0 % without the fifth)
@@ -774,7 +774,7 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     bool row_wise = false;
     const unsigned held = s.W % 4 != 0 && s.k <= 5 ? 10 : s.k == 7 && best >= 3 && cands[best].m == 6 ? 15 : 11;
     const long long ppm_before = best >= 0 ? ppm_of[best] : 0;      // what the forms below may not exceed
-    const bool free_choice = o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 && o.points_id == 0 &&
+    const bool free_choice = forms == FORMS_ALL && o.force_algo == MNN_ALGO_AUTO && o.force_m == 0 && o.operand == MNN_OPERAND_AUTO && o.passes == 0 && o.points_id == 0 &&
                              o.chunk_images == 0 && o.gemm_lhs == MNN_GEMM_LHS_AUTO && o.fused == 0;
     // Winograd takes over from Winograd only: it spreads an infinity over its tiles, which the GEMM scheme keeps to the windows.
     const bool winograd_before = best >= 3;

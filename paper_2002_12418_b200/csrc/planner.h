@@ -83,10 +83,11 @@ void winograd_chunking(const LayerShape& s, int m, int operand, int passes, cons
 // True when the layer's shape admits the fused Winograd F(2x2, 3x3) kernel.
 bool fused_shape_ok(const LayerShape& s);
 
-// Fills *d.  Returns MNN_OK or an mnn_status with *err set to a static reason.  packed_lines = false keeps the GEMM scheme from
-// packed lines, the one left operand chosen by itself whose workspace can far exceed the patch matrix's or the implicit
-// gather's.
-int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, bool packed_lines, Decision* d, const char** err);
+// The forms chosen by themselves whose workspace can exceed that of the form they replace.
+enum { FORMS_ALL, FORMS_NO_ROWS /* neither the convolution by rows nor row-wise Winograd */, FORMS_PLAIN /* nor packed lines */ };
+
+// Fills *d.  Returns MNN_OK or an mnn_status with *err set to a static reason.
+int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& cal, int forms, Decision* d, const char** err);
 
 // True when the Winograd kernels exist for (m, k).
 bool winograd_supported(int m, int k);

@@ -95,6 +95,32 @@ def test_static_workspace_where_the_packed_planes_do_not_fit(shape, lhs):
     assert_close(y.cpu().numpy(), oc.direct_conv(x, w, b, s, p, d, 1, True), B.PREC_TF32, "packed planes that do not fit")
 
 
+# Layers planned by rows whose weights, in channels padded to 16, do not fit the built-in array, but those of the patch matrix or of the
+# packed lines do: they run as the plan that asks for that operand, bit for bit.
+@pytest.mark.parametrize("shape,lhs", [((1, 27, 5655, 7, 9, 7, 1, 6, 1), B.GEMM_LHS_PATCHES), ((6, 32, 5324, 4, 8, 7, 1, 6, 1), B.GEMM_LHS_PACKED)])
+def test_static_workspace_where_the_weights_by_rows_do_not_fit(shape, lhs):
+    import torch
+    N, Cin, Cout, H, W_, k, s, p, d = shape
+    layer = W.ConvLayer("rows", N, Cin, Cout, H, W_, k, s, p, d, relu=True, seed=sum(shape))
+    x, w, b = W.make_inputs(layer)
+    xd, wd, bd = to_dev(torch, x), to_dev(torch, w), to_dev(torch, b)
+    plan = B.mnn_conv_plan_ex(*shape, B.make_opts(relu=1))
+    info = B.mnn_conv_plan_query(plan)
+    assert info.gemm_lhs == B.GEMM_LHS_ROWS and info.workspace_bytes > B.STATIC_WORKSPACE_BYTES
+    y = torch.full((N, Cout, info.OH, info.OW), float("nan"), device="cuda:0")
+    B.mnn_conv_run_static(plan, xd.data_ptr(), wd.data_ptr(), bd.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    B.mnn_conv_destroy(plan)
+    r = B.ConvLayerRunner(*shape, B.make_opts(relu=1, force_algo=B.ALGO_GEMM, operand=B.OPERAND_TF32, passes=1,
+                                              gemm_lhs=lhs if lhs != B.GEMM_LHS_PACKED else B.GEMM_LHS_AUTO))
+    assert r.info.gemm_lhs == lhs
+    y_ref = r.run(xd, wd, bd)
+    torch.cuda.synchronize()
+    assert r.device_status() == 0 and torch.equal(y, y_ref)
+    r.close()
+    at = np.random.default_rng(0).integers(0, y.numel(), 20000)
+    assert_close(y.cpu().numpy().ravel()[at], oc.direct_conv_at(x, w, b, at, s, p, d, 1, True), B.PREC_TF32, "weights by rows that do not fit")
+
+
 def test_static_workspace_rejects_plans_that_do_not_fit():
     import torch
     big = W.ConvLayer("big", 32, 256, 256, 56, 56, 3, 1, 1, seed=1)

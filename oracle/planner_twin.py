@@ -293,7 +293,7 @@ def _mma_cycles(n: int) -> int:
     return max(n // 2, 57 + n // 7)
 
 
-def rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, slots, rounds):
+def rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, slots, rounds, task_ps=595000):
     """Time of the convolution by rows in ps without its launch."""
     def moved(n):
         return 4096 + 32 * n
@@ -303,7 +303,7 @@ def rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split
     mma = tiles * (_mma_cycles(2 * bn) + _mma_cycles(bn) if mode == 2 else mode * _mma_cycles(bn)) * 461
     shared = tiles * (moved(2 * bn) + moved(bn) if mode == 2 else mode * moved(bn)) + steps * b_slot + a_slot
     x_bytes, tasks = rows * 64 * (1 if m == 1 else alpha), cdiv(rows, 32) * (1 if m == 1 else 2)
-    serial = cdiv(tasks, 10) * 595000 if m == 1 else cdiv(tasks, 12) * 1418000
+    serial = cdiv(tasks, 10) * task_ps if m == 1 else cdiv(tasks, 12) * 1418000
     stage = max(mma, (shared * 2 + x_bytes * (12 if m == 1 else 3)) * 193 // 100, serial) + steps * 51500
     drain, loop = 1098000 + 5700 * mt * bn * alpha * wide, slots * stage + 672000
     cost = rounds * max(loop, drain) + drain if bufs == 2 else rounds * (loop + drain)
@@ -328,6 +328,7 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
     if cells >= (1 << 31) - 65536 or span > 2048:
         return None
     stages, co16, room, best = cdiv(L.Cin, 16), cdiv(L.Cout, 16) * 16, 213 * 1024, None
+    from_memory = m == 1 and 4 * L.N * (L.Cin * L.H * L.W + L.Cout * L.OH * L.OW) > 16000000
     for mode in ([1] if passes == 1 else [3] if m == 2 else [2, 3]):
         halves, wide = (1 if mode == 1 else 2), (2 if mode == 2 else 1)
         for mt in ((1, 2) if m == 1 else (1,)):
@@ -353,10 +354,10 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
                     if split > 1 and (mt > 1 or items * split > sms or split == 4 and items > 32 or split == 8 and items > 8
                                       or stages < 2 * split or bn * m * 512 > room):
                         break
-                    cost = rows_time(k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, cdiv(stages, split),
-                                     cdiv(items * split, sms))
+                    args = (k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, cdiv(stages, split), cdiv(items * split, sms))
+                    cost = rows_time(*args)
                     if best is None or cost < best["time_ps"]:
-                        best = dict(time_ps=cost, mode=mode, mt=mt, bn=bn, split=split, items=items, rows=rows)
+                        best = dict(time_ps=cost, memory_ps=rows_time(*args, 900000) if from_memory else cost, mode=mode, mt=mt, bn=bn, split=split, items=items, rows=rows)
     return best
 
 
@@ -710,12 +711,11 @@ def plan(L: Layer, o: Options, c, ppm) -> Choice:
             pid, p = (0, ppm.get((1, L.k, 0, OPERAND_BF16, passes), -1)) if m == 1 else best_points(ppm, m, L.k, OPERAND_BF16, passes)
             now = ch.cost_ps[best]
             lines = not rows and side[best].get("lhs") == LHS_PACKED
-            if lines and L.Cout < 256:
-                continue
-            if lines:
-                now = min(now, packed_cost(L, _candidates()[best][2], c))
             cost = t["time_ps"] + c[5]
-            if p < 0 or p > ppm_before or cost * (10 if rows else 9 if lines else held) >= now * 10:
+            if lines:                           # by their own time; BF16: x from memory, and two overlapping kernels
+                now, cost = min(now, packed_cost(L, _candidates()[best][2], c)), (t["memory_ps"] if passes == 1 else t["time_ps"]) + c[5]
+            faster = (cost < now if rows else cost * 9 < now * 10 if lines and passes == 3 else cost * 19 + 80000000 < now * 20 if lines else cost * held < now * 10)
+            if p < 0 or p > ppm_before or not faster:
                 continue
             best, rows, ch.cost_ps[slot] = slot, True, cost
             side[slot] = dict(lhs=LHS_ROWS, ppm=p, pid=pid, chunk=L.N, n_chunks=1)

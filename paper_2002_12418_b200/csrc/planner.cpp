@@ -766,11 +766,14 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
     }
 
     // The convolution by rows, one kernel, where the planner is free and it is estimated faster than a tensor-core scheme that is not
-    // expected to be more accurate; a tenth is held against it, nothing on rows that are no multiple of 16 bytes (Winograd
-    // there measured 1.0 to 1.4 times its estimate, k <= 5), half against F(6, 7) (measured at 0.65 to 0.9 of its estimate); packed lines, of
-    // all layers with cold inputs, take a tenth more than theirs (256 channels 56 x 56 batch 64 BF16: 249 us, by rows 218): rows of Winograd F(2, 3) in hi + lo BF16 (booked as candidate 12), or the definition (as
-    // candidate 2), with hi + lo operands in the TF32 class.  One image, 3x3: 64 channels 56 x 56 13.1 -> 8.5 us, 128 channels
-    // 28 x 28 12.2 -> 8.6, 256 channels 14 x 14 11.3 -> 9.1.
+    // expected to be more accurate: rows of Winograd F(2, 3) in hi + lo BF16 (booked as candidate 12), or the definition (as candidate 2), with
+    // hi + lo operands in the TF32 class.  A tenth is held against it, nothing on rows that are no multiple of 16 bytes (Winograd
+    // there measured 1.0 to 1.4 times its estimate, k <= 5), half against F(6, 7) (measured at 0.65 to 0.9 of its estimate).
+    // Packed lines by their own time, from layers of any number of output channels measured in both forms with other inputs in each
+    // call.  BF16: x from memory, and the lines' two kernels take 4 us less than their estimate, and a twentieth more (328 layers lose 0.5 % against the
+    // better form each time, 3.6 % always in lines, 4.3 % by the rows' estimate from the L2); TF32: a tenth in favour of the rows (75 layers: 0.3 %,
+    // always in lines 53 %).  64 images 256 channels 56 x 56 BF16 to 256: 244 us in lines, 237 by rows; to 192: 226 and 203; to 96: 155 and 188.
+    // One image, 3x3: 64 channels 56 x 56 13.1 -> 8.5 us, 128 channels 28 x 28 12.2 -> 8.6, 256 channels 14 x 14 11.3 -> 9.1.
     bool row_wise = false;
     const unsigned held = s.W % 4 != 0 && s.k <= 5 ? 10 : s.k == 7 && best >= 3 && cands[best].m == 6 ? 15 : 11;
     const long long ppm_before = best >= 0 ? ppm_of[best] : 0;      // what the forms below may not exceed
@@ -790,10 +793,15 @@ int plan_layer(const LayerShape& s, const mnn_conv_opts& o, const Calibration& c
             if (m == 1) ppm = accuracy_ppm(1, s.k, 0, MNN_OPERAND_BF16, passes);
             uint64_t now = d->cost_ps[best];
             const bool lines = !d->rows && lhs_of[best] == MNN_GEMM_LHS_PACKED;
-            if (lines && s.Cout < 256) continue;      // (64 channels 56 x 56 batch 64: 50 us in lines, 51 by rows)
-            if (lines) now = std::min(now, packed_cost(s, cands[best].operand, cal));
-            const uint64_t cost = (uint64_t)rp.time_ps + (uint64_t)cal.c[5];
-            if (ppm < 0 || ppm > ppm_before || (u128)cost * (d->rows ? 10u : lines ? 9u : held) >= (u128)now * 10u) continue;
+            uint64_t cost = (uint64_t)rp.time_ps + (uint64_t)cal.c[5];
+            if (lines) {
+                now = std::min(now, packed_cost(s, cands[best].operand, cal));
+                if (passes == 1) cost = (uint64_t)rp.memory_ps + (uint64_t)cal.c[5];
+            }
+            const bool faster = d->rows ? cost < now
+                                : !lines ? (u128)cost * held < (u128)now * 10u
+                                : passes == 3 ? (u128)cost * 9u < (u128)now * 10u : (u128)cost * 19u + 80000000u < (u128)now * 20u;
+            if (ppm < 0 || ppm > ppm_before || !faster) continue;
             best = slot;
             d->rows = true;
             d->cost_ps[slot] = cost;

@@ -34,6 +34,7 @@ struct RowsPlan {
     int bn, n_co_blocks, split, a_slots, b_slots, acc_bufs;
     long long n_tile_blocks, n_items, u_bytes;
     long long time_ps;                   // estimated time of the kernel without its launch
+    long long memory_ps;                 // the same where x has to come from memory
 };
 
 bool rows_plan(const RowsShape& s, int num_sms, RowsPlan* p);

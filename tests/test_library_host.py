@@ -231,7 +231,7 @@ def test_a_subclass_chooses_the_stream_of_its_runs(monkeypatch):
 
 # What ran in the built-in workspace before a form with more padded weights was chosen still does: without a GPU the call must get
 # beyond the question of room.
-@pytest.mark.parametrize("shape", [(1, 27, 5655, 7, 9, 7, 1, 6, 1), (6, 32, 5324, 4, 8, 7, 1, 6, 1), (43, 32, 240, 120, 5, 7, 1, 1, 1)])
+@pytest.mark.parametrize("shape", [(1, 27, 5655, 7, 9, 7, 1, 6, 1), (5, 128, 7233, 5, 3, 3, 1, 1, 1), (43, 32, 240, 120, 5, 7, 1, 1, 1)])
 def test_static_runs_are_not_refused_for_the_chosen_form(shape):
     import torch
     if torch.cuda.is_available():

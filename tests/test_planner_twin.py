@@ -417,6 +417,25 @@ def test_winograd_by_rows_replaces_winograd_only(shape):
     assert info.algo == B.ALGO_GEMM and info.workspace_bytes <= B.STATIC_WORKSPACE_BYTES
 
 
+# Packed lines against the convolution by rows, at the sizes where either was measured faster by more than 4 % (us in lines and by rows):
+# neither the number of output channels nor the accuracy class decides alone.
+@pytest.mark.parametrize("shape,precision,rows", [
+    ((64, 256, 96, 56, 56, 3, 1), B.PREC_BF16, False),      # 155, 188
+    ((64, 256, 192, 56, 56, 3, 1), B.PREC_BF16, True),      # 226, 203
+    ((64, 256, 255, 56, 56, 3, 1), B.PREC_BF16, True),      # 252, 242
+    ((64, 256, 256, 56, 56, 3, 1), B.PREC_BF16, True),      # 244, 237 (262 and 302 call after call)
+    ((64, 256, 288, 56, 56, 3, 1), B.PREC_BF16, False),     # 295, 399
+    ((10, 256, 256, 95, 95, 3, 1), B.PREC_BF16, False),     # 124, 158
+    ((18, 64, 160, 28, 28, 3, 1), B.PREC_BF16, True),       # 12.5, 9.7
+    ((4, 192, 464, 26, 26, 2, 1), B.PREC_BF16, False),      # 11.1, 13.6
+    ((5, 64, 400, 15, 9, 3, 1), B.PREC_BF16, False),        # 6.3, 7.0
+    ((13, 6, 181, 62, 41, 3, 1), B.PREC_TF32, True)])       # 18.5, 11.9
+def test_rows_against_packed_lines(shape, precision, rows):
+    N, Cin, Cout, H, W_, k, pad = shape
+    info = compare(W.ConvLayer("lines", N, Cin, Cout, H, W_, k, 1, pad), dict(precision=precision), dict(precision=precision), B.mnn_get_calibration())
+    assert (info.gemm_lhs == B.GEMM_LHS_ROWS) == rows
+
+
 def test_routing_rules():
     t = ppm_table()
     for l in all_layers():

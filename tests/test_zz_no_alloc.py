@@ -97,7 +97,7 @@ def test_static_workspace_where_the_packed_planes_do_not_fit(shape, lhs):
 
 # Layers planned by rows whose weights, in channels padded to 16, do not fit the built-in array, but those of the patch matrix or of the
 # packed lines do: they run as the plan that asks for that operand, bit for bit.
-@pytest.mark.parametrize("shape,lhs", [((1, 27, 5655, 7, 9, 7, 1, 6, 1), B.GEMM_LHS_PATCHES), ((6, 32, 5324, 4, 8, 7, 1, 6, 1), B.GEMM_LHS_PACKED)])
+@pytest.mark.parametrize("shape,lhs", [((1, 27, 5655, 7, 9, 7, 1, 6, 1), B.GEMM_LHS_PATCHES), ((5, 128, 7233, 5, 3, 3, 1, 1, 1), B.GEMM_LHS_PACKED)])
 def test_static_workspace_where_the_weights_by_rows_do_not_fit(shape, lhs):
     import torch
     N, Cin, Cout, H, W_, k, s, p, d = shape

@@ -352,7 +352,7 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
                     continue
                 for split in (1, 2, 4, 8):
                     if split > 1 and (mt > 1 or items * split > sms or split == 4 and items > 32 or split == 8 and items > 8
-                                      or stages < 2 * split or bn * m * 512 > room):
+                                      or 2 * stages < 3 * split or bn * m * 512 > room):
                         break
                     args = (k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, cdiv(stages, split), cdiv(items * split, sms))
                     cost = rows_time(*args)

@@ -63,7 +63,9 @@ bool rows_plan(const RowsShape& s, int num_sms, RowsPlan* p)
             if (items >= (1ll << 31)) continue;
             for (int split = 1; split <= 8; split *= 2) {
                 // (clusters of four and eight that do not all fit the GPCs at once run in two waves: 36 of four 10 -> 20 us)
-                if (split > 1 && (mt > 1 || items * split > num_sms || (split == 4 && items > 32) || (split == 8 && items > 8) || p->k_slots < 2 * split ||
+                // A CTA may have one stage beside others with two: 112 channels (seven stages) 10 x 10 one image in four 7.5 us, in two 10.3 (three
+                // Winograd kernels 7.1 to 8), 96 channels 5 x 7 four images 7.5 and 9.5 (7.5 to 8).
+                if (split > 1 && (mt > 1 || items * split > num_sms || (split == 4 && items > 32) || (split == 8 && items > 8) || 2 * p->k_slots < 3 * split ||
                                   (long long)bn * s.m * 512 > room))
                     break;
                 // A stage: the instructions of its weight tiles (57 cycles for the left operand, more only from 128 channels on), or what

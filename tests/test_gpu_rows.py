@@ -61,7 +61,10 @@ SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "row
           ((9, 130, 1, 28, 29, 3, 1), "bf16"), ((2, 17, 100, 27, 7, 5, 0), "bf16"), ((1, 256, 1, 39, 35, 5, 4), "bf16"), ((17, 130, 1, 34, 36, 5, 4), "bf16"),
           ((1, 24, 72, 6, 13, 7, 3), "bf16"), ((1, 256, 64, 15, 12, 7, 0), "bf16"),
           ((32, 64, 64, 56, 56, 3, 1), "rows2"), ((17, 17, 17, 29, 37, 3, 1), "rows2"), ((17, 130, 1, 39, 30, 3, 0), "rows2"), ((17, 256, 1, 9, 33, 3, 1), "rows2"),
-          ((1, 256, 8, 37, 30, 3, 0), "rows2"), ((17, 256, 1, 33, 31, 5, 2), "wise"), ((17, 256, 1, 18, 9, 7, 3), "wise"), ((17, 130, 1, 33, 38, 7, 0), "wise"), ((64, 128, 128, 28, 28, 5, 2), "wise")]
+          ((1, 256, 8, 37, 30, 3, 0), "rows2"), 
+          # 3, 7, 12 and 13 stages shared out unevenly over clusters
+          ((8, 44, 16, 12, 19, 7, 6), "rows1"), ((1, 112, 100, 10, 10, 3, 1), "rows1"), ((1, 186, 40, 10, 10, 3, 1), "rows1"), ((2, 200, 100, 6, 5, 3, 1), "bf16"),
+          ((17, 256, 1, 33, 31, 5, 2), "wise"), ((17, 256, 1, 18, 9, 7, 3), "wise"), ((17, 130, 1, 33, 38, 7, 0), "wise"), ((64, 128, 128, 28, 28, 5, 2), "wise")]
 
 
 @pytest.mark.parametrize("shape,expected", SHAPES)

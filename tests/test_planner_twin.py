@@ -417,6 +417,18 @@ def test_winograd_by_rows_replaces_winograd_only(shape):
     assert info.algo == B.ALGO_GEMM and info.workspace_bytes <= B.STATIC_WORKSPACE_BYTES
 
 
+# Few items share their stages out over clusters, unevenly too (7 over 4): cut in two only, the first two lost to three Winograd kernels.
+@pytest.mark.parametrize("shape,precision,split", [((1, 112, 112, 10, 10, 3, 1), B.PREC_TF32, 4), ((2, 111, 111, 9, 9, 3, 1), B.PREC_BF16, 4),
+                                                   ((4, 96, 96, 5, 7, 3, 1), B.PREC_TF32, 4), ((1, 178, 178, 10, 10, 3, 1), B.PREC_BF16, 8),
+                                                   ((1, 64, 100, 11, 10, 3, 1), B.PREC_TF32, 1)])
+def test_rows_share_their_stages_unevenly(shape, precision, split):
+    N, Cin, Cout, H, W_, k, pad = shape
+    info = compare(W.ConvLayer("split", N, Cin, Cout, H, W_, k, 1, pad), dict(precision=precision), dict(precision=precision), B.mnn_get_calibration())
+    assert info.gemm_lhs == B.GEMM_LHS_ROWS
+    t = T.rows_tiling(T.Layer(N, Cin, Cout, H, W_, k, 1, pad, 1), 1, 3 if precision == B.PREC_TF32 else 1, 148)
+    assert t["split"] == split
+
+
 # Packed lines against the convolution by rows, at the sizes where either was measured faster by more than 4 % (us in lines and by rows):
 # neither the number of output channels nor the accuracy class decides alone.
 @pytest.mark.parametrize("shape,precision,rows", [

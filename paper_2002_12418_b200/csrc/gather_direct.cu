@@ -338,12 +338,13 @@ __device__ __forceinline__ void direct_tile_redo(const float* __restrict__ x, co
 template <int TCO, bool PAD>
 __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) direct_tile_kernel(const float* __restrict__ x, const float* __restrict__ w,
                                                                    const float* __restrict__ bias, float* __restrict__ y,
-                                                                   DirectGeom g, int kw, int pos_blocks, int co_tiles, long long T)
+                                                                   DirectGeom g, int kw, int pos_blocks, int co_tiles, long long T, int next_early)
 {
     constexpr int kRow = TCO >= 8 ? TCO + 4 : TCO;                  // padded: the transposing stores spread over the banks
     extern __shared__ __align__(16) unsigned char dt_raw[];
     float* s_w = reinterpret_cast<float*>(dt_raw);                  // [kTileChunk][kRow]; later the partial sums
     long long* s_off = reinterpret_cast<long long*>(dt_raw + sizeof(float) * kTileChunk * kRow);   // offset << 8 | a << 4 | b
+    if (next_early) asm volatile("griddepcontrol.launch_dependents;");       // (else behind the main loop)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cpg = g.Cin / g.groups, opg = g.Cout / g.groups, k2 = g.k * g.k, K = cpg * k2;
@@ -412,12 +413,7 @@ __global__ void __launch_bounds__(kTileThreads) __maxnreg__(TCO == 4 ? 40 : 64) 
         }
         for (; i < i1; ++i) fma_row(load(i), i);
     }
-    // Only now: let in at the start, the next kernel's blocks cost strided and small layers much of their time (passes in a graph, start
-    // and here: 19 -> 19 3 x 3 stride 2, 108 x 47, batch 2: 9.1 and 6.7 us; 96 in 3 groups stride 2, 57 x 57, batch 16: 65.8 and 51.9;
-    // 20 -> 44 in 4 groups, 15 x 15, batch 8: 6.1 and 4.8), while larger stride-1 layers lose their overlap of 0.1 to 0.4 us (64 in 8
-    // groups, 56 x 56, batch 8: 23.5 and 23.6; 128 in 32 groups, 28 x 28, batch 16: 22.1 and 22.4).  Why was not separated.
-    // The kernel with a thread per element is the other way round (5 x 5 depthwise 64 channels, 28 x 28, batch 8: 14.0 and 16.7).
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!next_early) asm volatile("griddepcontrol.launch_dependents;");
     int nan = 0;
     if (kw > 1) {
         __syncthreads();
@@ -1234,9 +1230,18 @@ cudaError_t launch_direct(const float* x, const float* w, const float* bias, flo
     const long long pos_blocks = (T + 32 * (8 / kw) - 1) / (32 * (8 / kw));
     if (pos_blocks * cts > 2147483647ll) return cudaErrorInvalidValue;
     const unsigned blocks = (unsigned)(pos_blocks * cts);
+    // The next kernel is let in at the start or only behind the main loop.  Its waiting CTAs take places on SMs where this kernel's CTAs are
+    // not all there yet, which presumably then settle unevenly on the others, so it waits where they fill from a sixteenth to three
+    // quarters of the chip: the same layer again and again, let in early and late, at 0.37 of it 12.9 and 8.9 us (80 -> 16 in 8 groups, 51 x 51, batch 2), at 0.54
+    // 69.9 and 53.1 (96 in 3 groups stride 2, 57 x 57, batch 16), at 0.73 28.2 and 25.7, but at 0.05 3.2 and 3.3, at 0.86 39.3 and 39.9, at 1.3
+    // 25.0 and 25.1 (64 in 8 groups, 56 x 56, batch 8).  Of 75 layers all from 0.14 to 0.73 are faster late, up to 0.05 and from 0.77 on early
+    // or the same to 0.3 %; between are five that differ by 4 % either way.
+    // The kernel with a thread per element is overlapped by a rule of its own (above).
+    const long long resident = 148ll * (tco == 4 ? 6 : 4);
+    const int next_early = 16ll * blocks < resident || 4ll * blocks >= 3 * resident ? 1 : 0;
 #define MNNB_DIRECT_TILE(TCO) do { \
         const size_t smem = sizeof(float) * kTileChunk * (TCO >= 8 ? TCO + 4 : TCO) + sizeof(long long) * kTileChunk; \
-        return launch_overlapped(g.pad > 0 ? direct_tile_kernel<TCO, true> : direct_tile_kernel<TCO, false>, dim3(blocks), dim3(kTileThreads), smem, stream, x, w, bias, y, g, kw, (int)pos_blocks, (int)co_tiles, T); } while (0)
+        return launch_overlapped(g.pad > 0 ? direct_tile_kernel<TCO, true> : direct_tile_kernel<TCO, false>, dim3(blocks), dim3(kTileThreads), smem, stream, x, w, bias, y, g, kw, (int)pos_blocks, (int)co_tiles, T, next_early); } while (0)
     if (tco == 16) MNNB_DIRECT_TILE(16); else if (tco == 8) MNNB_DIRECT_TILE(8); else MNNB_DIRECT_TILE(4);
 #undef MNNB_DIRECT_TILE
 }

@@ -622,3 +622,29 @@ def test_calibration_of_direct_and_gather(torch):
     got = [sorted(r[i] for r in runs)[2] for i in range(len(before))]
     assert all(c > 0 for c in got[:9]) and before[8] / 2 < got[8] < before[8] * 2
     assert before[13] / 2 < got[13] < before[13] * 2
+
+
+# The sliding-window tile kernel lets the next kernel in at its start or behind its main loop, by how much of the chip its CTAs fill: chains of
+# two layers, the second on the first one's output as it is written, on either side of both lines (a sixteenth and three quarters).
+@pytest.mark.parametrize("N,C,groups,H,stride", [(1, 8, 2, 9, 1), (5, 30, 2, 17, 1), (16, 96, 3, 57, 2), (6, 56, 8, 19, 1), (10, 56, 8, 19, 1), (8, 64, 8, 56, 1)])
+def test_chained_tile_layers(torch, N, C, groups, H, stride):
+    layers = [W.ConvLayer("tile%d" % i, N, C, C, h, h, 3, s, 1, groups=groups, relu=True, seed=700 + C + i)
+              for i, (h, s) in enumerate([(H, stride), ((H + 2 - 3) // stride + 1, 1)])]
+    ins = [W.make_inputs(l) for l in layers]
+    runners = [B.ConvLayerRunner(l.N, l.Cin, l.Cout, l.H, l.W, l.k, l.stride, l.pad, 1, B.make_opts(groups=groups, relu=1)) for l in layers]
+    assert all(r.info.algo == B.ALGO_DIRECT for r in runners)
+    x = to_dev(torch, ins[0][0])
+    dev = [(to_dev(torch, w), to_dev(torch, b) if b is not None else None) for _, w, b in ins]
+    outs = []
+    for _ in range(3):
+        y = x
+        for r, (w, b) in zip(runners, dev):
+            y = r.run(y, w, b)
+        outs.append(y)
+    torch.cuda.synchronize()
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
+    mid = oc.direct_conv(ins[0][0], ins[0][1], ins[0][2], stride, 1, 1, groups, True).astype(np.float32)
+    want = oc.direct_conv(mid, ins[1][1], ins[1][2], 1, 1, 1, groups, True)
+    assert rel_l2(outs[0].cpu().numpy(), want) <= 1e-5                 # fp32 sums of at most 288 terms, twice
+    for r in runners:
+        r.close()

@@ -341,7 +341,7 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
                 if wide * bn > 256 or alpha * mt * wide * bn > 512:
                     continue
                 bufs = 2 if 2 * alpha * mt * wide * bn <= 512 else 1
-                if mt == 2 and bufs == 1:
+                if mt == 2 and bufs == 1 or m == 1 and mode == 3 and k == 7 and mt == 1:
                     continue
                 rows = cdiv(128 * mt + span, 8) * 8
                 a_slot, b_slot = alpha * halves * rows * 32, taps * halves * bn * 32
@@ -351,7 +351,7 @@ def rows_tiling(L: Layer, m: int, passes: int, sms: int):
                 if items >= 1 << 31:
                     continue
                 for split in (1, 2, 4, 8):
-                    if split > 1 and (mt > 1 or items * split > sms or split == 4 and items > 32 or split == 8 and items > 8
+                    if split > 1 and (mt > 1 or m == 1 and mode == 3 and k >= 5 or items * split > sms or split == 4 and items > 32 or split == 8 and items > 8
                                       or 2 * stages < 3 * split or bn * m * 512 > room):
                         break
                     args = (k, m, mode, mt, bn, alpha, taps, rows, b_slot, a_slot, bufs, split, cdiv(stages, split), cdiv(items * split, sms))

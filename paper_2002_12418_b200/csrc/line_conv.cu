@@ -53,25 +53,6 @@ struct LineParams {
 // word, so that an instruction costs the issuing thread one addition per operand.
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 
-template <bool BF16>
-__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
-{
-#define MNNB_LINE_MMA(KIND)                                                                                                \
-    asm volatile(                                                                                                          \
-        "{\n\t"                                                                                                            \
-        ".reg .b64 da, db;\n\t"                                                                                            \
-        ".reg .pred p;\n\t"                                                                                                \
-        "mov.b64 da, {%1, %3};\n\t"                                                                                        \
-        "mov.b64 db, {%2, %3};\n\t"                                                                                        \
-        "setp.ne.b32 p, %5, 0;\n\t"                                                                                        \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %4, p;\n\t"                                                 \
-        "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate)                                 \
-        : "memory")
-    if (BF16) MNNB_LINE_MMA("f16");
-    else MNNB_LINE_MMA("tf32");
-#undef MNNB_LINE_MMA
-}
-
 // MT = tiles of 128 cells per item, KS = tensor-core steps per block of elements, G = weight tiles per step (slot, barrier and
 // commit), all fixed at compile time, with one issuing warp per tile of cells.  The issuing warp is on the critical path:
 // dilation-2 layer above, product only: 66 us with run-time loop bounds, 43.5 unrolled, 38 with up to three taps per step;
@@ -221,8 +202,8 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                                     if (j < n) {
 #pragma unroll
                                         for (int ks = 0; ks < KS; ++ks)
-                                            mma_lo<BF16>(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), idesc,
-                                                   (j | ks) ? 1u : accumulate);
+                                            ptx::mma_lo<BF16 ? 1 : 0>(d0, a_lo[j] + (uint32_t)(ks * 2), b_lo + (uint32_t)j * (b_tile_bytes >> 4) + (uint32_t)(ks * 2), kDescHi,
+                                                                      idesc, (j | ks) ? 1u : accumulate);
                                     }
                                 ptx::mma_commit(ptx::smem_u32(&b_empty[bs]));
                             }

@@ -11,13 +11,6 @@ namespace {
 long long cdiv(long long a, long long b) { return (a + b - 1) / b; }
 long long rup(long long a, long long b) { return cdiv(a, b) * b; }
 
-// Cells of one axis: `out` outputs, `lead` zero cells in front, data cells end before `end`, taps reach `reach` cells past an
-// output.  The smallest pitch that lets the zero cells behind the data be the next line's leading ones.
-int axis_pitch(int out, int lead, int end, int reach)
-{
-    return std::max(out, std::min(out + reach, std::max(end, out + reach - lead)));
-}
-
 }  // namespace
 
 bool line_plan(const LineShape& s, int num_sms, LinePlan* p)

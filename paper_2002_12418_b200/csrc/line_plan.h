@@ -11,6 +11,7 @@
 // into strips of about 16 columns, N x strips x Hq x Wq cells, so that a kernel row is a shift of 16 positions and not of a
 // whole row (3 -> 64 7x7 stride 2 at 224 x 224, batch 32: a region of 304 instead of 592 positions per 256 cells).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 namespace mnnb {
@@ -18,6 +19,13 @@ namespace mnnb {
 constexpr int kLineMaxTaps = 49, kLineMaxPlanes = 16, kLineMaxA = 4, kLineMaxB = 12;
 constexpr int kLineSmemBytes = 208 * 1024;
 constexpr int kLineMaxRegion = 1024;     // positions staged at a time
+
+// Cells of one axis: `out` outputs, `lead` zero cells in front, data cells end before `end`, taps reach `reach` cells past an
+// output.  The smallest pitch that lets the zero cells behind the data be the next line's leading ones.
+inline int axis_pitch(int out, int lead, int end, int reach)
+{
+    return std::max(out, std::min(out + reach, std::max(end, out + reach - lead)));
+}
 
 struct LineShape {
     int N, Cin, Cout, H, W, k, stride, dil, pad, OH, OW;

@@ -18,6 +18,7 @@
 #include <cstring>
 
 #include "contract_umma.h"
+#include "line_plan.h"
 #include "umma.cuh"
 
 namespace mnnb {
@@ -40,15 +41,6 @@ struct Params {
 
 // High word of the shared-memory descriptors: 8-row groups 512 bytes apart, version, 64-byte swizzle.
 constexpr uint32_t kDescHi = (512u >> 4) | (1u << 14) | (4u << 29);
-
-__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 
 template <int MT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -174,8 +166,8 @@ line_wino_kernel(const __grid_constant__ CUtensorMap map_v_hi, const __grid_cons
                             for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
                                 for (int m = 0; m < MT; ++m)
-                                    mma_lo(d0 + (uint32_t)(m * p.bn), a + (uint32_t)(m * 128 * (kRowBytes / 16) + ks * 2) + (pass == 1 ? a16 : 0u),
-                                           b + (uint32_t)(ks * 2) + (pass == 2 ? b16 : 0u), idesc, (pass | ks) ? 1u : accumulate);
+                                    ptx::mma_lo<1>(d0 + (uint32_t)(m * p.bn), a + (uint32_t)(m * 128 * (kRowBytes / 16) + ks * 2) + (pass == 1 ? a16 : 0u),
+                                           b + (uint32_t)(ks * 2) + (pass == 2 ? b16 : 0u), kDescHi, idesc, (pass | ks) ? 1u : accumulate);
                         ptx::mma_commit(ptx::smem_u32(&b_empty[bs]));
                     }
                     accumulate = 1u;
@@ -304,7 +296,7 @@ bool line_wino_plan(const LineWinoShape& s, int num_sms, LineWinoPlan* p)
     p->alpha = s.m + s.k - 1;
     if (p->alpha > 10 || s.k > 7) return false;
     const int reach = s.k - 1;
-    p->Hq = std::max(s.OH, std::min(s.OH + reach, std::max(s.H + s.pad, s.OH + reach - s.pad)));     // neighbours share their zero rows
+    p->Hq = axis_pitch(s.OH, s.pad, s.H + s.pad, reach);         // neighbours share their zero rows
     p->tiles_w = (int)cdiv(s.OW, s.m);
     p->T = (long long)s.N * p->Hq * p->tiles_w;
     p->cin_pad = (int)rup(s.Cin, 8);

@@ -55,21 +55,6 @@ struct RowsParams {
 // High word of the shared-memory descriptors: 8-row groups 256 bytes apart, version, 32-byte swizzle.
 constexpr uint32_t kDescHi = (256u >> 4) | (1u << 14) | (6u << 29);
 
-__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"
-        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
@@ -211,7 +196,7 @@ __global__ void __launch_bounds__(kRowsThreads<M>, 1) rows_conv_kernel(const __g
                 if (ptx::elect_one()) {
                     const uint32_t bar = ptx::smem_u32(&b_full[bs]);
                     ptx::mbar_expect_tx(bar, b_slot_bytes);
-                    bulk_load(b_base + bs * b_slot_bytes, src + (size_t)s * b_slot_bytes, b_slot_bytes, bar);
+                    ptx::bulk_load(b_base + bs * b_slot_bytes, src + (size_t)s * b_slot_bytes, b_slot_bytes, bar);
                 }
                 if (++bs == (uint32_t)p.b_slots) {
                     bs = 0;
@@ -261,7 +246,7 @@ __global__ void __launch_bounds__(kRowsThreads<M>, 1) rows_conv_kernel(const __g
                                     const uint32_t a = a_lo + (M == 1 ? (uint32_t)(t * p.tap_rows) * 2u : (uint32_t)(t * HL) * plane16) + (pass == 1 ? plane16 : 0u) + (uint32_t)mt * 256u;
                                     const uint32_t b = b_lo + (uint32_t)(t * HL + (pass == 2 ? 1 : 0)) * tile16;
                                     const uint32_t d = d0 + (uint32_t)(((M == 1 ? 0 : t) * MT + mt) * WIDE) * (uint32_t)p.bn;
-                                    mma_lo(d, a, b, MODE == 2 && pass == 0 ? idesc_wide : idesc, (pass || (M == 1 && t)) ? 1u : accumulate);
+                                    ptx::mma_lo<1>(d, a, b, kDescHi, MODE == 2 && pass == 0 ? idesc_wide : idesc, (pass || (M == 1 && t)) ? 1u : accumulate);
                                 }
                         ptx::mma_commit(ptx::smem_u32(&b_empty[bs]));
                     }
@@ -639,7 +624,11 @@ template <int KW, int MODE>
 RowsKernel rows_kernel_mode(const RowsPlan& p)
 {
     if (p.mt == 2) return rows_conv_kernel<1, KW, 2, MODE, false>;
-    return p.split > 1 ? rows_conv_kernel<1, KW, 1, MODE, true> : rows_conv_kernel<1, KW, 1, MODE, false>;
+    if constexpr (MODE != 3 || KW < 5)
+        if (p.split > 1) return rows_conv_kernel<1, KW, 1, MODE, true>;
+    if constexpr (MODE != 3 || KW < 7)
+        if (p.split == 1) return rows_conv_kernel<1, KW, 1, MODE, false>;
+    return nullptr;                                          // (no plan has it)
 }
 
 template <int KW>

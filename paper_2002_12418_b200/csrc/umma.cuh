@@ -191,6 +191,31 @@ __host__ __device__ constexpr uint32_t mma_idesc(int fmt, int M, int N, bool a_m
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// Contiguous bulk copy global -> shared memory of this CTA; completion counted in bytes on `bar`.
+__device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_smem),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// tcgen05.mma with both shared-memory descriptors given as their low words (start address) over one high word (stride between
+// 8-row groups, version, swizzle mode), so that an instruction costs the issuing thread one addition per operand.  KIND as below.
+template <int KIND>
+__device__ __forceinline__ void mma_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate)
+{
+#define MNNB_MMA_LO(NAME)                                                                                                  \
+    asm volatile(                                                                                                          \
+        "{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\t"                                                                      \
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\tsetp.ne.b32 p, %5, 0;\n\t"                                      \
+        "tcgen05.mma.cta_group::1.kind::" NAME " [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo),           \
+        "r"(desc_hi), "r"(idesc), "r"(accumulate)                                                                          \
+        : "memory")
+    if (KIND == 0) MNNB_MMA_LO("tf32");
+    else MNNB_MMA_LO("f16");
+#undef MNNB_MMA_LO
+}
+
 template <int KIND>   // 0 = tf32, 1 = bf16 (kind::f16)
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {

@@ -83,37 +83,12 @@ __host__ __device__ __forceinline__ uint32_t swz64(uint32_t row, uint32_t piece)
 
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Contiguous bulk copy global -> shared memory of this CTA; completion counted in bytes on `bar`.
-__device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_smem),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(taddr)
                  : "memory");
-}
-
-// tcgen05.mma kind::tf32 with both shared-memory descriptors given as their low words (start address) over a
-// common high word (stride between 8-row groups, version, swizzle mode).
-__device__ __forceinline__ void mma_tf32_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
-                                            uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t"
-        ".reg .b64 da, db;\n\t"
-        ".reg .pred p;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n\t"
-        "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // K-major operand of 64-byte rows, 64-byte swizzle: 8-row groups are 512 bytes apart.
@@ -207,7 +182,7 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                     const uint32_t bar = ptx::smem_u32(&u_full[slot]);
                     if (ptx::elect_one()) {
                         ptx::mbar_expect_tx(bar, kUSlotBytes);
-                        bulk_load(u_base + slot * kUSlotBytes, src + (size_t)c * kUSlotBytes, kUSlotBytes, bar);
+                        ptx::bulk_load(u_base + slot * kUSlotBytes, src + (size_t)c * kUSlotBytes, kUSlotBytes, bar);
                     }
                     if (++slot == kSlots) {
                         slot = 0;
@@ -261,7 +236,7 @@ fused_f2x2_3x3_kernel(const __grid_constant__ wino::MatBt2 Bt, MatAt4 At, FusedP
                             for (int ks = 0; ks < kKBlock / 8; ++ks)
 #pragma unroll
                                 for (int g = 0; g < kGroup; ++g)
-                                    mma_tf32_lo(d_t + g * kTiles, a_lo + g * (kUPosBytes >> 4) + ks * 2,
+                                    ptx::mma_lo<0>(d_t + g * kTiles, a_lo + g * (kUPosBytes >> 4) + ks * 2,
                                                 b_lo + g * (kVPosBytes >> 4) + ks * 2, kDescHi, idesc, ks != 0 ? 1u : acc0);
                             ptx::mma_commit(ptx::smem_u32(&u_empty[slot]));
                         }

@@ -92,3 +92,21 @@ def test_errors(torch):
             B.mnn_conv_plan_rect(*args, B.make_opts())
     with pytest.raises(B.MnnError):
         B.mnn_conv_plan_rect(1, 8, 8, 8, 8, 1, 7, 0, 3, B.make_opts(force_m=6))
+
+
+# 128-bit loads of the input transform at every tile size they are compiled for (rows of a multiple of four columns, padding that keeps the
+# size, hi + lo BF16), with channels off the 64 a block transforms and tiles off its 16; 64-bit ones at 1 x 7 and m = 2.
+@pytest.mark.parametrize("k,m,N,Cin,Cout,H,W", [(3, 4, 3, 70, 20, 5, 12), (3, 4, 1, 9, 33, 7, 4), (5, 4, 2, 66, 17, 6, 20), (7, 4, 2, 65, 24, 5, 16), (7, 2, 3, 70, 20, 7, 10)])
+def test_wide_loads_of_the_input_transform(torch, k, m, N, Cin, Cout, H, W):
+    x, w, b = make(N, Cin, Cout, H, W, 1, k, seed=k + m + H)
+    got, info = run_rect(torch, x, w, b, 0, k // 2, force_m=m, operand=B.OPERAND_BF16, passes=3)
+    assert info.m == m and rel_l2(got, oc.direct_conv_rect(x, w, b, 0, k // 2, True)) <= 1e-4      # F(4, 7): 8.5e-5
+
+
+# By rows the plan has no transform: m = 1, one launch, no V or M; alpha stays m + k - 1 = k.
+def test_info_of_a_plan_by_rows(torch):
+    x, w, b = make(4, 64, 64, 17, 17, 1, 7, seed=3)
+    got, info = run_rect(torch, x, w, b, 0, 3)
+    assert (info.algo, info.gemm_lhs, info.m, info.alpha) == (B.ALGO_GEMM, B.GEMM_LHS_ROWS, 1, 7)
+    assert (info.launches_per_run, info.v_bytes, info.m_bytes, info.passes) == (1, 0, 0, 3)
+    assert rel_l2(got, oc.direct_conv_rect(x, w, b, 0, 3, True)) <= 1e-5

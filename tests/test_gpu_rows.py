@@ -11,11 +11,10 @@ from tests.util import rel_l2, to_dev
 
 pytestmark = pytest.mark.gpu
 
-# hi + lo BF16 operands leave 2^-17 of each factor and drop lo * lo: 3 * 2^-17 of a product at most, half of that as a 2-norm over
-# many; F(2, 3) and the row-wise forms enlarge it by the norms of their matrices (2.4e-5 at most in fp64 simulation); one BF16
-# product 2 * 2^-9.
-BOUND = {"rows1": 2.3e-5, "rows2": 3e-5, "wise": 5e-5, "bf16": 4e-3}
-
+# The planner's own figures where it admits a form by them: F(2, 3) by rows 8 ppm, row-wise F(4, 5) and F(2, 7) 30, F(4, 3) 20.  The
+# definition with hi + lo operands is predicted at 4 to 5 ppm of an output tensor; with one output channel, or few channels, a
+# tensor's error strays to 7, so twice that.  One BF16 product: 2 * 2^-9.
+BOUND = {"rows1": 1e-5, "rows2": 8e-6, "wise": 3e-5, "wise3": 2e-5, "bf16": 4e-3}
 
 @pytest.fixture(scope="module")
 def torch():
@@ -48,7 +47,9 @@ def run(torch, shape, x, w, b, relu, cls=B.PREC_TF32, repeats=1):
     return ys[0].cpu().numpy(), info
 
 
-# (N, Cin, Cout, H, W, k, pad), one per kernel size, way of issuing the three products, tiles per item and CTAs per item
+# (N, Cin, Cout, H, W, k, pad); a shape at least per instantiation of the kernel by rows (kernel size, products and how they are issued, one or
+# two tiles per item or clusters: tests/test_planner_twin.py checks that), row-wise with one and several channel blocks, full and not, and
+# scalar, 64-bit and 128-bit loads; paddings up to more than k - 1, up to 860 input channels
 SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "rows1"), ((1, 200, 130, 8, 6, 2, 1), "rows1"), ((1, 256, 8, 26, 29, 2, 1), "rows1"),
           ((17, 16, 17, 33, 39, 2, 1), "rows1"), 
           ((1, 64, 100, 11, 10, 3, 1), "rows1"), ((9, 130, 1, 22, 30, 3, 2), "rows1"), ((1, 130, 64, 5, 17, 3, 1), "rows1"), ((2, 256, 33, 8, 9, 3, 0), "rows1"),
@@ -64,7 +65,13 @@ SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "row
           ((1, 256, 8, 37, 30, 3, 0), "rows2"), 
           # 3, 7, 12 and 13 stages shared out unevenly over clusters
           ((8, 44, 16, 12, 19, 7, 6), "rows1"), ((1, 112, 100, 10, 10, 3, 1), "rows1"), ((1, 186, 40, 10, 10, 3, 1), "rows1"), ((2, 200, 100, 6, 5, 3, 1), "bf16"),
-          ((17, 256, 1, 33, 31, 5, 2), "wise"), ((17, 256, 1, 18, 9, 7, 3), "wise"), ((17, 130, 1, 33, 38, 7, 0), "wise"), ((64, 128, 128, 28, 28, 5, 2), "wise")]
+          ((17, 256, 1, 33, 31, 5, 2), "wise"), ((17, 256, 1, 18, 9, 7, 3), "wise"), ((17, 130, 1, 33, 38, 7, 0), "wise"), ((64, 128, 128, 28, 28, 5, 2), "wise"),
+          ((39, 72, 17, 8, 4, 2, 1), "bf16"), ((19, 66, 56, 6, 5, 2, 1), "rows1"), ((36, 22, 1, 65, 45, 2, 1), "bf16"), ((5, 105, 57, 8, 5, 2, 1), "bf16"), ((2, 78, 10, 17, 108, 2, 0), "rows1"), ((39, 70, 1, 34, 31, 2, 0), "rows1"),
+          ((2, 186, 7, 7, 117, 2, 0), "rows1"), ((43, 26, 1, 37, 24, 3, 2), "bf16"), ((10, 8, 18, 51, 36, 3, 2), "rows1"), ((6, 45, 2, 16, 103, 3, 2), "rows1"),
+          ((2, 104, 6, 5, 94, 3, 2), "rows1"), ((21, 5, 68, 70, 9, 5, 4), "rows1"), ((5, 3, 264, 95, 5, 5, 4), "rows1"), ((55, 6, 8, 11, 45, 7, 0), "bf16"),
+          ((29, 6, 83, 7, 62, 7, 6), "rows1"), ((1, 512, 64, 7, 7, 3, 1), "rows1"), ((2, 40, 33, 12, 10, 5, 6), "rows1"), ((2, 48, 33, 14, 10, 3, 3), "rows1"),
+          ((28, 791, 1, 7, 21, 3, 4), "wise3"), ((16, 841, 667, 4, 6, 3, 4), "wise3"), ((7, 469, 29, 5, 39, 5, 6), "wise"), ((18, 323, 1, 14, 32, 5, 2), "wise"),
+          ((28, 59, 692, 14, 20, 5, 2), "wise"), ((5, 316, 434, 4, 4, 7, 8), "wise"), ((23, 160, 1, 10, 14, 7, 3), "wise"), ((22, 319, 136, 14, 6, 7, 3), "wise")]
 
 
 @pytest.mark.parametrize("shape,expected", SHAPES)
@@ -74,8 +81,14 @@ def test_against_the_oracle(torch, shape, expected):
     x, w, b = W.make_inputs(layer)
     cls = B.PREC_BF16 if expected == "bf16" else B.PREC_TF32
     got, info = run(torch, shape, x, w, b, True, cls, repeats=3)
-    assert form(info) == expected
-    assert rel_l2(got, oc.direct_conv(x, w, b, 1, pad, 1, 1, True)) <= BOUND[expected]
+    assert form(info) == expected.rstrip("3")
+    assert info.predicted_error_ppm * 1e-6 <= BOUND[expected]
+    if layer.direct_flops < 4e9:
+        ref = oc.direct_conv(x, w, b, 1, pad, 1, 1, True)
+    else:
+        at = np.random.default_rng(1).integers(0, got.size, 40000)
+        got, ref = got.ravel()[at], oc.direct_conv_at(x, w, b, at, 1, pad, 1, 1, True)
+    assert rel_l2(got, ref) <= BOUND[expected]
 
 
 # 1 x k and k x 1 kernels left to the plan take the same kernel: every kernel size, one tile and two per item, clusters, odd paddings.

@@ -417,6 +417,18 @@ def test_winograd_by_rows_replaces_winograd_only(shape):
     assert info.algo == B.ALGO_GEMM and info.workspace_bytes <= B.STATIC_WORKSPACE_BYTES
 
 
+def test_the_gpu_tests_reach_every_kernel_by_rows():
+    from tests.test_gpu_rows import SHAPES
+    got = set()
+    for s, expected in SHAPES:
+        if "wise" not in expected:
+            t = T.rows_tiling(T.Layer(*s[:6], 1, s[6], 1, 1), 2 if expected == "rows2" else 1, 1 if expected == "bf16" else 3, 148)
+            got.add((expected == "rows2", s[5], t["mode"], "two tiles" if t["mt"] == 2 else "cluster" if t["split"] > 1 else "one tile"))
+    want = {(False, k, mode, form) for k in (2, 3, 5, 7) for mode in (1, 2, 3) for form in ("one tile", "two tiles", "cluster")}
+    want -= {(False, 5, 3, "cluster"), (False, 7, 3, "cluster"), (False, 7, 3, "one tile")}      # not compiled
+    assert got == want | {(True, 3, 3, "one tile"), (True, 3, 3, "cluster")}
+
+
 # Few items share their stages out over clusters, unevenly too (7 over 4): cut in two only, the first two lost to three Winograd kernels.
 @pytest.mark.parametrize("shape,precision,split", [((1, 112, 112, 10, 10, 3, 1), B.PREC_TF32, 4), ((2, 111, 111, 9, 9, 3, 1), B.PREC_BF16, 4),
                                                    ((4, 96, 96, 5, 7, 3, 1), B.PREC_TF32, 4), ((1, 178, 178, 10, 10, 3, 1), B.PREC_BF16, 8),

@@ -196,7 +196,10 @@ MNN_API mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W,
  * the other axis: alpha = m + k - 1 transform positions) through the same tensor-core contraction.  opts as for
  * mnn_conv_plan_ex (relu, precision, operand, passes, force_m, points_id are read; force_m = 0 takes m = 4,
  * or 2 where m + k - 1 would pass 10; operand AUTO takes BF16 hi + lo under the TF32 accuracy class).
- * The plan is used with the same mnn_conv_* calls as any other; info.alpha is the number of transform positions. */
+ * Under the TF32 class, where none of force_algo, force_m, operand, passes, points_id, gemm_lhs and fused is given, the layer runs by
+ * rows instead where that is estimated faster: info reports MNN_ALGO_GEMM, MNN_GEMM_LHS_ROWS, BF16 hi + lo, m = 1, alpha = k (no
+ * transform positions; square plans by rows report 1), one launch, no V and no M, and the stages INPUT and OUTPUT do nothing.
+ * The plan is used with the same mnn_conv_* calls as any other. */
 MNN_API mnn_conv_plan_t mnn_conv_plan_rect(int N, int Cin, int Cout, int H, int W, int kh, int kw, int pad_h, int pad_w,
                                            const mnn_conv_opts* opts);
 

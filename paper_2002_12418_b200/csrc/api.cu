@@ -51,7 +51,8 @@ struct mnn_conv_plan_s {
     LayerShape s;
     mnn_conv_opts o;
     Decision d;
-    Decision d_static;               // for mnn_conv_run_static, where the workspace of packed lines or of a form by rows does not fit it
+    Decision d_plain;                // where d takes packed lines: the decision without them (mnn_conv_run_static)
+    Calibration cal;                 // what d was decided by
     int store_mode = STORE_TF32;
     int cin_pad = 0;                 // row length of U and V (Winograd: padded Cin; GEMM: padded Cin*k*k)
     long long chunk_tiles = 0;       // capacity of V / M in tiles (or GEMM columns)
@@ -361,6 +362,8 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
     const Calibration cal = current_calibration();
     if (cal.c[7] > 0) p->tiling_sms = (int)cal.c[7];
     int rc = plan_layer(s, o_plan, cal, FORMS_ALL, &p->d, &why);
+    if (rc == MNN_OK && p->d.gemm_lhs == MNN_GEMM_LHS_PACKED) rc = plan_layer(s, o_plan, cal, FORMS_PLAIN, &p->d_plain, &why);
+    p->cal = cal;
     if (rc == MNN_OK && p->strassen) {
         p->d.passes = o.passes;
         p->d.chosen = -1;
@@ -368,14 +371,6 @@ mnn_conv_plan_t mnn_conv_plan_ex(int N, int Cin, int Cout, int H, int W, int k, 
         p->d.error_ppm = accuracy_ppm(1, 1, 0, p->d.operand, p->d.passes);
     }
     if (rc == MNN_OK) rc = realise_decision(p, &why);
-    if (rc == MNN_OK && exceeds_static_workspace(p)) {
-        mnn_conv_plan_s t = *p;
-        for (int forms = FORMS_NO_ROWS; rc == MNN_OK && forms <= FORMS_PLAIN && exceeds_static_workspace(&t); ++forms) {
-            rc = plan_layer(s, o_plan, cal, forms, &t.d, &why);
-            if (rc == MNN_OK) rc = realise_decision(&t, &why);
-        }
-        p->d_static = t.d;
-    }
     if (rc != MNN_OK) {
         fail(rc, why);
         delete p;
@@ -1283,11 +1278,14 @@ extern "C" int mnn_conv_run_static(mnn_conv_plan_t p, const float* x, const floa
     // A private copy of the host-side plan whose workspace is the built-in array: the caller's
     // plan (its own workspace, prepared weights, profiling state) is left untouched.
     mnn_conv_plan_s local = *p;
-    if (exceeds_static_workspace(p)) {
-        // the layer as it is planned without these forms (the implicit gather stores the weights only, in fewer padded channels)
+    // Without the forms that do not fit: the implicit gather stores the weights only, in fewer padded channels.  Planned here for the forms by
+    // rows, whose weights alone seldom pass the limit (planning it ahead made 7 x 7 plans 152 -> 188 us).
+    for (int forms = FORMS_NO_ROWS; exceeds_static_workspace(&local); ++forms) {
         const char* why = "";
-        local.d = p->d_static;
-        const int rc = realise_decision(&local, &why);
+        int rc = MNN_OK;
+        if (p->packed) local.d = p->d_plain;
+        else rc = plan_layer(p->s, p->o, p->cal, forms, &local.d, &why);
+        if (rc == MNN_OK) rc = realise_decision(&local, &why);
         if (rc != MNN_OK) return fail(rc, why);
     }
     if (local.workspace_bytes > (long long)MNN_STATIC_WORKSPACE_BYTES)

@@ -163,7 +163,7 @@ line_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             }
         }
     } else if (warp <= MT) {
-        // ------------------------------ MMA issue: one thread per tile of 128 cells ------------------------------
+        // ------------------------------ MMA issue: one warp per tile of 128 cells ------------------------------
         {
             const uint32_t tile = (uint32_t)warp - 1u;
             const uint32_t idesc = ptx::mma_idesc(BF16 ? 1 : 2, 128, p.bn);

@@ -3,9 +3,10 @@
 // times the multiplications, but V and M are m / alpha as large ((alpha / m) times x and y instead of its square), and one
 // axis of rounding error less, which lets large kernels use BF16 hi + lo operands.
 //
-// Measured, three kernels: 5 x 5 128 channels 28 x 28 batch 64, F(4, 5): 18 + 43 + 20 us against 98 in two dimensions, error 2e-5
-// against 9e-5; 7 x 7, F(2, 7): 45 + 107 + 31 us against 208, error 2e-5 against 8e-5 (F(4, 7) takes 126 us, but with an
-// error of 9e-5).  The product reaches 0.75 of the tensor core's time: 128 x 128 x 16 instructions, 75 cycles each.
+// Measured, three kernels: 5 x 5 128 channels 28 x 28 batch 64, F(4, 5): 18 + 43 + 20 us against 98 in two dimensions; 7 x 7, F(2, 7):
+// 45 + 107 + 31 us against 208 (F(4, 7) takes 126 us for its product, but with an error of 9e-5).  Error against 64 bits over 27 random layers:
+// 1.5 to 1.6e-5 (3 x 3), 1.6 to 2.1e-5 (5 x 5), 1.8 to 2.7e-5 (7 x 7), at most 0.36 of the form each replaced.  The product reaches 0.75 of
+// the tensor core's time: 128 x 128 x 16 instructions, 75 cycles each.
 //
 // The product is the persistent pipeline of line_conv.cu over items (position xi, block of tiles, block of channels): a region of
 // 128 * mt + (k - 1) * tiles_w consecutive tiles x 32 channels, hi and lo, is staged once per block of channels in the 64-byte

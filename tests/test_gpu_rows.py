@@ -12,9 +12,10 @@ from tests.util import rel_l2, to_dev
 pytestmark = pytest.mark.gpu
 
 # The planner's own figures where it admits a form by them: F(2, 3) by rows 8 ppm, row-wise F(4, 5) and F(2, 7) 30, F(4, 3) 20.  The
-# definition with hi + lo operands is predicted at 4 to 5 ppm of an output tensor; with one output channel, or few channels, a
-# tensor's error strays to 7, so twice that.  One BF16 product: 2 * 2^-9.
+# definition: hi + lo BF16 operands leave 2^-17 of each factor and drop lo * lo, 3 * 2^-17 = 2.3e-5 of a product at most, as a 2-norm over
+# many terms of random sign a fifth of that (predicted 4 to 5 ppm; 7 with one output channel), so 1e-5.  One BF16 product: 2 * 2^-9.
 BOUND = {"rows1": 1e-5, "rows2": 8e-6, "wise": 3e-5, "wise3": 2e-5, "bf16": 4e-3}
+
 
 @pytest.fixture(scope="module")
 def torch():
@@ -49,7 +50,7 @@ def run(torch, shape, x, w, b, relu, cls=B.PREC_TF32, repeats=1):
 
 # (N, Cin, Cout, H, W, k, pad); a shape at least per instantiation of the kernel by rows (kernel size, products and how they are issued, one or
 # two tiles per item or clusters: tests/test_planner_twin.py checks that), row-wise with one and several channel blocks, full and not, and
-# scalar, 64-bit and 128-bit loads; paddings up to more than k - 1, up to 860 input channels
+# scalar, 64-bit and 128-bit loads; paddings up to more than k - 1, up to 841 input channels
 SHAPES = [((2, 100, 33, 8, 26, 2, 1), "rows1"), ((5, 130, 8, 26, 34, 2, 0), "rows1"), ((1, 200, 130, 8, 6, 2, 1), "rows1"), ((1, 256, 8, 26, 29, 2, 1), "rows1"),
           ((17, 16, 17, 33, 39, 2, 1), "rows1"), 
           ((1, 64, 100, 11, 10, 3, 1), "rows1"), ((9, 130, 1, 22, 30, 3, 2), "rows1"), ((1, 130, 64, 5, 17, 3, 1), "rows1"), ((2, 256, 33, 8, 9, 3, 0), "rows1"),
@@ -83,12 +84,7 @@ def test_against_the_oracle(torch, shape, expected):
     got, info = run(torch, shape, x, w, b, True, cls, repeats=3)
     assert form(info) == expected.rstrip("3")
     assert info.predicted_error_ppm * 1e-6 <= BOUND[expected]
-    if layer.direct_flops < 4e9:
-        ref = oc.direct_conv(x, w, b, 1, pad, 1, 1, True)
-    else:
-        at = np.random.default_rng(1).integers(0, got.size, 40000)
-        got, ref = got.ravel()[at], oc.direct_conv_at(x, w, b, at, 1, pad, 1, 1, True)
-    assert rel_l2(got, ref) <= BOUND[expected]
+    assert rel_l2(got, oc.direct_conv(x, w, b, 1, pad, 1, 1, True)) <= BOUND[expected]
 
 
 # 1 x k and k x 1 kernels left to the plan take the same kernel: every kernel size, one tile and two per item, clusters, odd paddings.
